@@ -1,4 +1,6 @@
-"""ctypes front end of the C-ABI library (``include/unionsparse.h``): argument marshalling only.
+"""Front end of the C-ABI library (``include/unionsparse.h``): argument marshalling only. Encoding and the host
+calls go through ctypes; the calls made per product go through a native module (``csrc/us_torch.cpp``), because
+marshalling them in Python takes longer than a small product takes on the GPU.
 
 Every step of the SpMM runs in the CUDA library; there is no CPU fallback. Importing this module
 fails loudly when the compiled library is missing (build it with ``python -m
@@ -12,9 +14,11 @@ from pathlib import Path
 import numpy as np
 
 _LIB_PATH = Path(__file__).resolve().parent / "libunionsparse.so"
-if not _LIB_PATH.exists():
-    raise ImportError(f"{_LIB_PATH} is missing: build the CUDA library first "
-                      "(python -m paper_2608_09291_b200.build)")
+_EXT_PATH = _LIB_PATH.with_name("_us_torch.so")
+for _p in (_LIB_PATH, _EXT_PATH):
+    if not _p.exists():
+        raise ImportError(f"{_p} is missing: build the CUDA library first "
+                          "(python -m paper_2608_09291_b200.build)")
 _lib = ctypes.CDLL(str(_LIB_PATH))
 
 US_OK = 0
@@ -73,6 +77,19 @@ class UsError(RuntimeError):
 def _check(status: int, where: str):
     if status != US_OK:
         raise UsError(status, where)
+
+
+_ext = None   # the native module: imported with the first tensor call, so that host-only use needs no torch
+
+
+def _native():
+    global _ext
+    if _ext is None:
+        import torch  # noqa: F401  (its libraries have to be loaded first)
+        from . import _us_torch
+        _us_torch.set_error(UsError)
+        _ext = _us_torch
+    return _ext
 
 
 def us_status_string(status: int) -> str:
@@ -233,14 +250,9 @@ def amax_values(buf, N: int):
 def absmax_f16(X16, out=None, stream=None):
     """Per-token absmax of a device float16 (N, K) tensor or view (unit column stride), as the
     absmax buffer the chained call takes."""
-    import torch
-    assert X16.dtype == torch.float16 and X16.stride(1) == 1
-    N, K = X16.shape
     if out is None:
         out = new_amax(X16.device)
-    if stream is None:
-        stream = torch.cuda.current_stream(X16.device).cuda_stream
-    us_absmax_f16(X16.data_ptr(), X16.stride(0), N, K, out.data_ptr(), stream)
+    (_ext or _native()).absmax_f16(X16, out, stream)
     return out
 
 
@@ -262,6 +274,7 @@ class SparseWeight:
 
     def __init__(self, W: np.ndarray, w_scale: np.ndarray | None = None, fmt: tuple | None = None,
                  max_N: int = 64, flags: int = 0):
+        _native()
         self.handle = us_encode(W, w_scale, fmt, max_N, flags)
         self.stats = us_get_stats(self.handle)
         self.M, self.K = self.stats["M"], self.stats["K"]
@@ -270,30 +283,14 @@ class SparseWeight:
     def spmm(self, X, N: int, x_scale=None, out=None, stream=None):
         """X: device uint8 tensor (N, ceil(K/2)); x_scale: device float16 (N,) or None.
         Returns a device tensor (N, M): int32, or float16 when x_scale is given."""
-        import torch
-        if out is None:
-            out = torch.empty((N, self.M), device=X.device,
-                              dtype=torch.float16 if x_scale is not None else torch.int32)
-        if stream is None:
-            stream = torch.cuda.current_stream(X.device).cuda_stream
-        us_spmm(self.handle, X.data_ptr(), N, x_scale.data_ptr() if x_scale is not None else None,
-                out.data_ptr(), stream)
-        return out
+        return _ext.spmm(self.handle, self.M, X, N, x_scale, out, stream)
 
     def spmm_requant(self, X16, N: int, x_amax, out=None, y_amax=None, amax_range=None, stream=None):
         """X16: device float16 tensor or view, (N, K) with unit column stride; x_amax: absmax buffer
         from absmax_f16 or an earlier call's y_amax. Returns the (N, M) float16 output; if y_amax
         (an absmax buffer) is given it receives the absmax of columns amax_range of the output."""
-        import torch
-        assert X16.dtype == torch.float16 and X16.stride(1) == 1 and X16.shape[1] == self.K
-        if out is None:
-            out = torch.empty((N, self.M), device=X16.device, dtype=torch.float16)
-        if stream is None:
-            stream = torch.cuda.current_stream(X16.device).cuda_stream
         m0, m1 = amax_range if amax_range is not None else (0, self.M)
-        us_spmm_requant(self.handle, X16.data_ptr(), X16.stride(0), x_amax.data_ptr(), N, out.data_ptr(),
-                        y_amax.data_ptr() if y_amax is not None else None, m0, m1, stream)
-        return out
+        return _ext.spmm_requant(self.handle, self.M, self.K, X16, N, x_amax, out, y_amax, m0, m1, stream)
 
     def check(self):
         st = us_last_error(self.handle)

@@ -1,43 +1,79 @@
-"""Builds the C-ABI shared library (in-tree) with nvcc for sm_100a."""
+"""Builds the native code in-tree: the C-ABI CUDA library (nvcc, sm_100a) and the Python front end on it."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
+import tempfile
+from concurrent.futures import ThreadPoolExecutor
 from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 LIB = PKG / "libunionsparse.so"
-SOURCES = [CSRC / "us_api.cu", CSRC / "us_encode.cpp"]
-HEADERS = [CSRC / "us_host.h", CSRC / "us_spmm_kernel.cuh", CSRC / "us_quant_kernels.cuh", PKG.parent / "include" / "unionsparse.h"]
+EXT = PKG / "_us_torch.so"
+# (source, extra flags, object): the kernels are one translation unit per N class, so that they build in parallel
+UNITS = [(CSRC / "us_api.cu", [], "us_api.o"), (CSRC / "us_encode.cpp", [], "us_encode.o")] + [
+    (CSRC / "us_kernels.cu", [f"-DUS_NT={nt}"], f"us_kernels_nt{nt}.o") for nt in (1, 2, 4, 8)]
+HEADERS = [CSRC / "us_host.h", CSRC / "us_launch.h", CSRC / "us_spmm_kernel.cuh", CSRC / "us_quant_kernels.cuh",
+           PKG.parent / "include" / "unionsparse.h"]
+EXT_SOURCE = CSRC / "us_torch.cpp"
 
 
-def nvcc_command(out: Path, verbose: bool = False) -> list[str]:
-    cmd = ["nvcc", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-           "-Xcompiler", "-fPIC,-O3,-Wall", "-shared", "-cudart", "shared"]
+def nvcc_flags(verbose: bool = False) -> list[str]:
+    cmd = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
+           "-Xcompiler", "-fPIC,-O3,-Wall", "-cudart", "shared"]
     if verbose:
         cmd += ["-Xptxas", "-v"]
-    cmd += os.environ.get("US_NVCC_FLAGS", "").split()
-    return cmd + [str(s) for s in SOURCES] + ["-o", str(out)]
+    return cmd + os.environ.get("US_NVCC_FLAGS", "").split()
+
+
+def ext_command(out: Path) -> list[str]:
+    import torch
+    from torch.utils import cpp_extension
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-Wall", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    cmd += [f"-I{p}" for p in cpp_extension.include_paths("cuda")] + [f"-I{sysconfig.get_paths()['include']}"]
+    cmd += [str(EXT_SOURCE), "-o", str(out)]
+    for p in cpp_extension.library_paths("cuda"):
+        cmd += [f"-L{p}", f"-Wl,-rpath,{p}"]
+    return cmd + [f"-L{PKG}", "-l:libunionsparse.so", "-Wl,-rpath,$ORIGIN", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda",
+                  "-ltorch", "-ltorch_python"]
+
+
+def _newest(paths) -> float:
+    return max(p.stat().st_mtime for p in paths)
 
 
 def is_stale() -> bool:
-    if not LIB.exists():
+    if not LIB.exists() or not EXT.exists():
         return True
-    t = LIB.stat().st_mtime
-    return any(p.stat().st_mtime > t for p in SOURCES + HEADERS)
+    return (LIB.stat().st_mtime < _newest([u[0] for u in UNITS] + HEADERS) or
+            EXT.stat().st_mtime < _newest([EXT_SOURCE, PKG.parent / "include" / "unionsparse.h"]))
+
+
+def _run(cmd: list[str], verbose: bool = False) -> None:
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose:
+        sys.stderr.write(r.stderr)
+    if r.returncode != 0:
+        raise RuntimeError(f"{cmd[0]} failed:\n" + r.stdout + r.stderr)
 
 
 def build(force: bool = False, verbose: bool = False) -> Path:
     if force or verbose or is_stale():
-        tmp = LIB.with_suffix(f".tmp{os.getpid()}.so")
-        r = subprocess.run(nvcc_command(tmp, verbose), capture_output=True, text=True)
-        if verbose:
-            sys.stderr.write(r.stderr)
-        if r.returncode != 0:
-            raise RuntimeError("nvcc failed:\n" + r.stdout + r.stderr)
-        os.replace(tmp, LIB)
+        with tempfile.TemporaryDirectory() as tmp, ThreadPoolExecutor(len(UNITS)) as pool:
+            objs = [str(Path(tmp) / o) for _, _, o in UNITS]
+            jobs = [pool.submit(_run, ["nvcc", *nvcc_flags(verbose), *flags, "-c", str(src), "-o", obj], verbose)
+                    for (src, flags, _), obj in zip(UNITS, objs)]
+            for j in jobs:
+                j.result()
+            new = LIB.with_suffix(f".tmp{os.getpid()}.so")
+            _run(["nvcc", *nvcc_flags(), "-shared", *objs, "-o", str(new)])
+            os.replace(new, LIB)
+        new = EXT.with_suffix(f".tmp{os.getpid()}.so")
+        _run(ext_command(new))
+        os.replace(new, EXT)
     return LIB
 
 

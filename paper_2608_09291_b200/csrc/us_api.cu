@@ -4,15 +4,31 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
 #include "us_host.h"
+#include "us_launch.h"
 #include "us_spmm_kernel.cuh"
 #include "us_quant_kernels.cuh"
 
+// How one N class is launched: fixed when the handle is made, so that a call is left with filling in its
+// pointers and launching.
+struct LaunchGeom {
+    int nt, cls, warps, stages, smem, lut_rep;
+    uint32_t slot_bytes;
+    bool xp;
+};
+struct ClassPlan {
+    bool ok = false;
+    LaunchGeom g{};
+    us::SpmmParams p{};   // everything but the call's pointers, N and the absmax range
+};
+
 struct us_handle {
     us::HostMatrix host;
+    ClassPlan plan[4];               // per N class (NT = 1, 2, 4, 8)
     bool on_device = false;
     int device = -1;
     int sm_count = 0;
@@ -65,12 +81,6 @@ constexpr int kLocalAccCap = 48 * 1024;      // ... and what is taken if nothing
 constexpr int kMinWarps = 12;                // warps the automatic K-range choice keeps room for
 constexpr int kCoresidentTiles = 16;         // most tiles per CTA for the half-SM plan
 constexpr int kHalfSmBytes = 228 * 1024 / 2 - 1024 - 512;   // shared memory of a half-SM CTA: 228 KB per SM, 1 KB reserved per CTA
-
-struct LaunchGeom {
-    int nt, cls, warps, stages, smem, lut_rep;
-    uint32_t slot_bytes;
-    bool xp;
-};
 
 // Segments per K range for an N class. The int8 activations of one K range live in shared memory
 // next to the warps' tile slots, so fewer, longer ranges (fewer partial-sum flushes) cost warps.
@@ -268,124 +278,6 @@ void plan_classes(us_handle* h, int n_cta, std::vector<uint32_t> (&sched)[4])
     }
 }
 
-template <int NT, int ST>
-cudaError_t launch_st(const us::SpmmParams& p, bool xp, int grid, int block, int smem, cudaStream_t st)
-{
-    // Launched with programmatic stream serialization: the kernel may start while its predecessor
-    // in the stream is still running; it waits (griddepcontrol.wait) before it touches anything
-    // an earlier kernel could produce or still use.
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = pdl_knob() ? 1 : 0;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const bool la = p.s_local > 0, timed = p.timers != nullptr;
-    if (p.w2)   // INT2 weights in folded tiles: plain kernels only (no packed X, timers or absmax)
-        return la ? cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<NT, ST, true, false, false, false, 2, true>, p)
-                  : cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<NT, ST, false, false, false, false, 2, true>, p);
-    if (p.fold_kb) {   // folded tiles (two column areas); stage timers for the N <= 8 kernels only
-        if (NT == 1 && timed && !xp)
-            return la ? cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<1, ST, true, true, false, false, 2>, p)
-                      : cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<1, ST, false, true, false, false, 2>, p);
-        if (NT <= 4 && xp && la) {
-            constexpr int NP = NT <= 4 ? NT : 4;
-            return cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<NP, ST, true, false, true, false, 2>, p);
-        }
-        return la ? cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<NT, ST, true, false, false, false, 2>, p)
-                  : cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<NT, ST, false, false, false, false, 2>, p);
-    }
-    if (p.y_amax) {   // chained call (never timed: enqueue_spmm leaves the timers off)
-        if (NT <= 4 && xp && la) {
-            constexpr int NP = NT <= 4 ? NT : 4;
-            return cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<NP, ST, true, false, true, true>, p);
-        }
-        return la ? cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<NT, ST, true, false, false, true>, p)
-                  : cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<NT, ST, false, false, false, true>, p);
-    }
-    if (NT <= 4 && xp && la) {   // packed X: planned for these classes and local mode only
-        constexpr int NP = NT <= 4 ? NT : 4;
-        return timed ? cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<NP, ST, true, true, true>, p)
-                     : cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<NP, ST, true, false, true>, p);
-    }
-    if (NT == 1 && p.N == 1 && !timed)   // a single token: dp4a beats the MMA (measured 2-3 %)
-        return la ? cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<1, ST, true, false, false, false, 1, false, true>, p)
-                  : cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<1, ST, false, false, false, false, 1, false, true>, p);
-    if (la && !timed) return cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<NT, ST, true, false>, p);
-    if (!la && !timed) return cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<NT, ST, false, false>, p);
-    if (la) return cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<NT, ST, true, true>, p);
-    return cudaLaunchKernelEx(&cfg, us::us_spmm_kernel<NT, ST, false, true>, p);
-}
-
-template <int NT>
-cudaError_t launch_nt(const us::SpmmParams& p, bool xp, int stages, int grid, int block, int smem, cudaStream_t st)
-{
-    return stages == 1 ? launch_st<NT, 1>(p, xp, grid, block, smem, st) : launch_st<NT, 2>(p, xp, grid, block, smem, st);
-}
-
-// Opt every kernel variant in to the device's full dynamic shared memory (once per handle, at
-// encode time, so that us_spmm itself is nothing but a launch).
-template <int NT, int ST>
-cudaError_t enable_large_smem_st(int bytes)
-{
-    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(us::us_spmm_kernel<NT, ST, true, false>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<NT, ST, false, false>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<NT, ST, true, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<NT, ST, false, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<NT, ST, true, false, false, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<NT, ST, false, false, false, true>, attr, bytes);
-    constexpr int NP = NT <= 4 ? NT : 4;   // packed-X kernels exist for N <= 32
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<NP, ST, true, false, true, true>, attr, bytes);
-    if (NT == 1) {   // single-token kernels
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<1, ST, true, false, false, false, 1, false, true>, attr, bytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<1, ST, false, false, false, false, 1, false, true>, attr, bytes);
-    }
-    // folded tiles, INT4 and INT2
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<NT, ST, true, false, false, false, 2, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<NT, ST, false, false, false, false, 2, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<NT, ST, true, false, false, false, 2>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<NT, ST, false, false, false, false, 2>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<NP, ST, true, false, true, false, 2>, attr, bytes);
-    if (NT == 1) {
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<1, ST, true, true, false, false, 2>, attr, bytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<1, ST, false, true, false, false, 2>, attr, bytes);
-    }
-    return e;
-}
-template <int NT>
-cudaError_t enable_large_smem_nt(int bytes)
-{
-    cudaError_t e = enable_large_smem_st<NT, 1>(bytes);
-    if (e == cudaSuccess) e = enable_large_smem_st<NT, 2>(bytes);
-    return e;
-}
-cudaError_t enable_large_smem(int bytes)
-{
-    cudaError_t e = enable_large_smem_nt<1>(bytes);
-    if (e == cudaSuccess) e = enable_large_smem_nt<2>(bytes);
-    if (e == cudaSuccess) e = enable_large_smem_nt<4>(bytes);
-    if (e == cudaSuccess) e = enable_large_smem_nt<8>(bytes);
-    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<2, 1, true, false, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<2, 2, true, false, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<2, 1, true, true, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<2, 2, true, true, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<1, 1, true, false, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<1, 2, true, false, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<1, 1, true, true, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<1, 2, true, true, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<4, 1, true, false, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<4, 2, true, false, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<4, 1, true, true, true>, attr, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(us::us_spmm_kernel<4, 2, true, true, true>, attr, bytes);
-    return e;
-}
-
 void free_device(us_handle* h)
 {
     cudaFree(h->d_blob); cudaFree(h->d_item_off);
@@ -415,25 +307,19 @@ us_status check_spmm_args(const us_handle* h, const void* X, int32_t N, const vo
     return US_OK;
 }
 
-// Fills the kernel parameters and launches: the one code path behind us_spmm and
-// us_spmm_static_scratch (they differ only in where the split-K scratch lives).
-// What a chained call adds to the plain one: the per-token absmax of a range of output rows, left
-// for the quantiser of the next call.
-struct ChainArgs {
-    void* y_amax = nullptr;
-    int64_t m0 = 0, m1 = 0;
-};
-
-us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_scale, void* Y, cudaStream_t st,
-                       int32_t* acc, uint32_t* cnt, bool timers, const ChainArgs* chain = nullptr)
+// Lays a class's launch down: geometry and every kernel parameter that no call changes.
+void build_plan(us_handle* h, int cls)
 {
-    LaunchGeom g;
-    if (!plan_launch(h, N, &g)) return US_ERR_UNSUPPORTED;
+    ClassPlan& pl = h->plan[cls];
+    LaunchGeom& g = pl.g;
+    pl.ok = plan_launch(h, 8 << cls, &g);
+    if (!pl.ok) return;
     const us::HostMatrix& hm = h->host;
-    us::SpmmParams p;
+    us::SpmmParams& p = pl.p;
+    std::memset(&p, 0, sizeof(p));
     p.blob = h->d_blob; p.item_off = h->d_item_off;
-    std::memcpy(p.cta_begin, h->cta_begin[g.cls].data(), h->cta_begin[g.cls].size() * sizeof(uint32_t));
-    p.G = h->G[g.cls]; p.s_local = h->s_local[g.cls]; p.lut_rep = g.lut_rep;
+    std::memcpy(p.cta_begin, h->cta_begin[cls].data(), h->cta_begin[cls].size() * sizeof(uint32_t));
+    p.G = h->G[cls]; p.s_local = h->s_local[cls]; p.lut_rep = g.lut_rep;
     {
         const int64_t n_kr = (hm.n_segs + p.G - 1) / p.G;
         const int64_t g_last = hm.n_segs - (n_kr - 1) * p.G;
@@ -452,21 +338,70 @@ us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_sca
         if ((hm.n_items + h->sm_count - 1) / std::max(1, h->sm_count) <= g.warps) p.run_len = 1;
     }
     p.row_order = h->d_row_order; p.w_scale = h->d_w_scale;
-    p.X = static_cast<const uint8_t*>(X);
-    p.x_scale = static_cast<const uint16_t*>(x_scale);
-    p.Y = Y; p.acc = acc; p.cnt = cnt; p.err = h->d_err;
-    // (no stage-timer builds of the absmax-tracking kernels, nor of the folded-tile kernels for N > 8 or with packed X:
-    // a timer build launched on a plan laid out for another variant would index shared memory wrongly)
-    p.timers = (timers && !(chain && chain->y_amax) && !(hm.fmt.C_A == 2 && (g.nt > 1 || g.xp)) && !hm.w2) ? h->d_timers : nullptr;
-    p.M = (int32_t)hm.M; p.K = (int32_t)hm.K; p.N = N;
+    p.err = h->d_err;
+    p.M = (int32_t)hm.M; p.K = (int32_t)hm.K;
     p.n_strips = (int32_t)hm.n_strips; p.n_segs = (int32_t)hm.n_segs;
     p.mask_rows = hm.mask_rows; p.K_L = hm.fmt.K_L;
     p.fold_kb = hm.fmt.C_A == 2 ? hm.nkb / 2 : 0;
     p.w2 = hm.w2 ? 1 : 0;
     p.slot_bytes = g.slot_bytes;
     p.x_fast = (hm.K % 32 == 0) ? 2 : (hm.K % 8 == 0) ? 1 : 0;
+}
+
+const void* kernel_for(int cls, const us::KernelKey& k)
+{
+    switch (cls) {
+        case 0: return us::kernel_nt1(k);
+        case 1: return us::kernel_nt2(k);
+        case 2: return us::kernel_nt4(k);
+        default: return us::kernel_nt8(k);
+    }
+}
+
+// Opt every kernel variant in to the device's full dynamic shared memory: once per device, when its first
+// handle is made, so that us_spmm itself is nothing but a launch.
+cudaError_t enable_large_smem(int device, int bytes)
+{
+    static std::mutex mu;
+    static std::vector<char> done;
+    std::lock_guard<std::mutex> lock(mu);
+    if (device < (int)done.size() && done[device]) return cudaSuccess;
+    for (int cls = 0; cls < 4; ++cls)
+        for (int bits = 0; bits < 256; ++bits) {
+            const us::KernelKey k{1 + (bits & 1), (bits & 2) != 0, (bits & 4) != 0, (bits & 8) != 0,
+                                  (bits & 16) != 0, (bits & 32) != 0, (bits & 64) != 0, (bits & 128) != 0};
+            const void* fn = kernel_for(cls, k);
+            if (!fn) continue;
+            const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+            if (e != cudaSuccess) return e;
+        }
+    if (device >= (int)done.size()) done.resize(device + 1, 0);
+    done[device] = 1;
+    return cudaSuccess;
+}
+
+// What a chained call adds to the plain one: the per-token absmax of a range of output rows, left
+// for the quantiser of the next call.
+struct ChainArgs {
+    void* y_amax = nullptr;
+    int64_t m0 = 0, m1 = 0;
+};
+
+// The one launch path behind us_spmm, us_spmm_static_scratch and us_spmm_requant: fills the call's own
+// parameters into a copy of the class's plan and launches.
+us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_scale, void* Y, cudaStream_t st,
+                       int32_t* acc, uint32_t* cnt, bool timers, const ChainArgs* chain = nullptr)
+{
+    const int cls = class_of(nt_for(N));
+    const ClassPlan& pl = h->plan[cls];
+    if (!pl.ok) return US_ERR_UNSUPPORTED;
+    const LaunchGeom& g = pl.g;
+    us::SpmmParams p = pl.p;
+    p.X = static_cast<const uint8_t*>(X);
+    p.x_scale = static_cast<const uint16_t*>(x_scale);
+    p.Y = Y; p.acc = acc; p.cnt = cnt;
+    p.N = N;
     p.fp16_out = x_scale ? 1 : 0;
-    p.y_amax = nullptr; p.amax_m0 = p.amax_m1 = 0;
     if (chain) {
         p.y_amax = static_cast<uint32_t*>(chain->y_amax);
         p.amax_m0 = (int32_t)chain->m0; p.amax_m1 = (int32_t)chain->m1;
@@ -474,13 +409,32 @@ us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_sca
     p.wait_ns_hi = h->wait_ns_hi;
     p.withhold = h->withhold;
 
-    cudaError_t e;
-    switch (g.nt) {
-        case 1: e = launch_nt<1>(p, g.xp, g.stages, h->sm_count, g.warps * 32, g.smem, st); break;
-        case 2: e = launch_nt<2>(p, g.xp, g.stages, h->sm_count, g.warps * 32, g.smem, st); break;
-        case 4: e = launch_nt<4>(p, g.xp, g.stages, h->sm_count, g.warps * 32, g.smem, st); break;
-        default: e = launch_nt<8>(p, g.xp, g.stages, h->sm_count, g.warps * 32, g.smem, st); break;
+    us::KernelKey k{g.stages, p.s_local > 0, timers, g.xp && p.s_local > 0, p.y_amax != nullptr, p.fold_kb != 0, p.w2 != 0, false};
+    // a single token: dp4a beats the MMA (measured 2-3 %)
+    k.dp = N == 1 && !k.timed && !k.xp && !k.am && !k.fold && !k.w2;
+    const void* fn = kernel_for(cls, k);
+    if (!fn && k.timed) {   // a variant without a timer build runs untimed
+        k.timed = false;
+        fn = kernel_for(cls, k);
     }
+    if (!fn) return US_ERR_UNSUPPORTED;
+    p.timers = k.timed ? h->d_timers : nullptr;
+
+    // Launched with programmatic stream serialization: the kernel may start while its predecessor
+    // in the stream is still running; it waits (griddepcontrol.wait) before it touches anything
+    // an earlier kernel could produce or still use.
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)h->sm_count);
+    cfg.blockDim = dim3((unsigned)g.warps * 32u);
+    cfg.dynamicSmemBytes = (size_t)g.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = pdl_knob() ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    void* args[1] = {&p};
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
     if (e != cudaSuccess) { h->sticky = e; return US_ERR_CUDA; }
     return US_OK;
 }
@@ -534,22 +488,22 @@ us_status us_encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_sca
         return US_OK;
     }
 
-    e = enable_large_smem(h->max_smem);
+    e = enable_large_smem(h->device, h->max_smem);
     if (e == cudaSuccess) {
         // Two N <= 8 CTAs share the SM's 64 K registers (allocated 8 per thread at a time).
         int regs = 0;
         // (the stage-timer builds need more and simply do not share an SM)
-        for (const void* fn : {(const void*)us::us_spmm_kernel<1, 1, true, false>, (const void*)us::us_spmm_kernel<1, 1, false, false>}) {
+        for (const bool local : {true, false}) {
             cudaFuncAttributes fa;
-            e = cudaFuncGetAttributes(&fa, fn);
+            e = cudaFuncGetAttributes(&fa, kernel_for(0, {1, local}));
             if (e != cudaSuccess) break;
             regs = std::max(regs, fa.numRegs);
         }
         if (e == cudaSuccess) h->co_warps = 32768 / (32 * ((regs + 7) / 8 * 8));
         cudaFuncAttributes fa2;
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa2, (const void*)us::us_spmm_kernel<2, 1, true, false, true>);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa2, kernel_for(1, {1, true, false, true}));
         if (e == cudaSuccess) h->co_warps2 = 32768 / (32 * ((fa2.numRegs + 7) / 8 * 8));
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa2, (const void*)us::us_spmm_kernel<1, 1, true, false, false, false, 2>);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa2, kernel_for(0, {1, true, false, false, false, true}));
         if (e == cudaSuccess) h->co_warps_fold = 32768 / (32 * ((fa2.numRegs + 7) / 8 * 8));
     }
     if (e != cudaSuccess) { delete h; return US_ERR_CUDA; }
@@ -580,8 +534,8 @@ us_status us_encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_sca
         return e == cudaErrorMemoryAllocation ? US_ERR_ALLOC : US_ERR_CUDA;
     }
     h->on_device = true;
-    LaunchGeom g;
-    if (!plan_launch(h, max_N, &g)) {  // a tile does not fit the shared-memory ring
+    for (int c = 0; c <= class_of(nt_max); ++c) build_plan(h, c);
+    if (!h->plan[class_of(nt_max)].ok) {  // a tile does not fit the shared-memory ring
         free_device(h);
         delete h;
         return US_ERR_UNSUPPORTED;

@@ -1,0 +1,24 @@
+// Which instantiation of us_spmm_kernel a launch needs. The kernels are compiled in one translation unit
+// per N class (us_kernels.cu with US_NT = 1, 2, 4, 8), so that they build in parallel.
+#pragma once
+
+namespace us {
+
+struct KernelKey {
+    int stages;        // ring slots per warp, 1 or 2
+    bool local;        // shared-memory strip sums
+    bool timed;        // stage-timer build
+    bool xp;           // activations staged packed
+    bool am;           // absmax of the output
+    bool fold;         // two column areas
+    bool w2;           // INT2 weights
+    bool dp;           // dp4a (a single token)
+};
+
+// The kernel for a key, or nullptr where no such variant is built.
+const void* kernel_nt1(const KernelKey& k);
+const void* kernel_nt2(const KernelKey& k);
+const void* kernel_nt4(const KernelKey& k);
+const void* kernel_nt8(const KernelKey& k);
+
+}  // namespace us
