@@ -11,6 +11,7 @@
 #include "us_host.h"
 #include "us_launch.h"
 #include "us_spmm_kernel.cuh"
+#include "us_spmm_tc.cuh"
 #include "us_quant_kernels.cuh"
 
 // How one N class is launched: fixed when the handle is made, so that a call is left with filling in its
@@ -26,8 +27,16 @@ struct ClassPlan {
     us::SpmmParams p{};   // everything but the call's pointers, N and the absmax range
 };
 
+// The same for us_spmm_tc_kernel, per number of 8-token groups.
+struct TcPlan {
+    bool ok = false;
+    int smem = 0;
+    us::TcParams p{};
+};
+
 struct us_handle {
     us::HostMatrix host;
+    TcPlan tc[9];                    // index: 8-token groups of the call
     ClassPlan plan[4];               // per N class (NT = 1, 2, 4, 8)
     bool on_device = false;
     int device = -1;
@@ -75,6 +84,7 @@ int pdl_knob() { static int v = env_int("US_PDL", 1); return v; }          // pr
 int stages_knob() { static int v = env_int("US_STAGES", 0); return v; }    // ring slots per warp, 0 = automatic
 // (up to 20 for the N <= 8 kernels; the other kernels are compiled for 16)
 int max_warps() { static int v = std::min(20, std::max(2, env_int("US_MAX_WARPS", 16))); return v; }
+int tc_knob() { static int v = env_int("US_TC", 1); return v; }   // tensor-memory kernel: 0 never, 1 by rule, 2 wherever it can run
 int coresident_knob() { static int v = env_int("US_CORESIDENT", 1); return v; }  // small problems: half an SM per CTA
 constexpr int kLocalAccBudget = 32 * 1024;   // local strip sums a K-range width is chosen with
 constexpr int kLocalAccCap = 48 * 1024;      // ... and what is taken if nothing fits that
@@ -348,6 +358,58 @@ void build_plan(us_handle* h, int cls)
     p.x_fast = (hm.K % 32 == 0) ? 2 : (hm.K % 8 == 0) ? 1 : 0;
 }
 
+// Lays a launch of us_spmm_tc_kernel down for calls of `ng` 8-token groups.
+void build_tc_plan(us_handle* h, int ng)
+{
+    TcPlan& pl = h->tc[ng];
+    pl.ok = false;
+    const us::HostMatrix& hm = h->host;
+    if (ng < 2) return;
+    us::TcParams& p = pl.p;
+    std::memset(&p, 0, sizeof(p));
+    const int64_t n_cta = h->sm_count;
+    const int n_stage = hm.fmt.C_A == 1 ? (hm.mask_rows + 1) / 2 : hm.mask_rows;   // 256-column stages per tile
+    const int64_t block_stages = hm.n_segs * n_stage, stages = (hm.n_strips + 15) / 16 * block_stages;
+    if (block_stages >= (1 << 16) || stages >= (1 << 24)) return;   // exact division by multiplication
+    // Where it is chosen. The kernel saves the X fragments, MMAs and split-K adds of every tile, and pays a longer
+    // prologue and a flush through the workspace per CTA (4 to 5 us together at N = 64). Against a plan that sums strips
+    // in shared memory it needs so many stages per CTA to win (measured at s = .5, us, that plan / this kernel: N = 16
+    // 13824 x 5120, 7 stages, 13.0 / 14.0, 28672 x 8192, 24 stages, 32.4 / 28.8; N = 32 4096 x 11008, 4.6 stages, sorted
+    // rows, 15.5 / 16.1, 13824 x 5120 18.8 / 17.0; N = 64 4096 x 4096, 1.7 stages, 14.4 / 17.3); against the direct
+    // mode it wins nearly always (N = 32 on 2 x 2 tiles 5120 x 5120 14.9 / 13.2; N = 64 4096 x 4096 with INT2 weights
+    // 21.8 / 16.5, 28672 x 8192 92 / 41, 8192 x 28672 83 / 41).
+    const bool sums_local = h->s_local[class_of(nt_for(8 * ng))] > 0;
+    const int64_t min_stages = !sums_local ? 3 * n_cta / 2 : (ng <= 2 ? 16 : ng <= 4 ? 6 : 4) * n_cta;
+    if (tc_knob() == 0 || (tc_knob() == 1 && stages < min_stages)) return;
+    p.slot_bytes = slot_bytes_for(hm);
+    const int limit = h->max_smem > 0 ? h->max_smem : 227 * 1024;
+    auto fixed_for = [&](int x_stages, int lut_rep) { return 256 * lut_rep * 4 + x_stages * ng * 2048 + 2048 + us::kTcFixedSmem; };
+    auto slots_for = [&](int x_stages, int lut_rep) {
+        return std::min(us::kTcMaxSlots, (limit - fixed_for(x_stages, lut_rep)) / (int)p.slot_bytes);
+    };
+    // tiles of a warp: a CTA's stages may begin and end inside a tile
+    const int64_t per_cta = (stages + n_cta - 1) / n_cta, tiles = (per_cta + n_stage - 1) / n_stage + (n_stage > 1 ? 1 : 0);
+    const int want = (int)std::min<int64_t>(24, 16 * tiles);   // slots worth having before the table gets its 32 copies
+    p.x_stages = 4;
+    while (p.x_stages > 2 && slots_for(p.x_stages, 8) < 16) --p.x_stages;
+    p.lut_rep = slots_for(p.x_stages, 32) >= want && per_cta >= 16 ? 32 : 8;
+    p.n_slots = std::min<int>(slots_for(p.x_stages, p.lut_rep), (int)(16 * tiles));
+    if (p.n_slots < 16) return;
+    pl.smem = fixed_for(p.x_stages, p.lut_rep) + p.n_slots * (int)p.slot_bytes;
+    for (int64_t c = 0; c <= n_cta; ++c) p.cta_begin[c] = (uint32_t)(stages * c / n_cta);
+    p.n_stage = n_stage; p.block_stages = (int32_t)block_stages;
+    p.mg_block = ((1ull << 40) / (uint64_t)block_stages) + 1ull;
+    p.blob = h->d_blob; p.item_off = h->d_item_off; p.row_order = h->d_row_order; p.w_scale = h->d_w_scale;
+    p.err = h->d_err;
+    p.M = (int32_t)hm.M; p.K = (int32_t)hm.K;
+    p.n_strips = (int32_t)hm.n_strips; p.n_segs = (int32_t)hm.n_segs;
+    p.mg_segs = ((1ull << 40) / (uint64_t)hm.n_segs) + 1ull;
+    p.mask_rows = hm.mask_rows; p.K_L = hm.fmt.K_L;
+    p.acc_nt = nt_for(8 * ng);
+    p.x_fast = hm.K % 32 == 0;
+    pl.ok = true;
+}
+
 const void* kernel_for(int cls, const us::KernelKey& k)
 {
     switch (cls) {
@@ -375,6 +437,11 @@ cudaError_t enable_large_smem(int device, int bytes)
             const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
             if (e != cudaSuccess) return e;
         }
+    for (int bits = 0; bits < 8; ++bits)
+        if (const void* fn = us::kernel_tc((bits & 1) != 0, (bits & 2) != 0, (bits & 4) != 0)) {
+            const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+            if (e != cudaSuccess) return e;
+        }
     if (device >= (int)done.size()) done.resize(device + 1, 0);
     done[device] = 1;
     return cudaSuccess;
@@ -387,11 +454,50 @@ struct ChainArgs {
     int64_t m0 = 0, m1 = 0;
 };
 
+us_status launch(us_handle* h, const void* fn, void* params, int threads, int smem, cudaStream_t st)
+{
+    // Launched with programmatic stream serialization: the kernel may start while its predecessor
+    // in the stream is still running; it waits (griddepcontrol.wait) before it touches anything
+    // an earlier kernel could produce or still use.
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)h->sm_count);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = pdl_knob() ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    void* args[1] = {params};
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
+    if (e != cudaSuccess) { h->sticky = e; return US_ERR_CUDA; }
+    return US_OK;
+}
+
 // The one launch path behind us_spmm, us_spmm_static_scratch and us_spmm_requant: fills the call's own
 // parameters into a copy of the class's plan and launches.
 us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_scale, void* Y, cudaStream_t st,
                        int32_t* acc, uint32_t* cnt, bool timers, const ChainArgs* chain = nullptr)
 {
+    const TcPlan& tc = h->tc[(N + 7) / 8];
+    if (tc.ok) {
+        us::TcParams p = tc.p;
+        p.X = static_cast<const uint8_t*>(X);
+        p.x_scale = static_cast<const uint16_t*>(x_scale);
+        p.Y = Y; p.acc = acc; p.cnt = cnt;
+        p.N = N;
+        p.fp16_out = x_scale ? 1 : 0;
+        if (chain) {
+            p.y_amax = static_cast<uint32_t*>(chain->y_amax);
+            p.amax_m0 = (int32_t)chain->m0; p.amax_m1 = (int32_t)chain->m1;
+        }
+        p.wait_ns_hi = h->wait_ns_hi;
+        p.withhold = h->withhold;
+        const void* fn = us::kernel_tc(h->host.fmt.C_A == 2, h->host.w2, p.y_amax != nullptr);
+        if (!fn) return US_ERR_UNSUPPORTED;
+        return launch(h, fn, &p, us::kTcThreads, tc.smem, st);
+    }
     const int cls = class_of(nt_for(N));
     const ClassPlan& pl = h->plan[cls];
     if (!pl.ok) return US_ERR_UNSUPPORTED;
@@ -420,23 +526,7 @@ us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_sca
     if (!fn) return US_ERR_UNSUPPORTED;
     p.timers = k.timed ? h->d_timers : nullptr;
 
-    // Launched with programmatic stream serialization: the kernel may start while its predecessor
-    // in the stream is still running; it waits (griddepcontrol.wait) before it touches anything
-    // an earlier kernel could produce or still use.
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)h->sm_count);
-    cfg.blockDim = dim3((unsigned)g.warps * 32u);
-    cfg.dynamicSmemBytes = (size_t)g.smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = pdl_knob() ? 1 : 0;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    void* args[1] = {&p};
-    const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
-    if (e != cudaSuccess) { h->sticky = e; return US_ERR_CUDA; }
-    return US_OK;
+    return launch(h, fn, &p, g.warps * 32, g.smem, st);
 }
 
 }  // namespace
@@ -535,6 +625,7 @@ us_status us_encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_sca
     }
     h->on_device = true;
     for (int c = 0; c <= class_of(nt_max); ++c) build_plan(h, c);
+    for (int ng = 1; ng <= (max_N + 7) / 8; ++ng) build_tc_plan(h, ng);
     if (!h->plan[class_of(nt_max)].ok) {  // a tile does not fit the shared-memory ring
         free_device(h);
         delete h;
@@ -574,6 +665,12 @@ us_status us_launch_info(const us_handle* h, int32_t N, int32_t* grid, int32_t* 
 {
     if (!h || N < 1 || N > h->max_N) return US_ERR_INVALID_ARG;
     if (!h->host.kernel_layout) return US_ERR_UNSUPPORTED;
+    if (h->tc[(N + 7) / 8].ok) {
+        if (grid) *grid = h->sm_count;
+        if (block) *block = us::kTcThreads;
+        if (smem_bytes) *smem_bytes = h->tc[(N + 7) / 8].smem;
+        return US_OK;
+    }
     LaunchGeom g;
     if (!plan_launch(h, N, &g)) return US_ERR_UNSUPPORTED;
     if (grid) *grid = h->sm_count > 0 ? h->sm_count : 148;

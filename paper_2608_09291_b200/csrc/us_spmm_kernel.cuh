@@ -364,7 +364,7 @@ struct ScalePre {
 // AM: also track the per-token absmax of the stored fp16 values (chained calls).
 template <int NT, bool AM>
 __device__ __forceinline__ void store_rows(const StoreCtx p, const int (&v)[NT][4], int lane, int m_lo, int m_hi,
-                                           const ScalePre<NT>* pre = nullptr, int rb = -2)
+                                           const ScalePre<NT>* pre = nullptr, int rb = -2, int n_base = 0)
 {
     const int t2 = (lane & 3) * 2;
     float sw_lo = 0.f, sw_hi = 0.f;
@@ -383,7 +383,7 @@ __device__ __forceinline__ void store_rows(const StoreCtx p, const int (&v)[NT][
         uint32_t big[2] = {0u, 0u};   // absmax (fp16 bits) of this lane's stored values of tokens t2, t2 + 1
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int n = nt * 8 + t2 + (j & 1);
+            const int n = n_base + nt * 8 + t2 + (j & 1);
             const int m = (j < 2) ? m_lo : m_hi;
             if (n >= p.N || m < 0) continue;
             const size_t o = (size_t)n * p.M + m;
@@ -406,7 +406,7 @@ __device__ __forceinline__ void store_rows(const StoreCtx p, const int (&v)[NT][
                 b = max(b, __shfl_xor_sync(0xffffffffu, b, 4));
                 b = max(b, __shfl_xor_sync(0xffffffffu, b, 8));
                 b = max(b, __shfl_xor_sync(0xffffffffu, b, 16));
-                if (lane < 4 && b) atomicMax(p.amax_s + nt * 8 + t2 + jj, b);
+                if (lane < 4 && b) atomicMax(p.amax_s + n_base + nt * 8 + t2 + jj, b);
             }
         }
     }
