@@ -95,7 +95,8 @@ typedef struct us_handle us_handle;
 
 /*
  * Offline encoder (paper Sec. V-A, Fig. 7: dense pruned INT4 -> union bitmaps, per-tile
- * offsets, packed INT4 values), followed by the upload to the current CUDA device.
+ * offsets, packed INT4 values), on the current CUDA device: the host packs the weight to INT4 and
+ * uploads it, kernels build the tiles (US_ENCODE_HOST_ONLY: all on the host).
  *   W        host, M x K row-major int8, values in [-8, 7], 0 = pruned. Not retained.
  *   w_scale  host, M fp16 bit patterns (per-output-channel scales), or NULL when only INT32
  *            output will be requested. Not retained.
@@ -113,8 +114,8 @@ us_status us_encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_sca
 us_status us_get_stats(const us_handle* h, us_stats* out);
 
 /*
- * Test hook: exact inverse of the encoder, from the handle's host copy of the encoded arrays
- * (paper Sec. V-A read backwards). W_out: host, M x K int8.
+ * Test hook: exact inverse of the encoder, from the encoded arrays themselves (fetched from the
+ * device where that is where they were encoded; paper Sec. V-A read backwards). W_out: host, M x K int8.
  */
 us_status us_decode(const us_handle* h, int8_t* W_out);
 

@@ -15,9 +15,10 @@ LIB = PKG / "libunionsparse.so"
 EXT = PKG / "_us_torch.so"
 # (source, extra flags, object): the kernels are one translation unit per N class, so that they build in parallel
 UNITS = [(CSRC / "us_api.cu", [], "us_api.o"), (CSRC / "us_encode.cpp", [], "us_encode.o"),
-         (CSRC / "us_spmm_tc.cu", [], "us_spmm_tc.o")] + [
+         (CSRC / "us_load.cu", [], "us_load.o"), (CSRC / "us_spmm_tc.cu", [], "us_spmm_tc.o")] + [
     (CSRC / "us_kernels.cu", [f"-DUS_NT={nt}"], f"us_kernels_nt{nt}.o") for nt in (1, 2, 4, 8)]
-HEADERS = [CSRC / "us_host.h", CSRC / "us_launch.h", CSRC / "us_spmm_kernel.cuh", CSRC / "us_spmm_tc.cuh", CSRC / "us_quant_kernels.cuh",
+HEADERS = [CSRC / "us_host.h", CSRC / "us_launch.h", CSRC / "us_load.h", CSRC / "us_device_encode.cuh",
+           CSRC / "us_spmm_kernel.cuh", CSRC / "us_spmm_tc.cuh", CSRC / "us_quant_kernels.cuh",
            PKG.parent / "include" / "unionsparse.h"]
 EXT_SOURCE = CSRC / "us_torch.cpp"
 

@@ -10,6 +10,7 @@
 
 #include "us_host.h"
 #include "us_launch.h"
+#include "us_load.h"
 #include "us_spmm_kernel.cuh"
 #include "us_spmm_tc.cuh"
 #include "us_quant_kernels.cuh"
@@ -249,7 +250,7 @@ void plan_classes(us_handle* h, int n_cta, std::vector<uint32_t> (&sched)[4])
         if (nt <= 4 && !h->host.w2) {   // (no packed-X kernel for INT2 weights)
             const int64_t n_segs = h->host.n_segs;
             const int64_t ranges = h->s_local[c] > 0 ? (n_segs + h->G[c] - 1) / h->G[c] : n_segs + 1;
-            const bool small_share = nt >= 2 && (int64_t)h->host.blob.size() / std::max(1, n_cta) < 128 * 1024;
+            const bool small_share = nt >= 2 && (int64_t)h->host.blob_bytes / std::max(1, n_cta) < 128 * 1024;
             // N <= 8: packed X when that is what lets the half-SM plan of plan_launch hold its eight warps
             // (4096 x 4096 at 30 % sparsity: tiles of 9.5 KB and 32 KB of int8 X do not fit half an SM, with
             // 16 KB of packed X they do: 5.6 -> 4.6 us; the same for the folded format at 50 %: 5.3 -> 4.35)
@@ -288,21 +289,20 @@ void plan_classes(us_handle* h, int n_cta, std::vector<uint32_t> (&sched)[4])
     }
 }
 
+// Gives the handle's device memory back, with its device current. Work that still uses it may be in flight on any
+// stream: wait for it first, as cudaFree did.
 void free_device(us_handle* h)
 {
-    cudaFree(h->d_blob); cudaFree(h->d_item_off);
-    cudaFree(h->d_row_order); cudaFree(h->d_w_scale); cudaFree(h->d_acc);
-    cudaFree(h->d_cnt); cudaFree(h->d_err); cudaFree(h->d_timers); cudaFree(h->d_xq);
+    int dev = -1;
+    cudaGetDevice(&dev);
+    if (dev != h->device) cudaSetDevice(h->device);
+    cudaDeviceSynchronize();
+    for (void* p : {(void*)h->d_blob, (void*)h->d_item_off, (void*)h->d_row_order, (void*)h->d_w_scale, (void*)h->d_acc,
+                    (void*)h->d_cnt, (void*)h->d_err, (void*)h->d_xq})
+        us::pool_free(h->device, p);
+    cudaFree(h->d_timers);
+    if (dev != h->device && dev >= 0) cudaSetDevice(dev);
 }
-
-template <class T>
-cudaError_t upload(T** dst, const void* src, size_t bytes)
-{
-    cudaError_t e = cudaMalloc((void**)dst, std::max<size_t>(bytes, 16));
-    if (e != cudaSuccess) return e;
-    return bytes ? cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) : cudaSuccess;
-}
-
 
 // Argument checks shared by the two SpMM entry points.
 us_status check_spmm_args(const us_handle* h, const void* X, int32_t N, const void* x_scale, const void* Y)
@@ -554,8 +554,18 @@ us_status us_encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_sca
     const int n_cta = h->sm_count > 0 ? h->sm_count : 148;   // host-only handles plan for a 148-SM part
     us_format f = fmt ? *fmt : us_format{16, us::default_K_L(M, K, n_cta), 2, 1};
     us_status s;
+    us::DeviceMatrix dm;
+    // the kernel's index arithmetic (exact division by multiplication) needs u * d < 2^40 for every
+    // position u < n_items and divisor d <= n_items
+    auto too_many = [&] { return h->host.n_items >= (1 << 20) || h->host.n_segs >= (1 << 16); };
     try {
-        s = us::encode_host(W, M, K, w_scale, f, flags, 0, &h->host);
+        if (host_only) {
+            s = us::encode_host(W, M, K, w_scale, f, flags, 0, &h->host);
+        } else {
+            s = us::encode_layout(W, M, K, w_scale, f, flags, 0, true, &h->host);
+            if (s == US_OK && too_many()) s = US_ERR_UNSUPPORTED;
+            if (s == US_OK) s = us::encode_device(W, h->device, flags, &h->host, &dm);
+        }
     } catch (const std::bad_alloc&) {
         s = US_ERR_ALLOC;
     }
@@ -565,9 +575,7 @@ us_status us_encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_sca
         *out = h;
         return US_OK;
     }
-    // the kernel's index arithmetic (exact division by multiplication) needs u * d < 2^40 for every
-    // position u < n_items and divisor d <= n_items
-    if (hm.n_items >= (1 << 20) || hm.n_segs >= (1 << 16)) {
+    if (too_many()) {
         delete h;
         return US_ERR_UNSUPPORTED;
     }
@@ -577,6 +585,7 @@ us_status us_encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_sca
         *out = h;
         return US_OK;
     }
+    h->d_blob = dm.blob; h->d_item_off = dm.item_off; h->d_row_order = dm.row_order;
 
     e = enable_large_smem(h->device, h->max_smem);
     if (e == cudaSuccess) {
@@ -596,27 +605,30 @@ us_status us_encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_sca
         if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa2, kernel_for(0, {1, true, false, false, false, true}));
         if (e == cudaSuccess) h->co_warps_fold = 32768 / (32 * ((fa2.numRegs + 7) / 8 * 8));
     }
-    if (e != cudaSuccess) { delete h; return US_ERR_CUDA; }
+    if (e != cudaSuccess) { free_device(h); delete h; return US_ERR_CUDA; }
 
     const int nt_max = nt_for(max_N);
     h->acc_bytes = (size_t)hm.n_strips * nt_max * 128 * sizeof(int32_t);
     h->cnt_bytes = (size_t)hm.n_strips * sizeof(uint32_t);
-    e = upload(&h->d_blob, hm.blob.data(), hm.blob.size());
-    if (e == cudaSuccess) e = upload(&h->d_item_off, hm.item_off.data(), hm.item_off.size() * 4);
     for (int c = 0; c < 4; ++c) h->cta_begin[c] = sched[c];
-    if (e == cudaSuccess) e = upload(&h->d_row_order, hm.row_order.data(), hm.row_order.size() * 4);
-    if (e == cudaSuccess && !hm.w_scale.empty()) e = upload(&h->d_w_scale, hm.w_scale.data(), hm.w_scale.size() * 2);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_acc, h->acc_bytes);
-    if (e == cudaSuccess) e = cudaMemset(h->d_acc, 0, h->acc_bytes);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_cnt, h->cnt_bytes);
-    if (e == cudaSuccess) e = cudaMemset(h->d_cnt, 0, h->cnt_bytes);
-    if (e == cudaSuccess && !hm.w_scale.empty()) {   // chained calls need fp16 output, hence weight scales
+    cudaStream_t ps = us::pool_stream(h->device);
+    auto alloc = [&](auto** p, size_t bytes) {
+        if (e == cudaSuccess) e = us::pool_alloc(h->device, (void**)p, bytes);
+    };
+    auto clear = [&](void* p, size_t bytes) {
+        if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, bytes, ps);
+    };
+    if (!hm.w_scale.empty()) {
+        alloc(&h->d_w_scale, hm.w_scale.size() * 2);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_w_scale, hm.w_scale.data(), hm.w_scale.size() * 2, cudaMemcpyHostToDevice, ps);
+        // chained calls need fp16 output, hence weight scales
         h->xq_bytes = (((size_t)max_N * (size_t)((hm.K + 1) / 2)) + 255) & ~(size_t)255;
-        e = cudaMalloc((void**)&h->d_xq, h->xq_bytes + 256);
+        alloc(&h->d_xq, h->xq_bytes + 256);
     }
-    if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_err, 16);
-    if (e == cudaSuccess) e = cudaMemset(h->d_err, 0, 16);
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    alloc(&h->d_acc, h->acc_bytes); clear(h->d_acc, h->acc_bytes);
+    alloc(&h->d_cnt, h->cnt_bytes); clear(h->d_cnt, h->cnt_bytes);
+    alloc(&h->d_err, 16); clear(h->d_err, 16);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ps);
     if (e != cudaSuccess) {
         free_device(h);
         delete h;
@@ -645,6 +657,18 @@ us_status us_get_stats(const us_handle* h, us_stats* out)
 us_status us_decode(const us_handle* h, int8_t* W_out)
 {
     if (!h || !W_out) return US_ERR_INVALID_ARG;
+    if (h->on_device && h->host.blob.empty()) {   // encoded on the GPU: fetch the tiles first
+        us::HostMatrix& host = const_cast<us_handle*>(h)->host;
+        try {
+            host.blob.resize((size_t)host.blob_bytes);
+        } catch (const std::bad_alloc&) {
+            return US_ERR_ALLOC;
+        }
+        if (cudaMemcpy(host.blob.data(), h->d_blob, host.blob.size(), cudaMemcpyDeviceToHost) != cudaSuccess) {
+            host.blob.clear();
+            return US_ERR_CUDA;
+        }
+    }
     us::decode_host(h->host, W_out);
     return US_OK;
 }

@@ -3,6 +3,8 @@
 // schedule. Pure C++: no CUDA here.
 #include <algorithm>
 #include <climits>
+#include <immintrin.h>
+
 #include <atomic>
 #include <cstdlib>
 #include <cstring>
@@ -224,10 +226,84 @@ void decode_generic(const HostMatrix& h, int8_t* W_out)
     }
 }
 
+// Two columns a byte from 2 n columns; ORs what falls outside the range into *bad, returns the nonzeros.
+__attribute__((target("avx2,popcnt"))) int64_t pack_avx2(const int8_t* s, uint8_t* d, int64_t n, int off, int keep, int* bad)
+{
+    int64_t nz = 0, i = 0;
+    __m256i wrong = _mm256_setzero_si256();
+    const __m256i voff = _mm256_set1_epi8((char)off), vkeep = _mm256_set1_epi8((char)~keep), lo = _mm256_set1_epi8(15),
+                  byte = _mm256_set1_epi16(255), zero = _mm256_setzero_si256();
+    for (; i + 32 <= n; i += 32) {
+        __m256i v[2];
+        for (int j = 0; j < 2; ++j) {
+            const __m256i x = _mm256_loadu_si256((const __m256i*)(s + 2 * i + 32 * j));
+            wrong = _mm256_or_si256(wrong, _mm256_and_si256(_mm256_add_epi8(x, voff), vkeep));
+            nz += 32 - __builtin_popcount((unsigned)_mm256_movemask_epi8(_mm256_cmpeq_epi8(x, zero)));
+            const __m256i t = _mm256_and_si256(x, lo);
+            v[j] = _mm256_and_si256(_mm256_or_si256(t, _mm256_srli_epi16(t, 4)), byte);
+        }
+        _mm256_storeu_si256((__m256i*)(d + i), _mm256_permute4x64_epi64(_mm256_packus_epi16(v[0], v[1]), 0xD8));
+    }
+    if (!_mm256_testz_si256(wrong, wrong)) *bad = 1;
+    for (; i < n; ++i) {
+        const int a = s[2 * i], b = s[2 * i + 1];
+        *bad |= (((a + off) | (b + off)) & ~keep) != 0;
+        nz += (a != 0) + (b != 0);
+        d[i] = (uint8_t)((a & 15) | ((b & 15) << 4));
+    }
+    return nz;
+}
+int64_t pack_plain(const int8_t* s, uint8_t* d, int64_t n, int off, int keep, int* bad)
+{
+    int64_t nz = 0;
+    int wrong = 0;
+    for (int64_t i = 0; i < n; ++i) {
+        const int a = s[2 * i], b = s[2 * i + 1];
+        wrong |= ((a + off) | (b + off)) & ~keep;
+        nz += (a != 0) + (b != 0);
+        d[i] = (uint8_t)((a & 15) | ((b & 15) << 4));
+    }
+    *bad |= wrong != 0;
+    return nz;
+}
+
 }  // namespace
 
-us_status encode_host(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_scale,
-                      const us_format& fmt, uint32_t flags, int threads, HostMatrix* out)
+bool pack_int4(const int8_t* W, int64_t K, int64_t ld, int64_t o0, int64_t o1, uint8_t* dst, bool w2,
+               std::atomic<int32_t>* row_nnz)
+{
+    static const bool avx2 = __builtin_cpu_supports("avx2") && __builtin_cpu_supports("popcnt");
+    const int off = w2 ? 2 : 8, keep = w2 ? 3 : 15;   // in range: value + off has no other bits
+    int bad = 0;
+    for (int64_t o = o0; o < o1;) {
+        const int64_t r = o / ld, c = o - r * ld, n = std::min(ld - c, o1 - o);   // bytes of row r from byte c on
+        const int64_t pairs = std::max<int64_t>(0, std::min(n, K / 2 - c));
+        const int8_t* s = W + r * K + 2 * c;
+        uint8_t* d = dst + (o - o0);
+        int64_t nz = (avx2 ? pack_avx2 : pack_plain)(s, d, pairs, off, keep, &bad);
+        if (pairs < n) std::memset(d + pairs, 0, (size_t)(n - pairs));
+        if ((K & 1) && K / 2 >= c && K / 2 < c + n) {   // the last column of an odd number
+            const int a = W[r * K + K - 1];
+            bad |= ((a + off) & ~keep) != 0;
+            nz += a != 0;
+            d[K / 2 - c] = (uint8_t)(a & 15);
+        }
+        row_nnz[r].fetch_add((int32_t)nz, std::memory_order_relaxed);
+        o += n;
+    }
+    return bad == 0;
+}
+
+void sort_rows(const std::vector<int64_t>& nonzeros, HostMatrix* h)
+{
+    std::vector<int32_t> idx(nonzeros.size());
+    std::iota(idx.begin(), idx.end(), 0);
+    std::stable_sort(idx.begin(), idx.end(), [&](int32_t a, int32_t b) { return nonzeros[a] < nonzeros[b]; });
+    std::copy(idx.begin(), idx.end(), h->row_order.begin());
+}
+
+us_status encode_layout(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_scale,
+                        const us_format& fmt, uint32_t flags, int threads, bool defer_sort, HostMatrix* out)
 {
     if (!W || !out || M <= 0 || K <= 0) return US_ERR_INVALID_ARG;
     if (fmt.H_L <= 0 || fmt.K_L <= 0 || fmt.R_A <= 0 || fmt.C_A <= 0) return US_ERR_SHAPE;
@@ -266,8 +342,7 @@ us_status encode_host(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_s
 
     // ---- row order -----------------------------------------------------------------------
     h.row_order.assign(h.Mp, -1);
-    std::atomic<int> bad{0};
-    if (flags & US_ENCODE_SORT_ROWS) {
+    if ((flags & US_ENCODE_SORT_ROWS) && !(defer_sort && !(flags & US_ENCODE_PAIR_ROWS))) {
         std::vector<int64_t> cnt(M, 0);
         parallel_for(M, threads, [&](int64_t r, int) {
             const int8_t* p = W + r * K;
@@ -275,15 +350,22 @@ us_status encode_host(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_s
             for (int64_t k = 0; k < K; ++k) c += p[k] != 0;
             cnt[r] = c;
         });
-        std::vector<int32_t> idx(M);
-        std::iota(idx.begin(), idx.end(), 0);
-        std::stable_sort(idx.begin(), idx.end(), [&](int32_t a, int32_t b) { return cnt[a] < cnt[b]; });
-        std::copy(idx.begin(), idx.end(), h.row_order.begin());
+        sort_rows(cnt, &h);
     } else {
         std::iota(h.row_order.begin(), h.row_order.begin() + M, 0);
     }
 
     if (flags & US_ENCODE_PAIR_ROWS) pair_rows(W, M, K, threads, &h);
+    return US_OK;
+}
+
+us_status encode_host(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_scale,
+                      const us_format& fmt, uint32_t flags, int threads, HostMatrix* out)
+{
+    const us_status laid = encode_layout(W, M, K, w_scale, fmt, flags, threads, false, out);
+    if (laid != US_OK || !out->kernel_layout) return laid;
+    HostMatrix& h = *out;
+    std::atomic<int> bad{0};
 
     // ---- build every tile blob (parallel over strips) ------------------------------------
     const int K_L = fmt.K_L, CA = fmt.C_A, nkb = h.nkb / CA, mask_rows = h.mask_rows;   // nkb: mask bytes per lane
@@ -389,6 +471,7 @@ us_status encode_host(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_s
     });
     h.nnz = nnz.load();
     h.sum_P = sum_P.load();
+    h.blob_bytes = h.blob.size();
     h.bytes_payload_padded = (int64_t)h.blob.size() - h.n_items * mask_bytes;
     return US_OK;
 }

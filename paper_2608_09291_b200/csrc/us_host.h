@@ -28,6 +28,7 @@
 // Any other valid IE-BME format (other H_L, R_A, C_A, narrow tiles) is encoded on the host in the
 // paper's own array layout (GenericArrays) for us_get_stats / us_decode; no kernel reads it.
 #pragma once
+#include <atomic>
 #include <cstdint>
 #include <vector>
 
@@ -55,7 +56,8 @@ struct HostMatrix {
     int64_t n_strips = 0, n_segs = 0, n_items = 0;
     std::vector<int32_t> row_order;   // Mp entries: original row at padded position, -1 = padding
     std::vector<uint32_t> item_off;   // n_items + 1, units of 16 bytes
-    std::vector<uint8_t> blob;        // all tile blobs back to back
+    std::vector<uint8_t> blob;        // all tile blobs back to back (empty until asked for where the GPU encoded them)
+    uint64_t blob_bytes = 0;
     std::vector<uint16_t> w_scale;    // M fp16 bit patterns (empty if none)
     int64_t nnz = 0, sum_P = 0, bytes_payload_padded = 0;
     uint32_t max_item_bytes = 0;
@@ -64,6 +66,17 @@ struct HostMatrix {
 // Returns US_OK or an error; `out` is filled on success. `threads` <= 0 picks the core count.
 us_status encode_host(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_scale,
                       const us_format& fmt, uint32_t flags, int threads, HostMatrix* out);
+// The steps before the tiles: checks, shape, row order. For a format without a kernel layout it encodes all there is.
+// With defer_sort the order by nonzero count (without row pairing) is left to sort_rows.
+us_status encode_layout(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_scale,
+                        const us_format& fmt, uint32_t flags, int threads, bool defer_sort, HostMatrix* out);
+void sort_rows(const std::vector<int64_t>& nonzeros, HostMatrix* h);
+
+// Packs bytes [o0, o1) of the INT4 form of W (rows of ld bytes, two columns a byte, zero beyond column K) into dst and
+// adds the nonzeros it meets to row_nnz. False if a value is out of range.
+bool pack_int4(const int8_t* W, int64_t K, int64_t ld, int64_t o0, int64_t o1, uint8_t* dst, bool w2,
+               std::atomic<int32_t>* row_nnz);
+
 void decode_host(const HostMatrix& h, int8_t* W_out);
 void fill_stats(const HostMatrix& h, us_stats* st);
 
