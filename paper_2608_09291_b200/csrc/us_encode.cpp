@@ -226,7 +226,9 @@ void decode_generic(const HostMatrix& h, int8_t* W_out)
     }
 }
 
-// Two columns a byte from 2 n columns; ORs what falls outside the range into *bad, returns the nonzeros.
+// Two columns a byte from 2 n columns, d 32-byte aligned. The stores go past the caches: a copy engine that finds the
+// staging buffer as dirty lines in 16 cores' caches reads it at 12 GB/s, from memory at 48 (22.5 MB: 1.8 ms against
+// 0.47). ORs what falls outside the range into *bad, returns the nonzeros.
 __attribute__((target("avx2,popcnt"))) int64_t pack_avx2(const int8_t* s, uint8_t* d, int64_t n, int off, int keep, int* bad)
 {
     int64_t nz = 0, i = 0;
@@ -242,8 +244,9 @@ __attribute__((target("avx2,popcnt"))) int64_t pack_avx2(const int8_t* s, uint8_
             const __m256i t = _mm256_and_si256(x, lo);
             v[j] = _mm256_and_si256(_mm256_or_si256(t, _mm256_srli_epi16(t, 4)), byte);
         }
-        _mm256_storeu_si256((__m256i*)(d + i), _mm256_permute4x64_epi64(_mm256_packus_epi16(v[0], v[1]), 0xD8));
+        _mm256_stream_si256((__m256i*)(d + i), _mm256_permute4x64_epi64(_mm256_packus_epi16(v[0], v[1]), 0xD8));
     }
+    _mm_sfence();
     if (!_mm256_testz_si256(wrong, wrong)) *bad = 1;
     for (; i < n; ++i) {
         const int a = s[2 * i], b = s[2 * i + 1];

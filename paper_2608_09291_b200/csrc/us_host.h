@@ -72,7 +72,7 @@ us_status encode_layout(const int8_t* W, int64_t M, int64_t K, const uint16_t* w
                         const us_format& fmt, uint32_t flags, int threads, bool defer_sort, HostMatrix* out);
 void sort_rows(const std::vector<int64_t>& nonzeros, HostMatrix* h);
 
-// Packs bytes [o0, o1) of the INT4 form of W (rows of ld bytes, two columns a byte, zero beyond column K) into dst and
+// Packs bytes [o0, o1) of the INT4 form of W (rows of ld bytes, two columns a byte, zero beyond column K) into dst (32-byte aligned, o0 and ld multiples of 32) and
 // adds the nonzeros it meets to row_nnz. False if a value is out of range.
 bool pack_int4(const int8_t* W, int64_t K, int64_t ld, int64_t o0, int64_t o1, uint8_t* dst, bool w2,
                std::atomic<int32_t>* row_nnz);
