@@ -355,7 +355,7 @@ void build_plan(us_handle* h, int cls)
     p.fold_kb = hm.fmt.C_A == 2 ? hm.nkb / 2 : 0;
     p.w2 = hm.w2 ? 1 : 0;
     p.slot_bytes = g.slot_bytes;
-    p.x_fast = (hm.K % 32 == 0) ? 2 : (hm.K % 8 == 0) ? 1 : 0;
+    p.x_fast = hm.K % 32 == 0;
 }
 
 // Lays a launch of us_spmm_tc_kernel down for calls of `ng` 8-token groups.

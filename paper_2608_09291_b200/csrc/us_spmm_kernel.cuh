@@ -64,7 +64,7 @@ struct SpmmParams {
     int32_t fold_kb;            // C_A = 2: k-blocks per column area (a mask bit also covers the column that many
                                 // k-blocks further on); 0 for C_A = 1
     uint32_t slot_bytes;        // ring slot size (max tile blob + slack), multiple of 128
-    int32_t x_fast;             // 2: K % 32 == 0 (16-byte loads); 1: K % 8 == 0 (4-byte loads); 0: bytes
+    int32_t x_fast;             // K % 32 == 0: 16-byte loads
     int32_t fp16_out;
     // Chained call: the epilogue leaves the per-token absmax of the fp16 outputs of rows
     // [amax_m0, amax_m1) in an absmax buffer (layout below) for the quantiser of the next call.
@@ -247,6 +247,71 @@ __device__ __forceinline__ uint32_t pack8(uint32_t v, int32_t& s)
     return (t.x >> 4) | t.y;
 }
 
+// Staging of a K range for any K (stage_x takes K a multiple of 32): a unit of 32 columns comes from two aligned 16-byte
+// loads, shifted into place. Kept short, one unit per thread at a time: a CTA runs this code once, and fetching it costs
+// more than the second round of loads does. It replaces eight byte loads in a row per 8 columns (5003 x 3001,
+// N = 5: 9.3 -> 7.0 us in the half-SM plan; 4096 x 4100, N = 16: 15.1 -> 8.8).
+template <int NT, bool XP>
+__device__ __forceinline__ void stage_x_any(const uint8_t* X, int K, int N, int K_L, int seg0, int n_seg, uint8_t* x8, int xstride,
+                                            int32_t* sx16)
+{
+    const int64_t ldx = ((int64_t)K + 1) / 2, bytes = (int64_t)N * ldx;
+    const int upr = K_L / 32, total = NT * 8 * n_seg * upr;   // a multiple of 32
+    const int sh_u = 31 - __clz(upr);
+    const bool pow2 = (1 << sh_u) == upr;
+#pragma unroll 1
+    for (int u = threadIdx.x; u < total; u += blockDim.x) {   // (whole warps)
+        const int pi = pow2 ? u >> sh_u : u / upr, q = u - pi * upr, sgl = pi / (NT * 8), n = pi & (NT * 8 - 1);
+        const int left = K - ((seg0 + sgl) * K_L + 32 * q);   // valid columns from the unit's first on
+        const int64_t at = (int64_t)n * ldx + (K - left) / 2, a = at & ~(int64_t)15;
+        int32_t s = 0;
+        if (n < N && left > 0 && (left < 32 || a + 32 > bytes)) {   // the end of a row, or of X: word by word, byte by byte
+#pragma unroll 1
+            for (int i = 0; i < 4; ++i) {
+                uint32_t v = 0;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int c = left - 8 * i - 2 * j;   // columns left at this byte
+                    if (c > 0) v |= (X[at + 4 * i + j] & (c > 1 ? 255u : 15u)) << (8 * j);
+                }
+                if (XP) *reinterpret_cast<uint32_t*>(x8 + n * xstride + (sgl * K_L + 32 * q) / 2 + 4 * i) = pack8(v, s);
+                else *reinterpret_cast<uint2*>(x8 + n * xstride + sgl * K_L + 32 * q + 8 * i) = expand8(v, s);
+            }
+        } else {
+            uint4 v = make_uint4(0, 0, 0, 0);
+            if (n < N && left > 0) {
+                const uint4 lo = __ldg(reinterpret_cast<const uint4*>(X + a)), hi = __ldg(reinterpret_cast<const uint4*>(X + a + 16));
+                uint32_t w[7] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z};
+                if (at & 8) { w[0] = w[2]; w[1] = w[3]; w[2] = w[4]; w[3] = w[5]; w[4] = w[6]; w[5] = hi.w; }
+                if (at & 4) { w[0] = w[1]; w[1] = w[2]; w[2] = w[3]; w[3] = w[4]; w[4] = w[5]; }
+                const uint32_t sh = 8u * (uint32_t)(at & 3);
+                v = make_uint4(__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh),
+                               __funnelshift_r(w[2], w[3], sh), __funnelshift_r(w[3], w[4], sh));
+            }
+            if (XP) {
+                uint4 pk;
+                pk.x = pack8(v.x, s); pk.y = pack8(v.y, s); pk.z = pack8(v.z, s); pk.w = pack8(v.w, s);
+                *reinterpret_cast<uint4*>(x8 + n * xstride + (sgl * K_L + 32 * q) / 2) = pk;
+            } else {
+                uint4 e, c;
+                uint2 t;
+                t = expand8(v.x, s); e.x = t.x; e.y = t.y;
+                t = expand8(v.y, s); e.z = t.x; e.w = t.y;
+                t = expand8(v.z, s); c.x = t.x; c.y = t.y;
+                t = expand8(v.w, s); c.z = t.x; c.w = t.y;
+                uint4* dst = reinterpret_cast<uint4*>(x8 + n * xstride + sgl * K_L + 32 * q);
+                dst[0] = e; dst[1] = c;
+            }
+        }
+        if (upr % 32 == 0) {   // the warp's units are of one (segment, token) pair: one add for all
+            s = __reduce_add_sync(0xffffffffu, s);
+            if ((threadIdx.x & 31) == 0) atomicAdd(sx16 + pi, s);
+        } else if (s) {
+            atomicAdd(sx16 + pi, s);
+        }
+    }
+}
+
 // sx16 must be zero on entry (the caller clears it and synchronises).
 // Units below `first_unit` (of the 16-byte path) were already staged by the caller.
 template <int NT, bool XP>
@@ -255,78 +320,53 @@ __device__ __forceinline__ void stage_x(const SpmmParams& p, int seg0, int n_seg
 {
     const int64_t ldx = ((int64_t)p.K + 1) / 2;
     const int rows = NT * 8;
-    if (p.x_fast == 2) {
-        // 16-byte units (32 activations); all loads of a batch are issued before any is used
-        const int upr = p.K_L / 32;                 // units per (segment, token)
-        const int total = rows * n_seg * upr;
-        constexpr int kBatch = 4;
-        for (int u0 = first_unit + threadIdx.x; u0 < total; u0 += kBatch * blockDim.x) {
-            uint4 v[kBatch];
-#pragma unroll
-            for (int b = 0; b < kBatch; ++b) {
-                const int u = u0 + b * blockDim.x;
-                v[b] = make_uint4(0, 0, 0, 0);
-                if (u < total) {
-                    const int pi = u / upr, q = u - pi * upr;
-                    const int sgl = pi / rows, n = pi - sgl * rows;
-                    const int64_t k = (int64_t)(seg0 + sgl) * p.K_L + 32 * q;
-                    if (n < p.N && k < p.K)
-                        v[b] = __ldg(reinterpret_cast<const uint4*>(p.X + (int64_t)n * ldx + k / 2));
-                }
-            }
-#pragma unroll
-            for (int b = 0; b < kBatch; ++b) {
-                const int u = u0 + b * blockDim.x;
-                if (u < total) {
-                    const int pi = u / upr, q = u - pi * upr;
-                    const int sgl = pi / rows, n = pi - sgl * rows;
-                    int32_t s = 0;
-                    if (XP) {
-                        uint4 pk;
-                        pk.x = pack8(v[b].x, s); pk.y = pack8(v[b].y, s);
-                        pk.z = pack8(v[b].z, s); pk.w = pack8(v[b].w, s);
-                        *reinterpret_cast<uint4*>(x8 + n * xstride + (sgl * p.K_L + 32 * q) / 2) = pk;
-                    } else {
-                        uint4 lo, hi;
-                        uint2 t;
-                        t = expand8(v[b].x, s); lo.x = t.x; lo.y = t.y;
-                        t = expand8(v[b].y, s); lo.z = t.x; lo.w = t.y;
-                        t = expand8(v[b].z, s); hi.x = t.x; hi.y = t.y;
-                        t = expand8(v[b].w, s); hi.z = t.x; hi.w = t.y;
-                        uint4* dst = reinterpret_cast<uint4*>(x8 + n * xstride + sgl * p.K_L + 32 * q);
-                        dst[0] = lo; dst[1] = hi;
-                    }
-                    if (s) atomicAdd(sx16 + pi, s);
-                }
-            }
-        }
+    if (!p.x_fast) {
+        stage_x_any<NT, XP>(p.X, p.K, p.N, p.K_L, seg0, n_seg, x8, xstride, sx16);
         return;
     }
-    // general path: 8 activations at a time, any K and alignment
-    const int wpr = p.K_L / 8;
-    const int total = rows * n_seg * wpr;
-    for (int u = threadIdx.x; u < total; u += blockDim.x) {
-        const int pi = u / wpr, wi = u - pi * wpr;
-        const int sgl = pi / rows, n = pi - sgl * rows;
-        const int64_t k = (int64_t)(seg0 + sgl) * p.K_L + 8 * wi;
-        uint32_t v = 0;
-        if (n < p.N) {
-            const uint8_t* src = p.X + (int64_t)n * ldx + k / 2;
-            if (p.x_fast == 1 && k + 8 <= p.K) {
-                v = __ldg(reinterpret_cast<const uint32_t*>(src));
-            } else {
-                for (int e = 0; e < 8; ++e) {
-                    if (k + e < p.K) {
-                        uint32_t byte = src[e >> 1];
-                        v |= ((e & 1) ? (byte >> 4) : (byte & 0xF)) << (4 * e);
-                    }
-                }
+    // 16-byte units (32 activations); all loads of a batch are issued before any is used
+    const int upr = p.K_L / 32;                 // units per (segment, token)
+    const int total = rows * n_seg * upr;
+    constexpr int kBatch = 4;
+    for (int u0 = first_unit + threadIdx.x; u0 < total; u0 += kBatch * blockDim.x) {
+        uint4 v[kBatch];
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            const int u = u0 + b * blockDim.x;
+            v[b] = make_uint4(0, 0, 0, 0);
+            if (u < total) {
+                const int pi = u / upr, q = u - pi * upr;
+                const int sgl = pi / rows, n = pi - sgl * rows;
+                const int64_t k = (int64_t)(seg0 + sgl) * p.K_L + 32 * q;
+                if (n < p.N && k < p.K)
+                    v[b] = __ldg(reinterpret_cast<const uint4*>(p.X + (int64_t)n * ldx + k / 2));
             }
         }
-        int32_t s = 0;
-        if (XP) *reinterpret_cast<uint32_t*>(x8 + n * xstride + (sgl * p.K_L + 8 * wi) / 2) = pack8(v, s);
-        else *reinterpret_cast<uint2*>(x8 + n * xstride + sgl * p.K_L + 8 * wi) = expand8(v, s);
-        if (s) atomicAdd(sx16 + pi, s);
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            const int u = u0 + b * blockDim.x;
+            if (u < total) {
+                const int pi = u / upr, q = u - pi * upr;
+                const int sgl = pi / rows, n = pi - sgl * rows;
+                int32_t s = 0;
+                if (XP) {
+                    uint4 pk;
+                    pk.x = pack8(v[b].x, s); pk.y = pack8(v[b].y, s);
+                    pk.z = pack8(v[b].z, s); pk.w = pack8(v[b].w, s);
+                    *reinterpret_cast<uint4*>(x8 + n * xstride + (sgl * p.K_L + 32 * q) / 2) = pk;
+                } else {
+                    uint4 lo, hi;
+                    uint2 t;
+                    t = expand8(v[b].x, s); lo.x = t.x; lo.y = t.y;
+                    t = expand8(v[b].y, s); lo.z = t.x; lo.w = t.y;
+                    t = expand8(v[b].z, s); hi.x = t.x; hi.y = t.y;
+                    t = expand8(v[b].w, s); hi.z = t.x; hi.w = t.y;
+                    uint4* dst = reinterpret_cast<uint4*>(x8 + n * xstride + sgl * p.K_L + 32 * q);
+                    dst[0] = lo; dst[1] = hi;
+                }
+                if (s) atomicAdd(sx16 + pi, s);
+            }
+        }
     }
 }
 
@@ -813,7 +853,7 @@ __global__ void __launch_bounds__((NT == 1 && CA == 1) ? 640 : 512, 1) us_spmm_k
     const int g_first = (kr_first == n_kr - 1) ? g_last : p.G;   // segments in that range
     constexpr int kXPre = NT <= 4 ? 8 : 0;   // 16-byte units of X a thread prefetches
     const int x_sh = 31 - __clz(p.K_L / 32);   // log2(units per (segment, token)) when a power of two
-    const bool x_early = kXPre > 0 && p.x_fast == 2 && (1 << x_sh) == p.K_L / 32;
+    const bool x_early = kXPre > 0 && p.x_fast && (1 << x_sh) == p.K_L / 32;
     uint4 xpre[kXPre > 0 ? kXPre : 1];
     const int x_upr = p.K_L / 32, x_total = NT * 8 * g_first * x_upr;
     if (x_early) {

@@ -190,17 +190,23 @@ __device__ __forceinline__ void decode_word(uint32_t mw, uint32_t pay_a, uint32_
     for (int s = 0; s < SR; ++s) { cw0[s] = w0[s][3]; cw1[s] = w1[s][3]; }
 }
 
-// 32 packed activations from byte address b of X on (column k of a token, a multiple of 32); columns from K on are
-// zero. Any K: rows start at any byte, so aligned words up to the one that holds the last column are shifted into
-// place. Out of line: the code of a CTA's first pass is fetched line by line, so what few shapes need stays away.
-inline __device__ __noinline__ uint4 load_x32_any(const uint8_t* X, int64_t b, int nv)
+// 32 packed activations from byte address b of X on (column k of a token, a multiple of 32), `nv` columns of them valid
+// and the rest zero; X holds `total` bytes. Any K: rows start at any byte, so aligned words are shifted into place. Out
+// of line: the code of a CTA's first pass is fetched line by line, so what few shapes need stays away.
+inline __device__ __noinline__ uint4 load_x32_any(const uint8_t* X, int64_t total, int64_t b, int nv)
 {
     nv = min(32, nv);
     const int64_t b4 = b & ~(int64_t)3, last = b + (nv - 1) / 2;
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(X + b4);
     uint32_t w[5];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) w[i] = b4 + 4 * i <= last ? __ldg(src + i) : 0u;
+    for (int i = 0; i < 5; ++i) {
+        const int64_t a = b4 + 4 * i;
+        w[i] = 0;
+        if (a <= last) {
+            if (a + 4 <= total) w[i] = __ldg(reinterpret_cast<const uint32_t*>(X + a));
+            else for (int j = 0; a + j < total; ++j) w[i] |= (uint32_t)X[a + j] << (8 * j);   // the end of X
+        }
+    }
     const uint32_t sh = 8u * (uint32_t)(b & 3);
     uint32_t o[4];
 #pragma unroll
@@ -211,12 +217,14 @@ inline __device__ __noinline__ uint4 load_x32_any(const uint8_t* X, int64_t b, i
     }
     return make_uint4(o[0], o[1], o[2], o[3]);
 }
+
+// 32 packed activations of token n from column k on.
 __device__ __forceinline__ uint4 load_x32(const TcParams& p, int64_t ldx, int n, int k)
 {
     uint4 v = make_uint4(0, 0, 0, 0);
     if (n >= p.N || k >= p.K) return v;
     const int64_t b = (int64_t)n * ldx + (k >> 1);
-    if (!p.x_fast) return load_x32_any(p.X, b, p.K - k);
+    if (!p.x_fast) return load_x32_any(p.X, (int64_t)p.N * ldx, b, p.K - k);
     // (volatile: the load is to be in flight from here on, not sunk to its use)
     asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p.X + b));
     return v;
