@@ -187,9 +187,15 @@ bool plan_launch(const us_handle* h, int N, LaunchGeom* g)
         int w = std::min(g->nt == 1 ? (fold ? h->co_warps_fold : h->co_warps) : h->co_warps2,
                          (g->nt == 1 && !fold) ? max_warps() : std::min(16, max_warps()));
         while (w >= 8 && fixed8 + w * (int)g->slot_bytes > half) --w;
+        // the most tiles a CTA has: cuts fall on strip boundaries, so it can be more than the average (5008 x 3008, 3 tiles to a
+        // strip: most CTAs have two strips, some three, and eight warps would need a second round for the ninth tile: 5.7 us
+        // against 5.2 with 16 warps on the whole SM; 3000 x 6000 11.7 against 8.7)
+        int64_t most = per_cta;
+        for (size_t c = 0; c + 1 < h->cta_begin[g->cls].size(); ++c)
+            most = std::max<int64_t>(most, (int64_t)h->cta_begin[g->cls][c + 1] - h->cta_begin[g->cls][c]);
         // (only if nearly every tile of the CTA finds a warp at once: 5120 x 5120 at 70 % sparsity, N = 16, has 11
         // tiles per CTA and room for 8 half-SM warps: 9.9 us against 8.9 with 16 warps on the whole SM)
-        if (w >= 8 && w >= std::min<int64_t>(per_cta, 10)) { stages = 1; lut_rep = 8; warps = w; fixed = fixed8; }
+        if (w >= 8 && w >= std::min<int64_t>(most, 10)) { stages = 1; lut_rep = 8; warps = w; fixed = fixed8; }
     }
     g->stages = stages;
     g->lut_rep = lut_rep;

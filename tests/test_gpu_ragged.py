@@ -28,3 +28,13 @@ def test_any_k(K, fmt):
             assert (y == oracle.spmm_dense(W, X[:N])).all(), (N, K, fmt)
     finally:
         sw.close()
+
+
+def test_plan_counts_the_largest_share():
+    """5008 x 3008 has CTAs of nine tiles: all its warps at once, not eight in half an SM; 4096 x 4096 has eight."""
+    from paper_2608_09291_b200 import binding as b
+    for M, K, wide in ((5008, 3008, True), (4096, 4096, False)):
+        W = workloads.make_weight(M, K, 0.5, seed=1)
+        h = b.us_encode(W, fmt=(16, 1024, 2, 2), max_N=8)
+        assert (b.us_launch_info(h, 8)["block"] > 384) == wide
+        b.us_destroy(h)
