@@ -535,6 +535,22 @@ us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_sca
     return launch(h, fn, &p, g.warps * 32, g.smem, st);
 }
 
+// A 256-thread kernel, launched with programmatic stream serialization like the SpMM.
+template <class... P, class... A>
+cudaError_t launch_small(void (*kernel)(P...), dim3 grid, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = pdl_knob() ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 }  // namespace
 
 extern "C" {
@@ -762,16 +778,8 @@ cudaError_t launch_quantize(const uint16_t* X16, int64_t ldx, int32_t N, int64_t
                             uint16_t* x_scale, cudaStream_t st)
 {
     const int64_t units = (K + 7) / 8;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(64, (units + 255) / 256)), (unsigned)N);
-    cfg.blockDim = dim3(256);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = pdl_knob() ? 1 : 0;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, us::us_quantize_f16_kernel, X16, ldx, K, amax, Xq, x_scale);
+    const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(64, (units + 255) / 256)), (unsigned)N);
+    return launch_small(us::us_quantize_f16_kernel, grid, st, X16, ldx, K, amax, Xq, x_scale);
 }
 }  // namespace
 
@@ -811,9 +819,9 @@ us_status us_absmax_f16(const void* X16, int64_t ldx, int32_t N, int64_t K, void
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int64_t units = (K + 7) / 8;
     const unsigned gx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(16, (units + 255) / 256));
-    us::us_absmax_f16_kernel<<<dim3(gx, (unsigned)N), 256, 0, st>>>(static_cast<const uint16_t*>(X16), ldx, K, N,
-                                                                    static_cast<uint32_t*>(amax));
-    if (cudaGetLastError() != cudaSuccess) return US_ERR_CUDA;
+    const cudaError_t e = launch_small(us::us_absmax_f16_kernel, dim3(gx, (unsigned)N), st, static_cast<const uint16_t*>(X16), ldx, K,
+                                       (int)N, static_cast<uint32_t*>(amax));
+    if (e != cudaSuccess) { cudaGetLastError(); return US_ERR_CUDA; }
     return US_OK;
 }
 

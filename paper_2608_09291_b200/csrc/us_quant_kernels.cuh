@@ -49,6 +49,9 @@ __global__ void __launch_bounds__(256) us_absmax_f16_kernel(const uint16_t* X16,
 {
     __shared__ uint32_t red[8];
     const int n = blockIdx.y;
+    // (launched like the other kernels: the next one may start its prologue, this one waits for what came before)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const uint16_t* row = X16 + (int64_t)n * ldx;
     uint32_t big = 0;
     const bool vec = (ldx % 8 == 0) && (reinterpret_cast<uintptr_t>(X16) % 16 == 0);
@@ -90,32 +93,38 @@ __global__ void __launch_bounds__(256) us_quantize_f16_kernel(const uint16_t* X1
     if (threadIdx.x == 0) am = 0;
     __syncthreads();
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    // The first unit's activations are requested before the absmax is reduced: two latencies side by side, not in a row.
+    const uint16_t* row = X16 + (int64_t)n * ldx;
+    const bool vec = (ldx % 8 == 0) && (reinterpret_cast<uintptr_t>(X16) % 16 == 0);
+    const int64_t units = (K + 7) / 8, u0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    auto load = [&](int64_t u) -> uint4 {
+        const int64_t k = 8 * u;
+        if (vec && k + 8 <= K) return __ldcg(reinterpret_cast<const uint4*>(row + k));
+        uint32_t w[4] = {0, 0, 0, 0};
+        for (int e = 0; e < 8; ++e)
+            if (k + e < K) w[e >> 1] |= (uint32_t)__ldcg(row + k + e) << (16 * (e & 1));
+        return make_uint4(w[0], w[1], w[2], w[3]);
+    };
+    uint4 h = u0 < units ? load(u0) : make_uint4(0, 0, 0, 0);
     {
+        // (a part beyond the number written is read but not used: all loads are in flight with the number itself)
         const int parts = min((int)__ldcg(amax), kAmaxParts);
         uint32_t big = 0;
-        for (int pt = threadIdx.x; pt < parts; pt += blockDim.x) big = max(big, __ldcg(amax + 64 + 64 * pt + n) & 0x7FFFu);
+        for (int pt = threadIdx.x; pt < kAmaxParts; pt += blockDim.x) {
+            const uint32_t v = __ldcg(amax + 64 + 64 * pt + n) & 0x7FFFu;
+            if (pt < parts) big = max(big, v);
+        }
         big = __reduce_max_sync(0xffffffffu, big);
         if ((threadIdx.x & 31) == 0 && big) atomicMax(&am, big);
     }
     __syncthreads();
-    const uint16_t* row = X16 + (int64_t)n * ldx;
     uint8_t* out = Xq + (int64_t)n * ((K + 1) / 2);
     const uint32_t iv = requant_inverse(am), inv2 = iv | (iv << 16);
     if (blockIdx.x == 0 && threadIdx.x == 0 && x_scale) x_scale[n] = __half_as_ushort(__float2half_rn(requant_scale(am)));
-    const bool vec = (ldx % 8 == 0) && (reinterpret_cast<uintptr_t>(X16) % 16 == 0);
     const bool vec_out = (((K + 1) / 2) % 4 == 0) && (reinterpret_cast<uintptr_t>(Xq) % 4 == 0);
-    const int64_t units = (K + 7) / 8;
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < units; u += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t u = u0; u < units; u += (int64_t)gridDim.x * blockDim.x) {
         const int64_t k = 8 * u;
-        uint4 h = make_uint4(0, 0, 0, 0);
-        if (vec && k + 8 <= K) {
-            h = __ldcg(reinterpret_cast<const uint4*>(row + k));
-        } else {
-            uint32_t w[4] = {0, 0, 0, 0};
-            for (int e = 0; e < 8; ++e)
-                if (k + e < K) w[e >> 1] |= (uint32_t)__ldcg(row + k + e) << (16 * (e & 1));
-            h = make_uint4(w[0], w[1], w[2], w[3]);
-        }
+        if (u != u0) h = load(u);
         const uint32_t v = requant8(h, inv2);
         if (vec_out && k + 8 <= K) {
             *reinterpret_cast<uint32_t*>(out + k / 2) = v;
