@@ -31,7 +31,7 @@ struct ClassPlan {
 // The same for us_spmm_tc_kernel, per number of 8-token groups.
 struct TcPlan {
     bool ok = false;
-    int smem = 0;
+    int octets = 2, threads = 0, smem = 0;
     us::TcParams p{};
 };
 
@@ -86,6 +86,7 @@ int stages_knob() { static int v = env_int("US_STAGES", 0); return v; }    // ri
 // (up to 20 for the N <= 8 kernels; the other kernels are compiled for 16)
 int max_warps() { static int v = std::min(20, std::max(2, env_int("US_MAX_WARPS", 16))); return v; }
 int tc_knob() { static int v = env_int("US_TC", 1); return v; }   // tensor-memory kernel: 0 never, 1 by rule, 2 wherever it can run
+int tc_oct_knob() { static int v = env_int("US_TC_OCT", 0); return v; }   // its octets: 0 by rule
 int coresident_knob() { static int v = env_int("US_CORESIDENT", 1); return v; }  // small problems: half an SM per CTA
 constexpr int kLocalAccBudget = 32 * 1024;   // local strip sums a K-range width is chosen with
 constexpr int kLocalAccCap = 48 * 1024;      // ... and what is taken if nothing fits that
@@ -375,32 +376,53 @@ void build_tc_plan(us_handle* h, int ng)
     std::memset(&p, 0, sizeof(p));
     const int64_t n_cta = h->sm_count;
     const int n_stage = hm.fmt.C_A == 1 ? (hm.mask_rows + 1) / 2 : hm.mask_rows;   // 256-column stages per tile
-    const int64_t block_stages = hm.n_segs * n_stage, stages = (hm.n_strips + 15) / 16 * block_stages;
+    const int64_t block_stages = hm.n_segs * n_stage;
+    int64_t stages = (hm.n_strips + 15) / 16 * block_stages;
     if (block_stages >= (1 << 16) || stages >= (1 << 24)) return;   // exact division by multiplication
-    // Where it is chosen. The kernel saves the X fragments, MMAs and split-K adds of every tile, and pays a longer
-    // prologue and a flush through the workspace per CTA (4 to 5 us together at N = 64). Against a plan that sums strips
-    // in shared memory it needs so many stages per CTA to win (measured at s = .5, us, that plan / this kernel: N = 16
-    // 13824 x 5120, 7 stages, 13.0 / 14.0, 28672 x 8192, 24 stages, 32.4 / 28.8; N = 32 4096 x 11008, 4.6 stages, sorted
-    // rows, 15.5 / 16.1, 13824 x 5120 18.8 / 17.0; N = 64 4096 x 4096, 1.7 stages, 14.4 / 17.3); against the direct
-    // mode it wins nearly always (N = 32 on 2 x 2 tiles 5120 x 5120 14.9 / 13.2; N = 64 4096 x 4096 with INT2 weights
-    // 21.8 / 16.5, 28672 x 8192 92 / 41, 8192 x 28672 83 / 41).
-    const bool sums_local = h->s_local[class_of(nt_for(8 * ng))] > 0;
-    const int64_t min_stages = !sums_local ? 3 * n_cta / 2 : (ng <= 2 ? 16 : ng <= 4 ? 6 : 4) * n_cta;
-    if (tc_knob() == 0 || (tc_knob() == 1 && stages < min_stages)) return;
+    // Where it is chosen. The kernel saves the X fragments, MMAs and split-K adds of every tile and gives all CTAs the same
+    // number of stages; it pays a longer prologue and a flush through the workspace per CTA (4 to 5 us together at N = 64).
+    // Against a plan that sums strips in shared memory, whose time follows the largest share of a CTA (cuts fall on strip
+    // boundaries), two straight lines in us fit what was measured at s = .5 and .6 within 5 %, `share` and `mean` being the
+    // largest and the average CTA share in stages:
+    //   N <= 16: that plan 4.5 + 1.08 share, this kernel 7.5 + 0.9 mean (20480 x 8192 26.2 / 23.3, 28672 x 8192 32.4 / 28.0,
+    //            27648 x 5120 21.0 / 20.9, 13824 x 5120 13.0 / 14.2). Half a us of margin, and from 10 stages on: among other
+    //            launches its code comes from L2 each time, and 5120 x 13824, 7 stages, alone 15.1 / 13.8, gained nothing in
+    //            a layer of seven projections.
+    //   N <= 32: 5.5 + 1.76 share, 9.7 + 0.97 mean (13824 x 5120 18.8 / 17.2, 28672 x 8192 51 / 33, 5120 x 5120 12.3 / 12.7);
+    //            2 us of margin, since matrices of uneven density cost this kernel more (4096 x 11008 sorted 15.5 / 16.1)
+    //   N <= 64: from 4 stages on (4096 x 4096, 1.7 stages, 14.4 / 17.3; 11008 x 4096, 4.6 stages, 35 / 20.6).
+    // Against the direct mode it wins nearly always (N = 32 on 2 x 2 tiles 5120 x 5120 14.9 / 12.9; N = 64 4096 x 4096 with
+    // INT2 weights 21.8 / 16.5, 28672 x 8192 92 / 41).
+    const int cls = class_of(nt_for(8 * ng));
+    uint32_t most = 0;
+    for (size_t c = 0; c + 1 < h->cta_begin[cls].size(); ++c) most = std::max(most, h->cta_begin[cls][c + 1] - h->cta_begin[cls][c]);
+    const double mean = (double)stages / (double)n_cta, share = (double)most * n_stage / 16;
+    const bool better = h->s_local[cls] == 0 ? mean >= 1.5
+                        : ng <= 2            ? mean >= 10 && 4.5 + 1.08 * share > 8.0 + 0.9 * mean
+                        : ng <= 4            ? 5.5 + 1.76 * share > 11.7 + 0.97 * mean
+                                             : mean >= 4;
+    if (tc_knob() == 0 || (tc_knob() == 1 && !better)) return;
     p.slot_bytes = slot_bytes_for(hm);
     const int limit = h->max_smem > 0 ? h->max_smem : 227 * 1024;
     auto fixed_for = [&](int x_stages, int lut_rep) { return 256 * lut_rep * 4 + x_stages * ng * 2048 + 2048 + us::kTcFixedSmem; };
     auto slots_for = [&](int x_stages, int lut_rep) {
         return std::min(us::kTcMaxSlots, (limit - fixed_for(x_stages, lut_rep)) / (int)p.slot_bytes);
     };
+    p.x_stages = 4;
+    // Three octets for N <= 16 and long shares (N = 16, two octets / three: 28672 x 8192 29.3 / 28.0, with INT2 weights
+    // 25.7 / 24.7; 13824 x 5120, 7 stages, INT2 12.75 / 12.86; N = 32 on 28672 x 8192 33.1 / 33.4).
+    const int64_t stages3 = (hm.n_strips + 23) / 24 * block_stages;
+    pl.octets = slots_for(3, 8) >= 24 && ng <= 4 && (tc_oct_knob() ? tc_oct_knob() == 3 : ng <= 2 && stages3 >= 8 * n_cta) ? 3 : 2;
+    if (pl.octets == 3) { stages = stages3; p.x_stages = slots_for(4, 8) >= 24 ? 4 : 3; }
+    const int warps = 8 * pl.octets;
+    pl.threads = pl.octets == 3 ? us::TcShape<3>::kThreads : us::TcShape<2>::kThreads;
     // tiles of a warp: a CTA's stages may begin and end inside a tile
     const int64_t per_cta = (stages + n_cta - 1) / n_cta, tiles = (per_cta + n_stage - 1) / n_stage + (n_stage > 1 ? 1 : 0);
-    const int want = (int)std::min<int64_t>(24, 16 * tiles);   // slots worth having before the table gets its 32 copies
-    p.x_stages = 4;
-    while (p.x_stages > 2 && slots_for(p.x_stages, 8) < 16) --p.x_stages;
+    const int want = (int)std::min<int64_t>(3 * warps / 2, warps * tiles);   // slots worth having before the table gets its 32 copies
+    while (p.x_stages > 2 && slots_for(p.x_stages, 8) < warps) --p.x_stages;
     p.lut_rep = slots_for(p.x_stages, 32) >= want && per_cta >= 16 ? 32 : 8;
-    p.n_slots = std::min<int>(slots_for(p.x_stages, p.lut_rep), (int)(16 * tiles));
-    if (p.n_slots < 16) return;
+    p.n_slots = std::min<int>(slots_for(p.x_stages, p.lut_rep), (int)(warps * tiles));
+    if (p.n_slots < warps) return;
     pl.smem = fixed_for(p.x_stages, p.lut_rep) + p.n_slots * (int)p.slot_bytes;
     for (int64_t c = 0; c <= n_cta; ++c) p.cta_begin[c] = (uint32_t)(stages * c / n_cta);
     p.n_stage = n_stage; p.block_stages = (int32_t)block_stages;
@@ -443,8 +465,8 @@ cudaError_t enable_large_smem(int device, int bytes)
             const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
             if (e != cudaSuccess) return e;
         }
-    for (int bits = 0; bits < 8; ++bits)
-        if (const void* fn = us::kernel_tc((bits & 1) != 0, (bits & 2) != 0, (bits & 4) != 0)) {
+    for (int bits = 0; bits < 16; ++bits)
+        if (const void* fn = us::kernel_tc(bits & 8 ? 3 : 2, (bits & 1) != 0, (bits & 2) != 0, (bits & 4) != 0)) {
             const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
             if (e != cudaSuccess) return e;
         }
@@ -500,9 +522,9 @@ us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_sca
         }
         p.wait_ns_hi = h->wait_ns_hi;
         p.withhold = h->withhold;
-        const void* fn = us::kernel_tc(h->host.fmt.C_A == 2, h->host.w2, p.y_amax != nullptr);
+        const void* fn = us::kernel_tc(tc.octets, h->host.fmt.C_A == 2, h->host.w2, p.y_amax != nullptr);
         if (!fn) return US_ERR_UNSUPPORTED;
-        return launch(h, fn, &p, us::kTcThreads, tc.smem, st);
+        return launch(h, fn, &p, tc.threads, tc.smem, st);
     }
     const int cls = class_of(nt_for(N));
     const ClassPlan& pl = h->plan[cls];
@@ -713,7 +735,7 @@ us_status us_launch_info(const us_handle* h, int32_t N, int32_t* grid, int32_t* 
     if (!h->host.kernel_layout) return US_ERR_UNSUPPORTED;
     if (h->tc[(N + 7) / 8].ok) {
         if (grid) *grid = h->sm_count;
-        if (block) *block = us::kTcThreads;
+        if (block) *block = h->tc[(N + 7) / 8].threads;
         if (smem_bytes) *smem_bytes = h->tc[(N + 7) / 8].smem;
         return US_OK;
     }

@@ -6,32 +6,41 @@
 // sparsity: 24 us at N = 8, 32 at 16, 50 at 32, 87 at 64). Here a decoded k-block leaves the registers once,
 // whatever N is; X is read from shared memory by the tensor core; partial sums stay in tensor memory over all of K.
 //
-//   decode    warps 0..15 in two octets. A warp decodes 16-row tiles; the 8 tiles of an octet (same K segment) fill
+//   decode    warps 0..15 in two octets (or 0..23 in three). A warp decodes 16-row tiles; the 8 tiles of an octet (same K segment) fill
 //             the 128 lanes of one A operand: tcgen05.st.16x256b puts the lane's fragment bytes (rows g and g + 8,
 //             columns 8t .. 8t + 7) where the MMA expects them, so the lane-stream layout needs no change.
-//   MMA       warp 16: one thread issues m128 nN k32 kind::i8 MMAs, 8 per 256-column stage, A from tensor memory.
-//   X         warps 17..24 expand the packed INT4 activations 256 columns at a time into a ring of operand-layout
+//   MMA       one warp, one thread of it issues m128 nN k32 kind::i8 MMAs, 8 per 256-column stage, A from tensor memory.
+//   X         the last warps expand the packed INT4 activations 256 columns at a time into a ring of operand-layout
 //             stages (8-token groups x 16-byte k-columns), and sum them for the excess-8 correction.
 //   flush     when an octet's run of K segments of one 128-row group ends, its warps read the sums back
 //             (tcgen05.ld.16x256b gives mma.sync's accumulator layout) and store Y, or add to the split-K workspace.
 //
-// Work is cut in stages: 256 rows x 256 columns (two octets, which share the stage's activations). A CTA owns a
-// contiguous range of the (256-row block, column stage) order, the same number of stages for every CTA whatever the
+// Work is cut in stages: 256 (384) rows x 256 columns (the octets share the stage's activations). A CTA owns a
+// contiguous range of the (row block, column stage) order, the same number of stages for every CTA whatever the
 // tile width: a warp enters a tile at any mask word by counting the set bits of the words before it.
 // Tile copies form one ring of slots over the CTA's tiles in processing order; the warp that empties a slot refills
-// it for whichever warp comes next, so any number of slots from 16 on can be used.
+// it for whichever warp comes next, so any number of slots from one per warp on can be used.
 #pragma once
 #include "us_spmm_kernel.cuh"
 
 namespace us {
 
-constexpr int kTcDecodeWarps = 16, kTcXWarps = 8;
-constexpr int kTcThreads = 32 * (kTcDecodeWarps + 1 + kTcXWarps);
+// The CTA by number of octets: two, or three for N <= 32 (see the kernel).
+template <int OCT>
+struct TcShape {
+    static constexpr int kDecode = 8 * OCT;              // decode warps
+    static constexpr int kX = OCT == 2 ? 8 : 3;          // X warps
+    static constexpr int kPair = OCT == 2 ? 2 : 1;       // X warps that share a stage
+    static constexpr int kThreads = 32 * (kDecode + 1 + kX);
+    static constexpr int kA = OCT == 2 ? 3 : 2;          // A stages per octet, 64 tensor-memory columns (256 of K) each
+    static constexpr int kD = OCT == 2 ? 64 : 32;        // tensor-memory columns of an octet's sums: the most tokens
+    static_assert(OCT * (kA * 64 + kD) <= 512, "tensor memory");
+};
+constexpr int kTcMaxOct = 3, kTcMaxA = 3;
 constexpr int kTcMaxSlots = 64;
-constexpr int kTcAStages = 3;         // A stages per octet, 64 tensor-memory columns (256 columns of K) each
 constexpr int kTcMaxXStages = 4;
 constexpr int kTcSxRing = 16;         // row blocks whose activation sums are kept (see the X warps)
-constexpr int kTcBars = kTcMaxSlots + 2 * 2 * kTcAStages + 2 * kTcMaxXStages + 4;
+constexpr int kTcBars = kTcMaxSlots + 2 * kTcMaxOct * kTcMaxA + 2 * kTcMaxXStages + kTcMaxOct + 1;
 constexpr int kTcMiscWords = 96 + kTcMaxSlots;
 constexpr int kTcFixedSmem = kTcSxRing * 64 * 4 + kTcBars * 8 + kTcMiscWords * 4 + 1024;
 
@@ -48,11 +57,11 @@ struct TcParams {
     uint32_t* err;
     int32_t M, K, N;
     int32_t n_strips, n_segs;
-    unsigned long long mg_segs, mg_block;   // floor(2^40 / d) + 1 for d = n_segs, stages per 256-row block
-    int32_t n_stage, block_stages;          // stages per tile, per 256-row block
+    unsigned long long mg_segs, mg_block;   // floor(2^40 / d) + 1 for d = n_segs, stages per row block
+    int32_t n_stage, block_stages;          // stages per tile, per row block
     int32_t mask_rows, K_L;
     uint32_t slot_bytes;
-    int32_t n_slots;              // ring slots, 16 .. kTcMaxSlots
+    int32_t n_slots;              // ring slots, one per decode warp .. kTcMaxSlots
     int32_t x_stages;             // X stages in the ring
     int32_t lut_rep;
     int32_t acc_nt;               // n-tiles of the workspace's strip layout
@@ -240,10 +249,17 @@ __device__ __noinline__ void store_block_tc(const StoreCtx& p, int v0, int v1, i
     store_rows<1, AM>(p, v, lane, m_lo, m_hi, nullptr, -2, n_base);
 }
 
-template <int CA, bool W2, bool AM>
-__global__ void __launch_bounds__(kTcThreads, 1) us_spmm_tc_kernel(const __grid_constant__ TcParams p)
+// OCT = 3: 24 decode warps, 384 rows to a stage, for N <= 32 (the sums of three octets of 64 tokens and two A stages each do
+// not fit tensor memory, nor 24 tile slots beside wide X stages shared memory). With 16 decode warps 0.59
+// instructions issue per cycle and scheduler; eight more warps hide more of the decode's latency (28672 x 8192, N = 16:
+// 29.3 -> 28.0 us, with INT2 weights 25.7 -> 24.7).
+template <int OCT, int CA, bool W2, bool AM>
+__global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(const __grid_constant__ TcParams p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
+    using S = TcShape<OCT>;
+    constexpr int kTcDecodeWarps = S::kDecode, kTcXWarps = S::kX, kTcAStages = S::kA;
+    constexpr uint32_t kDW = (uint32_t)S::kDecode;
     // (the warp number through a shuffle: the compiler then knows it to be the same in all lanes)
     const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
     const int ng = (p.N + 7) >> 3;                       // 8-token groups
@@ -259,9 +275,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) us_spmm_tc_kernel(const __grid_
     uint32_t* issued = misc + 96;                                   // phases started per slot
     uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(issued + kTcMaxSlots) + 127) & ~uintptr_t(127));
     const uint32_t bar0 = smem_u32(bars);
-    const uint32_t b_w = bar0, b_af = bar0 + 8 * kTcMaxSlots, b_ae = b_af + 8 * 2 * kTcAStages,
-                   b_xf = b_ae + 8 * 2 * kTcAStages, b_xe = b_xf + 8 * kTcMaxXStages, b_d = b_xe + 8 * kTcMaxXStages,
-                   b_drain = b_d + 16;
+    const uint32_t b_w = bar0, b_af = bar0 + 8 * kTcMaxSlots, b_ae = b_af + 8 * OCT * kTcAStages,
+                   b_xf = b_ae + 8 * OCT * kTcAStages, b_xe = b_xf + 8 * kTcMaxXStages, b_d = b_xe + 8 * kTcMaxXStages,
+                   b_drain = b_d + 8 * OCT;
     volatile uint32_t* dead = misc + 1;
 
     const uint32_t beg = p.cta_begin[blockIdx.x], end = p.cta_begin[blockIdx.x + 1];
@@ -274,7 +290,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) us_spmm_tc_kernel(const __grid_
         }
         return;
     }
-    // first stage of the range: 256-row block q0, segment seg0, stage st0 of its tiles; then stage by stage
+    // first stage of the range: row block q0 of 16 kDW rows, segment seg0, stage st0 of its tiles; then stage by stage
     const int n_stage = p.n_stage, total = (int)(end - beg);
     const int q0 = (int)fdiv(beg, p.mg_block), in_block = (int)beg - q0 * p.block_stages;
     const int seg0 = in_block / n_stage, st0 = in_block - seg0 * n_stage;
@@ -282,13 +298,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) us_spmm_tc_kernel(const __grid_
     const uint32_t n_tile = (uint32_t)((st0 + total + n_stage - 1) / n_stage);      // tiles of a warp
 
     const uint64_t w_policy = l2_evict_first_policy();
-    // Tile t of the CTA: warp t % 16, that warp's t / 16-th. Returns the tile index, kNull for a strip past the matrix
+    // Tile t of the CTA: warp t % kDW, that warp's t / kDW-th. Returns the tile index, kNull for a strip past the matrix
     // (its slot's phase is completed without a copy), kNone past the CTA's last tile.
     constexpr uint32_t kNone = 0xFFFFFFFFu, kNull = 0xFFFFFFFEu;
     auto tile_at = [&](uint32_t t) -> uint32_t {
-        if ((t >> 4) >= n_tile) return kNone;
-        const uint32_t u = tile0 + (t >> 4), q = fdiv(u, p.mg_segs), seg = u - q * (uint32_t)p.n_segs;
-        const uint32_t strip = 16u * q + (t & 15u);
+        if (t / kDW >= n_tile) return kNone;
+        const uint32_t u = tile0 + t / kDW, q = fdiv(u, p.mg_segs), seg = u - q * (uint32_t)p.n_segs;
+        const uint32_t strip = kDW * q + t % kDW;
         return strip < (uint32_t)p.n_strips ? strip * (uint32_t)p.n_segs + seg : kNull;
     };
     auto copy_tile = [&](uint32_t tile, uint32_t o0, uint32_t o1, uint32_t slot) {   // one lane
@@ -303,10 +319,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) us_spmm_tc_kernel(const __grid_
     // ---- prologue: first copies, barriers, tensor memory, selector table --------------------------------
     // lane j of a decode warp: the first copy into the warp's j-th slot. Only the warps' first tiles are requested at
     // once (they would otherwise arrive no sooner than everything the ring holds), the rest when those have arrived.
-    const uint32_t t_first = (uint32_t)(warp + 16 * lane);
+    const uint32_t t_first = (uint32_t)warp + kDW * (uint32_t)lane;
     uint32_t tile_first = kNone, of0 = 0, of1 = 0;
     if (warp < kTcDecodeWarps) {
-        if (lane < kTcMaxSlots / 16 && t_first < (uint32_t)p.n_slots) {
+        if (t_first < (uint32_t)p.n_slots) {
             tile_first = tile_at(t_first);
             if (tile_first < kNull) { of0 = __ldg(p.item_off + tile_first); of1 = __ldg(p.item_off + tile_first + 1); }
             mbar_init(b_w + 8u * t_first, 1);
@@ -316,15 +332,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) us_spmm_tc_kernel(const __grid_
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         if (tile_first != kNone && lane == 0) copy_tile(tile_first, of0, of1, t_first);
         // selector table: entry e by two threads, each writing half of its copies (conflict-free rotation)
-        const int e = threadIdx.x & 255, half = threadIdx.x >> 8, n_half = p.lut_rep / 2;
-        const uint32_t v = lut_entry(e);
-        const int rot = p.lut_rep == 32 ? lane : lane >> 2;
+        const int e = threadIdx.x & 255, part = threadIdx.x >> 8;
+        if (part < 2) {
+            const int n_half = p.lut_rep / 2;
+            const uint32_t v = lut_entry(e);
+            const int rot = p.lut_rep == 32 ? lane : lane >> 2;
 #pragma unroll 1
-        for (int i = 0; i < n_half; ++i) lut[e * p.lut_rep + ((rot + i + half * n_half) & (p.lut_rep - 1))] = v;
+            for (int i = 0; i < n_half; ++i) lut[e * p.lut_rep + ((rot + i + part * n_half) & (p.lut_rep - 1))] = v;
+        }
     } else if (warp == kTcDecodeWarps) {
-        if (lane < 2 * kTcAStages) { mbar_init(b_af + 8u * lane, 8); mbar_init(b_ae + 8u * lane, 1); }
-        if (lane < kTcMaxXStages) { mbar_init(b_xf + 8u * lane, 2); mbar_init(b_xe + 8u * lane, 1); }
-        if (lane < 3) mbar_init(b_d + 8u * lane, 1);   // (and b_drain)
+        if (lane < OCT * kTcAStages) { mbar_init(b_af + 8u * lane, 8); mbar_init(b_ae + 8u * lane, 1); }
+        if (lane < kTcMaxXStages) { mbar_init(b_xf + 8u * lane, S::kPair); mbar_init(b_xe + 8u * lane, 1); }
+        if (lane <= OCT) mbar_init(b_d + 8u * lane, 1);   // (and b_drain)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (lane == 0) { misc[1] = 0; misc[2] = 0; }
         __syncwarp();
@@ -342,8 +361,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) us_spmm_tc_kernel(const __grid_
     tc_fence_after();
     const uint32_t tm = *(volatile uint32_t*)misc;
     const uint32_t n16 = (uint32_t)(p.N + 15) / 16u;        // 16-token blocks
-    // tensor-memory columns: the A stages of the two octets, then their sums
-    const uint32_t tm_d = tm + 2u * kTcAStages * 64u;       // + o * 64
+    // tensor-memory columns: the A stages of the octets, then their sums
+    const uint32_t tm_d = tm + OCT * kTcAStages * 64u;      // + o * S::kD
 
     bool ok = true;
     if (warp < kTcDecodeWarps) {
@@ -368,10 +387,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) us_spmm_tc_kernel(const __grid_
         constexpr int WPS = CA == 1 ? 2 : 1;  // mask words per stage
 
         for (uint32_t i = 0; left > 0; ++i) {
-            const uint32_t strip = 16u * (uint32_t)q + (uint32_t)warp;
+            const uint32_t strip = kDW * (uint32_t)q + (uint32_t)warp;
             const bool valid = strip < (uint32_t)p.n_strips;
             // offsets of the tile that will take over this slot, fetched behind the decode
-            const uint32_t tile_next = tile_at(16u * i + (uint32_t)warp + (uint32_t)p.n_slots);
+            const uint32_t tile_next = tile_at(kDW * i + (uint32_t)warp + (uint32_t)p.n_slots);
             uint32_t no0 = 0, no1 = 0;
             if (lane == 0 && tile_next < kNull) { no0 = __ldg(p.item_off + tile_next); no1 = __ldg(p.item_off + tile_next + 1); }
             const uint32_t slot_a = smem_u32(ring + (size_t)slot * p.slot_bytes) + 4u * lane;
@@ -425,7 +444,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) us_spmm_tc_kernel(const __grid_
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 copy_tile(tile_next, no0, no1, slot);
             }
-            slot += 16;
+            slot += kDW;
             while (slot >= (uint32_t)p.n_slots) { slot -= (uint32_t)p.n_slots; ++pass; }
             left -= n_here;
             run_stages += n_here;
@@ -453,7 +472,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) us_spmm_tc_kernel(const __grid_
 #pragma unroll 1
                 for (int nt = 0; nt < ng; ++nt) {
                     int c[4], y[4];
-                    tc_ld4(tm_d + 64u * o + 8u * nt + lane_base, c);
+                    tc_ld4(tm_d + (uint32_t)(S::kD * o) + 8u * nt + lane_base, c);
                     const int s0 = sxp[8 * nt] >> 4, s1 = sxp[8 * nt + 1] >> 4;
                     if (W2) {
                         y[0] = (c[2] >> 4) - 2 * s0;
@@ -527,11 +546,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) us_spmm_tc_kernel(const __grid_
             ok = tc_wait_warp(b_xf + 8u * xst, x_par, p.wait_ns_hi, dead);
             const uint64_t b = bd0 + (uint64_t)((xst * x_stage_bytes) >> 4);
 #pragma unroll
-            for (int o = 0; o < 2; ++o) {
+            for (int o = 0; o < OCT; ++o) {
                 if (ok) ok = tc_wait_warp(b_af + 8u * (o * kTcAStages + as), a_par, p.wait_ns_hi, dead);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t a = tm + (uint32_t)o * kTcAStages * 64u + 64u * as, d = tm_d + 64u * o;
+                const uint32_t a = tm + (uint32_t)o * kTcAStages * 64u + 64u * as, d = tm_d + (uint32_t)(S::kD * o);
 #pragma unroll
                 for (uint32_t j = 0; j < 4; ++j) tc_mma_i8(leader, d, a + 8u * j, b + 16u * j, idesc, j == 0 ? more : 1u);
                 if (!half)
@@ -553,10 +572,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) us_spmm_tc_kernel(const __grid_
         __syncwarp();
     } else {
         // ================= X warps =================
-        // Whole stages in turn, so that the loads of several stages are in flight at once; two warps share a stage (even and
-        // odd token groups). (No more stages at once than the ring has: a warp one pass of the ring ahead could not tell the
+        // Whole stages in turn, so that the loads of several stages are in flight at once; with two octets two warps share a stage
+        // (even and odd token groups). (No more stages at once than the ring has: a warp one pass of the ring ahead could not tell the
         // barrier's phases apart.)
-        const int xw = warp - kTcDecodeWarps - 1, c0 = xw >> 1, W = min(kTcXWarps / 2, p.x_stages), g0 = xw & 1;
+        constexpr int P = S::kPair;
+        const int xw = warp - kTcDecodeWarps - 1, c0 = xw / P, W = min(kTcXWarps / P, p.x_stages), g0 = xw % P;
         const int64_t ldx = ((int64_t)p.K + 1) / 2;
         const int r = lane & 7, qq = lane >> 3;
         int xst = c0, q = q0, seg = seg0, st = st0 + c0;
@@ -575,13 +595,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) us_spmm_tc_kernel(const __grid_
             uint8_t* dst0 = xs + (size_t)xst * x_stage_bytes + g0 * 2048 + (2 * qq) * 128 + r * 16;
             int32_t* sxr = sx + ((q - q0) % kTcSxRing) * 64;
             uint4 v0 = load_x32(p, ldx, 8 * g0 + r, k0), v1 = load_x32(p, ldx, 8 * g0 + r, k1);
-            uint4 n0 = load_x32(p, ldx, 8 * g0 + 16 + r, k0), n1 = load_x32(p, ldx, 8 * g0 + 16 + r, k1);
+            uint4 n0 = load_x32(p, ldx, 8 * (g0 + P) + r, k0), n1 = load_x32(p, ldx, 8 * (g0 + P) + r, k1);
             ok = tc_wait_warp(b_xe + 8u * xst, x_par, p.wait_ns_hi, dead);
             if (!ok) break;
 #pragma unroll 1
-            for (int g = g0; g < ng; g += 2) {
+            for (int g = g0; g < ng; g += P) {
                 uint4 f0 = make_uint4(0, 0, 0, 0), f1 = f0;   // two groups ahead
-                if (g + 4 < ng) { f0 = load_x32(p, ldx, (g + 4) * 8 + r, k0); f1 = load_x32(p, ldx, (g + 4) * 8 + r, k1); }
+                if (g + 2 * P < ng) { f0 = load_x32(p, ldx, (g + 2 * P) * 8 + r, k0); f1 = load_x32(p, ldx, (g + 2 * P) * 8 + r, k1); }
                 int s = 0;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -596,7 +616,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) us_spmm_tc_kernel(const __grid_
                     dst[0] = a;
                     dst[8] = b;
                 }
-                dst0 += 4096;
+                dst0 += 2048 * P;
                 s += __shfl_xor_sync(0xffffffffu, s, 8);
                 s += __shfl_xor_sync(0xffffffffu, s, 16);
                 if (lane < 8) atomicAdd(sxr + g * 8 + lane, s);

@@ -33,7 +33,7 @@ def run_edges():
         X = workloads.make_x(K, N, seed=N)
         s_w, s_x = workloads.make_scales(M, N, seed=M)
         sw = b.SparseWeight(W, s_w, fmt=fmt, max_N=N, flags=flags)
-        assert b.us_launch_info(sw.handle, N)["block"] == 800
+        assert b.us_launch_info(sw.handle, N)["block"] in (800, 896)
         Xd, xs = torch.from_numpy(b.pack_int4(X)).cuda(), torch.from_numpy(s_x.copy()).cuda()
         ref = oracle.spmm_dense(W, X)
         for _ in range(2):     # the second call checks the self-cleaning workspace
@@ -51,9 +51,10 @@ def run_edges():
         sw.close()
 
 
-def test_edges_forced():
+@pytest.mark.parametrize("octets", ["2", "3"])
+def test_edges_forced(octets):
     r = subprocess.run([sys.executable, "-c", "import sys; sys.path[:0] = ['.', 'tests']; import test_gpu_tc; test_gpu_tc.run_edges()"],
-                       cwd=ROOT, env=dict(os.environ, US_TC="2"), capture_output=True, text=True, timeout=600)
+                       cwd=ROOT, env=dict(os.environ, US_TC="2", US_TC_OCT=octets), capture_output=True, text=True, timeout=600)
     assert r.returncode == 0, r.stdout[-1500:] + r.stderr[-1500:]
 
 
