@@ -434,7 +434,6 @@ void build_tc_plan(us_handle* h, int ng)
     p.mg_segs = ((1ull << 40) / (uint64_t)hm.n_segs) + 1ull;
     p.mask_rows = hm.mask_rows; p.K_L = hm.fmt.K_L;
     p.acc_nt = nt_for(8 * ng);
-    p.x_fast = hm.K % 32 == 0;
     pl.ok = true;
 }
 
@@ -465,8 +464,8 @@ cudaError_t enable_large_smem(int device, int bytes)
             const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
             if (e != cudaSuccess) return e;
         }
-    for (int bits = 0; bits < 16; ++bits)
-        if (const void* fn = us::kernel_tc(bits & 8 ? 3 : 2, (bits & 1) != 0, (bits & 2) != 0, (bits & 4) != 0)) {
+    for (int bits = 0; bits < 32; ++bits)
+        if (const void* fn = us::kernel_tc(bits & 8 ? 3 : 2, (bits & 16) != 0, (bits & 1) != 0, (bits & 2) != 0, (bits & 4) != 0)) {
             const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
             if (e != cudaSuccess) return e;
         }
@@ -522,7 +521,7 @@ us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_sca
         }
         p.wait_ns_hi = h->wait_ns_hi;
         p.withhold = h->withhold;
-        const void* fn = us::kernel_tc(tc.octets, h->host.fmt.C_A == 2, h->host.w2, p.y_amax != nullptr);
+        const void* fn = us::kernel_tc(tc.octets, h->host.K % 32 != 0, h->host.fmt.C_A == 2, h->host.w2, p.y_amax != nullptr);
         if (!fn) return US_ERR_UNSUPPORTED;
         return launch(h, fn, &p, tc.threads, tc.smem, st);
     }

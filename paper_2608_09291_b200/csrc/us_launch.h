@@ -21,7 +21,7 @@ const void* kernel_nt2(const KernelKey& k);
 const void* kernel_nt4(const KernelKey& k);
 const void* kernel_nt8(const KernelKey& k);
 
-// us_spmm_tc_kernel (us_spmm_tc.cu) with two or three octets: fold = two column areas; am = absmax of the output (default format only).
-const void* kernel_tc(int octets, bool fold, bool w2, bool am);
+// us_spmm_tc_kernel (us_spmm_tc.cu) with two or three octets: any_k = K is not a multiple of 32; fold = two column areas; am = absmax of the output (default format only).
+const void* kernel_tc(int octets, bool any_k, bool fold, bool w2, bool am);
 
 }  // namespace us

@@ -65,7 +65,6 @@ struct TcParams {
     int32_t x_stages;             // X stages in the ring
     int32_t lut_rep;
     int32_t acc_nt;               // n-tiles of the workspace's strip layout
-    int32_t x_fast;               // K % 32 == 0: 16-byte loads
     int32_t fp16_out;
     uint32_t* y_amax;
     int32_t amax_m0, amax_m1;
@@ -199,44 +198,61 @@ __device__ __forceinline__ void decode_word(uint32_t mw, uint32_t pay_a, uint32_
     for (int s = 0; s < SR; ++s) { cw0[s] = w0[s][3]; cw1[s] = w1[s][3]; }
 }
 
-// 32 packed activations from byte address b of X on (column k of a token, a multiple of 32), `nv` columns of them valid
-// and the rest zero; X holds `total` bytes. Any K: rows start at any byte, so aligned words are shifted into place. Out
-// of line: the code of a CTA's first pass is fetched line by line, so what few shapes need stays away.
-inline __device__ __noinline__ uint4 load_x32_any(const uint8_t* X, int64_t total, int64_t b, int nv)
+// 32 packed activations of token n from column k (a multiple of 32) on; columns from K on are zero. Where K is not a
+// multiple of 32 rows start at any byte: two aligned 16-byte loads hold the unit (in flight from here on: volatile, not
+// sunk to their use), and unit_x shifts it into place. The end of a row, or of X, is fetched byte by byte out of line.
+struct UnitX {
+    uint4 lo, hi;
+};
+inline __device__ __noinline__ uint4 load_x_tail(const uint8_t* src, int left)
 {
-    nv = min(32, nv);
-    const int64_t b4 = b & ~(int64_t)3, last = b + (nv - 1) / 2;
-    uint32_t w[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        const int64_t a = b4 + 4 * i;
-        w[i] = 0;
-        if (a <= last) {
-            if (a + 4 <= total) w[i] = __ldg(reinterpret_cast<const uint32_t*>(X + a));
-            else for (int j = 0; a + j < total; ++j) w[i] |= (uint32_t)X[a + j] << (8 * j);   // the end of X
-        }
-    }
-    const uint32_t sh = 8u * (uint32_t)(b & 3);
     uint32_t o[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        o[i] = __funnelshift_r(w[i], w[i + 1], sh);
-        const int left = nv - 8 * i;   // valid columns of this word
-        if (left < 8) o[i] = left <= 0 ? 0u : o[i] & ((1u << (4 * left)) - 1u);
+        o[i] = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int c = left - 8 * i - 2 * j;   // columns left at this byte
+            if (c > 0) o[i] |= (src[4 * i + j] & (c > 1 ? 255u : 15u)) << (8 * j);
+        }
     }
     return make_uint4(o[0], o[1], o[2], o[3]);
 }
-
-// 32 packed activations of token n from column k on.
-__device__ __forceinline__ uint4 load_x32(const TcParams& p, int64_t ldx, int n, int k)
+__device__ __forceinline__ uint4 ldg_now(const uint8_t* a)
 {
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (n >= p.N || k >= p.K) return v;
-    const int64_t b = (int64_t)n * ldx + (k >> 1);
-    if (!p.x_fast) return load_x32_any(p.X, (int64_t)p.N * ldx, b, p.K - k);
-    // (volatile: the load is to be in flight from here on, not sunk to its use)
-    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p.X + b));
+    uint4 v;
+    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(a));
     return v;
+}
+template <bool ANY>
+__device__ __forceinline__ UnitX load_x32(const TcParams& p, int64_t ldx, int n, int k)
+{
+    UnitX u;
+    u.lo = u.hi = make_uint4(0, 0, 0, 0);
+    if (n >= p.N || k >= p.K) return u;
+    const int64_t b = (int64_t)n * ldx + (k >> 1);
+    if (!ANY) {
+        u.lo = ldg_now(p.X + b);
+    } else if (p.K - k >= 32 && (b & ~(int64_t)15) + 32 <= (int64_t)p.N * ldx) {
+        u.lo = ldg_now(p.X + (b & ~(int64_t)15));
+        u.hi = ldg_now(p.X + (b & ~(int64_t)15) + 16);
+    } else {
+        u.lo = load_x_tail(p.X + b, p.K - k);
+    }
+    return u;
+}
+template <bool ANY>
+__device__ __forceinline__ uint4 unit_x(const TcParams& p, int64_t ldx, int n, int k, const UnitX& u)
+{
+    if (!ANY) return u.lo;
+    const int64_t b = (int64_t)n * ldx + (k >> 1);
+    if (p.K - k < 32 || (b & ~(int64_t)15) + 32 > (int64_t)p.N * ldx) return u.lo;
+    uint32_t w[7] = {u.lo.x, u.lo.y, u.lo.z, u.lo.w, u.hi.x, u.hi.y, u.hi.z};
+    if (b & 8) { w[0] = w[2]; w[1] = w[3]; w[2] = w[4]; w[3] = w[5]; w[4] = w[6]; w[5] = u.hi.w; }
+    if (b & 4) { w[0] = w[1]; w[1] = w[2]; w[2] = w[3]; w[3] = w[4]; w[4] = w[5]; }
+    const uint32_t sh = 8u * (uint32_t)(b & 3);
+    return make_uint4(__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh), __funnelshift_r(w[2], w[3], sh),
+                      __funnelshift_r(w[3], w[4], sh));
 }
 
 // Stores the 16 x 8 results of one 8-token block (store_rows). Out of line, like everything that runs once or twice per
@@ -249,11 +265,12 @@ __device__ __noinline__ void store_block_tc(const StoreCtx& p, int v0, int v1, i
     store_rows<1, AM>(p, v, lane, m_lo, m_hi, nullptr, -2, n_base);
 }
 
+// ANY: K is not a multiple of 32 (load_x32).
 // OCT = 3: 24 decode warps, 384 rows to a stage, for N <= 32 (the sums of three octets of 64 tokens and two A stages each do
 // not fit tensor memory, nor 24 tile slots beside wide X stages shared memory). With 16 decode warps 0.59
 // instructions issue per cycle and scheduler; eight more warps hide more of the decode's latency (28672 x 8192, N = 16:
 // 29.3 -> 28.0 us, with INT2 weights 25.7 -> 24.7).
-template <int OCT, int CA, bool W2, bool AM>
+template <int OCT, int CA, bool W2, bool AM, bool ANY>
 __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(const __grid_constant__ TcParams p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -594,18 +611,25 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
             const int k1 = CA == 1 && 2 * st + 1 >= p.mask_rows ? p.K : k0 + k_second;
             uint8_t* dst0 = xs + (size_t)xst * x_stage_bytes + g0 * 2048 + (2 * qq) * 128 + r * 16;
             int32_t* sxr = sx + ((q - q0) % kTcSxRing) * 64;
-            uint4 v0 = load_x32(p, ldx, 8 * g0 + r, k0), v1 = load_x32(p, ldx, 8 * g0 + r, k1);
-            uint4 n0 = load_x32(p, ldx, 8 * (g0 + P) + r, k0), n1 = load_x32(p, ldx, 8 * (g0 + P) + r, k1);
+            UnitX v0 = load_x32<ANY>(p, ldx, 8 * g0 + r, k0), v1 = load_x32<ANY>(p, ldx, 8 * g0 + r, k1);
+            UnitX n0, n1;   // a group ahead
+            if (!ANY) { n0 = load_x32<ANY>(p, ldx, 8 * (g0 + P) + r, k0); n1 = load_x32<ANY>(p, ldx, 8 * (g0 + P) + r, k1); }
             ok = tc_wait_warp(b_xe + 8u * xst, x_par, p.wait_ns_hi, dead);
             if (!ok) break;
 #pragma unroll 1
             for (int g = g0; g < ng; g += P) {
-                uint4 f0 = make_uint4(0, 0, 0, 0), f1 = f0;   // two groups ahead
-                if (g + 2 * P < ng) { f0 = load_x32(p, ldx, (g + 2 * P) * 8 + r, k0); f1 = load_x32(p, ldx, (g + 2 * P) * 8 + r, k1); }
+                // the group after next, or (any K: twice the registers) the next
+                constexpr int kAhead = ANY ? 1 : 2;
+                UnitX f0, f1;
+                f0.lo = f0.hi = f1.lo = f1.hi = make_uint4(0, 0, 0, 0);
+                if (g + kAhead * P < ng) {
+                    f0 = load_x32<ANY>(p, ldx, (g + kAhead * P) * 8 + r, k0);
+                    f1 = load_x32<ANY>(p, ldx, (g + kAhead * P) * 8 + r, k1);
+                }
                 int s = 0;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const uint4 v = h ? v1 : v0;
+                    const uint4 v = unit_x<ANY>(p, ldx, 8 * g + r, h ? k1 : k0, h ? v1 : v0);
                     uint4 a, b;
                     uint2 t;
                     t = expand8(v.x, s); a.x = t.x; a.y = t.y;
@@ -620,7 +644,8 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
                 s += __shfl_xor_sync(0xffffffffu, s, 8);
                 s += __shfl_xor_sync(0xffffffffu, s, 16);
                 if (lane < 8) atomicAdd(sxr + g * 8 + lane, s);
-                v0 = n0; v1 = n1; n0 = f0; n1 = f1;
+                if (ANY) { v0 = f0; v1 = f1; }
+                else { v0 = n0; v1 = n1; n0 = f0; n1 = f1; }
             }
             // the row block's last stage: clear the sums of the block eight further on (those of the block eight back, which
             // shared their place, were read long ago)
