@@ -92,6 +92,8 @@ constexpr int kLocalAccBudget = 32 * 1024;   // local strip sums a K-range width
 constexpr int kLocalAccCap = 48 * 1024;      // ... and what is taken if nothing fits that
 constexpr int kMinWarps = 12;                // warps the automatic K-range choice keeps room for
 constexpr int kCoresidentTiles = 16;         // most tiles per CTA for the half-SM plan
+constexpr int kCoresidentK = 5120;           // ... and widest K: its few threads stage all of X (N = 8, half SM / whole: 2304 x 8192 6.8 / 5.9 us,
+                                             // 2304 x 6144 6.4 / 5.6, 4096 x 4096 4.6 / 5.6)
 constexpr int kHalfSmBytes = 228 * 1024 / 2 - 1024 - 512;   // shared memory of a half-SM CTA: 228 KB per SM, 1 KB reserved per CTA
 
 // Segments per K range for an N class. The int8 activations of one K range live in shared memory
@@ -177,26 +179,28 @@ bool plan_launch(const us_handle* h, int N, LaunchGeom* g)
     // Measured on 4096 x 4096, N = 8: 6.6 -> 5.7 us; not worth it from ~20 tiles per CTA on.
     const int64_t n_cta = h->sm_count > 0 ? h->sm_count : 148;
     const int64_t per_cta = (h->host.n_items + n_cta - 1) / n_cta;
+    // the most tiles a CTA has: cuts fall on strip boundaries, so it can be more than the average (5008 x 3008, 3 tiles to a
+    // strip: most CTAs have two strips, some three, and eight warps would need a second round for the ninth tile: 5.7 us
+    // against 5.2 with 16 warps on the whole SM; 3000 x 6000 11.7 against 8.7; 512 x 8192, where 32 CTAs have a strip of 32
+    // tiles each and the others none: 8.9 against 5.8)
+    int64_t most = per_cta;
+    for (size_t c = 0; c + 1 < h->cta_begin[g->cls].size(); ++c)
+        most = std::max<int64_t>(most, (int64_t)h->cta_begin[g->cls][c + 1] - h->cta_begin[g->cls][c]);
     int fixed = fixed_base + 32 * stages * 8;
     // (N = 9..16 too, where the plan stages X packed and in local mode: that kernel is as lean.)
     // (Tried at N = 32 as well: 8 warps per CTA, slower.)
     const bool co_class = g->nt == 1 || (g->nt == 2 && g->xp && s_local > 0);
-    if (coresident_knob() && co_class && per_cta <= kCoresidentTiles && stages_knob() == 0) {
+    if (coresident_knob() && co_class && most <= kCoresidentTiles && stages_knob() == 0 && h->host.Kp <= kCoresidentK) {
         const int half = kHalfSmBytes;
         const int fixed8 = fixed_for(8) + 32 * 8;
         const bool fold = h->host.fmt.C_A == 2;
         int w = std::min(g->nt == 1 ? (fold ? h->co_warps_fold : h->co_warps) : h->co_warps2,
                          (g->nt == 1 && !fold) ? max_warps() : std::min(16, max_warps()));
         while (w >= 8 && fixed8 + w * (int)g->slot_bytes > half) --w;
-        // the most tiles a CTA has: cuts fall on strip boundaries, so it can be more than the average (5008 x 3008, 3 tiles to a
-        // strip: most CTAs have two strips, some three, and eight warps would need a second round for the ninth tile: 5.7 us
-        // against 5.2 with 16 warps on the whole SM; 3000 x 6000 11.7 against 8.7)
-        int64_t most = per_cta;
-        for (size_t c = 0; c + 1 < h->cta_begin[g->cls].size(); ++c)
-            most = std::max<int64_t>(most, (int64_t)h->cta_begin[g->cls][c + 1] - h->cta_begin[g->cls][c]);
-        // (only if nearly every tile of the CTA finds a warp at once: 5120 x 5120 at 70 % sparsity, N = 16, has 11
-        // tiles per CTA and room for 8 half-SM warps: 9.9 us against 8.9 with 16 warps on the whole SM)
-        if (w >= 8 && w >= std::min<int64_t>(most, 10)) { stages = 1; lut_rep = 8; warps = w; fixed = fixed8; }
+        // (only if every tile of the CTA finds a warp at once: 5120 x 5120 at 70 % sparsity, N = 16, has 11 tiles per CTA
+        // and room for 8 half-SM warps: 9.9 us against 8.9 with 16 warps on the whole SM; 1500 x 6000 has 12 and room for 10:
+        // N = 8 8.6 against 6.0)
+        if (w >= 8 && w >= most) { stages = 1; lut_rep = 8; warps = w; fixed = fixed8; }
     }
     g->stages = stages;
     g->lut_rep = lut_rep;
@@ -262,7 +266,7 @@ void plan_classes(us_handle* h, int n_cta, std::vector<uint32_t> (&sched)[4])
             // (4096 x 4096 at 30 % sparsity: tiles of 9.5 KB and 32 KB of int8 X do not fit half an SM, with
             // 16 KB of packed X they do: 5.6 -> 4.6 us; the same for the folded format at 50 %: 5.3 -> 4.35)
             bool for_half_sm = false;
-            if (nt == 1 && ranges == 1 && coresident_knob()) {
+            if (nt == 1 && ranges == 1 && coresident_knob() && h->host.Kp <= kCoresidentK) {
                 const int64_t per_cta = (h->host.n_items + n_cta - 1) / std::max(1, n_cta);
                 const int64_t need = 8;
                 auto fits = [&](bool xp, int s_loc) {

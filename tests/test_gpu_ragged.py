@@ -31,10 +31,16 @@ def test_any_k(K, fmt):
 
 
 def test_plan_counts_the_largest_share():
-    """5008 x 3008 has CTAs of nine tiles: all its warps at once, not eight in half an SM; 4096 x 4096 has eight."""
+    """512 x 8192 (one strip of 32 tiles to a CTA) and 1500 x 6000 (12 tiles): all warps of the SM; 4096 x 4096 (eight
+    tiles) and 2304 x 4096 (one strip to a CTA, none gets two): half an SM."""
     from paper_2608_09291_b200 import binding as b
-    for M, K, wide in ((5008, 3008, True), (4096, 4096, False)):
+    for M, K, wide in ((512, 8192, True), (1500, 6000, True), (4096, 4096, False), (2304, 4096, False)):
         W = workloads.make_weight(M, K, 0.5, seed=1)
-        h = b.us_encode(W, fmt=(16, 1024, 2, 2), max_N=8)
-        assert (b.us_launch_info(h, 8)["block"] > 384) == wide
-        b.us_destroy(h)
+        X = workloads.make_x(K, 8, seed=1)
+        sw = b.SparseWeight(W, max_N=8)
+        info = b.us_launch_info(sw.handle, 8)
+        assert (info["smem_bytes"] > 114 * 1024 or info["block"] > 384) == wide, (M, K, info)
+        y = sw.spmm(torch.from_numpy(b.pack_int4(X)).cuda(), 8).cpu().numpy()
+        sw.check()
+        assert (y == oracle.spmm_dense(W, X)).all(), (M, K)
+        sw.close()
