@@ -94,6 +94,9 @@ constexpr int kMinWarps = 12;                // warps the automatic K-range choi
 constexpr int kCoresidentTiles = 16;         // most tiles per CTA for the half-SM plan
 constexpr int kCoresidentK = 5120;           // ... and widest K: its few threads stage all of X (N = 8, half SM / whole: 2304 x 8192 6.8 / 5.9 us,
                                              // 2304 x 6144 6.4 / 5.6, 4096 x 4096 4.6 / 5.6)
+// The same where K is not a multiple of 32 and staging takes a thread one unit at a time (half SM / whole: N = 8
+// 1500 x 4500 6.7 / 5.8 (N = 1, which shares the plan, 5.3 / 5.6), 2304 x 4500 7.3 / 6.5, 2304 x 3000 5.5 / 5.4; N = 1 there 4.4 / 5.2; N = 16 5003 x 3001 9.0 / 8.0).
+int64_t coresident_K(int64_t K, int nt) { return K % 32 == 0 ? kCoresidentK : nt == 1 ? 3072 : 2048; }
 constexpr int kHalfSmBytes = 228 * 1024 / 2 - 1024 - 512;   // shared memory of a half-SM CTA: 228 KB per SM, 1 KB reserved per CTA
 
 // Segments per K range for an N class. The int8 activations of one K range live in shared memory
@@ -190,7 +193,7 @@ bool plan_launch(const us_handle* h, int N, LaunchGeom* g)
     // (N = 9..16 too, where the plan stages X packed and in local mode: that kernel is as lean.)
     // (Tried at N = 32 as well: 8 warps per CTA, slower.)
     const bool co_class = g->nt == 1 || (g->nt == 2 && g->xp && s_local > 0);
-    if (coresident_knob() && co_class && most <= kCoresidentTiles && stages_knob() == 0 && h->host.Kp <= kCoresidentK) {
+    if (coresident_knob() && co_class && most <= kCoresidentTiles && stages_knob() == 0 && h->host.Kp <= coresident_K(h->host.K, g->nt)) {
         const int half = kHalfSmBytes;
         const int fixed8 = fixed_for(8) + 32 * 8;
         const bool fold = h->host.fmt.C_A == 2;
@@ -266,7 +269,7 @@ void plan_classes(us_handle* h, int n_cta, std::vector<uint32_t> (&sched)[4])
             // (4096 x 4096 at 30 % sparsity: tiles of 9.5 KB and 32 KB of int8 X do not fit half an SM, with
             // 16 KB of packed X they do: 5.6 -> 4.6 us; the same for the folded format at 50 %: 5.3 -> 4.35)
             bool for_half_sm = false;
-            if (nt == 1 && ranges == 1 && coresident_knob() && h->host.Kp <= kCoresidentK) {
+            if (nt == 1 && ranges == 1 && coresident_knob() && h->host.Kp <= coresident_K(h->host.K, nt)) {
                 const int64_t per_cta = (h->host.n_items + n_cta - 1) / std::max(1, n_cta);
                 const int64_t need = 8;
                 auto fits = [&](bool xp, int s_loc) {
