@@ -413,12 +413,11 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
             const uint32_t slot_a = smem_u32(ring + (size_t)slot * p.slot_bytes) + 4u * lane;
             uint32_t b8 = 0, cw0[SR], cw1[SR], mw = 0;
             int words = p.mask_rows - WPS * st;       // mask words of the tile from here on
-            if (valid) {
-                // (another warp may not even have had its own tile in this slot yet, and the barrier's parity alone could not
-                // tell: wait for the pass to begin, then for its copy)
-                ok = tc_wait_count(issued + slot, pass + 1u, p.wait_ns_hi, dead) && tc_wait_warp(b_w + 8u * slot, pass & 1u, p.wait_ns_hi, dead);
-                if (!ok) break;
-            }
+            // (another warp may not even have had its own tile in this slot yet, and the barrier's parity alone could not
+            // tell: wait for the pass to begin, then for its copy. A warp whose strip lies past the matrix too: it refills
+            // the slot below, and the warp that had it before may still be decoding)
+            ok = tc_wait_count(issued + slot, pass + 1u, p.wait_ns_hi, dead) && tc_wait_warp(b_w + 8u * slot, pass & 1u, p.wait_ns_hi, dead);
+            if (!ok) break;
             if (i == 0 && lane > 0 && tile_first != kNone) copy_tile(tile_first, of0, of1, t_first);
             const uint32_t pay_a = slot_a + 128u * p.mask_rows;
             uint32_t mask_a = slot_a;

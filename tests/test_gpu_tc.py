@@ -78,3 +78,24 @@ def test_rule_and_withheld_copy():
             assert (y == ref).all()
     finally:
         sw.close()
+
+
+@pytest.mark.parametrize("s,fmt", [(0.5, (16, 512, 2, 2)), (0.3, (16, 512, 2, 1))])
+def test_idle_warps_keep_off_tiles_in_use(s, fmt):
+    """The last row block has 14 strips for 16 warps, and the tile ring a number of slots (between 16 and 32) that 16 does
+    not divide: the two idle warps refill slots that other warps decode from, at two stages per tile."""
+    from paper_2608_09291_b200 import binding as b
+    M, K, N = 8160, 9216, 64
+    W = workloads.make_weight(M, K, s, seed=11)
+    X = workloads.make_x(K, N, seed=11)
+    sw = b.SparseWeight(W, fmt=fmt, max_N=N)
+    try:
+        assert b.us_launch_info(sw.handle, N)["block"] == 800
+        Xd = torch.from_numpy(b.pack_int4(X)).cuda()
+        ref = torch.from_numpy(oracle.spmm_dense(W, X)).cuda()
+        for _ in range(20):
+            y = sw.spmm(Xd, N)
+            sw.check()
+            assert torch.equal(y, ref), int((y != ref).sum())
+    finally:
+        sw.close()
