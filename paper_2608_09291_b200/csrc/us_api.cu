@@ -425,6 +425,7 @@ void build_tc_plan(us_handle* h, int ng)
     pl.threads = pl.octets == 3 ? us::TcShape<3>::kThreads : us::TcShape<2>::kThreads;
     // tiles of a warp: a CTA's stages may begin and end inside a tile
     const int64_t per_cta = (stages + n_cta - 1) / n_cta, tiles = (per_cta + n_stage - 1) / n_stage + (n_stage > 1 ? 1 : 0);
+    if (std::min(per_cta, block_stages) > us::tc_max_run(hm.w2)) return;   // (from 5 * 10^9 weights on: the other kernel sums tile by tile)
     const int want = (int)std::min<int64_t>(3 * warps / 2, warps * tiles);   // slots worth having before the table gets its 32 copies
     while (p.x_stages > 2 && slots_for(p.x_stages, 8) < warps) --p.x_stages;
     p.lut_rep = slots_for(p.x_stages, 32) >= want && per_cta >= 16 ? 32 : 8;

@@ -44,6 +44,10 @@ constexpr int kTcBars = kTcMaxSlots + 2 * kTcMaxOct * kTcMaxA + 2 * kTcMaxXStage
 constexpr int kTcMiscWords = 96 + kTcMaxSlots;
 constexpr int kTcFixedSmem = kTcSxRing * 64 * 4 + kTcBars * 8 + kTcMiscWords * 4 + 1024;
 
+// The most stages a run of one row block may have: its sums of 256 products per stage stay in tensor memory as INT32.
+// INT4: raw byte (-128 .. 127) x 16 x (-128 .. 112), 2^14 at most -> 511; INT2: 4-bit field x 16 x, 15 * 128 -> 4369.
+constexpr int64_t tc_max_run(bool w2) { return 0x7FFFFFFFll / (256 * (w2 ? 15 * 128 : 128 * 128)); }
+
 struct TcParams {
     const uint8_t* blob;
     const uint32_t* item_off;

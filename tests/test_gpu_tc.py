@@ -99,3 +99,28 @@ def test_idle_warps_keep_off_tiles_in_use(s, fmt):
             assert torch.equal(y, ref), int((y != ref).sum())
     finally:
         sw.close()
+
+
+def test_sums_stay_exact_at_the_largest_k():
+    """37888 x 131072 gives every CTA one row block of 512 stages, whose sums of extreme values would leave 32 bits by one:
+    the other kernel takes it. (Nearly all rows are empty, so that the matrix costs no host memory.)"""
+    from paper_2608_09291_b200 import binding as b
+    M, K = 37888, 131072
+    W = np.zeros((M, K), np.int8)
+    rows = [0, 8, 20000, 37887]     # both halves of a strip
+    W[rows] = -8
+    X = workloads.make_x(K, 64, seed=3)
+    X[0], X[1] = -8, 7
+    sw = b.SparseWeight(W, max_N=64)
+    try:
+        Xd = torch.from_numpy(b.pack_int4(X)).cuda()
+        want = torch.from_numpy((-8 * X.astype(np.int64).sum(axis=1)).astype(np.int32)).cuda()
+        for N in (16, 64):
+            y = sw.spmm(Xd[:N], N)
+            sw.check()
+            assert all(torch.equal(y[:, r], want[:N]) for r in rows), (N, y[:2, rows].tolist(), want[:2].tolist())
+            y[:, rows] = 0
+            assert int(y.count_nonzero()) == 0, N
+            assert b.us_launch_info(sw.handle, N)["block"] <= 512
+    finally:
+        sw.close()
