@@ -407,76 +407,77 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
         constexpr int SR = W2 ? 1 : CA;
         constexpr int WPS = CA == 1 ? 2 : 1;  // mask words per stage
 
-        for (uint32_t i = 0; left > 0; ++i) {
-            const uint32_t strip = kDW * (uint32_t)q + (uint32_t)warp;
-            const bool valid = strip < (uint32_t)p.n_strips;
-            // offsets of the tile that will take over this slot, fetched behind the decode
-            const uint32_t tile_next = tile_at(kDW * i + (uint32_t)warp + (uint32_t)p.n_slots);
-            uint32_t no0 = 0, no1 = 0;
-            if (lane == 0 && tile_next < kNull) { no0 = __ldg(p.item_off + tile_next); no1 = __ldg(p.item_off + tile_next + 1); }
-            const uint32_t slot_a = smem_u32(ring + (size_t)slot * p.slot_bytes) + 4u * lane;
-            uint32_t b8 = 0, cw0[SR], cw1[SR], mw = 0;
-            int words = p.mask_rows - WPS * st;       // mask words of the tile from here on
-            // (another warp may not even have had its own tile in this slot yet, and the barrier's parity alone could not
-            // tell: wait for the pass to begin, then for its copy. A warp whose strip lies past the matrix too: it refills
-            // the slot below, and the warp that had it before may still be decoding)
+        // The warp's i-th tile is in its slot: another warp may not even have had its own tile there yet, and the barrier's
+        // parity alone could not tell, so wait for the pass to begin, then for its copy.
+        auto wait_tile = [&](uint32_t i) {
             ok = tc_wait_count(issued + slot, pass + 1u, p.wait_ns_hi, dead) && tc_wait_warp(b_w + 8u * slot, pass & 1u, p.wait_ns_hi, dead);
-            if (!ok) break;
-            if (i == 0 && lane > 0 && tile_first != kNone) copy_tile(tile_first, of0, of1, t_first);
-            const uint32_t pay_a = slot_a + 128u * p.mask_rows;
-            uint32_t mask_a = slot_a;
-            if (valid) {
-#pragma unroll 1
-                for (int w = WPS * st; w > 0; --w) {  // entered in its middle: the stream position there
-                    b8 += 8u * (uint32_t)__popc(lds32(mask_a));
-                    mask_a += 128u;
-                }
-                mw = lds32(mask_a);
-                const uint32_t a = pay_a + (b8 >> 5) * (uint32_t)(128 * SR);
-#pragma unroll
-                for (int s = 0; s < SR; ++s) { cw0[s] = lds32(a + 128u * s); cw1[s] = lds32(a + 128u * (SR + s)); }
-            }
-            const int n_here = min(n_stage - st, left);
-            for (int j = 0; j < n_here; ++j) {
-                ok = tc_wait_warp(b_ae + 8u * (o * kTcAStages + as), a_par, p.wait_ns_hi, dead);
-                if (!ok) break;
-                if (valid) {
-                    tc_fence_after();
-                    const uint32_t dst = tm_a + 64u * as;
-#pragma unroll
-                    for (int h = 0; h < WPS; ++h) {
-                        if (h == 1 && words <= 0) break;   // (an odd number of mask words: the last stage is half a stage)
-                        const uint32_t m = mw;
-                        mask_a += 128u;
-                        if (--words > 0) mw = lds32(mask_a);
-                        uint32_t r[CA][16];
-                        decode_word<CA, W2>(m, pay_a, lut_a, lut_stride, b8, cw0, cw1, r);
-                        tc_st16(dst + 32u * h, r[0]);
-                        if (CA == 2) tc_st16(dst + 32u, r[CA - 1]);
-                    }
-                }
-                announce(b_af + 8u * (o * kTcAStages + as));
-                if (++as == kTcAStages) { as = 0; a_par ^= 1u; }
-            }
-            if (!ok) break;
-            // the slot is free: refill it for the tile that comes n_slots later
+            if (ok && i == 0 && lane > 0 && tile_first != kNone) copy_tile(tile_first, of0, of1, t_first);
+            return ok;
+        };
+        // offsets of the tile that will take over that slot, fetched behind the decode
+        uint32_t tile_next, no0 = 0, no1 = 0;
+        auto look_ahead = [&](uint32_t i) {
+            tile_next = tile_at(kDW * i + (uint32_t)warp + (uint32_t)p.n_slots);
+            if (lane == 0 && tile_next < kNull) { no0 = __ldg(p.item_off + tile_next); no1 = __ldg(p.item_off + tile_next + 1); }
+        };
+        auto refill = [&]() {   // the slot is free: refill it for the tile that comes n_slots later, go to the next
             if (lane == 0 && tile_next != kNone) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 copy_tile(tile_next, no0, no1, slot);
             }
             slot += kDW;
             while (slot >= (uint32_t)p.n_slots) { slot -= (uint32_t)p.n_slots; ++pass; }
+        };
+
+        uint32_t i = 0;
+        for (; left > 0; ++i) {
+            const uint32_t strip = kDW * (uint32_t)q + (uint32_t)warp;
+            if (strip >= (uint32_t)p.n_strips) break;
+            look_ahead(i);
+            const uint32_t slot_a = smem_u32(ring + (size_t)slot * p.slot_bytes) + 4u * lane;
+            uint32_t b8 = 0, cw0[SR], cw1[SR], mw = 0;
+            int words = p.mask_rows - WPS * st;       // mask words of the tile from here on
+            if (!wait_tile(i)) break;
+            const uint32_t pay_a = slot_a + 128u * p.mask_rows;
+            uint32_t mask_a = slot_a;
+#pragma unroll 1
+            for (int w = WPS * st; w > 0; --w) {  // entered in its middle: the stream position there
+                b8 += 8u * (uint32_t)__popc(lds32(mask_a));
+                mask_a += 128u;
+            }
+            mw = lds32(mask_a);
+            const uint32_t a0 = pay_a + (b8 >> 5) * (uint32_t)(128 * SR);
+#pragma unroll
+            for (int s = 0; s < SR; ++s) { cw0[s] = lds32(a0 + 128u * s); cw1[s] = lds32(a0 + 128u * (SR + s)); }
+            const int n_here = min(n_stage - st, left);
+            for (int j = 0; j < n_here; ++j) {
+                ok = tc_wait_warp(b_ae + 8u * (o * kTcAStages + as), a_par, p.wait_ns_hi, dead);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t dst = tm_a + 64u * as;
+#pragma unroll
+                for (int h = 0; h < WPS; ++h) {
+                    if (h == 1 && words <= 0) break;   // (an odd number of mask words: the last stage is half a stage)
+                    const uint32_t m = mw;
+                    mask_a += 128u;
+                    if (--words > 0) mw = lds32(mask_a);
+                    uint32_t r[CA][16];
+                    decode_word<CA, W2>(m, pay_a, lut_a, lut_stride, b8, cw0, cw1, r);
+                    tc_st16(dst + 32u * h, r[0]);
+                    if (CA == 2) tc_st16(dst + 32u, r[CA - 1]);
+                }
+                announce(b_af + 8u * (o * kTcAStages + as));
+                if (++as == kTcAStages) { as = 0; a_par ^= 1u; }
+            }
+            if (!ok) break;
+            refill();
             left -= n_here;
             run_stages += n_here;
             st = 0;
             if (++seg < p.n_segs && left > 0) continue;
 
             // ---- the run of this row block ends: read the sums back ----
-            int m_lo = -1, m_hi = -1;
-            if (valid) {
-                m_lo = __ldg(p.row_order + strip * 16 + (lane >> 2));
-                m_hi = __ldg(p.row_order + strip * 16 + (lane >> 2) + 8);
-            }
+            const int m_lo = __ldg(p.row_order + strip * 16 + (lane >> 2)), m_hi = __ldg(p.row_order + strip * 16 + (lane >> 2) + 8);
             ok = tc_wait_warp(b_d + 8u * o, d_par, p.wait_ns_hi, dead);
             if (!ok) break;
             d_par ^= 1u;
@@ -484,69 +485,84 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
                 asm volatile("griddepcontrol.wait;" ::: "memory");
                 waited = true;
             }
-            if (valid) {
-                tc_fence_after();
-                const int32_t* sxp = sx + ((q - q0) % kTcSxRing) * 64 + 2 * (lane & 3);
-                const bool whole = run_stages == p.block_stages;
-                int32_t* accp = p.acc + (size_t)strip * (p.acc_nt * 128) + lane;
+            tc_fence_after();
+            const int32_t* sxp = sx + ((q - q0) % kTcSxRing) * 64 + 2 * (lane & 3);
+            const bool whole = run_stages == p.block_stages;
+            int32_t* accp = p.acc + (size_t)strip * (p.acc_nt * 128) + lane;
 #pragma unroll 1
-                for (int nt = 0; nt < ng; ++nt) {
-                    int c[4], y[4];
-                    tc_ld4(tm_d + (uint32_t)(S::kD * o) + 8u * nt + lane_base, c);
-                    const int s0 = sxp[8 * nt] >> 4, s1 = sxp[8 * nt + 1] >> 4;
-                    if (W2) {
-                        y[0] = (c[2] >> 4) - 2 * s0;
-                        y[1] = (c[3] >> 4) - 2 * s1;
-                        y[2] = ((c[0] - c[2]) >> 6) - 2 * s0;
-                        y[3] = ((c[1] - c[3]) >> 6) - 2 * s1;
-                    } else {
-                        y[0] = (c[2] >> 4) - 8 * s0;
-                        y[1] = (c[3] >> 4) - 8 * s1;
-                        y[2] = (c[0] - c[2]) >> 8;
-                        y[3] = (c[1] - c[3]) >> 8;
-                    }
-                    if (whole) {
-                        store_block_tc<AM>(sctx, y[0], y[1], y[2], y[3], lane, m_lo, m_hi, 8 * nt);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) atomicAdd(accp + nt * 128 + j * 32, y[j]);
-                    }
+            for (int nt = 0; nt < ng; ++nt) {
+                int c[4], y[4];
+                tc_ld4(tm_d + (uint32_t)(S::kD * o) + 8u * nt + lane_base, c);
+                const int s0 = sxp[8 * nt] >> 4, s1 = sxp[8 * nt + 1] >> 4;
+                if (W2) {
+                    y[0] = (c[2] >> 4) - 2 * s0;
+                    y[1] = (c[3] >> 4) - 2 * s1;
+                    y[2] = ((c[0] - c[2]) >> 6) - 2 * s0;
+                    y[3] = ((c[1] - c[3]) >> 6) - 2 * s1;
+                } else {
+                    y[0] = (c[2] >> 4) - 8 * s0;
+                    y[1] = (c[3] >> 4) - 8 * s1;
+                    y[2] = (c[0] - c[2]) >> 8;
+                    y[3] = (c[1] - c[3]) >> 8;
                 }
-                tc_fence_before();
-                if (!whole) {
+                if (whole) {
+                    store_block_tc<AM>(sctx, y[0], y[1], y[2], y[3], lane, m_lo, m_hi, 8 * nt);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) atomicAdd(accp + nt * 128 + j * 32, y[j]);
+                }
+            }
+            tc_fence_before();
+            if (!whole) {
+                __syncwarp();
+                uint32_t old = 0;
+                if (lane == 0)
+                    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p.cnt + strip), "r"(run_stages) : "memory");
+                old = __shfl_sync(0xffffffffu, old, 0);
+                if (old + (uint32_t)run_stages == (uint32_t)p.block_stages) {
+                    // the strip is complete: take the sums (two blocks ahead), leave workspace and counter zeroed
                     __syncwarp();
-                    uint32_t old = 0;
-                    if (lane == 0)
-                        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p.cnt + strip), "r"(run_stages) : "memory");
-                    old = __shfl_sync(0xffffffffu, old, 0);
-                    if (old + (uint32_t)run_stages == (uint32_t)p.block_stages) {
-                        // the strip is complete: take the sums (two blocks ahead), leave workspace and counter zeroed
-                        __syncwarp();
-                        int v[3][4];
+                    int v[3][4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        v[0][j] = __ldcg(accp + j * 32);
+                        v[1][j] = ng > 1 ? __ldcg(accp + 128 + j * 32) : 0;
+                    }
+#pragma unroll 1
+                    for (int nt = 0; nt < ng; ++nt) {
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            v[0][j] = __ldcg(accp + j * 32);
-                            v[1][j] = ng > 1 ? __ldcg(accp + 128 + j * 32) : 0;
+                            v[2][j] = nt + 2 < ng ? __ldcg(accp + 256 + j * 32) : 0;
+                            __stcg(accp + j * 32, 0);
                         }
-#pragma unroll 1
-                        for (int nt = 0; nt < ng; ++nt) {
+                        store_block_tc<AM>(sctx, v[0][0], v[0][1], v[0][2], v[0][3], lane, m_lo, m_hi, 8 * nt);
+                        accp += 128;
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                v[2][j] = nt + 2 < ng ? __ldcg(accp + 256 + j * 32) : 0;
-                                __stcg(accp + j * 32, 0);
-                            }
-                            store_block_tc<AM>(sctx, v[0][0], v[0][1], v[0][2], v[0][3], lane, m_lo, m_hi, 8 * nt);
-                            accp += 128;
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) { v[0][j] = v[1][j]; v[1][j] = v[2][j]; }
-                        }
-                        if (lane == 0) p.cnt[strip] = 0;
+                        for (int j = 0; j < 4; ++j) { v[0][j] = v[1][j]; v[1][j] = v[2][j]; }
                     }
+                    if (lane == 0) p.cnt[strip] = 0;
                 }
             }
             run_stages = 0;
             seg = 0;
             ++q;
+        }
+        // In the last row block a warp's strip may lie past the matrix. Such a warp announces its part of every stage as it
+        // is, and passes its ring slots on: not before they are filled, the warp before it may still be decoding from them.
+        for (; ok && left > 0; ++i) {
+            look_ahead(i);
+            if (!wait_tile(i)) break;
+            const int n_here = min(n_stage - st, left);
+            for (int j = 0; j < n_here && ok; ++j) {
+                ok = tc_wait_warp(b_ae + 8u * (o * kTcAStages + as), a_par, p.wait_ns_hi, dead);
+                if (!ok) break;
+                announce(b_af + 8u * (o * kTcAStages + as));
+                if (++as == kTcAStages) { as = 0; a_par ^= 1u; }
+            }
+            if (!ok) break;
+            refill();
+            left -= n_here;
+            st = 0;
         }
         if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
     } else if (warp == kTcDecodeWarps) {
