@@ -44,9 +44,6 @@ struct us_handle {
     int sm_count = 0;
     int max_N = 0;
     int max_smem = 0;
-    int co_warps = 10;   // warps of an N <= 8 CTA when two CTAs share an SM's registers
-    int co_warps2 = 8;   // the same for the N = 9..16 kernel with packed activations
-    int co_warps_fold = 8;   // the same for the folded-tile (two column areas) N <= 8 kernel
     uint8_t* d_blob = nullptr;
     uint32_t* d_item_off = nullptr;
     std::vector<uint32_t> cta_begin[4];  // schedule per N class (NT = 1, 2, 4, 8)
@@ -137,6 +134,35 @@ int segs_per_range(const us::HostMatrix& hm, int nt, int limit, int64_t min_rang
     return 1;
 }
 
+const void* kernel_for(int cls, const us::KernelKey& k)
+{
+    switch (cls) {
+        case 0: return us::kernel_nt1(k);
+        case 1: return us::kernel_nt2(k);
+        case 2: return us::kernel_nt4(k);
+        default: return us::kernel_nt8(k);
+    }
+}
+
+// The most warps with which two CTAs of every kernel that calls on this handle launch under the given plan share an SM's
+// registers: 16384 to a scheduler, allocated 8 a thread at a time. (The stage-timer builds need more and do not share one.)
+int half_sm_warps(const us_handle* h, int cls, bool local, bool xp)
+{
+    const us::HostMatrix& hm = h->host;
+    const bool fold = hm.fmt.C_A == 2;
+    if (h->device < 0) return cls == 0 && !fold ? 12 : 10;   // host-only handle
+    int regs = 0;
+    for (int form = 0; form < 3; ++form) {   // plain, chained, single token
+        us::KernelKey k{1, local, false, xp, form == 1, fold, hm.w2, form == 2, hm.K % 32 != 0};
+        const void* fn = kernel_for(cls, k);
+        if (!fn) continue;
+        cudaFuncAttributes fa;
+        if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) { cudaGetLastError(); return 0; }
+        regs = std::max(regs, fa.numRegs);
+    }
+    return regs ? 2 * (16384 / (32 * ((regs + 7) / 8 * 8))) : 0;
+}
+
 // Shared-memory layout of us_spmm_kernel: selector table, int8 X of one K range, per-(segment,
 // token) sums, mbarriers, claim counter, local strip accumulators + counters, per-warp rings.
 bool plan_launch(const us_handle* h, int N, LaunchGeom* g)
@@ -196,9 +222,8 @@ bool plan_launch(const us_handle* h, int N, LaunchGeom* g)
     if (coresident_knob() && co_class && most <= kCoresidentTiles && stages_knob() == 0 && h->host.Kp <= coresident_K(h->host.K, g->nt)) {
         const int half = kHalfSmBytes;
         const int fixed8 = fixed_for(8) + 32 * 8;
-        const bool fold = h->host.fmt.C_A == 2;
-        int w = std::min(g->nt == 1 ? (fold ? h->co_warps_fold : h->co_warps) : h->co_warps2,
-                         (g->nt == 1 && !fold) ? max_warps() : std::min(16, max_warps()));
+        // (two column areas: 10 at most; 3001 x 2000, N = 8 4.10 us with 10, 4.18 with 12)
+        int w = std::min({half_sm_warps(h, g->cls, s_local > 0, g->xp && s_local > 0), h->host.fmt.C_A == 2 ? 10 : 16, max_warps()});
         while (w >= 8 && fixed8 + w * (int)g->slot_bytes > half) --w;
         // (only if every tile of the CTA finds a warp at once: 5120 x 5120 at 70 % sparsity, N = 16, has 11 tiles per CTA
         // and room for 8 half-SM warps: 9.9 us against 8.9 with 16 warps on the whole SM; 1500 x 6000 has 12 and room for 10:
@@ -369,7 +394,6 @@ void build_plan(us_handle* h, int cls)
     p.fold_kb = hm.fmt.C_A == 2 ? hm.nkb / 2 : 0;
     p.w2 = hm.w2 ? 1 : 0;
     p.slot_bytes = g.slot_bytes;
-    p.x_fast = hm.K % 32 == 0;
 }
 
 // Lays a launch of us_spmm_tc_kernel down for calls of `ng` 8-token groups.
@@ -445,35 +469,26 @@ void build_tc_plan(us_handle* h, int ng)
     pl.ok = true;
 }
 
-const void* kernel_for(int cls, const us::KernelKey& k)
-{
-    switch (cls) {
-        case 0: return us::kernel_nt1(k);
-        case 1: return us::kernel_nt2(k);
-        case 2: return us::kernel_nt4(k);
-        default: return us::kernel_nt8(k);
-    }
-}
-
-// Opt every kernel variant in to the device's full dynamic shared memory: once per device, when its first
-// handle is made, so that us_spmm itself is nothing but a launch.
-cudaError_t enable_large_smem(int device, int bytes)
+// Opt the kernel variants for a K (any_k: no multiple of 32) in to the device's full dynamic shared memory: once per
+// device, when the first handle with such a K is made, so that us_spmm itself is nothing but a launch.
+cudaError_t enable_large_smem(int device, int bytes, bool any_k)
 {
     static std::mutex mu;
-    static std::vector<char> done;
+    static std::vector<char> enabled[2];
     std::lock_guard<std::mutex> lock(mu);
+    std::vector<char>& done = enabled[any_k];
     if (device < (int)done.size() && done[device]) return cudaSuccess;
     for (int cls = 0; cls < 4; ++cls)
         for (int bits = 0; bits < 256; ++bits) {
             const us::KernelKey k{1 + (bits & 1), (bits & 2) != 0, (bits & 4) != 0, (bits & 8) != 0,
-                                  (bits & 16) != 0, (bits & 32) != 0, (bits & 64) != 0, (bits & 128) != 0};
+                                  (bits & 16) != 0, (bits & 32) != 0, (bits & 64) != 0, (bits & 128) != 0, any_k};
             const void* fn = kernel_for(cls, k);
             if (!fn) continue;
             const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
             if (e != cudaSuccess) return e;
         }
-    for (int bits = 0; bits < 32; ++bits)
-        if (const void* fn = us::kernel_tc(bits & 8 ? 3 : 2, (bits & 16) != 0, (bits & 1) != 0, (bits & 2) != 0, (bits & 4) != 0)) {
+    for (int bits = 0; bits < 16; ++bits)
+        if (const void* fn = us::kernel_tc(bits & 8 ? 3 : 2, any_k, (bits & 1) != 0, (bits & 2) != 0, (bits & 4) != 0)) {
             const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
             if (e != cudaSuccess) return e;
         }
@@ -550,7 +565,8 @@ us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_sca
     p.wait_ns_hi = h->wait_ns_hi;
     p.withhold = h->withhold;
 
-    us::KernelKey k{g.stages, p.s_local > 0, timers, g.xp && p.s_local > 0, p.y_amax != nullptr, p.fold_kb != 0, p.w2 != 0, false};
+    us::KernelKey k{g.stages, p.s_local > 0, timers, g.xp && p.s_local > 0, p.y_amax != nullptr, p.fold_kb != 0, p.w2 != 0, false,
+                    h->host.K % 32 != 0};
     // a single token: dp4a beats the MMA (measured 2-3 %)
     k.dp = N == 1 && !k.timed && !k.xp && !k.am && !k.fold && !k.w2;
     const void* fn = kernel_for(cls, k);
@@ -638,24 +654,7 @@ us_status us_encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_sca
     }
     h->d_blob = dm.blob; h->d_item_off = dm.item_off; h->d_row_order = dm.row_order;
 
-    e = enable_large_smem(h->device, h->max_smem);
-    if (e == cudaSuccess) {
-        // Two N <= 8 CTAs share the SM's 64 K registers (allocated 8 per thread at a time).
-        int regs = 0;
-        // (the stage-timer builds need more and simply do not share an SM)
-        for (const bool local : {true, false}) {
-            cudaFuncAttributes fa;
-            e = cudaFuncGetAttributes(&fa, kernel_for(0, {1, local}));
-            if (e != cudaSuccess) break;
-            regs = std::max(regs, fa.numRegs);
-        }
-        if (e == cudaSuccess) h->co_warps = 32768 / (32 * ((regs + 7) / 8 * 8));
-        cudaFuncAttributes fa2;
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa2, kernel_for(1, {1, true, false, true}));
-        if (e == cudaSuccess) h->co_warps2 = 32768 / (32 * ((fa2.numRegs + 7) / 8 * 8));
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa2, kernel_for(0, {1, true, false, false, false, true}));
-        if (e == cudaSuccess) h->co_warps_fold = 32768 / (32 * ((fa2.numRegs + 7) / 8 * 8));
-    }
+    e = enable_large_smem(h->device, h->max_smem, hm.K % 32 != 0);
     if (e != cudaSuccess) { free_device(h); delete h; return US_ERR_CUDA; }
 
     const int nt_max = nt_for(max_N);

@@ -13,6 +13,7 @@ struct KernelKey {
     bool fold;         // two column areas
     bool w2;           // INT2 weights
     bool dp;           // dp4a (a single token)
+    bool any_k;        // K is not a multiple of 32
 };
 
 // The kernel for a key, or nullptr where no such variant is built.

@@ -64,7 +64,6 @@ struct SpmmParams {
     int32_t fold_kb;            // C_A = 2: k-blocks per column area (a mask bit also covers the column that many
                                 // k-blocks further on); 0 for C_A = 1
     uint32_t slot_bytes;        // ring slot size (max tile blob + slack), multiple of 128
-    int32_t x_fast;             // K % 32 == 0: 16-byte loads
     int32_t fp16_out;
     // Chained call: the epilogue leaves the per-token absmax of the fp16 outputs of rows
     // [amax_m0, amax_m1) in an absmax buffer (layout below) for the quantiser of the next call.
@@ -313,14 +312,14 @@ __device__ __forceinline__ void stage_x_any(const uint8_t* X, int K, int N, int 
 }
 
 // sx16 must be zero on entry (the caller clears it and synchronises).
-// Units below `first_unit` (of the 16-byte path) were already staged by the caller.
-template <int NT, bool XP>
+// ANY: K is not a multiple of 32. Units below `first_unit` (of the 16-byte path) were already staged by the caller.
+template <int NT, bool XP, bool ANY>
 __device__ __forceinline__ void stage_x(const SpmmParams& p, int seg0, int n_seg, uint8_t* x8,
                                         int xstride, int32_t* sx16, int first_unit)
 {
     const int64_t ldx = ((int64_t)p.K + 1) / 2;
     const int rows = NT * 8;
-    if (!p.x_fast) {
+    if (ANY) {
         stage_x_any<NT, XP>(p.X, p.K, p.N, p.K_L, seg0, n_seg, x8, xstride, sx16);
         return;
     }
@@ -608,6 +607,16 @@ __device__ __forceinline__ uint32_t fdiv(uint32_t u, unsigned long long m)
 constexpr int kWarpRec = 16, kMaxWarpsPerCta = 24;
 constexpr int kTimerWords = kWarpRec * kMaxWarpsPerCta * kMaxCtas;
 
+// Threads a kernel is compiled for, which bounds its registers. N <= 8 kernels run up to 20 warps (more than 16 per full-SM
+// CTA were measured and do not pay). Two are held to fewer registers than the compiler would take, for the half-SM plan:
+// direct mode to 80, as local mode uses, so that 12 warps of each of two CTAs share an SM instead of 10 (24000 x 1024, 11
+// tiles per CTA, N = 8: 5.8 -> 4.8 us); folded tiles at a K that is no multiple of 32 to 96, 10 warps instead of 8
+// (4001 x 2500, N = 8: 5.4 -> 4.5).
+template <bool ANY, int NT, int STAGES, bool LA, bool TIMED, int CA, bool W2>
+constexpr int kMaxThreads = NT != 1    ? 512
+                            : CA == 1  ? (STAGES == 1 && !LA && !TIMED ? 768 : 640)
+                                       : (STAGES == 1 && ANY && !TIMED && !W2 ? 640 : 512);
+
 // LA = local mode (shared-memory strip accumulators), else direct mode.
 // TIMED = record the diagnostic stage timers (a separate instantiation, so that the production
 // kernel carries none of their clock reads and branches).
@@ -615,11 +624,12 @@ constexpr int kTimerWords = kWarpRec * kMaxWarpsPerCta * kMaxCtas;
 // fp16 store measured 2.5 % slower with the tracking compiled in behind a run-time flag).
 // CA = column areas of the weight format (2: folded tiles).
 // W2 = INT2 weights (folded format only). DP = dp4a instead of the MMA: the N = 1 kernels of the default format.
-template <int NT, int STAGES, bool LA, bool TIMED, bool XP = false, bool AM = false, int CA = 1, bool W2 = false,
+// ANY = K is not a multiple of 32 (stage_x_any). Separate instantiations: with both forms of staging behind a run-time
+// flag the kernels took up to 13 registers more (N <= 8: chained 79 -> 92, direct mode 80 -> 83), and two half-SM CTAs of
+// a chained call no longer shared an SM.
+template <bool ANY, int NT, int STAGES, bool LA, bool TIMED, bool XP = false, bool AM = false, int CA = 1, bool W2 = false,
           bool DP = false>
-// (N <= 8 kernels are compiled for up to 20 warps: 80 registers instead of 90, which lets 12 instead of 10 warps of
-// two half-SM CTAs share an SM; more than 16 warps per full-SM CTA were measured and do not pay.)
-__global__ void __launch_bounds__((NT == 1 && CA == 1) ? 640 : 512, 1) us_spmm_kernel(const SpmmParams p)
+__global__ void __launch_bounds__(kMaxThreads<ANY, NT, STAGES, LA, TIMED, CA, W2>, 1) us_spmm_kernel(const SpmmParams p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
@@ -851,9 +861,9 @@ __global__ void __launch_bounds__((NT == 1 && CA == 1) ? 640 : 512, 1) us_spmm_k
         spre.have_sx = true;
     }
     const int g_first = (kr_first == n_kr - 1) ? g_last : p.G;   // segments in that range
-    constexpr int kXPre = NT <= 4 ? 8 : 0;   // 16-byte units of X a thread prefetches
+    constexpr int kXPre = NT <= 4 && !ANY ? 8 : 0;   // 16-byte units of X a thread prefetches
     const int x_sh = 31 - __clz(p.K_L / 32);   // log2(units per (segment, token)) when a power of two
-    const bool x_early = kXPre > 0 && p.x_fast && (1 << x_sh) == p.K_L / 32;
+    const bool x_early = kXPre > 0 && (1 << x_sh) == p.K_L / 32;
     uint4 xpre[kXPre > 0 ? kXPre : 1];
     const int x_upr = p.K_L / 32, x_total = NT * 8 * g_first * x_upr;
     if (x_early) {
@@ -960,9 +970,9 @@ __global__ void __launch_bounds__((NT == 1 && CA == 1) ? 640 : 512, 1) us_spmm_k
                     }
                 }
             }
-            stage_x<NT, XP>(p, kr * p.G, g_kr, x8, xstride, sx16, kXPre * (int)blockDim.x);
+            stage_x<NT, XP, ANY>(p, kr * p.G, g_kr, x8, xstride, sx16, kXPre * (int)blockDim.x);
         } else {
-            stage_x<NT, XP>(p, kr * p.G, g_kr, x8, xstride, sx16, 0);
+            stage_x<NT, XP, ANY>(p, kr * p.G, g_kr, x8, xstride, sx16, 0);
         }
         __syncthreads();
     };

@@ -178,3 +178,28 @@ def test_layer_13b_chain(b, j, s):
     finally:
         for m in mats:
             m["sw"].close()
+
+
+@pytest.mark.parametrize("M,K,fmt,warps", [(2048, 2048, None, 12),                    # local mode
+                                           (11500, 1000, (16, 512, 2, 1), 12),        # local mode, one range of two segments
+                                           (24000, 1024, None, 11),                   # direct mode, 11 tiles per CTA
+                                           (4001, 2500, (16, 512, 2, 2), 10)])        # two column areas, K no multiple of 32
+def test_half_sm_plan_counts_the_registers_of_every_kernel(b, M, K, fmt, warps):
+    """Plain, single-token and chained calls are different kernels under one plan: its warps are what two CTAs of each of
+    them share an SM with (2048 x 2048 had 11 while the direct mode's kernel was counted and the chained one was not)."""
+    W = workloads.make_weight(M, K, 0.5, seed=M + K)
+    s_w = workloads.make_chain_weight_scales(M, K, 5)
+    sw = b.SparseWeight(W, s_w, fmt=fmt, max_N=8)
+    try:
+        info = b.us_launch_info(sw.handle, 8)
+        assert info["smem_bytes"] <= 114 * 1024 and info["block"] == 32 * warps, info
+        X = workloads.make_x(K, 8, seed=1)
+        ref = oracle.spmm_dense(W, X)
+        for N in (1, 8):
+            y = sw.spmm(torch.from_numpy(b.pack_int4(X[:N])).cuda(), N).cpu().numpy()
+            sw.check()
+            assert (y == ref[:N]).all(), N
+        if fmt is None or fmt[3] == 1:
+            _check_requant_call(b, sw, W, s_w, workloads.make_x_f16(K, 8, seed=2), 8, 0, M)
+    finally:
+        sw.close()
