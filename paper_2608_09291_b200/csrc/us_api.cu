@@ -707,19 +707,18 @@ us_status us_get_stats(const us_handle* h, us_stats* out)
 us_status us_decode(const us_handle* h, int8_t* W_out)
 {
     if (!h || !W_out) return US_ERR_INVALID_ARG;
-    if (h->on_device && h->host.blob.empty()) {   // encoded on the GPU: fetch the tiles first
-        us::HostMatrix& host = const_cast<us_handle*>(h)->host;
+    std::vector<uint8_t> fetched;   // (the handle is read only: several threads may decode it at once)
+    const uint8_t* blob = h->host.blob.data();
+    if (h->on_device) {
         try {
-            host.blob.resize((size_t)host.blob_bytes);
+            fetched.resize((size_t)h->host.blob_bytes);
         } catch (const std::bad_alloc&) {
             return US_ERR_ALLOC;
         }
-        if (cudaMemcpy(host.blob.data(), h->d_blob, host.blob.size(), cudaMemcpyDeviceToHost) != cudaSuccess) {
-            host.blob.clear();
-            return US_ERR_CUDA;
-        }
+        if (cudaMemcpy(fetched.data(), h->d_blob, fetched.size(), cudaMemcpyDeviceToHost) != cudaSuccess) return US_ERR_CUDA;
+        blob = fetched.data();
     }
-    us::decode_host(h->host, W_out);
+    us::decode_host(h->host, blob, W_out);
     return US_OK;
 }
 

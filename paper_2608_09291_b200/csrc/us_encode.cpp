@@ -479,14 +479,14 @@ us_status encode_host(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_s
     return US_OK;
 }
 
-void decode_host(const HostMatrix& h, int8_t* W_out)
+void decode_host(const HostMatrix& h, const uint8_t* blob, int8_t* W_out)
 {
     std::memset(W_out, 0, (size_t)(h.M * h.K));
     if (!h.kernel_layout) { decode_generic(h, W_out); return; }
     const int CA = h.fmt.C_A, nkb = h.nkb / CA, mask_rows = h.mask_rows, K_L = h.fmt.K_L, K_B = K_L / CA;
     for (int64_t t = 0; t < h.n_items; ++t) {
         const int64_t rb = t / h.n_segs, sg = t % h.n_segs;
-        const uint8_t* b = h.blob.data() + (size_t)h.item_off[t] * 16;
+        const uint8_t* b = blob + (size_t)h.item_off[t] * 16;
         const uint8_t* pay = b + (size_t)mask_rows * 128;
         for (int lane = 0; lane < 32; ++lane) {
             const int g = lane >> 2, tt = lane & 3;

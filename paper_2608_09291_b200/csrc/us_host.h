@@ -56,7 +56,7 @@ struct HostMatrix {
     int64_t n_strips = 0, n_segs = 0, n_items = 0;
     std::vector<int32_t> row_order;   // Mp entries: original row at padded position, -1 = padding
     std::vector<uint32_t> item_off;   // n_items + 1, units of 16 bytes
-    std::vector<uint8_t> blob;        // all tile blobs back to back (empty until asked for where the GPU encoded them)
+    std::vector<uint8_t> blob;        // all tile blobs back to back (empty where the GPU encoded them)
     uint64_t blob_bytes = 0;
     std::vector<uint16_t> w_scale;    // M fp16 bit patterns (empty if none)
     int64_t nnz = 0, sum_P = 0, bytes_payload_padded = 0;
@@ -77,7 +77,7 @@ void sort_rows(const std::vector<int64_t>& nonzeros, HostMatrix* h);
 bool pack_int4(const int8_t* W, int64_t K, int64_t ld, int64_t o0, int64_t o1, uint8_t* dst, bool w2,
                std::atomic<int32_t>* row_nnz);
 
-void decode_host(const HostMatrix& h, int8_t* W_out);
+void decode_host(const HostMatrix& h, const uint8_t* blob, int8_t* W_out);   // blob: unused for a format without a kernel layout
 void fill_stats(const HostMatrix& h, us_stats* st);
 
 // Byte-balanced split of the processing order (K range of G segments, strip, segment) over

@@ -76,3 +76,24 @@ def test_concurrent_loads_and_products(b):
     for t in threads:
         t.join()
     assert not wrong
+
+
+def test_concurrent_decodes_of_one_handle(b):
+    """Reading a handle is no call on it that must not overlap: several threads decode the same one."""
+    W = workloads.make_weight(3000, 2000, 0.5, seed=9)
+    h = b.us_encode(W, max_N=8)
+    wrong = []
+
+    def work():
+        if not (b.us_decode(h) == W).all():
+            wrong.append(1)
+
+    try:
+        threads = [threading.Thread(target=work) for _ in range(8)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        assert not wrong
+    finally:
+        b.us_destroy(h)
