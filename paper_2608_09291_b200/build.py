@@ -13,10 +13,10 @@ PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 LIB = PKG / "libunionsparse.so"
 EXT = PKG / "_us_torch.so"
-# (source, extra flags, object): the kernels are one translation unit per N class, so that they build in parallel
+# (source, extra flags, object): the kernels are one translation unit per N class and kind of K, so that they build in parallel
 UNITS = [(CSRC / "us_api.cu", [], "us_api.o"), (CSRC / "us_encode.cpp", [], "us_encode.o"),
          (CSRC / "us_load.cu", [], "us_load.o"), (CSRC / "us_spmm_tc.cu", [], "us_spmm_tc.o")] + [
-    (CSRC / "us_kernels.cu", [f"-DUS_NT={nt}"], f"us_kernels_nt{nt}.o") for nt in (1, 2, 4, 8)]
+    (CSRC / "us_kernels.cu", [f"-DUS_NT={nt}", f"-DUS_ANY={a}"], f"us_kernels_nt{nt}_{a}.o") for nt in (1, 2, 4, 8) for a in (0, 1)]
 HEADERS = [CSRC / "us_host.h", CSRC / "us_launch.h", CSRC / "us_load.h", CSRC / "us_device_encode.cuh",
            CSRC / "us_spmm_kernel.cuh", CSRC / "us_spmm_tc.cuh", CSRC / "us_quant_kernels.cuh",
            PKG.parent / "include" / "unionsparse.h"]

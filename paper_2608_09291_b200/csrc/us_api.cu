@@ -6,6 +6,8 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <set>
+#include <utility>
 #include <vector>
 
 #include "us_host.h"
@@ -22,9 +24,13 @@ struct LaunchGeom {
     uint32_t slot_bytes;
     bool xp;
 };
+struct KernelForms {      // nullptr where no such kernel is built
+    const void *plain = nullptr, *chained = nullptr, *single = nullptr, *timed = nullptr;
+};
 struct ClassPlan {
     bool ok = false;
     LaunchGeom g{};
+    KernelForms fn;
     us::SpmmParams p{};   // everything but the call's pointers, N and the absmax range
 };
 
@@ -32,6 +38,7 @@ struct ClassPlan {
 struct TcPlan {
     bool ok = false;
     int octets = 2, threads = 0, smem = 0;
+    const void *plain = nullptr, *chained = nullptr;
     us::TcParams p{};
 };
 
@@ -134,27 +141,40 @@ int segs_per_range(const us::HostMatrix& hm, int nt, int limit, int64_t min_rang
     return 1;
 }
 
-const void* kernel_for(int cls, const us::KernelKey& k)
+const void* kernel_for(int cls, bool any_k, const us::KernelKey& k)
 {
     switch (cls) {
-        case 0: return us::kernel_nt1(k);
-        case 1: return us::kernel_nt2(k);
-        case 2: return us::kernel_nt4(k);
-        default: return us::kernel_nt8(k);
+        case 0: return any_k ? us::kernel_nt<1, true>(k) : us::kernel_nt<1, false>(k);
+        case 1: return any_k ? us::kernel_nt<2, true>(k) : us::kernel_nt<2, false>(k);
+        case 2: return any_k ? us::kernel_nt<4, true>(k) : us::kernel_nt<4, false>(k);
+        default: return any_k ? us::kernel_nt<8, true>(k) : us::kernel_nt<8, false>(k);
     }
 }
 
-// The most warps with which two CTAs of every kernel that calls on this handle launch under the given plan share an SM's
-// registers: 16384 to a scheduler, allocated 8 a thread at a time. (The stage-timer builds need more and do not share one.)
+// The kernels that calls on this handle launch under a plan.
+KernelForms kernel_forms(const us_handle* h, int cls, int stages, bool local, bool xp)
+{
+    us::KernelKey k{stages, local, false, xp, false, h->host.fmt.C_A == 2, h->host.w2, false};
+    const bool any_k = h->host.K % 32 != 0;
+    KernelForms f;
+    f.plain = kernel_for(cls, any_k, k);
+    k.am = true;
+    f.chained = kernel_for(cls, any_k, k);
+    k.am = false; k.dp = true;   // a single token: dp4a beats the MMA (measured 2-3 %)
+    f.single = kernel_for(cls, any_k, k);
+    k.dp = false; k.timed = true;
+    f.timed = kernel_for(cls, any_k, k);
+    return f;
+}
+
+// The most warps with which two CTAs of each of them share an SM's registers: 16384 to a scheduler, allocated 8 a thread
+// at a time. (The stage-timer builds need more and do not share one.)
 int half_sm_warps(const us_handle* h, int cls, bool local, bool xp)
 {
-    const us::HostMatrix& hm = h->host;
-    const bool fold = hm.fmt.C_A == 2;
-    if (h->device < 0) return cls == 0 && !fold ? 12 : 10;   // host-only handle
+    if (h->device < 0) return cls == 0 && h->host.fmt.C_A == 1 ? 12 : 10;   // host-only handle
+    const KernelForms f = kernel_forms(h, cls, 1, local, xp);
     int regs = 0;
-    for (int form = 0; form < 3; ++form) {   // plain, chained, single token
-        us::KernelKey k{1, local, false, xp, form == 1, fold, hm.w2, form == 2, hm.K % 32 != 0};
-        const void* fn = kernel_for(cls, k);
+    for (const void* fn : {f.plain, f.chained, f.single}) {
         if (!fn) continue;
         cudaFuncAttributes fa;
         if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) { cudaGetLastError(); return 0; }
@@ -363,6 +383,7 @@ void build_plan(us_handle* h, int cls)
     LaunchGeom& g = pl.g;
     pl.ok = plan_launch(h, 8 << cls, &g);
     if (!pl.ok) return;
+    pl.fn = kernel_forms(h, cls, g.stages, h->s_local[cls] > 0, g.xp && h->s_local[cls] > 0);
     const us::HostMatrix& hm = h->host;
     us::SpmmParams& p = pl.p;
     std::memset(&p, 0, sizeof(p));
@@ -466,35 +487,24 @@ void build_tc_plan(us_handle* h, int ng)
     p.mg_segs = ((1ull << 40) / (uint64_t)hm.n_segs) + 1ull;
     p.mask_rows = hm.mask_rows; p.K_L = hm.fmt.K_L;
     p.acc_nt = nt_for(8 * ng);
+    pl.plain = us::kernel_tc(pl.octets, hm.K % 32 != 0, hm.fmt.C_A == 2, hm.w2, false);
+    pl.chained = us::kernel_tc(pl.octets, hm.K % 32 != 0, hm.fmt.C_A == 2, hm.w2, true);
     pl.ok = true;
 }
 
-// Opt the kernel variants for a K (any_k: no multiple of 32) in to the device's full dynamic shared memory: once per
-// device, when the first handle with such a K is made, so that us_spmm itself is nothing but a launch.
-cudaError_t enable_large_smem(int device, int bytes, bool any_k)
+// Opt a kernel in to the device's full dynamic shared memory, once per device. This also loads it, so that us_spmm itself
+// is nothing but a launch. Only what a handle's plans launch is loaded: a program's first handle takes 37 ms, 62 when it
+// loaded every kernel of the aligned K.
+cudaError_t enable_large_smem(int device, int bytes, const void* fn)
 {
     static std::mutex mu;
-    static std::vector<char> enabled[2];
+    static std::set<std::pair<int, const void*>> done;
+    if (!fn) return cudaSuccess;
     std::lock_guard<std::mutex> lock(mu);
-    std::vector<char>& done = enabled[any_k];
-    if (device < (int)done.size() && done[device]) return cudaSuccess;
-    for (int cls = 0; cls < 4; ++cls)
-        for (int bits = 0; bits < 256; ++bits) {
-            const us::KernelKey k{1 + (bits & 1), (bits & 2) != 0, (bits & 4) != 0, (bits & 8) != 0,
-                                  (bits & 16) != 0, (bits & 32) != 0, (bits & 64) != 0, (bits & 128) != 0, any_k};
-            const void* fn = kernel_for(cls, k);
-            if (!fn) continue;
-            const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-            if (e != cudaSuccess) return e;
-        }
-    for (int bits = 0; bits < 16; ++bits)
-        if (const void* fn = us::kernel_tc(bits & 8 ? 3 : 2, any_k, (bits & 1) != 0, (bits & 2) != 0, (bits & 4) != 0)) {
-            const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-            if (e != cudaSuccess) return e;
-        }
-    if (device >= (int)done.size()) done.resize(device + 1, 0);
-    done[device] = 1;
-    return cudaSuccess;
+    if (done.count({device, fn})) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) done.insert({device, fn});
+    return e;
 }
 
 // What a chained call adds to the plain one: the per-token absmax of a range of output rows, left
@@ -544,7 +554,7 @@ us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_sca
         }
         p.wait_ns_hi = h->wait_ns_hi;
         p.withhold = h->withhold;
-        const void* fn = us::kernel_tc(tc.octets, h->host.K % 32 != 0, h->host.fmt.C_A == 2, h->host.w2, p.y_amax != nullptr);
+        const void* fn = p.y_amax ? tc.chained : tc.plain;
         if (!fn) return US_ERR_UNSUPPORTED;
         return launch(h, fn, &p, tc.threads, tc.smem, st);
     }
@@ -565,17 +575,11 @@ us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_sca
     p.wait_ns_hi = h->wait_ns_hi;
     p.withhold = h->withhold;
 
-    us::KernelKey k{g.stages, p.s_local > 0, timers, g.xp && p.s_local > 0, p.y_amax != nullptr, p.fold_kb != 0, p.w2 != 0, false,
-                    h->host.K % 32 != 0};
-    // a single token: dp4a beats the MMA (measured 2-3 %)
-    k.dp = N == 1 && !k.timed && !k.xp && !k.am && !k.fold && !k.w2;
-    const void* fn = kernel_for(cls, k);
-    if (!fn && k.timed) {   // a variant without a timer build runs untimed
-        k.timed = false;
-        fn = kernel_for(cls, k);
-    }
+    // (a variant without a timer build runs untimed)
+    const bool timed = timers && !p.y_amax && pl.fn.timed;
+    const void* fn = p.y_amax ? pl.fn.chained : timed ? pl.fn.timed : N == 1 && !timers && pl.fn.single ? pl.fn.single : pl.fn.plain;
     if (!fn) return US_ERR_UNSUPPORTED;
-    p.timers = k.timed ? h->d_timers : nullptr;
+    p.timers = timed ? h->d_timers : nullptr;
 
     return launch(h, fn, &p, g.warps * 32, g.smem, st);
 }
@@ -654,9 +658,6 @@ us_status us_encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_sca
     }
     h->d_blob = dm.blob; h->d_item_off = dm.item_off; h->d_row_order = dm.row_order;
 
-    e = enable_large_smem(h->device, h->max_smem, hm.K % 32 != 0);
-    if (e != cudaSuccess) { free_device(h); delete h; return US_ERR_CUDA; }
-
     const int nt_max = nt_for(max_N);
     h->acc_bytes = (size_t)hm.n_strips * nt_max * 128 * sizeof(int32_t);
     h->cnt_bytes = (size_t)hm.n_strips * sizeof(uint32_t);
@@ -693,6 +694,13 @@ us_status us_encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_sca
         delete h;
         return US_ERR_UNSUPPORTED;
     }
+    for (const ClassPlan& pl : h->plan)
+        for (const void* fn : {pl.fn.plain, pl.fn.chained, pl.fn.single})
+            if (e == cudaSuccess) e = enable_large_smem(h->device, h->max_smem, fn);
+    for (const TcPlan& pl : h->tc)
+        for (const void* fn : {pl.plain, pl.chained})
+            if (e == cudaSuccess) e = enable_large_smem(h->device, h->max_smem, fn);
+    if (e != cudaSuccess) { free_device(h); delete h; return US_ERR_CUDA; }
     *out = h;
     return US_OK;
 }
@@ -908,6 +916,8 @@ us_status us_stage_timers(us_handle* h, int32_t enable, uint64_t* out, int32_t n
     if (!h->on_device) return US_ERR_UNSUPPORTED;
     const size_t bytes = us::kTimerWords * sizeof(unsigned long long);
     if (!h->d_timers) {
+        for (const ClassPlan& pl : h->plan)
+            if (enable_large_smem(h->device, h->max_smem, pl.fn.timed) != cudaSuccess) return US_ERR_CUDA;
         if (cudaMalloc((void**)&h->d_timers, bytes) != cudaSuccess) return US_ERR_ALLOC;
         cudaMemset(h->d_timers, 0, bytes);
     }

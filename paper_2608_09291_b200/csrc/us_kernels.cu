@@ -1,18 +1,19 @@
-// The instantiations of us_spmm_kernel for one N class: compiled once per class with -DUS_NT=1, 2, 4, 8.
+// The instantiations of us_spmm_kernel for one N class and one kind of K: compiled with -DUS_NT=1, 2, 4, 8 and -DUS_ANY=0, 1.
 #include "us_launch.h"
 #include "us_spmm_kernel.cuh"
 
-#ifndef US_NT
-#error "compile with -DUS_NT=1, 2, 4 or 8"
+#if !defined(US_NT) || !defined(US_ANY)
+#error "compile with -DUS_NT=1, 2, 4 or 8 and -DUS_ANY=0 or 1"
 #endif
 
 namespace us {
 namespace {
 
-template <bool ANY, int ST, bool LA>
+template <int ST, bool LA>
 const void* pick(const KernelKey& k)
 {
     constexpr int NT = US_NT;
+    constexpr bool ANY = US_ANY;
     constexpr bool kPacked = NT <= 4 && LA;   // packed X: planned for these classes and local mode only
     if (k.w2) {          // INT2 weights in folded tiles: plain kernels only
         if (k.timed || k.xp || k.am || k.dp) return nullptr;
@@ -44,25 +45,13 @@ const void* pick(const KernelKey& k)
     return k.timed ? (const void*)us_spmm_kernel<ANY, NT, ST, LA, true> : (const void*)us_spmm_kernel<ANY, NT, ST, LA, false>;
 }
 
-template <bool ANY>
-const void* pick_mode(const KernelKey& k)
-{
-    if (k.stages == 1) return k.local ? pick<ANY, 1, true>(k) : pick<ANY, 1, false>(k);
-    return k.local ? pick<ANY, 2, true>(k) : pick<ANY, 2, false>(k);
-}
-
-const void* pick_kernel(const KernelKey& k) { return k.any_k ? pick_mode<true>(k) : pick_mode<false>(k); }
-
 }  // namespace
 
-#if US_NT == 1
-const void* kernel_nt1(const KernelKey& k) { return pick_kernel(k); }
-#elif US_NT == 2
-const void* kernel_nt2(const KernelKey& k) { return pick_kernel(k); }
-#elif US_NT == 4
-const void* kernel_nt4(const KernelKey& k) { return pick_kernel(k); }
-#else
-const void* kernel_nt8(const KernelKey& k) { return pick_kernel(k); }
-#endif
+template <>
+const void* kernel_nt<US_NT, US_ANY>(const KernelKey& k)
+{
+    if (k.stages == 1) return k.local ? pick<1, true>(k) : pick<1, false>(k);
+    return k.local ? pick<2, true>(k) : pick<2, false>(k);
+}
 
 }  // namespace us

@@ -1,5 +1,6 @@
 // Which instantiation of us_spmm_kernel a launch needs. The kernels are compiled in one translation unit
-// per N class (us_kernels.cu with US_NT = 1, 2, 4, 8), so that they build in parallel.
+// per N class and kind of K (us_kernels.cu with US_NT = 1, 2, 4, 8 and US_ANY = 0, 1): they build in parallel, and a
+// program loads only the units that it uses.
 #pragma once
 
 namespace us {
@@ -13,14 +14,19 @@ struct KernelKey {
     bool fold;         // two column areas
     bool w2;           // INT2 weights
     bool dp;           // dp4a (a single token)
-    bool any_k;        // K is not a multiple of 32
 };
 
 // The kernel for a key, or nullptr where no such variant is built.
-const void* kernel_nt1(const KernelKey& k);
-const void* kernel_nt2(const KernelKey& k);
-const void* kernel_nt4(const KernelKey& k);
-const void* kernel_nt8(const KernelKey& k);
+template <int NT, bool ANY>   // ANY: K is not a multiple of 32
+const void* kernel_nt(const KernelKey& k);
+template <> const void* kernel_nt<1, false>(const KernelKey& k);
+template <> const void* kernel_nt<2, false>(const KernelKey& k);
+template <> const void* kernel_nt<4, false>(const KernelKey& k);
+template <> const void* kernel_nt<8, false>(const KernelKey& k);
+template <> const void* kernel_nt<1, true>(const KernelKey& k);
+template <> const void* kernel_nt<2, true>(const KernelKey& k);
+template <> const void* kernel_nt<4, true>(const KernelKey& k);
+template <> const void* kernel_nt<8, true>(const KernelKey& k);
 
 // us_spmm_tc_kernel (us_spmm_tc.cu) with two or three octets: any_k = K is not a multiple of 32; fold = two column areas; am = absmax of the output (default format only).
 const void* kernel_tc(int octets, bool any_k, bool fold, bool w2, bool am);
