@@ -4,6 +4,8 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <exception>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <set>
@@ -600,18 +602,22 @@ cudaError_t launch_small(void (*kernel)(P...), dim3 grid, cudaStream_t st, A... 
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
-}  // namespace
+// Frees a handle, whole or in the making.
+struct DeleteHandle {
+    void operator()(us_handle* h) const
+    {
+        if (h->d_blob) free_device(h);
+        delete h;
+    }
+};
+using HandlePtr = std::unique_ptr<us_handle, DeleteHandle>;
 
-extern "C" {
-
-us_status us_encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_scale,
-                    const us_format* fmt, int32_t max_N, uint32_t flags, us_handle** out)
+// us_encode after the checks of its arguments. May throw.
+us_status encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_scale, const us_format* fmt, int32_t max_N, uint32_t flags,
+                 HandlePtr* out)
 {
-    if (out) *out = nullptr;
-    if (!W || !out || M <= 0 || K <= 0 || max_N < 1 || max_N > 64) return US_ERR_INVALID_ARG;
-    if (M > 0x7FFFFFF0ll || K > 0x7FFFFFF0ll) return US_ERR_INVALID_ARG;
-    us_handle* h = new (std::nothrow) us_handle();
-    if (!h) return US_ERR_ALLOC;
+    HandlePtr owner(new us_handle());
+    us_handle* h = owner.get();
     h->max_N = max_N;
     const bool host_only = (flags & US_ENCODE_HOST_ONLY) != 0;
     cudaError_t e = cudaSuccess;
@@ -619,44 +625,37 @@ us_status us_encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_sca
         e = cudaGetDevice(&h->device);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-        if (e != cudaSuccess) { delete h; return US_ERR_CUDA; }
+        if (e != cudaSuccess) return US_ERR_CUDA;
         if (h->sm_count > us::kMaxCtas) h->sm_count = us::kMaxCtas;
     }
     const int n_cta = h->sm_count > 0 ? h->sm_count : 148;   // host-only handles plan for a 148-SM part
     us_format f = fmt ? *fmt : us_format{16, us::default_K_L(M, K, n_cta), 2, 1};
     us_status s;
-    us::DeviceMatrix dm;
     // the kernel's index arithmetic (exact division by multiplication) needs u * d < 2^40 for every
     // position u < n_items and divisor d <= n_items
     auto too_many = [&] { return h->host.n_items >= (1 << 20) || h->host.n_segs >= (1 << 16); };
-    try {
-        if (host_only) {
-            s = us::encode_host(W, M, K, w_scale, f, flags, 0, &h->host);
-        } else {
-            s = us::encode_layout(W, M, K, w_scale, f, flags, 0, true, &h->host);
-            if (s == US_OK && too_many()) s = US_ERR_UNSUPPORTED;
-            if (s == US_OK) s = us::encode_device(W, h->device, flags, &h->host, &dm);
-        }
-    } catch (const std::bad_alloc&) {
-        s = US_ERR_ALLOC;
+    if (host_only) {
+        s = us::encode_host(W, M, K, w_scale, f, flags, 0, &h->host);
+    } else {
+        us::DeviceMatrix dm;
+        s = us::encode_layout(W, M, K, w_scale, f, flags, 0, true, &h->host);
+        if (s == US_OK && too_many()) s = US_ERR_UNSUPPORTED;
+        if (s == US_OK) s = us::encode_device(W, h->device, flags, &h->host, &dm);
+        h->d_blob = dm.blob; h->d_item_off = dm.item_off; h->d_row_order = dm.row_order;
     }
-    if (s != US_OK) { delete h; return s; }
+    if (s != US_OK) return s;
     const us::HostMatrix& hm = h->host;
     if (!hm.kernel_layout) {   // a format without a kernel: statistics and decoding only
-        *out = h;
+        *out = std::move(owner);
         return US_OK;
     }
-    if (too_many()) {
-        delete h;
-        return US_ERR_UNSUPPORTED;
-    }
+    if (too_many()) return US_ERR_UNSUPPORTED;
     std::vector<uint32_t> sched[4];
     plan_classes(h, n_cta, sched);
     if (host_only) {
-        *out = h;
+        *out = std::move(owner);
         return US_OK;
     }
-    h->d_blob = dm.blob; h->d_item_off = dm.item_off; h->d_row_order = dm.row_order;
 
     const int nt_max = nt_for(max_N);
     h->acc_bytes = (size_t)hm.n_strips * nt_max * 128 * sizeof(int32_t);
@@ -681,28 +680,42 @@ us_status us_encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_sca
     alloc(&h->d_err, 16); clear(h->d_err, 16);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ps);
     if (e != cudaSuccess) {
-        free_device(h);
-        delete h;
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? US_ERR_ALLOC : US_ERR_CUDA;
     }
     h->on_device = true;
     for (int c = 0; c <= class_of(nt_max); ++c) build_plan(h, c);
     for (int ng = 1; ng <= (max_N + 7) / 8; ++ng) build_tc_plan(h, ng);
-    if (!h->plan[class_of(nt_max)].ok) {  // a tile does not fit the shared-memory ring
-        free_device(h);
-        delete h;
-        return US_ERR_UNSUPPORTED;
-    }
+    if (!h->plan[class_of(nt_max)].ok) return US_ERR_UNSUPPORTED;   // a tile does not fit the shared-memory ring
     for (const ClassPlan& pl : h->plan)
         for (const void* fn : {pl.fn.plain, pl.fn.chained, pl.fn.single})
             if (e == cudaSuccess) e = enable_large_smem(h->device, h->max_smem, fn);
     for (const TcPlan& pl : h->tc)
         for (const void* fn : {pl.plain, pl.chained})
             if (e == cudaSuccess) e = enable_large_smem(h->device, h->max_smem, fn);
-    if (e != cudaSuccess) { free_device(h); delete h; return US_ERR_CUDA; }
-    *out = h;
+    if (e != cudaSuccess) return US_ERR_CUDA;
+    *out = std::move(owner);
     return US_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+us_status us_encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_scale,
+                    const us_format* fmt, int32_t max_N, uint32_t flags, us_handle** out)
+{
+    if (out) *out = nullptr;
+    if (!W || !out || M <= 0 || K <= 0 || max_N < 1 || max_N > 64) return US_ERR_INVALID_ARG;
+    if (M > 0x7FFFFFF0ll || K > 0x7FFFFFF0ll) return US_ERR_INVALID_ARG;
+    try {
+        HandlePtr h;
+        const us_status s = encode(W, M, K, w_scale, fmt, max_N, flags, &h);
+        *out = h.release();
+        return s;
+    } catch (const std::exception&) {   // no host memory
+        return US_ERR_ALLOC;
+    }
 }
 
 us_status us_get_stats(const us_handle* h, us_stats* out)
@@ -965,9 +978,7 @@ us_status us_stage_timers(us_handle* h, int32_t enable, uint64_t* out, int32_t n
 
 us_status us_destroy(us_handle* h)
 {
-    if (!h) return US_OK;
-    if (h->on_device) free_device(h);
-    delete h;
+    if (h) DeleteHandle()(h);
     return US_OK;
 }
 

@@ -8,6 +8,8 @@
 #include <atomic>
 #include <cstdlib>
 #include <cstring>
+#include <exception>
+#include <mutex>
 #include <numeric>
 #include <thread>
 
@@ -25,25 +27,33 @@ int pick_threads(int threads, int64_t work_units)
     return std::min(threads, 64);
 }
 
+// f(i, thread) for all i < n. Where fewer threads can be started, those do it; what f throws is thrown again here.
 template <class F>
 void parallel_for(int64_t n, int threads, F&& f)
 {
     threads = pick_threads(threads, n);
-    if (threads == 1) {
-        for (int64_t i = 0; i < n; ++i) f(i, 0);
-        return;
-    }
-    std::vector<std::thread> pool;
     std::atomic<int64_t> next{0};
-    for (int t = 0; t < threads; ++t)
-        pool.emplace_back([&, t] {
-            for (;;) {
-                int64_t i = next.fetch_add(1);
-                if (i >= n) break;
-                f(i, t);
-            }
-        });
+    std::exception_ptr failed;
+    std::mutex mu;
+    auto work = [&](int t) {
+        (void)std::uncaught_exceptions();   // has the thread's exception state allocated now: where that fails later, the C library aborts
+        try {
+            for (int64_t i; (i = next.fetch_add(1)) < n;) f(i, t);
+        } catch (...) {
+            next.store(n);
+            std::lock_guard<std::mutex> lock(mu);
+            failed = std::current_exception();
+        }
+    };
+    std::vector<std::thread> pool;
+    pool.reserve((size_t)threads);
+    try {
+        for (int t = 1; t < threads; ++t) pool.emplace_back(work, t);
+    } catch (const std::exception&) {
+    }
+    work(0);
     for (auto& th : pool) th.join();
+    if (failed) std::rethrow_exception(failed);
 }
 
 // Bitmap-aware row reordering (paper Sec. V-B, Alg. 1) in its per-strip form: within each strip
@@ -462,12 +472,7 @@ us_status encode_host(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_s
         if (off16 > 0xFFFFFFFFull) { h = HostMatrix(); return US_ERR_ALLOC; }
     }
     h.item_off[h.n_items] = (uint32_t)off16;
-    try {
-        h.blob.assign((size_t)off16 * 16, 0);
-    } catch (...) {
-        h = HostMatrix();
-        return US_ERR_ALLOC;
-    }
+    h.blob.assign((size_t)off16 * 16, 0);
     parallel_for(h.n_items, threads, [&](int64_t t, int) {
         std::memcpy(h.blob.data() + (size_t)h.item_off[t] * 16, blobs[t].data(), blobs[t].size());
         std::vector<uint8_t>().swap(blobs[t]);

@@ -1,6 +1,7 @@
 // Bringing a weight onto the GPU: packing on the host's cores, upload and encoding overlapped, device memory from a pool.
 #include <algorithm>
 #include <atomic>
+#include <exception>
 #include <mutex>
 #include <thread>
 
@@ -52,6 +53,25 @@ cudaError_t open_device(int device, Device** out)
     return e;
 }
 
+// What encode_device holds, given back on every way out: its temporaries in stream order, the matrix too unless it is done.
+struct Scratch {
+    cudaStream_t st;
+    DeviceMatrix* out;
+    uint8_t* dense = nullptr;
+    uint32_t* size16 = nullptr;
+    unsigned long long* sums = nullptr;   // total size, largest size, sum of P
+    bool done = false;
+    ~Scratch()
+    {
+        if (!done) cudaStreamSynchronize(st);
+        for (void* p : {(void*)dense, (void*)size16, (void*)sums}) if (p) cudaFreeAsync(p, st);
+        if (done) return;
+        for (void* p : {(void*)out->blob, (void*)out->item_off, (void*)out->row_order}) if (p) cudaFreeAsync(p, st);
+        *out = DeviceMatrix();
+        cudaGetLastError();
+    }
+};
+
 }  // namespace
 
 cudaError_t pool_alloc(int device, void** p, size_t bytes)
@@ -84,24 +104,12 @@ us_status encode_device(const int8_t* W, int device, uint32_t flags, HostMatrix*
     if (open_device(device, &d) != cudaSuccess) return US_ERR_CUDA;
     cudaStream_t st = d->stream;
 
-    uint8_t* dense = nullptr;
-    uint32_t* size16 = nullptr;
-    unsigned long long* sums = nullptr;   // total size, largest size, sum of P
-    auto give_back = [&](us_status s) {
-        cudaStreamSynchronize(st);
-        for (void* p : {(void*)dense, (void*)size16, (void*)sums}) if (p) cudaFreeAsync(p, st);
-        if (s != US_OK) {
-            for (void* p : {(void*)out->blob, (void*)out->item_off, (void*)out->row_order}) if (p) cudaFreeAsync(p, st);
-            *out = DeviceMatrix();
-            cudaGetLastError();
-        }
-        return s;
-    };
+    Scratch t{st, out};
     auto alloc = [&](auto** p, size_t bytes) { return cudaMallocFromPoolAsync((void**)p, std::max<size_t>(bytes, 16), d->pool, st); };
-    if (alloc(&dense, (size_t)total) != cudaSuccess || alloc(&size16, (size_t)h.n_items * 4) != cudaSuccess ||
-        alloc(&sums, 24) != cudaSuccess || alloc(&out->item_off, (size_t)(h.n_items + 1) * 4) != cudaSuccess ||
+    if (alloc(&t.dense, (size_t)total) != cudaSuccess || alloc(&t.size16, (size_t)h.n_items * 4) != cudaSuccess ||
+        alloc(&t.sums, 24) != cudaSuccess || alloc(&out->item_off, (size_t)(h.n_items + 1) * 4) != cudaSuccess ||
         alloc(&out->row_order, (size_t)h.Mp * 4) != cudaSuccess)
-        return give_back(US_ERR_ALLOC);
+        return US_ERR_ALLOC;
 
     // ---- pack to INT4 (range check, nonzeros per row) and upload, chunk by chunk on all cores ----------------------
     const size_t chunk = (size_t)std::min<int64_t>(kChunk, std::max<int64_t>(32 * 1024, (total / (2 * kMaxThreads) + 4095) / 4096 * 4096));
@@ -111,28 +119,32 @@ us_status encode_device(const int8_t* W, int device, uint32_t flags, HostMatrix*
     for (auto& c : row_nnz) c.store(0, std::memory_order_relaxed);
     std::atomic<int64_t> next{0};
     std::atomic<int> bad{0}, failed{0};
-    auto work = [&](int t) {
-        if (t > 0 && cudaSetDevice(device) != cudaSuccess) { failed = 1; return; }
+    auto work = [&](int i) {
+        if (i > 0 && cudaSetDevice(device) != cudaSuccess) { failed = 1; return; }
         for (int k = 0;; ++k) {
             const int64_t c = next.fetch_add(1);
             if (c >= n_chunks || bad.load(std::memory_order_relaxed)) break;
-            const int b = 2 * t + (k & 1);
+            const int b = 2 * i + (k & 1);
             uint8_t* buf = d->staging + (size_t)b * kChunk;
             if (k >= 2 && cudaEventSynchronize(d->copied[b]) != cudaSuccess) { failed = 1; break; }
             const int64_t o0 = c * (int64_t)chunk, o1 = std::min<int64_t>(total, o0 + (int64_t)chunk);
             if (!pack_int4(W, K, ld, o0, o1, buf, h.w2, row_nnz.data())) { bad = 1; break; }
-            if (cudaMemcpyAsync(dense + o0, buf, (size_t)(o1 - o0), cudaMemcpyHostToDevice, st) != cudaSuccess ||
+            if (cudaMemcpyAsync(t.dense + o0, buf, (size_t)(o1 - o0), cudaMemcpyHostToDevice, st) != cudaSuccess ||
                 cudaEventRecord(d->copied[b], st) != cudaSuccess) { failed = 1; break; }
         }
     };
     {
         std::vector<std::thread> pool;
-        for (int t = 1; t < n_thr; ++t) pool.emplace_back(work, t);
+        pool.reserve((size_t)n_thr);
+        try {
+            for (int i = 1; i < n_thr; ++i) pool.emplace_back(work, i);
+        } catch (const std::exception&) {   // fewer threads do it too
+        }
         work(0);
-        for (auto& t : pool) t.join();
+        for (auto& th : pool) th.join();
     }
-    if (bad) return give_back(US_ERR_VALUE_RANGE);
-    if (failed) return give_back(US_ERR_CUDA);
+    if (bad) return US_ERR_VALUE_RANGE;
+    if (failed) return US_ERR_CUDA;
     if (sort) {
         std::vector<int64_t> cnt((size_t)M);
         for (int64_t r = 0; r < M; ++r) cnt[r] = row_nnz[r].load(std::memory_order_relaxed);
@@ -143,30 +155,30 @@ us_status encode_device(const int8_t* W, int device, uint32_t flags, HostMatrix*
 
     // ---- tile sizes, offsets, tiles ---------------------------------------------------------------------------------
     EncodeParams p = {};
-    p.W = dense; p.row_order = out->row_order; p.ld = ld;
+    p.W = t.dense; p.row_order = out->row_order; p.ld = ld;
     p.n_segs = (int32_t)h.n_segs; p.n_items = (int32_t)h.n_items; p.K_L = h.fmt.K_L; p.mask_rows = h.mask_rows;
     p.fold = h.fmt.C_A == 2; p.w2 = h.w2;
-    p.size16 = size16; p.item_off = out->item_off; p.sum_P = sums + 2;
-    cudaMemsetAsync(sums, 0, 24, st);
+    p.size16 = t.size16; p.item_off = out->item_off; p.sum_P = t.sums + 2;
+    cudaMemsetAsync(t.sums, 0, 24, st);
     cudaMemcpyAsync(out->row_order, h.row_order.data(), (size_t)h.Mp * 4, cudaMemcpyHostToDevice, st);
     const unsigned blocks = (unsigned)((h.n_items + 7) / 8);
     us_encode_size_kernel<<<blocks, 256, 0, st>>>(p);
-    us_encode_scan_kernel<<<1, 1024, 0, st>>>(size16, out->item_off, p.n_items, sums);
+    us_encode_scan_kernel<<<1, 1024, 0, st>>>(t.size16, out->item_off, p.n_items, t.sums);
     unsigned long long got[3] = {0, 0, 0};
     h.item_off.resize((size_t)h.n_items + 1);
-    cudaMemcpyAsync(got, sums, sizeof(got), cudaMemcpyDeviceToHost, st);
+    cudaMemcpyAsync(got, t.sums, sizeof(got), cudaMemcpyDeviceToHost, st);
     cudaMemcpyAsync(h.item_off.data(), out->item_off, h.item_off.size() * 4, cudaMemcpyDeviceToHost, st);
-    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return give_back(US_ERR_CUDA);
-    if (got[0] > 0xFFFFFFFFull) return give_back(US_ERR_ALLOC);
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return US_ERR_CUDA;
+    if (got[0] > 0xFFFFFFFFull) return US_ERR_ALLOC;
     h.blob_bytes = got[0] * 16;
     h.max_item_bytes = (uint32_t)got[1] * 16u;
     h.sum_P = (int64_t)got[2];
     h.bytes_payload_padded = (int64_t)h.blob_bytes - h.n_items * (int64_t)h.mask_rows * 128;
-    if (alloc(&out->blob, (size_t)h.blob_bytes) != cudaSuccess) return give_back(US_ERR_ALLOC);
+    if (alloc(&out->blob, (size_t)h.blob_bytes) != cudaSuccess) return US_ERR_ALLOC;
     p.blob = out->blob;
     us_encode_write_kernel<<<blocks, 256, 0, st>>>(p);
-    if (cudaGetLastError() != cudaSuccess) return give_back(US_ERR_CUDA);
-    for (void* q : {(void*)dense, (void*)size16, (void*)sums}) cudaFreeAsync(q, st);   // (in stream order)
+    if (cudaGetLastError() != cudaSuccess) return US_ERR_CUDA;
+    t.done = true;
     return US_OK;
 }
 

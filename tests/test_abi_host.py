@@ -1,7 +1,10 @@
 """Host side of the C-ABI library: exported symbols, encoder / decoder / statistics against the
 oracle, error behaviour, schedule geometry. No GPU needed (US_ENCODE_HOST_ONLY)."""
 import ctypes
+import os
 import re
+import subprocess
+import sys
 from pathlib import Path
 
 import numpy as np
@@ -216,3 +219,37 @@ def test_w2_errors(b):
 def test_pack_int4(b):
     X = np.array([[1, -2, 7, -8, 0]], np.int8)
     assert list(b.pack_int4(X)[0]) == [0x1 | (0xE << 4), 0x7 | (0x8 << 4), 0x0]
+
+
+_NO_MEMORY = """
+import resource, sys
+sys.path.insert(0, '.')
+import numpy as np
+from paper_2608_09291_b200 import binding as b, workloads
+W = np.tile(workloads.make_weight(64, 4096, 0.5, seed=1), (64, 1))
+refused = 0
+for fmt, flags in (((16, 512, 2, 1), 0), ((16, 128, 2, 1), 2), ((16, 512, 2, 1), 4), ((16, 64, 2, 2), 0)):
+    for extra in (1, 3, 6, 9, 12, 20):   # MB of address space left
+        used = int(open('/proc/self/statm').read().split()[0]) * resource.getpagesize()
+        resource.setrlimit(resource.RLIMIT_AS, (used + (extra << 20), resource.RLIM_INFINITY))
+        try:
+            b.us_destroy(b.us_encode(W, fmt=fmt, flags=b.US_ENCODE_HOST_ONLY | flags))
+        except b.UsError as e:
+            assert e.status == 5, e
+            refused += 1
+        finally:
+            resource.setrlimit(resource.RLIMIT_AS, (resource.RLIM_INFINITY, resource.RLIM_INFINITY))
+    h = b.us_encode(W, fmt=fmt, flags=b.US_ENCODE_HOST_ONLY | flags)
+    assert (b.us_decode(h) == W).all()
+    b.us_destroy(h)
+print('refused', refused)
+"""
+
+
+def test_no_host_memory_is_a_status():
+    """Where memory or threads run out, at whatever step, us_encode returns US_ERR_ALLOC: no exception leaves the C ABI, no
+    thread is left behind, and the next call works."""
+    r = subprocess.run([sys.executable, "-c", _NO_MEMORY], cwd=ROOT, capture_output=True, text=True, timeout=300,
+                       env=dict(os.environ, MALLOC_ARENA_MAX="1"))
+    assert r.returncode == 0, (r.returncode, r.stdout[-500:], r.stderr[-1500:])
+    assert int(r.stdout.split()[-1]) >= 4, r.stdout
