@@ -3,8 +3,8 @@ calls go through ctypes; the calls made per product go through a native module (
 marshalling them in Python takes longer than a small product takes on the GPU.
 
 Every step of the SpMM runs in the CUDA library; there is no CPU fallback. Importing this module
-fails loudly when the compiled library is missing (build it with ``python -m
-paper_2608_09291_b200.build`` or ``__graft_entry__.build()``).
+fails loudly when the compiled library is missing, and the first call that takes tensors when the native
+module is (build them with ``python -m paper_2608_09291_b200.build`` or ``__graft_entry__.build()``).
 """
 from __future__ import annotations
 
@@ -15,10 +15,9 @@ import numpy as np
 
 _LIB_PATH = Path(__file__).resolve().parent / "libunionsparse.so"
 _EXT_PATH = _LIB_PATH.with_name("_us_torch.so")
-for _p in (_LIB_PATH, _EXT_PATH):
-    if not _p.exists():
-        raise ImportError(f"{_p} is missing: build the CUDA library first "
-                          "(python -m paper_2608_09291_b200.build)")
+if not _LIB_PATH.exists():
+    raise ImportError(f"{_LIB_PATH} is missing: build the CUDA library first "
+                      "(python -m paper_2608_09291_b200.build)")
 _lib = ctypes.CDLL(str(_LIB_PATH))
 
 US_OK = 0
@@ -86,6 +85,8 @@ def _native():
     global _ext
     if _ext is None:
         import torch  # noqa: F401  (its libraries have to be loaded first)
+        if not _EXT_PATH.exists():
+            raise ImportError(f"{_EXT_PATH} is missing: build it first (python -m paper_2608_09291_b200.build)")
         from . import _us_torch
         _us_torch.set_error(UsError)
         _ext = _us_torch

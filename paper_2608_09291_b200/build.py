@@ -1,6 +1,8 @@
-"""Builds the native code in-tree: the C-ABI CUDA library (nvcc, sm_100a) and the Python front end on it."""
+"""Builds the native code in-tree: the C-ABI CUDA library (nvcc, sm_100a) and, where torch is installed, the native module
+of the Python front end on it (the calls that take tensors)."""
 from __future__ import annotations
 
+import importlib.util
 import os
 import subprocess
 import sys
@@ -47,11 +49,18 @@ def _newest(paths) -> float:
     return max(p.stat().st_mtime for p in paths)
 
 
+def _lib_stale() -> bool:
+    return not LIB.exists() or LIB.stat().st_mtime < _newest([u[0] for u in UNITS] + HEADERS)
+
+
+def _ext_stale() -> bool:
+    if importlib.util.find_spec("torch") is None:   # nothing to build it for
+        return False
+    return not EXT.exists() or EXT.stat().st_mtime < _newest([EXT_SOURCE, PKG.parent / "include" / "unionsparse.h"])
+
+
 def is_stale() -> bool:
-    if not LIB.exists() or not EXT.exists():
-        return True
-    return (LIB.stat().st_mtime < _newest([u[0] for u in UNITS] + HEADERS) or
-            EXT.stat().st_mtime < _newest([EXT_SOURCE, PKG.parent / "include" / "unionsparse.h"]))
+    return _lib_stale() or _ext_stale()
 
 
 def _run(cmd: list[str], verbose: bool = False) -> None:
@@ -63,7 +72,7 @@ def _run(cmd: list[str], verbose: bool = False) -> None:
 
 
 def build(force: bool = False, verbose: bool = False) -> Path:
-    if force or verbose or is_stale():
+    if force or verbose or _lib_stale():
         with tempfile.TemporaryDirectory() as tmp, ThreadPoolExecutor(len(UNITS)) as pool:
             objs = [str(Path(tmp) / o) for _, _, o in UNITS]
             jobs = [pool.submit(_run, ["nvcc", *nvcc_flags(verbose), *flags, "-c", str(src), "-o", obj], verbose)
@@ -73,6 +82,9 @@ def build(force: bool = False, verbose: bool = False) -> Path:
             new = LIB.with_suffix(f".tmp{os.getpid()}.so")
             _run(["nvcc", *nvcc_flags(), "-shared", *objs, "-o", str(new)])
             os.replace(new, LIB)
+    if importlib.util.find_spec("torch") is None:
+        sys.stderr.write(f"torch is not installed: {EXT.name} (the calls that take tensors) is not built\n")
+    elif force or verbose or _ext_stale():
         new = EXT.with_suffix(f".tmp{os.getpid()}.so")
         _run(ext_command(new))
         os.replace(new, EXT)

@@ -3,6 +3,7 @@ oracle, error behaviour, schedule geometry. No GPU needed (US_ENCODE_HOST_ONLY).
 import ctypes
 import os
 import re
+import shutil
 import subprocess
 import sys
 from pathlib import Path
@@ -253,3 +254,35 @@ def test_no_host_memory_is_a_status():
                        env=dict(os.environ, MALLOC_ARENA_MAX="1"))
     assert r.returncode == 0, (r.returncode, r.stdout[-500:], r.stderr[-1500:])
     assert int(r.stdout.split()[-1]) >= 4, r.stdout
+
+
+_NO_TORCH = """
+import sys
+sys.path.insert(0, sys.argv[1])
+if sys.argv[2] == "hide":
+    sys.modules["torch"] = None
+import numpy as np
+if sys.argv[2] == "hide":
+    from paper_2608_09291_b200 import build
+    assert not build.is_stale()
+    build.build()
+from paper_2608_09291_b200 import binding as b
+W = np.eye(16, 256, dtype=np.int8)
+h = b.us_encode(W, flags=b.US_ENCODE_HOST_ONLY)
+assert (b.us_decode(h) == W).all() and b.us_get_stats(h)["nnz"] == 16
+b.us_destroy(h)
+try:
+    b.SparseWeight(W)
+except ImportError as e:
+    print("ImportError", e)
+"""
+
+
+@pytest.mark.parametrize("torch_is", ["hide", "keep"])
+def test_host_calls_need_neither_torch_nor_the_native_module(tmp_path, torch_is):
+    """Encoding, statistics and decoding on the host work from the C library alone; what takes tensors fails loudly."""
+    for d in ("paper_2608_09291_b200", "include"):
+        shutil.copytree(ROOT / d, tmp_path / d, ignore=shutil.ignore_patterns("_us_torch*", "__pycache__"))
+    r = subprocess.run([sys.executable, "-c", _NO_TORCH, str(tmp_path), torch_is], cwd=tmp_path, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-1500:]
+    assert "ImportError" in r.stdout and ("torch" if torch_is == "hide" else "_us_torch.so is missing") in r.stdout
