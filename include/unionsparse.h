@@ -256,7 +256,8 @@ us_status us_destroy(us_handle* h);
 /* Algorithmic bytes one us_spmm call moves: encoded W as stored + X + Y + scales. */
 int64_t us_spmm_bytes(const us_handle* h, int32_t N, int32_t fp16_out);
 
-/* Launch geometry of the next us_spmm(N): CTAs, threads per CTA, dynamic shared memory. */
+/* Launch geometry of the next us_spmm(N): CTAs, threads per CTA, dynamic shared memory. For a host-only handle, what a
+ * handle on a B200 would have. */
 us_status us_launch_info(const us_handle* h, int32_t N, int32_t* grid, int32_t* block,
                          int32_t* smem_bytes);
 

@@ -50,9 +50,9 @@ struct us_handle {
     ClassPlan plan[4];               // per N class (NT = 1, 2, 4, 8)
     bool on_device = false;
     int device = -1;
-    int sm_count = 0;
+    int sm_count = 148;               // (host-only handles plan for a 148-SM part)
     int max_N = 0;
-    int max_smem = 0;
+    int max_smem = 227 * 1024;
     uint8_t* d_blob = nullptr;
     uint32_t* d_item_off = nullptr;
     std::vector<uint32_t> cta_begin[4];  // schedule per N class (NT = 1, 2, 4, 8)
@@ -201,7 +201,7 @@ bool plan_launch(const us_handle* h, int N, LaunchGeom* g)
                            us::kClaimWords * 4 + s_local * (g->nt * 128 + 1) * 4 + 2 * us::kOffTable * 4 + 128;
     };
     int fixed_base = fixed_for(lut_rep);
-    const int limit = h->max_smem > 0 ? h->max_smem : 227 * 1024;
+    const int limit = h->max_smem;
     // Ring depth: two slots per warp when that still gives (nearly) all the warps; else one slot per
     // warp and more warps -- measured on the 70B-shaped FFN: 16 warps x 1 slot beat 9 warps x 2.
     auto warps_for = [&](int stages) {
@@ -215,7 +215,7 @@ bool plan_launch(const us_handle* h, int N, LaunchGeom* g)
         const int w8 = std::max(warps_for(1), warps_for(2));
         // 32 copies only for long-running CTAs (measured: 1 % faster on the 70B-shaped FFN, but the
         // 4096 x 4096 case -- about one tile per warp -- loses 5 % to the bigger table)
-        const int64_t n_cta = h->sm_count > 0 ? h->sm_count : 148;
+        const int64_t n_cta = h->sm_count;
         const bool long_run = (h->host.n_items + n_cta - 1) / n_cta >= 4 * (int64_t)w8;
         if (w32 >= w8 && long_run) { lut_rep = 32; fixed_base = fixed_for(32); } else { lut_rep = 8; }
     }
@@ -228,7 +228,7 @@ bool plan_launch(const us_handle* h, int N, LaunchGeom* g)
     // under this one's work; with one CTA per SM, programmatic dependent launch alone hides only the
     // launch latency, because all CTAs of a launch end at about the same time.
     // Measured on 4096 x 4096, N = 8: 6.6 -> 5.7 us; not worth it from ~20 tiles per CTA on.
-    const int64_t n_cta = h->sm_count > 0 ? h->sm_count : 148;
+    const int64_t n_cta = h->sm_count;
     const int64_t per_cta = (h->host.n_items + n_cta - 1) / n_cta;
     // the most tiles a CTA has: cuts fall on strip boundaries, so it can be more than the average (5008 x 3008, 3 tiles to a
     // strip: most CTAs have two strips, some three, and eight warps would need a second round for the ninth tile: 5.7 us
@@ -261,9 +261,11 @@ bool plan_launch(const us_handle* h, int N, LaunchGeom* g)
 
 // Chooses, per N class, the K-range width, whether strips are summed in shared memory, and whether
 // X is staged packed.
-void plan_classes(us_handle* h, int n_cta, std::vector<uint32_t> (&sched)[4])
+void plan_classes(us_handle* h)
 {
-    const int limit = h->max_smem > 0 ? h->max_smem : 227 * 1024;
+    const int n_cta = h->sm_count;
+    std::vector<uint32_t> (&sched)[4] = h->cta_begin;
+    const int limit = h->max_smem;
     for (int c = 0; c < 4; ++c) {
         const int nt = 1 << c;
         // Local mode needs the strip sums of a CTA's share of one K range in shared memory; a short
@@ -311,13 +313,13 @@ void plan_classes(us_handle* h, int n_cta, std::vector<uint32_t> (&sched)[4])
         if (nt <= 4 && !h->host.w2) {   // (no packed-X kernel for INT2 weights)
             const int64_t n_segs = h->host.n_segs;
             const int64_t ranges = h->s_local[c] > 0 ? (n_segs + h->G[c] - 1) / h->G[c] : n_segs + 1;
-            const bool small_share = nt >= 2 && (int64_t)h->host.blob_bytes / std::max(1, n_cta) < 128 * 1024;
+            const bool small_share = nt >= 2 && (int64_t)h->host.blob_bytes / n_cta < 128 * 1024;
             // N <= 8: packed X when that is what lets the half-SM plan of plan_launch hold its eight warps
             // (4096 x 4096 at 30 % sparsity: tiles of 9.5 KB and 32 KB of int8 X do not fit half an SM, with
             // 16 KB of packed X they do: 5.6 -> 4.6 us; the same for the folded format at 50 %: 5.3 -> 4.35)
             bool for_half_sm = false;
             if (nt == 1 && ranges == 1 && coresident_knob() && h->host.Kp <= coresident_K(h->host.K, nt)) {
-                const int64_t per_cta = (h->host.n_items + n_cta - 1) / std::max(1, n_cta);
+                const int64_t per_cta = (h->host.n_items + n_cta - 1) / n_cta;
                 const int64_t need = 8;
                 auto fits = [&](bool xp, int s_loc) {
                     const int64_t fixed8 = 256 * 8 * 4 + (int64_t)us::kLutScratchBytes + x_bytes(nt, n_segs, h->host.fmt.K_L, xp) +
@@ -402,12 +404,12 @@ void build_plan(us_handle* h, int cls)
         // Claim runs of up to a whole strip's segments of the range (the partial sums of a run stay
         // in registers; the kernel shortens the runs towards the end of a CTA's range), but never
         // so long that a CTA's warps run out of runs to share.
-        const int64_t per_cta = std::max<int64_t>(1, hm.n_items / std::max(1, h->sm_count));
+        const int64_t per_cta = std::max<int64_t>(1, hm.n_items / h->sm_count);
         const int balanced = (int)std::max<int64_t>(1, per_cta / (4 * (int64_t)g.warps));
         p.run_len = std::max(1, std::min(std::min(p.G, 2 * balanced), p.G));
         // Fewer tiles than warps: one tile per warp, all at once (1024 x 1024, N = 8: 4.1 -> 3.1 us); with more
         // tiles than warps, runs of two keep a run's sums in registers and win (4096 x 4096: 5.7 against 6.3 us).
-        if ((hm.n_items + h->sm_count - 1) / std::max(1, h->sm_count) <= g.warps) p.run_len = 1;
+        if ((hm.n_items + h->sm_count - 1) / h->sm_count <= g.warps) p.run_len = 1;
     }
     p.row_order = h->d_row_order; p.w_scale = h->d_w_scale;
     p.err = h->d_err;
@@ -457,7 +459,7 @@ void build_tc_plan(us_handle* h, int ng)
                                              : mean >= 4;
     if (tc_knob() == 0 || (tc_knob() == 1 && !better)) return;
     p.slot_bytes = slot_bytes_for(hm);
-    const int limit = h->max_smem > 0 ? h->max_smem : 227 * 1024;
+    const int limit = h->max_smem;
     auto fixed_for = [&](int x_stages, int lut_rep) { return 256 * lut_rep * 4 + x_stages * ng * 2048 + 2048 + us::kTcFixedSmem; };
     auto slots_for = [&](int x_stages, int lut_rep) {
         return std::min(us::kTcMaxSlots, (limit - fixed_for(x_stages, lut_rep)) / (int)p.slot_bytes);
@@ -628,8 +630,7 @@ us_status encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_scale,
         if (e != cudaSuccess) return US_ERR_CUDA;
         if (h->sm_count > us::kMaxCtas) h->sm_count = us::kMaxCtas;
     }
-    const int n_cta = h->sm_count > 0 ? h->sm_count : 148;   // host-only handles plan for a 148-SM part
-    us_format f = fmt ? *fmt : us_format{16, us::default_K_L(M, K, n_cta), 2, 1};
+    us_format f = fmt ? *fmt : us_format{16, us::default_K_L(M, K, h->sm_count), 2, 1};
     us_status s;
     // the kernel's index arithmetic (exact division by multiplication) needs u * d < 2^40 for every
     // position u < n_items and divisor d <= n_items
@@ -650,17 +651,20 @@ us_status encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_scale,
         return US_OK;
     }
     if (too_many()) return US_ERR_UNSUPPORTED;
-    std::vector<uint32_t> sched[4];
-    plan_classes(h, n_cta, sched);
+    const int nt_max = nt_for(max_N);
+    auto lay_plans = [&] {
+        for (int c = 0; c <= class_of(nt_max); ++c) build_plan(h, c);
+        for (int ng = 1; ng <= (max_N + 7) / 8; ++ng) build_tc_plan(h, ng);
+    };
+    plan_classes(h);
     if (host_only) {
+        lay_plans();   // (for us_launch_info)
         *out = std::move(owner);
         return US_OK;
     }
 
-    const int nt_max = nt_for(max_N);
     h->acc_bytes = (size_t)hm.n_strips * nt_max * 128 * sizeof(int32_t);
     h->cnt_bytes = (size_t)hm.n_strips * sizeof(uint32_t);
-    for (int c = 0; c < 4; ++c) h->cta_begin[c] = sched[c];
     cudaStream_t ps = us::pool_stream(h->device);
     auto alloc = [&](auto** p, size_t bytes) {
         if (e == cudaSuccess) e = us::pool_alloc(h->device, (void**)p, bytes);
@@ -684,8 +688,7 @@ us_status encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_scale,
         return e == cudaErrorMemoryAllocation ? US_ERR_ALLOC : US_ERR_CUDA;
     }
     h->on_device = true;
-    for (int c = 0; c <= class_of(nt_max); ++c) build_plan(h, c);
-    for (int ng = 1; ng <= (max_N + 7) / 8; ++ng) build_tc_plan(h, ng);
+    lay_plans();
     if (!h->plan[class_of(nt_max)].ok) return US_ERR_UNSUPPORTED;   // a tile does not fit the shared-memory ring
     for (const ClassPlan& pl : h->plan)
         for (const void* fn : {pl.fn.plain, pl.fn.chained, pl.fn.single})
@@ -759,17 +762,12 @@ us_status us_launch_info(const us_handle* h, int32_t N, int32_t* grid, int32_t* 
 {
     if (!h || N < 1 || N > h->max_N) return US_ERR_INVALID_ARG;
     if (!h->host.kernel_layout) return US_ERR_UNSUPPORTED;
-    if (h->tc[(N + 7) / 8].ok) {
-        if (grid) *grid = h->sm_count;
-        if (block) *block = h->tc[(N + 7) / 8].threads;
-        if (smem_bytes) *smem_bytes = h->tc[(N + 7) / 8].smem;
-        return US_OK;
-    }
-    LaunchGeom g;
-    if (!plan_launch(h, N, &g)) return US_ERR_UNSUPPORTED;
-    if (grid) *grid = h->sm_count > 0 ? h->sm_count : 148;
-    if (block) *block = g.warps * 32;
-    if (smem_bytes) *smem_bytes = g.smem;
+    const TcPlan& tc = h->tc[(N + 7) / 8];
+    const ClassPlan& pl = h->plan[class_of(nt_for(N))];
+    if (!tc.ok && !pl.ok) return US_ERR_UNSUPPORTED;
+    if (grid) *grid = h->sm_count;
+    if (block) *block = tc.ok ? tc.threads : pl.g.warps * 32;
+    if (smem_bytes) *smem_bytes = tc.ok ? tc.smem : pl.g.smem;
     return US_OK;
 }
 

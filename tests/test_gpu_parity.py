@@ -460,3 +460,18 @@ def test_stage_timers_on_every_plan_variant(b):
             assert d["warps"] >= 0
         finally:
             sw.close()
+
+
+@pytest.mark.parametrize("M,K,fmt,flags", [(1024, 1024, None, 0), (4096, 4096, None, 0), (512, 8192, None, 0), (24000, 1024, None, 0),
+                                           (5003, 3001, (16, 512, 2, 2), 0), (4001, 2500, (16, 512, 2, 2), 8), (8160, 9216, None, 0)])
+def test_launch_info_of_a_host_only_handle(b, M, K, fmt, flags):
+    """One plan serves the launches and us_launch_info, and a host-only handle lays the same."""
+    W = (workloads.make_weight_w2 if flags & 8 else workloads.make_weight)(M, K, 0.5, seed=1)
+    dev = b.us_encode(W, fmt=fmt, max_N=64, flags=flags)
+    host = b.us_encode(W, fmt=fmt, max_N=64, flags=flags | b.US_ENCODE_HOST_ONLY)
+    try:
+        for N in (1, 8, 9, 16, 17, 32, 33, 64):
+            assert b.us_launch_info(dev, N) == b.us_launch_info(host, N), N
+    finally:
+        b.us_destroy(dev)
+        b.us_destroy(host)
