@@ -101,7 +101,7 @@ constexpr int kCoresidentTiles = 16;         // most tiles per CTA for the half-
 constexpr int kCoresidentK = 5120;           // ... and widest K: its few threads stage all of X (N = 8, half SM / whole: 2304 x 8192 6.8 / 5.9 us,
                                              // 2304 x 6144 6.4 / 5.6, 4096 x 4096 4.6 / 5.6)
 // The same where K is not a multiple of 32 and staging takes a thread one unit at a time (half SM / whole: N = 8
-// 1500 x 4500 6.7 / 5.8 (N = 1, which shares the plan, 5.3 / 5.6), 2304 x 4500 7.3 / 6.5, 2304 x 3000 5.5 / 5.4; N = 1 there 4.4 / 5.2; N = 16 5003 x 3001 9.0 / 8.0).
+// 1500 x 4500 6.7 / 5.8 (N = 1, which shares the plan, loses by it, 5.3 / 5.6), 2304 x 4500 7.3 / 6.5, 2304 x 3000 5.5 / 5.4; N = 1 there 4.4 / 5.2; N = 16 5003 x 3001 9.0 / 8.0).
 int64_t coresident_K(int64_t K, int nt) { return K % 32 == 0 ? kCoresidentK : nt == 1 ? 3072 : 2048; }
 constexpr int kHalfSmBytes = 228 * 1024 / 2 - 1024 - 512;   // shared memory of a half-SM CTA: 228 KB per SM, 1 KB reserved per CTA
 
@@ -443,9 +443,10 @@ void build_tc_plan(us_handle* h, int ng)
     //   N <= 16: that plan 4.5 + 1.08 share, this kernel 7.5 + 0.9 mean (20480 x 8192 26.2 / 23.3, 28672 x 8192 32.4 / 28.0,
     //            27648 x 5120 21.0 / 20.9, 13824 x 5120 13.0 / 14.2). Half a us of margin, and from 10 stages on: among other
     //            launches its code comes from L2 each time, and 5120 x 13824, 7 stages, alone 15.1 / 13.8, gained nothing in
-    //            a layer of seven projections.
+    //            a layer of seven projections (called by itself again and again it would).
     //   N <= 32: 5.5 + 1.76 share, 9.7 + 0.97 mean (13824 x 5120 18.8 / 17.2, 28672 x 8192 51 / 33, 5120 x 5120 12.3 / 12.7);
-    //            2 us of margin, since matrices of uneven density cost this kernel more (4096 x 11008 sorted 15.5 / 16.1)
+    //            2 us of margin, since matrices of uneven density cost this kernel more (4096 x 11008 sorted 15.5 / 16.1).
+    //            Even ones pay for that: 13824 x 5120 falls inside the margin and keeps the slower plan.
     //   N <= 64: from 4 stages on (4096 x 4096, 1.7 stages, 14.4 / 17.3; 11008 x 4096, 4.6 stages, 35 / 20.6).
     // Against the direct mode it wins nearly always (N = 32 on 2 x 2 tiles 5120 x 5120 14.9 / 12.9; N = 64 4096 x 4096 with
     // INT2 weights 21.8 / 16.5, 28672 x 8192 92 / 41).
@@ -465,10 +466,10 @@ void build_tc_plan(us_handle* h, int ng)
         return std::min(us::kTcMaxSlots, (limit - fixed_for(x_stages, lut_rep)) / (int)p.slot_bytes);
     };
     p.x_stages = 4;
-    // Three octets for N <= 16 and long shares (N = 16, two octets / three: 28672 x 8192 29.3 / 28.0, with INT2 weights
-    // 25.7 / 24.7; 13824 x 5120, 7 stages, INT2 12.75 / 12.86; N = 32 on 28672 x 8192 33.1 / 33.4).
+    // Three octets (a kernel for N <= 16) where shares are long: two / three on 28672 x 8192, N = 16 29.3 / 28.0, with INT2
+    // weights 25.7 / 24.7; 13824 x 5120, 7 stages, INT2 12.75 / 12.86.
     const int64_t stages3 = (hm.n_strips + 23) / 24 * block_stages;
-    pl.octets = slots_for(3, 8) >= 24 && ng <= 4 && (tc_oct_knob() ? tc_oct_knob() == 3 : ng <= 2 && stages3 >= 8 * n_cta) ? 3 : 2;
+    pl.octets = slots_for(3, 8) >= 24 && ng <= 2 && (tc_oct_knob() ? tc_oct_knob() == 3 : stages3 >= 8 * n_cta) ? 3 : 2;
     if (pl.octets == 3) { stages = stages3; p.x_stages = slots_for(4, 8) >= 24 ? 4 : 3; }
     const int warps = 8 * pl.octets;
     pl.threads = pl.octets == 3 ? us::TcShape<3>::kThreads : us::TcShape<2>::kThreads;

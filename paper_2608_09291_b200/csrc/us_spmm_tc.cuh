@@ -25,7 +25,7 @@
 
 namespace us {
 
-// The CTA by number of octets: two, or three for N <= 32 (see the kernel).
+// The CTA by number of octets: two, or three for N <= 16 (see the kernel).
 template <int OCT>
 struct TcShape {
     static constexpr int kDecode = 8 * OCT;              // decode warps
@@ -33,7 +33,7 @@ struct TcShape {
     static constexpr int kPair = OCT == 2 ? 2 : 1;       // X warps that share a stage
     static constexpr int kThreads = 32 * (kDecode + 1 + kX);
     static constexpr int kA = OCT == 2 ? 3 : 2;          // A stages per octet, 64 tensor-memory columns (256 of K) each
-    static constexpr int kD = OCT == 2 ? 64 : 32;        // tensor-memory columns of an octet's sums: the most tokens
+    static constexpr int kD = OCT == 2 ? 64 : 32;        // tensor-memory columns of an octet's sums, one a token
     static_assert(OCT * (kA * 64 + kD) <= 512, "tensor memory");
 };
 constexpr int kTcMaxOct = 3, kTcMaxA = 3;
@@ -270,10 +270,9 @@ __device__ __noinline__ void store_block_tc(const StoreCtx& p, int v0, int v1, i
 }
 
 // ANY: K is not a multiple of 32 (load_x32).
-// OCT = 3: 24 decode warps, 384 rows to a stage, for N <= 32 (the sums of three octets of 64 tokens and two A stages each do
-// not fit tensor memory, nor 24 tile slots beside wide X stages shared memory). With 16 decode warps 0.59
-// instructions issue per cycle and scheduler; eight more warps hide more of the decode's latency (28672 x 8192, N = 16:
-// 29.3 -> 28.0 us, with INT2 weights 25.7 -> 24.7).
+// OCT = 3: 24 decode warps, 384 rows to a stage, for N <= 16. With 16 decode warps 0.59 instructions issue per cycle and
+// scheduler; eight more warps hide more of the decode's latency (28672 x 8192, N = 16: 29.3 -> 28.0 us, with INT2 weights
+// 25.7 -> 24.7). Their A operands leave an octet two stages and the CTA three X warps: at N = 32 33.4 us against 33.1.
 template <int OCT, int CA, bool W2, bool AM, bool ANY>
 __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(const __grid_constant__ TcParams p)
 {
