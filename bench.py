@@ -1,16 +1,16 @@
 #!/usr/bin/env python
-"""Benchmark of the W4A4 bitmap-sparse SpMM (one JSON line on stdout).
+"""Benchmark of the W4A4 bitmap-sparse SpMM (one JSON line on stdout, the other configurations on stderr).
 
 Workload of the headline line: LLaMA-2-7B-shaped attention projections, W 4096x4096 INT4 at 50 %
 uniform sparsity, X 4096xN INT4 with N = 8, fused fp16 dequant output. One pass = one SpMM on each
 of R distinct encoded weight buffers (R * bytes > 3x the L2 size, so every launch streams its
 weights from HBM); one step = as many passes as make the timed region at least half a second. The
 other configurations (1024x1024; sparsity {30, 50, 70 %} x N {1, 8, 16, 32}; the 7B-shaped FFN with
-row-varying density; the 13B-shaped decoder layer; the 70B-shaped FFN N sweep) are reported in the
-same line under "sweep".
+row-varying density; the 13B-shaped decoder layer; the 70B-shaped FFN N sweep) are one JSON line each on
+stderr: with them the stdout line was 50 KB, too long for a reader that takes the end of it.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--no-sweep]
-  python bench.py --only M,K,s,N[,int32|fp16[,K_L[,N_max[,q4]]]]     one case with the kernel's stage
+  python bench.py --only M,K,s,N[,int32|fp16[,K_L[,N_max[,q4|w2]]]]  one case with the kernel's stage
                                                                timers (the command of the ncu captures)
 
 With --gpus N > 1 and no torchrun environment the script starts itself N times under
@@ -455,9 +455,10 @@ def run_ours(args, rank: int, local_rank: int, world: int):
     }
     head.close()
 
+    rows = []
     if rank == 0 and not args.no_sweep:
-        out["sweep"] = sweep(binding, torch, workloads, l2, peak_gbs)
-        big = [r for r in out["sweep"] if r["case"] == "ffn70b_up" and r["N"] == 8]
+        rows = sweep(binding, torch, workloads, l2, peak_gbs)
+        big = [r for r in rows if r["case"] == "ffn70b_up" and r["N"] == 8]
         if big:   # the shape on which a bandwidth roofline is physically reachable
             r = big[0]
             out["roofline_large"] = {"bound": "hbm", "achieved": r["gbs"], "peak": peak_gbs, "unit": "GB/s",
@@ -469,7 +470,7 @@ def run_ours(args, rank: int, local_rank: int, world: int):
         # fewer decode instructions per weight; its own byte count, time and fractions
         for key, case_name, shape in (("roofline_q4", "attn7b_q4", "4096x4096 s=0.5 N=8 fp16"),
                                       ("roofline_large_q4", "ffn70b_up_q4", "28672x8192 s=0.6 N=8 int32")):
-            hit = [r for r in out["sweep"] if r["case"] == case_name and r["N"] == 8 and r["sparsity"] in (0.5, 0.6)]
+            hit = [r for r in rows if r["case"] == case_name and r["N"] == 8 and r["sparsity"] in (0.5, 0.6)]
             if hit:
                 r = hit[0]
                 out[key] = {"bound": "hbm", "achieved": r["gbs"], "peak": peak_gbs, "unit": "GB/s",
@@ -478,16 +479,25 @@ def run_ours(args, rank: int, local_rank: int, world: int):
                             "kernel": r["kernel"] + " on " + shape}
     if rank == 0:
         out["cpu_baseline"] = cpu_baseline(W, Xall[:N], s_w, s_x[:N], pstats)
-        print(json.dumps(out))
+        report(out, rows)
     if dist is not None:
         dist.barrier()
         dist.destroy_process_group()
 
 
+def report(out, rows):
+    """The result line on stdout, the sweep's rows on stderr before it."""
+    for r in rows:
+        print(json.dumps(r), file=sys.stderr)
+    sys.stderr.flush()
+    print(json.dumps(out), flush=True)
+
+
 def kernel_label(binding, handle, N):
     """The dominant (only) kernel of a call and its launch geometry."""
     g = binding.us_launch_info(handle, N)
-    return (f"us_spmm_kernel (n-tiles {max(1, 1 << (max(N, 1) - 1).bit_length()) // 8 or 1}, {g['grid']} CTAs x "
+    name = "us_spmm_tc_kernel" if g["block"] in (800, 896) else "us_spmm_kernel"   # (two or three octets; no other block is as wide)
+    return (f"{name} (n-tiles {max(1, 1 << (max(N, 1) - 1).bit_length()) // 8 or 1}, {g['grid']} CTAs x "
             f"{g['block'] // 32} warps, {g['smem_bytes']} B shared memory)")
 
 
@@ -732,18 +742,20 @@ def run_only(args):
     f = args.only.split(",")
     M, K, s, N = int(f[0]), int(f[1]), float(f[2]), int(f[3])
     fp16 = len(f) > 4 and f[4] == "fp16"
-    # K_L > 0 picks the tile width; a seventh field "q4" the folded format (16, K_L, 2, 2)
-    fmt = (16, int(f[5]), 2, 2 if (len(f) > 7 and f[7] == "q4") else 1) if len(f) > 5 and int(f[5]) > 0 else None
+    # K_L > 0 picks the tile width; an eighth field "q4" the folded format (16, K_L, 2, 2), "w2" INT2 weights in it
+    kind = f[7] if len(f) > 7 else ""
+    fmt = (16, int(f[5]), 2, 2 if kind in ("q4", "w2") else 1) if len(f) > 5 and int(f[5]) > 0 else None
+    flags = binding.US_ENCODE_W2 if kind == "w2" else 0
     n_max = int(f[6]) if len(f) > 6 else N   # largest N the handles are encoded for
     torch.cuda.set_device(0)
     l2 = torch.cuda.get_device_properties(0).L2_cache_size or L2_BYTES_FALLBACK
-    W = workloads.make_weight(M, K, s, seed=1)
+    W = (workloads.make_weight_w2 if kind == "w2" else workloads.make_weight)(M, K, s, seed=1)
     X = workloads.make_x(K, n_max, seed=1)
     s_w, s_x = workloads.make_scales(M, n_max, seed=1)
-    probe = binding.us_encode(W, None, fmt, n_max, binding.US_ENCODE_HOST_ONLY)
+    probe = binding.us_encode(W, None, fmt, n_max, binding.US_ENCODE_HOST_ONLY | flags)
     st = binding.us_get_stats(probe)
     binding.us_destroy(probe)
-    case = Case(binding, torch, W, s_w, X, s_x, n_max, replicas_for(st, l2), fmt=fmt)
+    case = Case(binding, torch, W, s_w, X, s_x, n_max, replicas_for(st, l2), fmt=fmt, flags=flags)
     for _ in range(max(1, args.warmup)):
         case.enqueue_pass(N, fp16)
     torch.cuda.synchronize()
@@ -812,7 +824,7 @@ def main(argv=None):
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--no-sweep", action="store_true")
-    ap.add_argument("--only", default=None, metavar="M,K,s,N[,int32|fp16[,K_L[,N_max[,q4]]]]",
+    ap.add_argument("--only", default=None, metavar="M,K,s,N[,int32|fp16[,K_L[,N_max[,q4|w2]]]]",
                     help="time one case only, with the kernel's stage timers: the small run of the ncu captures")
     ap.add_argument("--chain", action="store_true",
                     help="time only the 13B-shaped layer, as seven plain calls and as a chain of four chained calls")

@@ -88,3 +88,12 @@ def test_gpus_flag_starts_replicas_or_refuses(monkeypatch):
         raise AssertionError("a contradicting world size must be refused")
     except SystemExit as e:
         assert "WORLD_SIZE=2" in str(e)
+
+
+def test_result_line_is_short_and_alone_on_stdout(capsys):
+    """The sweep's rows go to stderr: the stdout line has to be parsed by readers that keep its end only."""
+    row = {"case": "attn7b", "M": 4096, "K": 4096, "us": 4.6, "kernel": "k" * 120}
+    bench.report({"metric": bench.METRIC, "value": 1.0, "roofline": {"kernel": "k" * 120}}, [row] * 60)
+    got = capsys.readouterr()
+    assert got.out.count("\n") == 1 and json.loads(got.out)["value"] == 1.0
+    assert [json.loads(line) for line in got.err.splitlines()] == [row] * 60
