@@ -173,7 +173,7 @@ KernelForms kernel_forms(const us_handle* h, int cls, int stages, bool local, bo
 // at a time. (The stage-timer builds need more and do not share one.)
 int half_sm_warps(const us_handle* h, int cls, bool local, bool xp)
 {
-    if (h->device < 0) return cls == 0 && h->host.fmt.C_A == 1 ? 12 : 10;   // host-only handle
+    if (h->device < 0) return (cls == 0 ? 12 : 10) - (h->host.fmt.C_A == 2 ? 2 : 0);   // host-only handle: what it comes to today
     const KernelForms f = kernel_forms(h, cls, 1, local, xp);
     int regs = 0;
     for (const void* fn : {f.plain, f.chained, f.single}) {
@@ -923,7 +923,7 @@ us_status us_debug_withhold_copy(us_handle* h, int64_t position, int64_t wait_us
 }
 
 us_status us_stage_timers(us_handle* h, int32_t enable, uint64_t* out, int32_t n_out)
-{
+try {
     if (!h || (out && n_out < 8)) return US_ERR_INVALID_ARG;
     if (!h->on_device) return US_ERR_UNSUPPORTED;
     const size_t bytes = us::kTimerWords * sizeof(unsigned long long);
@@ -973,6 +973,8 @@ us_status us_stage_timers(us_handle* h, int32_t enable, uint64_t* out, int32_t n
     }
     if (enable >= 0) h->timers_on = enable != 0;
     return US_OK;
+} catch (const std::exception&) {   // no host memory
+    return US_ERR_ALLOC;
 }
 
 us_status us_destroy(us_handle* h)

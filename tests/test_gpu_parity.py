@@ -463,7 +463,8 @@ def test_stage_timers_on_every_plan_variant(b):
 
 
 @pytest.mark.parametrize("M,K,fmt,flags", [(1024, 1024, None, 0), (4096, 4096, None, 0), (512, 8192, None, 0), (24000, 1024, None, 0),
-                                           (5003, 3001, (16, 512, 2, 2), 0), (4001, 2500, (16, 512, 2, 2), 8), (8160, 9216, None, 0)])
+                                           (5003, 3001, (16, 512, 2, 2), 0), (4001, 2500, (16, 512, 2, 2), 8), (8160, 9216, None, 0),
+                                           (4500, 2048, (16, 512, 2, 2), 0), (4500, 2048, (16, 512, 2, 1), 0)])
 def test_launch_info_of_a_host_only_handle(b, M, K, fmt, flags):
     """One plan serves the launches and us_launch_info, and a host-only handle lays the same."""
     W = (workloads.make_weight_w2 if flags & 8 else workloads.make_weight)(M, K, 0.5, seed=1)
