@@ -928,10 +928,19 @@ try {
     if (!h->on_device) return US_ERR_UNSUPPORTED;
     const size_t bytes = us::kTimerWords * sizeof(unsigned long long);
     if (!h->d_timers) {
+        int dev = -1;
+        cudaGetDevice(&dev);
+        if (dev != h->device) cudaSetDevice(h->device);
+        cudaError_t e = cudaSuccess;
         for (const ClassPlan& pl : h->plan)
-            if (enable_large_smem(h->device, h->max_smem, pl.fn.timed) != cudaSuccess) return US_ERR_CUDA;
-        if (cudaMalloc((void**)&h->d_timers, bytes) != cudaSuccess) return US_ERR_ALLOC;
-        cudaMemset(h->d_timers, 0, bytes);
+            if (e == cudaSuccess) e = enable_large_smem(h->device, h->max_smem, pl.fn.timed);
+        if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_timers, bytes);
+        if (e == cudaSuccess) e = cudaMemset(h->d_timers, 0, bytes);
+        if (dev != h->device && dev >= 0) cudaSetDevice(dev);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return e == cudaErrorMemoryAllocation ? US_ERR_ALLOC : US_ERR_CUDA;
+        }
     }
     if (out) {
         if (cudaDeviceSynchronize() != cudaSuccess) return US_ERR_CUDA;
