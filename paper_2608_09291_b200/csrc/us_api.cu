@@ -5,12 +5,14 @@
 #include <cstdlib>
 #include <cstring>
 #include <exception>
+#include <map>
 #include <memory>
 #include <mutex>
 #include <new>
-#include <set>
 #include <utility>
 #include <vector>
+
+#include <cuda.h>
 
 #include "us_host.h"
 #include "us_launch.h"
@@ -26,8 +28,12 @@ struct LaunchGeom {
     uint32_t slot_bytes;
     bool xp;
 };
-struct KernelForms {      // nullptr where no such kernel is built
-    const void *plain = nullptr, *chained = nullptr, *single = nullptr, *timed = nullptr;
+struct Kernel {
+    const void* symbol = nullptr;      // nullptr where no such kernel is built
+    cudaFunction_t fn = nullptr;       // on the handle's device, once it is loaded (load_kernel)
+};
+struct KernelForms {
+    Kernel plain, chained, single, timed;
 };
 struct ClassPlan {
     bool ok = false;
@@ -40,7 +46,7 @@ struct ClassPlan {
 struct TcPlan {
     bool ok = false;
     int octets = 2, threads = 0, smem = 0;
-    const void *plain = nullptr, *chained = nullptr;
+    Kernel plain, chained;
     us::TcParams p{};
 };
 
@@ -159,13 +165,13 @@ KernelForms kernel_forms(const us_handle* h, int cls, int stages, bool local, bo
     us::KernelKey k{stages, local, false, xp, false, h->host.fmt.C_A == 2, h->host.w2, false};
     const bool any_k = h->host.K % 32 != 0;
     KernelForms f;
-    f.plain = kernel_for(cls, any_k, k);
+    f.plain.symbol = kernel_for(cls, any_k, k);
     k.am = true;
-    f.chained = kernel_for(cls, any_k, k);
+    f.chained.symbol = kernel_for(cls, any_k, k);
     k.am = false; k.dp = true;   // a single token: dp4a beats the MMA (measured 2-3 %)
-    f.single = kernel_for(cls, any_k, k);
+    f.single.symbol = kernel_for(cls, any_k, k);
     k.dp = false; k.timed = true;
-    f.timed = kernel_for(cls, any_k, k);
+    f.timed.symbol = kernel_for(cls, any_k, k);
     return f;
 }
 
@@ -176,7 +182,7 @@ int half_sm_warps(const us_handle* h, int cls, bool local, bool xp)
     if (h->device < 0) return (cls == 0 ? 12 : 10) - (h->host.fmt.C_A == 2 ? 2 : 0);   // host-only handle: what it comes to today
     const KernelForms f = kernel_forms(h, cls, 1, local, xp);
     int regs = 0;
-    for (const void* fn : {f.plain, f.chained, f.single}) {
+    for (const void* fn : {f.plain.symbol, f.chained.symbol, f.single.symbol}) {
         if (!fn) continue;
         cudaFuncAttributes fa;
         if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) { cudaGetLastError(); return 0; }
@@ -492,23 +498,28 @@ void build_tc_plan(us_handle* h, int ng)
     p.mg_segs = ((1ull << 40) / (uint64_t)hm.n_segs) + 1ull;
     p.mask_rows = hm.mask_rows; p.K_L = hm.fmt.K_L;
     p.acc_nt = nt_for(8 * ng);
-    pl.plain = us::kernel_tc(pl.octets, hm.K % 32 != 0, hm.fmt.C_A == 2, hm.w2, false);
-    pl.chained = us::kernel_tc(pl.octets, hm.K % 32 != 0, hm.fmt.C_A == 2, hm.w2, true);
+    pl.plain.symbol = us::kernel_tc(pl.octets, hm.K % 32 != 0, hm.fmt.C_A == 2, hm.w2, false);
+    pl.chained.symbol = us::kernel_tc(pl.octets, hm.K % 32 != 0, hm.fmt.C_A == 2, hm.w2, true);
     pl.ok = true;
 }
 
-// Opt a kernel in to the device's full dynamic shared memory, once per device. This also loads it, so that us_spmm itself
-// is nothing but a launch. Only what a handle's plans launch is loaded: a program's first handle takes 37 ms, 62 when it
-// loaded every kernel of the aligned K.
-cudaError_t enable_large_smem(int device, int bytes, const void* fn)
+// Loads a kernel, opted in to the device's full dynamic shared memory (once per device, with that device current), so that
+// us_spmm itself is nothing but a launch. Only what a handle's plans launch is loaded: a program's first handle takes 37 ms,
+// 62 when it loaded every kernel of the aligned K.
+cudaError_t load_kernel(int device, int smem_bytes, Kernel* k)
 {
     static std::mutex mu;
-    static std::set<std::pair<int, const void*>> done;
-    if (!fn) return cudaSuccess;
+    static std::map<std::pair<int, const void*>, cudaFunction_t> loaded;
+    if (!k->symbol) return cudaSuccess;
     std::lock_guard<std::mutex> lock(mu);
-    if (done.count({device, fn})) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) done.insert({device, fn});
+    const auto it = loaded.find({device, k->symbol});
+    if (it != loaded.end()) {
+        k->fn = it->second;
+        return cudaSuccess;
+    }
+    cudaError_t e = cudaFuncSetAttribute(k->symbol, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    if (e == cudaSuccess) e = cudaGetFuncBySymbol(&k->fn, k->symbol);
+    if (e == cudaSuccess) loaded[{device, k->symbol}] = k->fn;
     return e;
 }
 
@@ -519,11 +530,46 @@ struct ChainArgs {
     int64_t m0 = 0, m1 = 0;
 };
 
-us_status launch(us_handle* h, const void* fn, void* params, int threads, int smem, cudaStream_t st)
+// The driver's launch call, or nullptr. The runtime's looks the kernel up by its symbol on every call, among all that the
+// library holds. 1024 x 1024, N = 8 into a new output, us of host time on two machines: 3.5 and 3.35 with the 128 kernels
+// that there were before ragged K had its own, 3.9 with 240, 3.65 and 3.2 with the function in hand.
+using DriverLaunch = CUresult (*)(const CUlaunchConfig*, CUfunction, void**, void**);
+DriverLaunch driver_launch()
+{
+    static const DriverLaunch f = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPointByVersion("cuLaunchKernelEx", &p, 12000, cudaEnableDefault, &r) != cudaSuccess) cudaGetLastError();
+        return reinterpret_cast<DriverLaunch>(p);
+    }();
+    return f;
+}
+
+us_status launch(us_handle* h, const Kernel& kernel, void* params, int threads, int smem, cudaStream_t st)
 {
     // Launched with programmatic stream serialization: the kernel may start while its predecessor
     // in the stream is still running; it waits (griddepcontrol.wait) before it touches anything
     // an earlier kernel could produce or still use.
+    void* args[1] = {params};
+    if (const DriverLaunch f = driver_launch()) {
+        CUlaunchAttribute attr[1];
+        attr[0].id = CU_LAUNCH_ATTRIBUTE_PROGRAMMATIC_STREAM_SERIALIZATION;
+        attr[0].value.programmaticStreamSerializationAllowed = pdl_knob() ? 1 : 0;
+        CUlaunchConfig cfg = {};
+        cfg.gridDimX = (unsigned)h->sm_count;
+        cfg.blockDimX = (unsigned)threads;
+        cfg.gridDimY = cfg.gridDimZ = cfg.blockDimY = cfg.blockDimZ = 1;
+        cfg.sharedMemBytes = (unsigned)smem;
+        cfg.hStream = st;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        const CUresult r = f(&cfg, kernel.fn, args, nullptr);
+        if (r == CUDA_SUCCESS) return US_OK;
+        if (r != CUDA_ERROR_INVALID_CONTEXT) {   // (a thread that has made no runtime call yet has none: the runtime makes it current)
+            h->sticky = (cudaError_t)r;          // (the codes are the runtime's)
+            return US_ERR_CUDA;
+        }
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)h->sm_count);
     cfg.blockDim = dim3((unsigned)threads);
@@ -534,8 +580,7 @@ us_status launch(us_handle* h, const void* fn, void* params, int threads, int sm
     attr[0].val.programmaticStreamSerializationAllowed = pdl_knob() ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    void* args[1] = {params};
-    const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, kernel.symbol, args);
     if (e != cudaSuccess) { h->sticky = e; return US_ERR_CUDA; }
     return US_OK;
 }
@@ -559,9 +604,9 @@ us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_sca
         }
         p.wait_ns_hi = h->wait_ns_hi;
         p.withhold = h->withhold;
-        const void* fn = p.y_amax ? tc.chained : tc.plain;
-        if (!fn) return US_ERR_UNSUPPORTED;
-        return launch(h, fn, &p, tc.threads, tc.smem, st);
+        const Kernel& k = p.y_amax ? tc.chained : tc.plain;
+        if (!k.fn) return US_ERR_UNSUPPORTED;
+        return launch(h, k, &p, tc.threads, tc.smem, st);
     }
     const int cls = class_of(nt_for(N));
     const ClassPlan& pl = h->plan[cls];
@@ -581,12 +626,12 @@ us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_sca
     p.withhold = h->withhold;
 
     // (a variant without a timer build runs untimed)
-    const bool timed = timers && !p.y_amax && pl.fn.timed;
-    const void* fn = p.y_amax ? pl.fn.chained : timed ? pl.fn.timed : N == 1 && !timers && pl.fn.single ? pl.fn.single : pl.fn.plain;
-    if (!fn) return US_ERR_UNSUPPORTED;
+    const bool timed = timers && !p.y_amax && pl.fn.timed.fn;
+    const Kernel& k = p.y_amax ? pl.fn.chained : timed ? pl.fn.timed : N == 1 && !timers && pl.fn.single.fn ? pl.fn.single : pl.fn.plain;
+    if (!k.fn) return US_ERR_UNSUPPORTED;
     p.timers = timed ? h->d_timers : nullptr;
 
-    return launch(h, fn, &p, g.warps * 32, g.smem, st);
+    return launch(h, k, &p, g.warps * 32, g.smem, st);
 }
 
 // A 256-thread kernel, launched with programmatic stream serialization like the SpMM.
@@ -691,12 +736,12 @@ us_status encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_scale,
     h->on_device = true;
     lay_plans();
     if (!h->plan[class_of(nt_max)].ok) return US_ERR_UNSUPPORTED;   // a tile does not fit the shared-memory ring
-    for (const ClassPlan& pl : h->plan)
-        for (const void* fn : {pl.fn.plain, pl.fn.chained, pl.fn.single})
-            if (e == cudaSuccess) e = enable_large_smem(h->device, h->max_smem, fn);
-    for (const TcPlan& pl : h->tc)
-        for (const void* fn : {pl.plain, pl.chained})
-            if (e == cudaSuccess) e = enable_large_smem(h->device, h->max_smem, fn);
+    for (ClassPlan& pl : h->plan)
+        for (Kernel* k : {&pl.fn.plain, &pl.fn.chained, &pl.fn.single})
+            if (e == cudaSuccess) e = load_kernel(h->device, h->max_smem, k);
+    for (TcPlan& pl : h->tc)
+        for (Kernel* k : {&pl.plain, &pl.chained})
+            if (e == cudaSuccess) e = load_kernel(h->device, h->max_smem, k);
     if (e != cudaSuccess) return US_ERR_CUDA;
     *out = std::move(owner);
     return US_OK;
@@ -932,8 +977,8 @@ try {
         cudaGetDevice(&dev);
         if (dev != h->device) cudaSetDevice(h->device);
         cudaError_t e = cudaSuccess;
-        for (const ClassPlan& pl : h->plan)
-            if (e == cudaSuccess) e = enable_large_smem(h->device, h->max_smem, pl.fn.timed);
+        for (ClassPlan& pl : h->plan)
+            if (e == cudaSuccess) e = load_kernel(h->device, h->max_smem, &pl.fn.timed);
         if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_timers, bytes);
         if (e == cudaSuccess) e = cudaMemset(h->d_timers, 0, bytes);
         if (dev != h->device && dev >= 0) cudaSetDevice(dev);

@@ -97,3 +97,30 @@ def test_concurrent_decodes_of_one_handle(b):
         assert not wrong
     finally:
         b.us_destroy(h)
+
+
+def test_first_call_of_a_thread(b):
+    """A thread whose first use of CUDA is a launch: it has no context yet."""
+    W = workloads.make_weight(512, 1024, 0.5, seed=4)
+    X = workloads.make_x(1024, 24, seed=4)
+    h = b.us_encode(W, max_N=24)
+    try:
+        Xd = torch.from_numpy(b.pack_int4(X)).cuda()
+        Y = torch.zeros((24, 512), dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        failed = []
+
+        def work():
+            try:
+                b.us_spmm(h, Xd.data_ptr(), 24, None, Y.data_ptr(), None)
+            except Exception as e:
+                failed.append(e)
+
+        t = threading.Thread(target=work)
+        t.start()
+        t.join()
+        assert not failed, failed
+        assert b.us_last_error(h) == 0
+        assert (Y.cpu().numpy() == oracle.spmm_dense(W, X)).all()
+    finally:
+        b.us_destroy(h)
