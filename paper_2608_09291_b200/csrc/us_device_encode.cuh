@@ -22,14 +22,14 @@ struct EncodeParams {
     uint8_t* blob;
 };
 
-// nibbles of v that are not zero -> one bit each, in order
+// nibbles of v that are not zero -> one bit each, in slot order: nibbles 0, 2, 4, 6, then 1, 3, 5, 7
 __device__ __forceinline__ uint32_t nonzero_nibbles(uint32_t v)
 {
     uint32_t n = v | (v >> 1);
-    n = (n | (n >> 2)) & 0x11111111u;
-    n = (n | (n >> 3)) & 0x03030303u;
-    n = (n | (n >> 6)) & 0x000F000Fu;
-    return (n | (n >> 12)) & 0xFFu;
+    n |= n >> 2;                 // bits 4 i
+    // four bits 8 apart to bits 24 .. 27 by one multiplication (no two of its terms share a bit)
+    const uint32_t even = ((n & 0x01010101u) * 0x01020408u) >> 24, odd = (((n >> 4) & 0x01010101u) * 0x01020408u) >> 24;
+    return (even & 15u) | ((odd & 15u) << 4);
 }
 
 // The lane's words of mask byte kb: v[area][row half].
@@ -142,8 +142,9 @@ __global__ void __launch_bounds__(256) us_encode_write_kernel(const EncodeParams
             mw |= m << (8 * i);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const uint32_t a0 = (v[0][0] >> (4 * j)) & 15u, b0 = (v[0][1] >> (4 * j)) & 15u;
-                const uint32_t a1 = (v[1][0] >> (4 * j)) & 15u, b1 = (v[1][1] >> (4 * j)) & 15u;
+                const int c = 4 * (2 * (j & 3) + (j >> 2));   // (slot_column)
+                const uint32_t a0 = (v[0][0] >> c) & 15u, b0 = (v[0][1] >> c) & 15u;
+                const uint32_t a1 = (v[1][0] >> c) & 15u, b1 = (v[1][1] >> c) & 15u;
                 if ((m >> j) & 1u) {
                     if (p.w2) {
                         acc[0] |= (unsigned long long)(((a0 + 2u) & 3u) | (((b0 + 2u) & 3u) << 2) | (((a1 + 2u) & 3u) << 4) | (((b1 + 2u) & 3u) << 6)) << (8 * n);

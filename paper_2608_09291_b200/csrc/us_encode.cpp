@@ -408,14 +408,14 @@ us_status encode_host(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_s
             for (int g = 0; g < 8; ++g) {
                 const int8_t* pa = rows[g];
                 const int8_t* pb = rows[g + 8];
-                // kk = column within the column area; with C_A = 2 one mask bit covers columns kk and
-                // kk + K_B of the tile (rows g and g + 8 of each), and the two columns' bytes go to two
+                // kk = mask bit within the column area (a column of it, in slot order); with C_A = 2 one mask bit covers
+                // that column and the one K_B further on of the tile (rows g and g + 8 of each), and the two columns' bytes go to two
                 // streams of equal length
                 for (int kk = 0; kk < K_B; ++kk) {
                     int v[2][2];   // [column area][row half]
                     int any = 0;
                     for (int ca = 0; ca < CA; ++ca) {
-                        const int64_t k = k0 + kk + (int64_t)ca * K_B;
+                        const int64_t k = k0 + (kk & ~7) + slot_column(kk & 7) + (int64_t)ca * K_B;
                         v[ca][0] = (pa && k < K) ? pa[k] : 0;
                         v[ca][1] = (pb && k < K) ? pb[k] : 0;
                         any |= v[ca][0] | v[ca][1];
@@ -502,7 +502,7 @@ void decode_host(const HostMatrix& h, const uint8_t* blob, int8_t* W_out)
                 for (int j = 0; j < 8; ++j) {
                     if (!((m >> j) & 1)) continue;
                     for (int ca = 0; ca < CA; ++ca) {
-                        const int64_t k = sg * K_L + (int64_t)ca * K_B + 32 * kb + 8 * tt + j;
+                        const int64_t k = sg * K_L + (int64_t)ca * K_B + 32 * kb + 8 * tt + slot_column(j);
                         if (k >= h.K) continue;
                         int lo, hi;
                         if (h.w2) {

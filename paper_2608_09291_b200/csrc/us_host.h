@@ -7,9 +7,11 @@
 //   * a tile is decoded by one warp; lane l = 4*g + t owns, for every 32-column k-block kb of
 //     the tile, the 8 columns 32*kb + 8*t + j (j = 0..7) of strip rows g and g+8 -- exactly
 //     the A-fragment slots of that lane in an m16n8k32 integer MMA.
-//   * union mask: bit j of the lane's mask byte for k-block kb is set iff W[g][k] or W[g+8][k]
-//     is nonzero (one bit covers Q = 2 values, area 0 = strip rows 0..7, area 1 = rows 8..15).
-//   * payload: one byte per set bit, in (kb, j) order: high nibble = W[g+8][k] (two's
+//   * union mask: bit b of the lane's mask byte for k-block kb is set iff W[g][k] or W[g+8][k]
+//     is nonzero (one bit covers Q = 2 values, area 0 = strip rows 0..7, area 1 = rows 8..15), k = column j =
+//     slot_column(b) of the lane's eight: the even columns first, then the odd ones. A word of packed activations
+//     then is its two B-fragment words with no byte moved: (x << 4) & 0xF0F0F0F0 and x & 0xF0F0F0F0.
+//   * payload: one byte per set bit, in (kb, b) order: high nibble = W[g+8][k] (two's
 //     complement), low nibble = W[g][k] + 8 (excess-8). A cleared bit stands for the byte 0x08.
 //   * tile blob = mask matrix [K_L/128 rows][32 lanes] u32 (byte i of word w = k-block 4w+i)
 //                 followed by the payload matrix [J rows][32 lanes] u32, J = the longest lane
@@ -35,6 +37,9 @@
 #include "../../include/unionsparse.h"
 
 namespace us {
+
+// Column, of a lane's eight of a k-block, that mask bit b stands for.
+constexpr int slot_column(int b) { return 2 * (b & 3) + (b >> 2); }
 
 // The paper's three arrays for an arbitrary (H_L, K_L, R_A, C_A) (Sec. V-A "Storage Arrays"): what
 // a format without a kernel is encoded into, for us_get_stats / us_decode.

@@ -226,24 +226,24 @@ __device__ __forceinline__ uint2 lds64(uint32_t a)
 }
 
 // ---- X staging: INT4 -> int8 (x16) for one K range, plus 16 * sum_k x per (segment, token) -----
-// expands 8 packed activations (one 32-bit word) into two words of int8 (x16) and adds 16 * their sum
+// expands 8 packed activations (one 32-bit word) into two words of int8 (x16), the even columns and the odd ones as the
+// mask bits stand for them, and adds 16 * their sum
 __device__ __forceinline__ uint2 expand8(uint32_t v, int32_t& s)
 {
     const uint32_t te = (v << 4) & 0xF0F0F0F0u;  // 16*x for k even
     const uint32_t to = v & 0xF0F0F0F0u;         // 16*x for k odd
     s = __dp4a((int)te, 0x01010101, s);
     s = __dp4a((int)to, 0x01010101, s);
-    return make_uint2(prmt(te, to, 0x5140), prmt(te, to, 0x7362));
+    return make_uint2(te, to);
 }
 
-// Packed staging (XP): the same 8 activations as one word q whose even nibbles are k 0..3 and odd
-// nibbles k 4..7, so that the decode loop gets its two B-fragment words (x16, as int8) with
-// (q << 4) & 0xF0F0F0F0 and q & 0xF0F0F0F0. Half the shared memory of the int8 form for three more
+// Packed staging (XP): the word q of 8 activations stays as it is; the decode loop gets its two B-fragment words (x16, as
+// int8) with (q << 4) & 0xF0F0F0F0 and q & 0xF0F0F0F0. Half the shared memory of the int8 form for three more
 // integer instructions per n-tile and k-block.
 __device__ __forceinline__ uint32_t pack8(uint32_t v, int32_t& s)
 {
-    const uint2 t = expand8(v, s);
-    return (t.x >> 4) | t.y;
+    expand8(v, s);
+    return v;
 }
 
 // Staging of a K range for any K (stage_x takes K a multiple of 32): a unit of 32 columns comes from two aligned 16-byte
