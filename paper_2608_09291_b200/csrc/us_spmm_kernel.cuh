@@ -227,7 +227,8 @@ __device__ __forceinline__ uint2 lds64(uint32_t a)
 
 // ---- X staging: INT4 -> int8 (x16) for one K range, plus 16 * sum_k x per (segment, token) -----
 // expands 8 packed activations (one 32-bit word) into two words of int8 (x16), the even columns and the odd ones as the
-// mask bits stand for them, and adds 16 * their sum
+// mask bits stand for them, and adds 16 * their sum. (With the mask bits in column order two byte permutes a word had to
+// follow: 4096 x 4096, N = 32 9.06 us against 8.75, a 13B-shaped layer at N = 16 74.6 against 72.9.)
 __device__ __forceinline__ uint2 expand8(uint32_t v, int32_t& s)
 {
     const uint32_t te = (v << 4) & 0xF0F0F0F0u;  // 16*x for k even
