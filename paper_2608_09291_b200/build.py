@@ -20,7 +20,7 @@ UNITS = [(CSRC / "us_api.cu", [], "us_api.o"), (CSRC / "us_encode.cpp", [], "us_
          (CSRC / "us_load.cu", [], "us_load.o"), (CSRC / "us_spmm_tc.cu", [], "us_spmm_tc.o")] + [
     (CSRC / "us_kernels.cu", [f"-DUS_NT={nt}", f"-DUS_ANY={a}"], f"us_kernels_nt{nt}_{a}.o") for nt in (1, 2, 4, 8) for a in (0, 1)]
 HEADERS = [CSRC / "us_host.h", CSRC / "us_launch.h", CSRC / "us_load.h", CSRC / "us_device_encode.cuh",
-           CSRC / "us_spmm_kernel.cuh", CSRC / "us_spmm_tc.cuh", CSRC / "us_quant_kernels.cuh",
+           CSRC / "us_spmm_kernel.cuh", CSRC / "us_spmm_tc.cuh", CSRC / "us_spmm_ahead.cuh", CSRC / "us_quant_kernels.cuh",
            PKG.parent / "include" / "unionsparse.h"]
 EXT_SOURCE = CSRC / "us_torch.cpp"
 

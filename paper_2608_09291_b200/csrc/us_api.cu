@@ -19,6 +19,7 @@
 #include "us_load.h"
 #include "us_spmm_kernel.cuh"
 #include "us_spmm_tc.cuh"
+#include "us_spmm_ahead.cuh"
 #include "us_quant_kernels.cuh"
 
 // How one N class is launched: fixed when the handle is made, so that a call is left with filling in its
@@ -50,8 +51,17 @@ struct TcPlan {
     us::TcParams p{};
 };
 
+// The same for us_spmm_ahead_kernel, per N class.
+struct AheadPlan {
+    bool ok = false, chain_ok = false;   // chain_ok: chained calls, too
+    int threads = 0, smem = 0;
+    Kernel plain, chained;
+    us::AheadParams p{};
+};
+
 struct us_handle {
     us::HostMatrix host;
+    AheadPlan ahead[3];              // NT = 1, 2, 4
     TcPlan tc[9];                    // index: 8-token groups of the call
     ClassPlan plan[4];               // per N class (NT = 1, 2, 4, 8)
     bool on_device = false;
@@ -99,6 +109,7 @@ int stages_knob() { static int v = env_int("US_STAGES", 0); return v; }    // ri
 int max_warps() { static int v = std::min(20, std::max(2, env_int("US_MAX_WARPS", 16))); return v; }
 int tc_knob() { static int v = env_int("US_TC", 1); return v; }   // tensor-memory kernel: 0 never, 1 by rule, 2 wherever it can run
 int tc_oct_knob() { static int v = env_int("US_TC_OCT", 0); return v; }   // its octets: 0 by rule
+int ahead_knob() { static int v = env_int("US_AHEAD", 1); return v; }   // decode-ahead kernel: 0 never, 1 by rule, 2 wherever it can run
 int coresident_knob() { static int v = env_int("US_CORESIDENT", 1); return v; }  // small problems: half an SM per CTA
 constexpr int kLocalAccBudget = 32 * 1024;   // local strip sums a K-range width is chosen with
 constexpr int kLocalAccCap = 48 * 1024;      // ... and what is taken if nothing fits that
@@ -128,7 +139,7 @@ uint32_t slot_bytes_for(const us::HostMatrix& hm)
 
 int64_t x_bytes(int nt, int64_t G, int K_L, bool xp)
 {
-    return xp ? (int64_t)nt * 8 * (G * K_L / 2 + 16) : (int64_t)nt * 8 * (G * K_L + 32);
+    return (int64_t)nt * 8 * us::x_row_bytes((int)(G * K_L), xp);
 }
 
 int segs_per_range(const us::HostMatrix& hm, int nt, int limit, int64_t min_ranges, bool xp)
@@ -244,10 +255,8 @@ bool plan_launch(const us_handle* h, int N, LaunchGeom* g)
     for (size_t c = 0; c + 1 < h->cta_begin[g->cls].size(); ++c)
         most = std::max<int64_t>(most, (int64_t)h->cta_begin[g->cls][c + 1] - h->cta_begin[g->cls][c]);
     int fixed = fixed_base + 32 * stages * 8;
-    // (N = 9..16 too, where the plan stages X packed and in local mode: that kernel is as lean.)
-    // (Tried at N = 32 as well: 8 warps per CTA, slower.)
-    const bool co_class = g->nt == 1 || (g->nt == 2 && g->xp && s_local > 0);
-    if (coresident_knob() && co_class && most <= kCoresidentTiles && stages_knob() == 0 && h->host.Kp <= coresident_K(h->host.K, g->nt)) {
+    // (us_spmm_ahead_kernel takes nearly all of these calls; what is left for this plan is said at build_ahead_plan.)
+    if (coresident_knob() && g->nt == 1 && most <= kCoresidentTiles && stages_knob() == 0 && h->host.Kp <= coresident_K(h->host.K, g->nt)) {
         const int half = kHalfSmBytes;
         const int fixed8 = fixed_for(8) + 32 * 8;
         // (two column areas: 10 at most; 3001 x 2000, N = 8 4.10 us with 10, 4.18 with 12)
@@ -320,24 +329,7 @@ void plan_classes(us_handle* h)
             const int64_t n_segs = h->host.n_segs;
             const int64_t ranges = h->s_local[c] > 0 ? (n_segs + h->G[c] - 1) / h->G[c] : n_segs + 1;
             const bool small_share = nt >= 2 && (int64_t)h->host.blob_bytes / n_cta < 128 * 1024;
-            // N <= 8: packed X when that is what lets the half-SM plan of plan_launch hold its eight warps
-            // (4096 x 4096 at 30 % sparsity: tiles of 9.5 KB and 32 KB of int8 X do not fit half an SM, with
-            // 16 KB of packed X they do: 5.6 -> 4.6 us; the same for the folded format at 50 %: 5.3 -> 4.35)
-            bool for_half_sm = false;
-            if (nt == 1 && ranges == 1 && coresident_knob() && h->host.Kp <= coresident_K(h->host.K, nt)) {
-                const int64_t per_cta = (h->host.n_items + n_cta - 1) / n_cta;
-                const int64_t need = 8;
-                auto fits = [&](bool xp, int s_loc) {
-                    const int64_t fixed8 = 256 * 8 * 4 + (int64_t)us::kLutScratchBytes + x_bytes(nt, n_segs, h->host.fmt.K_L, xp) +
-                                           n_segs * nt * 8 * 4 + us::kClaimWords * 4 + (int64_t)s_loc * (nt * 128 + 1) * 4 +
-                                           2 * us::kOffTable * 4 + 128 + 32 * 8;
-                    return fixed8 + need * (int64_t)slot_bytes_for(h->host) <= kHalfSmBytes;
-                };
-                // (only where every tile then finds its own warp: 5120 x 5120 at 70 % sparsity, 11 tiles per CTA,
-                // runs 7.7 us in a 12-warp half-SM CTA against 6.3 us with 16 warps on the whole SM)
-                for_half_sm = per_cta <= 8 && !fits(false, h->s_local[c]) && fits(true, h->s_local[c]);
-            }
-            if (ranges > 1 || small_share || for_half_sm) {
+            if (ranges > 1 || small_share) {
                 std::vector<uint32_t> alt;
                 int sl2 = 0;
                 const int G2 = local_plan(true, &alt, &sl2);
@@ -503,6 +495,102 @@ void build_tc_plan(us_handle* h, int ng)
     pl.ok = true;
 }
 
+// Lays a launch of us_spmm_ahead_kernel down for the calls of an N class.
+//
+// Where it is chosen (us per call, us_spmm_kernel's plan / this, replayed graph; s = .5 unless it says; tiles: of 1024 columns,
+// the largest CTA's share):
+//   N <= 8: up to 64 tiles (1024 x 1024 3.1 / 2.2, 4096 x 4096 4.75 / 3.8, 11008 x 4096 8.8 / 6.6, 15360 x 5120, 33 tiles, 13.7 / 11.3,
+//     27648 x 5120, 60 tiles, 19.0 / 18.7; 28672 x 8192 at .6, 97 tiles, 26.4 / 31.2: the other kernel's 16 warps on one CTA count from
+//     there on), 46 with two column areas (20480 x 5120, 45 tiles, 14.6 / 14.6), 40 where K is cut in ranges (5120 x 13824, 31 tiles, 14.7 / 12.5).
+//   N <= 16: up to 42 tiles (5120 x 5120 7.9 / 6.6, 11008 x 4096 10.1 / 8.2, 13824 x 5120, 30 tiles, 13.0 / 12.9, 22016 x 4096, 40 tiles,
+//     16.7 / 15.9; 20480 x 5120, 45 tiles, 17.6 / 18.5). It is taken where alone it is no better, too: a CTA of the whole SM and one of
+//     half an SM cannot overlap, and a change between the two kinds costs 3 to 8 us (the seven projections of a 13B-shaped
+//     layer, four of 5120 x 5120, two of 13824 x 5120, one of 5120 x 13824: all whole 74, the first four half 73.5, all half 65).
+//     Cut in ranges where the other plan has one range: 24 (4096 x 11008 13.4 / 10.7; 8192 x 8192, 28 tiles, 13.0 / 14.4). Two column areas: 28
+//     and 24 (13824 x 5120 INT2 10.5 / 11.4, 5120 x 13824 16.2 / 17.7, 16384 x 4096, 28 tiles, INT2 12.7 / 11.2).
+//   N <= 32: where all tiles are parked (4096 x 4096 8.7 / 6.4, 5120 x 5120 11.6 / 9.3; 11008 x 4096, 20 tiles, 13.7 / 16.9).
+//   One segment to a strip and more than 8 tiles at N <= 8: not (24000 x 1024, 11 tiles, 4.9 / 5.6: the other half-SM plan has a warp
+//     for every tile).
+//   Chained calls: where all tiles are parked. The quantiser between two products takes the time in which later tiles would
+//     have been decoded (13B-shaped chain, all half 80, like this 72, all whole 74).
+void build_ahead_plan(us_handle* h, int cls)
+{
+    if (cls > 2 || ahead_knob() == 0) return;
+    AheadPlan& pl = h->ahead[cls];
+    const us::HostMatrix& hm = h->host;
+    const int nt = 1 << cls;
+    const bool plain = hm.fmt.C_A == 1;
+    us::AheadParams& p = pl.p;
+    std::memset(&p, 0, sizeof(p));
+    p.slot_bytes = slot_bytes_for(hm);
+    p.tile_cols = hm.mask_rows * hm.fmt.C_A * 8;
+    const int places = us::kAheadCols / p.tile_cols;   // of parked tiles in each quarter of the tensor memory
+    // The fewest K ranges whose X leaves room for six tile slots (5120 x 13824, N = 8: one range with five 16.3 us, two with
+    // eight 12.5; N = 16: two with four 16.2, three with six 15.1).
+    int64_t most = 0;
+    int warps = 8;
+    for (int64_t r = 1; r <= 8 && p.n_ranges == 0; ++r) {
+        const int64_t G = (hm.n_segs + r - 1) / r;
+        if ((hm.n_segs + G - 1) / G != r) continue;
+        const int64_t x = (int64_t)nt * 8 * us::ahead_x_row((int)std::min<int64_t>(G * hm.fmt.K_L, 1 << 20), hm.K % 32 != 0);
+        if (x > kHalfSmBytes) continue;
+        std::vector<uint32_t> begin;
+        int strips = 1;
+        us::make_schedule(hm, h->sm_count, (int)G, &begin, &strips);
+        most = 1;
+        bool one_range = true;   // to every CTA
+        for (int c = 0; c < h->sm_count; ++c) {
+            if (begin[c + 1] <= begin[c]) continue;
+            most = std::max<int64_t>(most, (int64_t)begin[c + 1] - begin[c]);
+            one_range = one_range && begin[c] / (hm.n_strips * G) == (begin[c + 1] - 1) / (hm.n_strips * G);
+        }
+        if (!one_range || most > us::kAheadMaxTiles) continue;
+        // Twelve decode warps and three that copy where 64 registers a thread do and there is work for them (with eight: 11008 x 4096,
+        // N = 8 7.05, with twelve 6.6; 13824 x 5120, N = 16 13.5 / 12.9; 2048 x 2048, N = 8 the other way, 2.5 / 2.6). One copying warp less
+        // is slower (20480 x 5120, N = 16 20.5 with one, 18.5 with three): each copy takes the issuing warp some 500 cycles.
+        const bool wide = plain && (nt == 1 ? hm.K > kCoresidentK || most > 16 : nt == 2);
+        warps = wide ? 12 : 8;
+        pl.threads = 32 * (wide ? 16 : nt == 1 && plain ? 12 : nt <= 2 && most > 16 ? 12 : 10);
+        if (4 * places < warps) continue;
+        const int64_t fixed = us::ahead_fixed_smem(nt, strips);
+        auto slots_in = [&](int64_t bytes) { return (int32_t)std::min<int64_t>(most, std::max<int64_t>(0, bytes) / (int64_t)p.slot_bytes); };
+        p.parked = (int32_t)std::min<int64_t>(most, 4 * places);
+        p.n_slots = slots_in(kHalfSmBytes - fixed - x);
+        p.x_over = p.parked == most && p.n_slots < std::min<int64_t>(most, warps) && fixed + x <= kHalfSmBytes ? 1 : 0;
+        if (p.x_over) p.n_slots = slots_in(kHalfSmBytes - fixed);
+        if (p.n_slots < std::min<int64_t>(most, 6)) continue;
+        pl.smem = (int)(fixed + (p.x_over ? std::max<int64_t>(x, (int64_t)p.n_slots * p.slot_bytes) : x + (int64_t)p.n_slots * p.slot_bytes));
+        std::copy(begin.begin(), begin.end(), p.cta_begin);
+        p.n_ranges = (int32_t)r; p.G = (int32_t)G; p.s_local = strips;
+    }
+    if (p.n_ranges == 0) return;
+    const int64_t share = most * hm.fmt.K_L / 1024;
+    const bool more_ranges = p.n_ranges > 1 && h->s_local[cls] > 0 && h->G[cls] == hm.n_segs;   // than the other plan's one
+    const bool better = cls == 0   ? share <= (p.n_ranges > 1 ? 40 : plain ? 64 : 46) && (hm.n_segs > 1 || most <= 8)
+                        : cls == 1 ? share <= (more_ranges || (!plain && p.n_ranges > 1) ? 24 : plain ? 42 : 28)
+                                   : p.parked == most;
+    if (ahead_knob() == 1 && !better) return;
+    p.tm_cols = 32;
+    while (p.tm_cols < (p.parked + 3) / 4 * p.tile_cols) p.tm_cols *= 2;
+    p.blob = h->d_blob; p.item_off = h->d_item_off; p.row_order = h->d_row_order; p.w_scale = h->d_w_scale;
+    p.err = h->d_err;
+    p.M = (int32_t)hm.M; p.K = (int32_t)hm.K;
+    p.n_strips = (int32_t)hm.n_strips; p.n_segs = (int32_t)hm.n_segs;
+    auto magic = [](int64_t d) { return ((1ull << 40) / (uint64_t)d) + 1ull; };
+    p.mg_g = magic(p.G); p.mg_last = magic(hm.n_segs - (int64_t)(p.n_ranges - 1) * p.G); p.mg_range = magic(hm.n_strips * p.G);
+    p.mask_rows = hm.mask_rows; p.K_L = hm.fmt.K_L;
+    auto symbol = [&](bool am) {
+        const bool any = hm.K % 32 != 0, fold = !plain;
+        if (cls == 0) return any ? us::kernel_ahead<1, true>(warps, pl.threads, fold, hm.w2, am) : us::kernel_ahead<1, false>(warps, pl.threads, fold, hm.w2, am);
+        if (cls == 1) return any ? us::kernel_ahead<2, true>(warps, pl.threads, fold, hm.w2, am) : us::kernel_ahead<2, false>(warps, pl.threads, fold, hm.w2, am);
+        return any ? us::kernel_ahead<4, true>(warps, pl.threads, fold, hm.w2, am) : us::kernel_ahead<4, false>(warps, pl.threads, fold, hm.w2, am);
+    };
+    pl.plain.symbol = symbol(false);
+    pl.chained.symbol = symbol(true);
+    pl.ok = true;
+    pl.chain_ok = p.parked == most;
+}
+
 // Loads a kernel, opted in to the device's full dynamic shared memory (once per device, with that device current), so that
 // us_spmm itself is nothing but a launch. Only what a handle's plans launch is loaded: a program's first handle takes 37 ms,
 // 62 when it loaded every kernel of the aligned K.
@@ -610,6 +698,24 @@ us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_sca
     }
     const int cls = class_of(nt_for(N));
     const ClassPlan& pl = h->plan[cls];
+    if (cls <= 2 && h->ahead[cls].ok && !(chain && !h->ahead[cls].chain_ok) && !(timers && !chain && pl.fn.timed.fn)) {   // (the stage timers are the other kernel's)
+        const AheadPlan& ah = h->ahead[cls];
+        us::AheadParams p = ah.p;
+        p.X = static_cast<const uint8_t*>(X);
+        p.x_scale = static_cast<const uint16_t*>(x_scale);
+        p.Y = Y; p.acc = acc; p.cnt = cnt;
+        p.N = N;
+        p.fp16_out = x_scale ? 1 : 0;
+        if (chain) {
+            p.y_amax = static_cast<uint32_t*>(chain->y_amax);
+            p.amax_m0 = (int32_t)chain->m0; p.amax_m1 = (int32_t)chain->m1;
+        }
+        p.wait_ns_hi = h->wait_ns_hi;
+        p.withhold = h->withhold;
+        const Kernel& k = p.y_amax ? ah.chained : ah.plain;
+        if (!k.fn) return US_ERR_UNSUPPORTED;
+        return launch(h, k, &p, ah.threads, ah.smem, st);
+    }
     if (!pl.ok) return US_ERR_UNSUPPORTED;
     const LaunchGeom& g = pl.g;
     us::SpmmParams p = pl.p;
@@ -699,7 +805,7 @@ us_status encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_scale,
     if (too_many()) return US_ERR_UNSUPPORTED;
     const int nt_max = nt_for(max_N);
     auto lay_plans = [&] {
-        for (int c = 0; c <= class_of(nt_max); ++c) build_plan(h, c);
+        for (int c = 0; c <= class_of(nt_max); ++c) { build_plan(h, c); build_ahead_plan(h, c); }
         for (int ng = 1; ng <= (max_N + 7) / 8; ++ng) build_tc_plan(h, ng);
     };
     plan_classes(h);
@@ -736,9 +842,17 @@ us_status encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_scale,
     h->on_device = true;
     lay_plans();
     if (!h->plan[class_of(nt_max)].ok) return US_ERR_UNSUPPORTED;   // a tile does not fit the shared-memory ring
-    for (ClassPlan& pl : h->plan)
-        for (Kernel* k : {&pl.fn.plain, &pl.fn.chained, &pl.fn.single})
-            if (e == cudaSuccess) e = load_kernel(h->device, h->max_smem, k);
+    for (int c = 0; c < 4; ++c)
+        if (c < 3 && h->ahead[c].ok) {
+            for (Kernel* k : {&h->ahead[c].plain, &h->ahead[c].chained})
+                if (e == cudaSuccess) e = load_kernel(h->device, h->max_smem, k);
+            if (!h->ahead[c].chain_ok)
+                for (Kernel* k : {&h->plan[c].fn.plain, &h->plan[c].fn.chained, &h->plan[c].fn.single})
+                    if (e == cudaSuccess) e = load_kernel(h->device, h->max_smem, k);
+        } else {
+            for (Kernel* k : {&h->plan[c].fn.plain, &h->plan[c].fn.chained, &h->plan[c].fn.single})
+                if (e == cudaSuccess) e = load_kernel(h->device, h->max_smem, k);
+        }
     for (TcPlan& pl : h->tc)
         for (Kernel* k : {&pl.plain, &pl.chained})
             if (e == cudaSuccess) e = load_kernel(h->device, h->max_smem, k);
@@ -809,11 +923,13 @@ us_status us_launch_info(const us_handle* h, int32_t N, int32_t* grid, int32_t* 
     if (!h || N < 1 || N > h->max_N) return US_ERR_INVALID_ARG;
     if (!h->host.kernel_layout) return US_ERR_UNSUPPORTED;
     const TcPlan& tc = h->tc[(N + 7) / 8];
-    const ClassPlan& pl = h->plan[class_of(nt_for(N))];
-    if (!tc.ok && !pl.ok) return US_ERR_UNSUPPORTED;
+    const int cls = class_of(nt_for(N));
+    const ClassPlan& pl = h->plan[cls];
+    const AheadPlan* ah = cls <= 2 && h->ahead[cls].ok ? &h->ahead[cls] : nullptr;
+    if (!tc.ok && !ah && !pl.ok) return US_ERR_UNSUPPORTED;
     if (grid) *grid = h->sm_count;
-    if (block) *block = tc.ok ? tc.threads : pl.g.warps * 32;
-    if (smem_bytes) *smem_bytes = tc.ok ? tc.smem : pl.g.smem;
+    if (block) *block = tc.ok ? tc.threads : ah ? ah->threads : pl.g.warps * 32;
+    if (smem_bytes) *smem_bytes = tc.ok ? tc.smem : ah ? ah->smem : pl.g.smem;
     return US_OK;
 }
 

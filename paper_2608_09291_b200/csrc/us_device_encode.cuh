@@ -1,8 +1,8 @@
 // Encoder kernels: the lane-stream layout of us_host.h built on the GPU from the weight as packed INT4 (two columns a
 // byte, even column in the low nibble; W2: the same nibbles), rows of `ld` bytes, zero beyond K.
 //
-// One warp per tile; lane 4g + t reads what it will own: for every 32-column k-block the 8 columns 32 kb + 8t .. of strip
-// rows g and g + 8, one 32-bit word per row (and column area). Two passes over the 22 MB of an 11008 x 4096 matrix,
+// One warp per tile; lane 4g + t reads what it will own: for every mask word w (four k-blocks) the 32 columns 128 w + 32 t ..
+// of strip rows g and g + 8, one 16-byte load per row (and column area). Two passes over the 22 MB of an 11008 x 4096 matrix,
 // sizes then bytes, about 20 us each; the host encoder needed 13 ms on 16 threads for the same, most of it byte by byte.
 #pragma once
 #include <cuda_runtime.h>
@@ -32,7 +32,7 @@ __device__ __forceinline__ uint32_t nonzero_nibbles(uint32_t v)
     return (even & 15u) | ((odd & 15u) << 4);
 }
 
-// The lane's words of mask byte kb: v[area][row half].
+// The lane's weights of a mask word, a 32-bit word per k-block: v[area][row half][k-block].
 struct EncodeLane {
     const uint8_t *a, *b;   // rows g and g + 8 at the tile's first column, nullptr = padding row
     int64_t second;         // bytes to the second column area
@@ -41,19 +41,24 @@ struct EncodeLane {
     {
         const int rb = item / p.n_segs, sg = item - rb * p.n_segs;
         const int ra = p.row_order[rb * 16 + (lane >> 2)], rw = p.row_order[rb * 16 + (lane >> 2) + 8];
-        const int64_t col = (int64_t)sg * (p.K_L / 2) + 4 * (lane & 3);
+        const int64_t col = (int64_t)sg * (p.K_L / 2) + 16 * (lane & 3);
         a = ra < 0 ? nullptr : p.W + (int64_t)ra * p.ld + col;
         b = rw < 0 ? nullptr : p.W + (int64_t)rw * p.ld + col;
         second = p.K_L / 4;
         fold = p.fold != 0;
     }
-    __device__ __forceinline__ void load(int kb, uint32_t (&v)[2][2]) const
+    __device__ __forceinline__ static void load16(const uint8_t* s, uint32_t (&v)[4])
     {
-        const int64_t o = 16 * (int64_t)kb;
-        v[0][0] = a ? __ldg(reinterpret_cast<const uint32_t*>(a + o)) : 0u;
-        v[0][1] = b ? __ldg(reinterpret_cast<const uint32_t*>(b + o)) : 0u;
-        v[1][0] = fold && a ? __ldg(reinterpret_cast<const uint32_t*>(a + o + second)) : 0u;
-        v[1][1] = fold && b ? __ldg(reinterpret_cast<const uint32_t*>(b + o + second)) : 0u;
+        const uint4 q = s ? __ldg(reinterpret_cast<const uint4*>(s)) : make_uint4(0, 0, 0, 0);
+        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+    }
+    __device__ __forceinline__ void load(int w, uint32_t (&v)[2][2][4]) const
+    {
+        const int64_t o = 64 * (int64_t)w;
+        load16(a ? a + o : nullptr, v[0][0]);
+        load16(b ? b + o : nullptr, v[0][1]);
+        load16(fold && a ? a + o + second : nullptr, v[1][0]);
+        load16(fold && b ? b + o + second : nullptr, v[1][1]);
     }
 };
 
@@ -62,13 +67,13 @@ __global__ void __launch_bounds__(256) us_encode_size_kernel(const EncodeParams 
     const int lane = threadIdx.x & 31, item = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (item >= p.n_items) return;
     const EncodeLane l(p, item, lane);
-    const int nkb = p.mask_rows * 4;   // mask bytes per lane
     int len = 0;
-#pragma unroll 4
-    for (int kb = 0; kb < nkb; ++kb) {
-        uint32_t v[2][2];
-        l.load(kb, v);
-        len += __popc(nonzero_nibbles(v[0][0] | v[0][1] | v[1][0] | v[1][1]));
+#pragma unroll 2
+    for (int w = 0; w < p.mask_rows; ++w) {
+        uint32_t v[2][2][4];
+        l.load(w, v);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) len += __popc(nonzero_nibbles(v[0][0][i] | v[0][1][i] | v[1][0][i] | v[1][1][i]));
     }
     const int longest = __reduce_max_sync(0xffffffffu, len), sum = __reduce_add_sync(0xffffffffu, len);
     if (lane == 0) {
@@ -133,18 +138,17 @@ __global__ void __launch_bounds__(256) us_encode_write_kernel(const EncodeParams
     unsigned long long acc[2] = {0, 0};   // bytes not yet stored, per stream
     int n = 0, at = 0;                    // how many; payload row they go to
     for (int w = 0; w < p.mask_rows; ++w) {
-        uint32_t mw = 0;
+        uint32_t mw = 0, v[2][2][4];
+        l.load(w, v);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            uint32_t v[2][2];
-            l.load(4 * w + i, v);
-            const uint32_t m = nonzero_nibbles(v[0][0] | v[0][1] | v[1][0] | v[1][1]);
+            const uint32_t m = nonzero_nibbles(v[0][0][i] | v[0][1][i] | v[1][0][i] | v[1][1][i]);
             mw |= m << (8 * i);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int c = 4 * (2 * (j & 3) + (j >> 2));   // (slot_column)
-                const uint32_t a0 = (v[0][0] >> c) & 15u, b0 = (v[0][1] >> c) & 15u;
-                const uint32_t a1 = (v[1][0] >> c) & 15u, b1 = (v[1][1] >> c) & 15u;
+                const uint32_t a0 = (v[0][0][i] >> c) & 15u, b0 = (v[0][1][i] >> c) & 15u;
+                const uint32_t a1 = (v[1][0][i] >> c) & 15u, b1 = (v[1][1][i] >> c) & 15u;
                 if ((m >> j) & 1u) {
                     if (p.w2) {
                         acc[0] |= (unsigned long long)(((a0 + 2u) & 3u) | (((b0 + 2u) & 3u) << 2) | (((a1 + 2u) & 3u) << 4) | (((b1 + 2u) & 3u) << 6)) << (8 * n);

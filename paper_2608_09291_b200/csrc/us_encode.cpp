@@ -415,7 +415,7 @@ us_status encode_host(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_s
                     int v[2][2];   // [column area][row half]
                     int any = 0;
                     for (int ca = 0; ca < CA; ++ca) {
-                        const int64_t k = k0 + (kk & ~7) + slot_column(kk & 7) + (int64_t)ca * K_B;
+                        const int64_t k = k0 + lane_column(kk >> 5, (kk >> 3) & 3) + slot_column(kk & 7) + (int64_t)ca * K_B;
                         v[ca][0] = (pa && k < K) ? pa[k] : 0;
                         v[ca][1] = (pb && k < K) ? pb[k] : 0;
                         any |= v[ca][0] | v[ca][1];
@@ -502,7 +502,7 @@ void decode_host(const HostMatrix& h, const uint8_t* blob, int8_t* W_out)
                 for (int j = 0; j < 8; ++j) {
                     if (!((m >> j) & 1)) continue;
                     for (int ca = 0; ca < CA; ++ca) {
-                        const int64_t k = sg * K_L + (int64_t)ca * K_B + 32 * kb + 8 * tt + slot_column(j);
+                        const int64_t k = sg * K_L + (int64_t)ca * K_B + lane_column(kb, tt) + slot_column(j);
                         if (k >= h.K) continue;
                         int lo, hi;
                         if (h.w2) {

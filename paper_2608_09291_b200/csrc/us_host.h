@@ -4,9 +4,10 @@
 // order chosen for the sm_100a kernel):
 //   * rows are cut into strips of 16 (after an optional row order); columns into segments of
 //     K_L; one (strip, segment) pair is a tile ("item"), tile index = strip * n_segs + segment.
-//   * a tile is decoded by one warp; lane l = 4*g + t owns, for every 32-column k-block kb of
-//     the tile, the 8 columns 32*kb + 8*t + j (j = 0..7) of strip rows g and g+8 -- exactly
-//     the A-fragment slots of that lane in an m16n8k32 integer MMA.
+//   * a tile is decoded by one warp; lane l = 4*g + t owns, of every 128 columns (four k-blocks kb = 4*w .. 4*w + 3), the
+//     32 columns 128*w + 32*t .. of strip rows g and g+8: k-block 4*w + i takes the 8 columns 128*w + 32*t + 8*i + j
+//     (j = 0..7), the A-fragment slots of that lane in an m16n8k32 integer MMA. (The order of a contraction's terms is
+//     free: so a lane's activations of a mask word are 16 consecutive packed bytes of a token.)
 //   * union mask: bit b of the lane's mask byte for k-block kb is set iff W[g][k] or W[g+8][k]
 //     is nonzero (one bit covers Q = 2 values, area 0 = strip rows 0..7, area 1 = rows 8..15), k = column j =
 //     slot_column(b) of the lane's eight: the even columns first, then the odd ones. A word of packed activations
@@ -40,6 +41,9 @@ namespace us {
 
 // Column, of a lane's eight of a k-block, that mask bit b stands for.
 constexpr int slot_column(int b) { return 2 * (b & 3) + (b >> 2); }
+
+// First column, in its column area, of the eight that lane 4 g + t owns in k-block kb.
+constexpr int lane_column(int kb, int t) { return 128 * (kb >> 2) + 32 * t + 8 * (kb & 3); }
 
 // The paper's three arrays for an arbitrary (H_L, K_L, R_A, C_A) (Sec. V-A "Storage Arrays"): what
 // a format without a kernel is encoded into, for us_get_stats / us_decode.

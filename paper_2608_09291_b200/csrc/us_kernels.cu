@@ -1,5 +1,6 @@
-// The instantiations of us_spmm_kernel for one N class and one kind of K: compiled with -DUS_NT=1, 2, 4, 8 and -DUS_ANY=0, 1.
+// The instantiations of us_spmm_kernel and us_spmm_ahead_kernel for one N class and one kind of K: compiled with -DUS_NT=1, 2, 4, 8 and -DUS_ANY=0, 1.
 #include "us_launch.h"
+#include "us_spmm_ahead.cuh"
 #include "us_spmm_kernel.cuh"
 
 #if !defined(US_NT) || !defined(US_ANY)
@@ -53,5 +54,32 @@ const void* kernel_nt<US_NT, US_ANY>(const KernelKey& k)
     if (k.stages == 1) return k.local ? pick<1, true>(k) : pick<1, false>(k);
     return k.local ? pick<2, true>(k) : pick<2, false>(k);
 }
+
+#if US_NT <= 4
+template <>
+const void* kernel_ahead<US_NT, US_ANY>(int warps, int threads, bool fold, bool w2, bool am)
+{
+    constexpr int NT = US_NT;
+    constexpr bool ANY = US_ANY;
+    if (!fold) {
+        if constexpr (NT == 1)
+            if (warps == 8 && threads == 32 * 12)
+                return am ? (const void*)us_spmm_ahead_kernel<NT, 1, false, true, ANY, 8, 12> : (const void*)us_spmm_ahead_kernel<NT, 1, false, false, ANY, 8, 12>;
+        if constexpr (NT <= 2)
+            if (warps == 12 && threads == 32 * 16)
+                return am ? (const void*)us_spmm_ahead_kernel<NT, 1, false, true, ANY, 12, 16> : (const void*)us_spmm_ahead_kernel<NT, 1, false, false, ANY, 12, 16>;
+        if constexpr (NT > 2)
+            if (warps == 8 && threads == 32 * 10)
+                return am ? (const void*)us_spmm_ahead_kernel<NT, 1, false, true, ANY, 8, 10> : (const void*)us_spmm_ahead_kernel<NT, 1, false, false, ANY, 8, 10>;
+        return nullptr;
+    }
+    if (warps != 8 || am) return nullptr;
+    if constexpr (NT <= 2)
+        if (threads == 32 * 12)
+            return w2 ? (const void*)us_spmm_ahead_kernel<NT, 2, true, false, ANY, 8, 12> : (const void*)us_spmm_ahead_kernel<NT, 2, false, false, ANY, 8, 12>;
+    if (threads != 32 * 10) return nullptr;
+    return w2 ? (const void*)us_spmm_ahead_kernel<NT, 2, true, false, ANY, 8, 10> : (const void*)us_spmm_ahead_kernel<NT, 2, false, false, ANY, 8, 10>;
+}
+#endif
 
 }  // namespace us

@@ -28,6 +28,16 @@ template <> const void* kernel_nt<2, true>(const KernelKey& k);
 template <> const void* kernel_nt<4, true>(const KernelKey& k);
 template <> const void* kernel_nt<8, true>(const KernelKey& k);
 
+// us_spmm_ahead_kernel for N <= 8 NT (NT = 1, 2, 4) with so many decode warps and threads, in the same units; am = absmax of the output (default format only).
+template <int NT, bool ANY>
+const void* kernel_ahead(int warps, int threads, bool fold, bool w2, bool am);
+template <> const void* kernel_ahead<1, false>(int warps, int threads, bool fold, bool w2, bool am);
+template <> const void* kernel_ahead<2, false>(int warps, int threads, bool fold, bool w2, bool am);
+template <> const void* kernel_ahead<4, false>(int warps, int threads, bool fold, bool w2, bool am);
+template <> const void* kernel_ahead<1, true>(int warps, int threads, bool fold, bool w2, bool am);
+template <> const void* kernel_ahead<2, true>(int warps, int threads, bool fold, bool w2, bool am);
+template <> const void* kernel_ahead<4, true>(int warps, int threads, bool fold, bool w2, bool am);
+
 // us_spmm_tc_kernel (us_spmm_tc.cu) with two or three octets: any_k = K is not a multiple of 32; fold = two column areas; am = absmax of the output (default format only).
 const void* kernel_tc(int octets, bool any_k, bool fold, bool w2, bool am);
 

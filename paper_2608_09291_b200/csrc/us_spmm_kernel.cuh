@@ -87,6 +87,13 @@ constexpr int kNoRow = -2;        // "row ids not loaded yet" marker (-1 is a pa
 constexpr int kClaimWords = 96;   // shared-memory words of the claim counter and its neighbours
 constexpr int kOffTable = 256;   // tile offsets of a CTA kept in shared memory (start, end pairs)
 
+// Bytes of one token's row of staged X, `cols` columns (a multiple of 128): int8, or packed (xp). A lane reads 16 bytes at a
+// time, eight lanes (two tokens, t = 0..3) in one pass: the pad puts the second token on the banks that the first leaves free.
+__host__ __device__ constexpr int x_row_bytes(int cols, bool xp)
+{
+    return xp ? cols / 2 + 64 - (cols / 2) % 128 : cols + 16;
+}
+
 // ---- selector table -------------------------------------------------------------------------
 // entry(m): low 16 bits  = prmt selector for mask bits 0..3 reading the 4 bytes AT the lane's
 //                          stream position (nibble j = rank of bit j, or 4 = neutral byte);
@@ -126,6 +133,11 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t c)
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
+}
+// (without an arrival)
+__device__ __forceinline__ void mbar_expect_tx_only(uint32_t bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
 {
@@ -192,6 +204,17 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
         ::"r"(dst), "l"(src), "r"(bytes), "r"(bar), "l"(policy)
         : "memory");
 }
+__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+__device__ __forceinline__ uint4 lds128(uint32_t a)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
 __device__ __forceinline__ void mma_s8(int (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
                                        uint32_t a3, uint32_t b0, uint32_t b1)
 {
@@ -216,12 +239,6 @@ __device__ __forceinline__ uint32_t lds32_at(uint32_t a)
 {
     uint32_t v;
     asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(a), "n"(OFF));
-    return v;
-}
-__device__ __forceinline__ uint2 lds64(uint32_t a)
-{
-    uint2 v;
-    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
     return v;
 }
 
@@ -481,15 +498,21 @@ __device__ __forceinline__ void process_tile(uint32_t slot_a, uint32_t lut_a, ui
     const uint32_t mask_a = slot_a + 4u * lane;
     const uint32_t pay_a = slot_a + 128u * mask_rows + 4u * lane;
     constexpr bool kPreX = NT <= 2 && CA == 1;   // small N: fetch the X fragments together with the windows
-    constexpr uint32_t kXStep = XP ? 16u : 32u;   // bytes of a token's row per k-block
+    constexpr uint32_t kXWord = XP ? 64u : 128u;  // bytes of a token's row per mask word
+    constexpr int kXR = XP ? 4 : 8;               // registers of a lane's activations of a mask word
     constexpr int SR = W2 ? 1 : CA;               // payload streams per lane
     constexpr int kRow = 128 * SR;                // bytes from one payload row of a stream to its next
-    auto ldx = [&](uint32_t a) -> uint2 {         // the lane's two B-fragment words at address a
-        if (XP) {
-            const uint32_t q = lds32(a);
-            return make_uint2((q * 16u) & 0xF0F0F0F0u, q & 0xF0F0F0F0u);
+    auto packed_b = [](uint32_t q) { return make_uint2((q * 16u) & 0xF0F0F0F0u, q & 0xF0F0F0F0u); };   // B fragment of 8 packed activations
+    auto mma_block = [&](int nt, uint32_t d0, uint32_t d1, uint2 b) {   // one k-block
+        int (&cc)[4] = c[nt];
+        constexpr uint32_t low = W2 ? 0x03030303u : 0x0F0F0F0Fu;
+        const uint32_t e0 = d0 & low, e1 = d1 & low;
+        if (DP) {
+            cc[0] = __dp4a((int)d0, (int)b.x, cc[0]); cc[0] = __dp4a((int)d1, (int)b.y, cc[0]);
+            cc[2] = __dp4a((int)e0, (int)b.x, cc[2]); cc[2] = __dp4a((int)e1, (int)b.y, cc[2]);
+        } else {
+            mma_s8(cc, d0, e0, d1, e1, b.x, b.y);
         }
-        return lds64(a);
     };
     uint32_t b8 = 0;                                     // 8 * (byte position in the lane's payload stream)
     uint32_t cw0[SR], cw1[SR];                           // carried window: the words at / after the position
@@ -498,7 +521,7 @@ __device__ __forceinline__ void process_tile(uint32_t slot_a, uint32_t lut_a, ui
     const uint32_t xb_fold_a = xb_a + x_fold;            // X fragments of the second column area
     for (int w = 0; w < mask_rows; ++w) {
         uint32_t pos[5], wm1[SR][4], w0[SR][4], w1[SR][4], e[4];
-        uint2 xf[4][kPreX ? NT : 1];
+        uint32_t xf[kPreX ? NT : 1][kXR];
         const uint32_t mw = lds32(mask_a + 128u * w);
         pos[0] = b8;
 #pragma unroll
@@ -520,53 +543,61 @@ __device__ __forceinline__ void process_tile(uint32_t slot_a, uint32_t lut_a, ui
                 w1[SR - 1][i] = lds32_at<128 + kRow>(a);
             }
             e[i] = lds32(e[i]);
-            if (kPreX) {
+            if (kPreX && i == 0) {
 #pragma unroll
-                for (int nt = 0; nt < NT; ++nt) xf[i][nt] = ldx(xb_a + kXStep * (4 * w + i) + nt * 8 * xstride);
+                for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+                    for (int h = 0; h < kXR / 4; ++h) {   // the lane's activations of the word: 32 consecutive columns
+                        const uint4 q = lds128(xb_a + kXWord * w + nt * 8 * xstride + 16 * h);
+                        xf[nt][4 * h] = q.x; xf[nt][4 * h + 1] = q.y; xf[nt][4 * h + 2] = q.z; xf[nt][4 * h + 3] = q.w;
+                    }
             }
         }
+        uint32_t d[CA][8];   // the word's fragment bytes, rows g: two registers per k-block
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            if (W2) {
-                const uint32_t s0 = (i == 0) ? cw0[0] : w0[0][i - 1];
-                const uint32_t s1 = (i == 0) ? cw1[0] : w1[0][i - 1];
-                const uint32_t lo = __funnelshift_r(s0, s1, pos[i]);
-                const uint32_t prev = __funnelshift_r(wm1[0][i], w0[0][i], pos[i + 1]);
-                const uint32_t g0 = prmt(lo, kFillW2, e[i]);
-                const uint32_t g1 = prmt(prev, kFillW2, e[i] >> 16);
 #pragma unroll
-                for (int ca = 0; ca < 2; ++ca) {
-                    const uint32_t d0 = (ca ? g0 >> 4 : g0) & 0x0F0F0F0Fu, d1 = (ca ? g1 >> 4 : g1) & 0x0F0F0F0Fu;
-                    const uint32_t e0 = d0 & 0x03030303u, e1 = d1 & 0x03030303u;
-#pragma unroll
-                    for (int nt = 0; nt < NT; ++nt) {
-                        const uint2 b = ldx((ca ? xb_fold_a : xb_a) + kXStep * (4 * w + i) + nt * 8 * xstride);
-                        mma_s8(c[nt], d0, e0, d1, e1, b.x, b.y);
-                    }
-                }
-            } else {
-#pragma unroll
-            for (int ca = 0; ca < CA; ++ca) {
+            for (int sr = 0; sr < SR; ++sr) {
                 // first four bytes: the window starting at pos[i] (carried, or the previous block's)
-                const uint32_t s0 = (i == 0) ? cw0[ca] : w0[ca][i - 1];
-                const uint32_t s1 = (i == 0) ? cw1[ca] : w1[ca][i - 1];
+                const uint32_t s0 = (i == 0) ? cw0[sr] : w0[sr][i == 0 ? 0 : i - 1];
+                const uint32_t s1 = (i == 0) ? cw1[sr] : w1[sr][i == 0 ? 0 : i - 1];
                 const uint32_t lo = __funnelshift_r(s0, s1, pos[i]);
-                const uint32_t prev = __funnelshift_r(wm1[ca][i], w0[ca][i], pos[i + 1]);
-                const uint32_t d0 = prmt(lo, kFill, e[i]);
-                const uint32_t d1 = prmt(prev, kFill, e[i] >> 16);
-                const uint32_t e0 = d0 & 0x0F0F0F0Fu, e1 = d1 & 0x0F0F0F0Fu;
-                if (DP) {
-                    const uint2 b = kPreX ? xf[i][0] : ldx(xb_a + kXStep * (4 * w + i));
-                    c[0][0] = __dp4a((int)d0, (int)b.x, c[0][0]); c[0][0] = __dp4a((int)d1, (int)b.y, c[0][0]);
-                    c[0][2] = __dp4a((int)e0, (int)b.x, c[0][2]); c[0][2] = __dp4a((int)e1, (int)b.y, c[0][2]);
-                } else {
+                const uint32_t prev = __funnelshift_r(wm1[sr][i], w0[sr][i], pos[i + 1]);
+                const uint32_t g0 = prmt(lo, W2 ? kFillW2 : kFill, e[i]);
+                const uint32_t g1 = prmt(prev, W2 ? kFillW2 : kFill, e[i] >> 16);
+                if (W2) {
 #pragma unroll
-                    for (int nt = 0; nt < NT; ++nt) {
-                        const uint2 b = kPreX ? xf[i][nt] : ldx((ca ? xb_fold_a : xb_a) + kXStep * (4 * w + i) + nt * 8 * xstride);
-                        mma_s8(c[nt], d0, e0, d1, e1, b.x, b.y);
+                    for (int ca = 0; ca < CA; ++ca) {
+                        d[ca][2 * i] = (ca ? g0 >> 4 : g0) & 0x0F0F0F0Fu;
+                        d[ca][2 * i + 1] = (ca ? g1 >> 4 : g1) & 0x0F0F0F0Fu;
                     }
+                } else {
+                    d[sr][2 * i] = g0; d[sr][2 * i + 1] = g1;
                 }
             }
+            if (kPreX) {
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt) mma_block(nt, d[0][2 * i], d[0][2 * i + 1], XP ? packed_b(xf[nt][XP ? i : 0]) : make_uint2(xf[nt][XP ? 0 : 2 * i], xf[nt][XP ? 0 : 2 * i + 1]));
+            } else if (XP ? i == 3 : i & 1) {
+                // the word's k-blocks in twos (packed X: all four, a 16-byte load holds them), token groups in twos (fours): MMAs
+                // on different sums follow each other
+                constexpr int GN = NT == 8 ? 1 : NT < (XP ? 4 : 2) ? NT : (XP ? 4 : 2);
+#pragma unroll
+                for (int ca = 0; ca < CA; ++ca)
+#pragma unroll
+                    for (int n0 = 0; n0 < NT; n0 += GN) {
+                        uint32_t x[GN][4];
+#pragma unroll
+                        for (int nt = 0; nt < GN; ++nt) {
+                            const uint4 q = lds128((ca ? xb_fold_a : xb_a) + kXWord * w + (XP ? 0 : 16 * (i / 2)) + (n0 + nt) * 8 * xstride);
+                            x[nt][0] = q.x; x[nt][1] = q.y; x[nt][2] = q.z; x[nt][3] = q.w;
+                        }
+#pragma unroll
+                        for (int ii = XP ? 0 : i - 1; ii <= i; ++ii)
+#pragma unroll
+                            for (int nt = 0; nt < GN; ++nt)
+                                mma_block(n0 + nt, d[ca][2 * ii], d[ca][2 * ii + 1], XP ? packed_b(x[nt][ii]) : make_uint2(x[nt][2 * (ii & 1)], x[nt][2 * (ii & 1) + 1]));
+                    }
             }
         }
 #pragma unroll
@@ -640,9 +671,7 @@ __global__ void __launch_bounds__(kMaxThreads<ANY, NT, STAGES, LA, TIMED, CA, W2
     const unsigned long long g_start = timing ? global_timer_ns() : 0;
 
     // ---- shared-memory carve-up (mirrored by plan_launch on the host) --------------------------
-    // bytes of one token's row of staged X: int8, or packed (XP); the pad keeps the 8 tokens of an
-    // n-tile on different banks
-    const int xstride = XP ? p.G * p.K_L / 2 + 16 : p.G * p.K_L + 32;
+    const int xstride = x_row_bytes(p.G * p.K_L, XP);
     uint32_t* lut = reinterpret_cast<uint32_t*>(smem);                       // [256][lut_rep]
     uint32_t* lut1 = lut + 256 * p.lut_rep;                                  // [256] built first
     uint8_t* x8 = reinterpret_cast<uint8_t*>(lut1 + 256);
@@ -1028,10 +1057,10 @@ __global__ void __launch_bounds__(kMaxThreads<ANY, NT, STAGES, LA, TIMED, CA, W2
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) c[nt][0] = c[nt][1] = c[nt][2] = c[nt][3] = 0;
             const uint32_t slot_a = smem_u32(my_ring + (size_t)cur * p.slot_bytes);
-            const uint32_t xb_a = XP ? smem_u32(x8) + (lane >> 2) * xstride + 4 * (lane & 3) + sgl * (p.K_L / 2)
-                                     : smem_u32(x8) + (lane >> 2) * xstride + 8 * (lane & 3) + sgl * p.K_L;
+            const uint32_t xb_a = XP ? smem_u32(x8) + (lane >> 2) * xstride + 16 * (lane & 3) + sgl * (p.K_L / 2)
+                                     : smem_u32(x8) + (lane >> 2) * xstride + 32 * (lane & 3) + sgl * p.K_L;
             if (DP) {
-                const uint32_t xb0 = smem_u32(x8) + 8 * (lane & 3) + sgl * p.K_L;   // token 0, this lane's columns
+                const uint32_t xb0 = smem_u32(x8) + 32 * (lane & 3) + sgl * p.K_L;   // token 0, this lane's columns
                 process_tile<NT, XP, CA, W2, true>(slot_a, lut_a, 4u * (uint32_t)p.lut_rep, xb0, xstride, p.mask_rows, lane, c, 0u);
                 // the four lanes of a row group hold parts of the same two sums; the first keeps them in the
                 // accumulator slots of token 0, the slots of tokens 1..7 stay zero

@@ -301,8 +301,8 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
     volatile uint32_t* dead = misc + 1;
 
     const uint32_t beg = p.cta_begin[blockIdx.x], end = p.cta_begin[blockIdx.x + 1];
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (beg >= end) {
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         if (AM && threadIdx.x < 64) {
             asm volatile("griddepcontrol.wait;" ::: "memory");
             p.y_amax[64 + 64 * blockIdx.x + threadIdx.x] = 0;
@@ -369,6 +369,8 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
         __syncwarp();
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(misc)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        // Only now: a dependent's CTA that fits beside this one takes tensor memory of its own, and then waits for this kernel.
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     } else {
         const int x = threadIdx.x - 32 * (kTcDecodeWarps + 1);
         for (int i = x; i < kTcSxRing * 64; i += 32 * kTcXWarps) sx[i] = 0;
@@ -633,7 +635,8 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
             // columns of this lane's two 32-column units: CA = 1 consecutive; CA = 2 half of the stage from each column area
             const int k0 = seg * p.K_L + (CA == 1 ? 256 : 128) * st + 32 * qq;
             const int k1 = CA == 1 && 2 * st + 1 >= p.mask_rows ? p.K : k0 + k_second;
-            uint8_t* dst0 = xs + (size_t)xst * x_stage_bytes + g0 * 2048 + (2 * qq) * 128 + r * 16;
+            // (the lane's 32 columns are lane t = qq of a fragment: 8 of them in each of the unit's four k-blocks)
+            uint8_t* dst0 = xs + (size_t)xst * x_stage_bytes + g0 * 2048 + (qq >> 1) * 128 + r * 16 + (qq & 1) * 8;
             int32_t* sxr = sx + ((q - q0) % kTcSxRing) * 64;
             UnitX v0 = load_x32<ANY>(p, ldx, 8 * g0 + r, k0), v1 = load_x32<ANY>(p, ldx, 8 * g0 + r, k1);
             UnitX n0, n1;   // a group ahead
@@ -654,15 +657,11 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const uint4 v = unit_x<ANY>(p, ldx, 8 * g + r, h ? k1 : k0, h ? v1 : v0);
-                    uint4 a, b;
-                    uint2 t;
-                    t = expand8(v.x, s); a.x = t.x; a.y = t.y;
-                    t = expand8(v.y, s); a.z = t.x; a.w = t.y;
-                    t = expand8(v.z, s); b.x = t.x; b.y = t.y;
-                    t = expand8(v.w, s); b.z = t.x; b.w = t.y;
-                    uint4* dst = reinterpret_cast<uint4*>(dst0 + h * 1024);
-                    dst[0] = a;
-                    dst[8] = b;
+                    uint8_t* dst = dst0 + h * 1024;
+                    *reinterpret_cast<uint2*>(dst) = expand8(v.x, s);
+                    *reinterpret_cast<uint2*>(dst + 256) = expand8(v.y, s);
+                    *reinterpret_cast<uint2*>(dst + 512) = expand8(v.z, s);
+                    *reinterpret_cast<uint2*>(dst + 768) = expand8(v.w, s);
                 }
                 dst0 += 2048 * P;
                 s += __shfl_xor_sync(0xffffffffu, s, 8);
