@@ -59,8 +59,15 @@ struct AheadPlan {
     us::AheadParams p{};
 };
 
+// A split of the tiles over the CTAs (make_schedule), for one length of K ranges.
+struct Schedule {
+    std::vector<uint32_t> begin;
+    int strips = 1;
+};
+
 struct us_handle {
     us::HostMatrix host;
+    std::map<int, Schedule> schedules;   // by segments of a K range, while the plans are laid
     AheadPlan ahead[3];              // NT = 1, 2, 4
     TcPlan tc[9];                    // index: 8-token groups of the call
     ClassPlan plan[4];               // per N class (NT = 1, 2, 4, 8)
@@ -140,6 +147,16 @@ uint32_t slot_bytes_for(const us::HostMatrix& hm)
 int64_t x_bytes(int nt, int64_t G, int K_L, bool xp)
 {
     return (int64_t)nt * 8 * us::x_row_bytes((int)(G * K_L), xp);
+}
+
+// The schedule for K ranges of G segments: the classes and both kernels ask for the same ones.
+const Schedule& schedule(us_handle* h, int G)
+{
+    const auto it = h->schedules.find(G);
+    if (it != h->schedules.end()) return it->second;
+    Schedule& s = h->schedules[G];
+    us::make_schedule(h->host, h->sm_count, G, &s.begin, &s.strips);
+    return s;
 }
 
 int segs_per_range(const us::HostMatrix& hm, int nt, int limit, int64_t min_ranges, bool xp)
@@ -298,7 +315,9 @@ void plan_classes(us_handle* h)
                     if (Gr == G) continue;
                     G = Gr;
                     if (G <= 1) break;
-                    us::make_schedule(h->host, n_cta, G, out, &worst);
+                    const Schedule& sc = schedule(h, G);
+                    *out = sc.begin;
+                    worst = sc.strips;
                     const int need = worst * nt * 512;
                     if (pass == 0 && need <= kLocalAccBudget) { *s_local = worst; return G; }
                     if (pass == 1 && need <= kLocalAccCap) {
@@ -345,8 +364,7 @@ void plan_classes(us_handle* h)
         }
         // direct mode: one segment per range, every tile goes to the global workspace (longer ranges
         // and runs were measured: no gain at N = 32, the bigger X costs more than the adds it saves)
-        int worst = 1;
-        if (h->s_local[c] == 0) us::make_schedule(h->host, n_cta, 1, &sched[c], &worst);
+        if (h->s_local[c] == 0) sched[c] = schedule(h, 1).begin;
     }
 }
 
@@ -501,7 +519,8 @@ void build_tc_plan(us_handle* h, int ng)
 // the largest CTA's share):
 //   N <= 8: up to 64 tiles (1024 x 1024 3.1 / 2.2, 4096 x 4096 4.75 / 3.8, 11008 x 4096 8.8 / 6.6, 15360 x 5120, 33 tiles, 13.7 / 11.3,
 //     27648 x 5120, 60 tiles, 19.0 / 18.7; 28672 x 8192 at .6, 97 tiles, 26.4 / 31.2: the other kernel's 16 warps on one CTA count from
-//     there on), 46 with two column areas (20480 x 5120, 45 tiles, 14.6 / 14.6), 40 where K is cut in ranges (5120 x 13824, 31 tiles, 14.7 / 12.5).
+//     there on), 46 with two column areas (20480 x 5120, 45 tiles, 14.6 / 14.6), 40 where K is cut in ranges or fewer than eight
+//     slots are left (5120 x 13824, 31 tiles, 14.7 / 12.5; 11136 x 9388, 50 tiles and seven slots, 17.9 / 19.5).
 //   N <= 16: up to 42 tiles (5120 x 5120 7.9 / 6.6, 11008 x 4096 10.1 / 8.2, 13824 x 5120, 30 tiles, 13.0 / 12.9, 22016 x 4096, 40 tiles,
 //     16.7 / 15.9; 20480 x 5120, 45 tiles, 17.6 / 18.5). It is taken where alone it is no better, too: a CTA of the whole SM and one of
 //     half an SM cannot overlap, and a change between the two kinds costs 3 to 8 us (the seven projections of a 13B-shaped
@@ -534,9 +553,9 @@ void build_ahead_plan(us_handle* h, int cls)
         if ((hm.n_segs + G - 1) / G != r) continue;
         const int64_t x = (int64_t)nt * 8 * us::ahead_x_row((int)std::min<int64_t>(G * hm.fmt.K_L, 1 << 20), hm.K % 32 != 0);
         if (x > kHalfSmBytes) continue;
-        std::vector<uint32_t> begin;
-        int strips = 1;
-        us::make_schedule(hm, h->sm_count, (int)G, &begin, &strips);
+        const Schedule& sc = schedule(h, (int)G);
+        const std::vector<uint32_t>& begin = sc.begin;
+        const int strips = sc.strips;
         most = 1;
         bool one_range = true;   // to every CTA
         for (int c = 0; c < h->sm_count; ++c) {
@@ -566,7 +585,7 @@ void build_ahead_plan(us_handle* h, int cls)
     if (p.n_ranges == 0) return;
     const int64_t share = most * hm.fmt.K_L / 1024;
     const bool more_ranges = p.n_ranges > 1 && h->s_local[cls] > 0 && h->G[cls] == hm.n_segs;   // than the other plan's one
-    const bool better = cls == 0   ? share <= (p.n_ranges > 1 ? 40 : plain ? 64 : 46) && (hm.n_segs > 1 || most <= 8)
+    const bool better = cls == 0   ? share <= (p.n_ranges > 1 || p.n_slots < 8 ? 40 : plain ? 64 : 46) && (hm.n_segs > 1 || most <= 8)
                         : cls == 1 ? share <= (more_ranges || (!plain && p.n_ranges > 1) ? 24 : plain ? 42 : 28)
                                    : p.parked == most;
     if (ahead_knob() == 1 && !better) return;
@@ -807,6 +826,7 @@ us_status encode(const int8_t* W, int64_t M, int64_t K, const uint16_t* w_scale,
     auto lay_plans = [&] {
         for (int c = 0; c <= class_of(nt_max); ++c) { build_plan(h, c); build_ahead_plan(h, c); }
         for (int ng = 1; ng <= (max_N + 7) / 8; ++ng) build_tc_plan(h, ng);
+        h->schedules.clear();
     };
     plan_classes(h);
     if (host_only) {

@@ -543,14 +543,13 @@ __device__ __forceinline__ void process_tile(uint32_t slot_a, uint32_t lut_a, ui
                 w1[SR - 1][i] = lds32_at<128 + kRow>(a);
             }
             e[i] = lds32(e[i]);
-            if (kPreX && i == 0) {
+            if (kPreX && (i == 0 || (!XP && i == 2))) {   // the lane's activations of the word (int8: of two k-blocks): consecutive columns
 #pragma unroll
-                for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                    for (int h = 0; h < kXR / 4; ++h) {   // the lane's activations of the word: 32 consecutive columns
-                        const uint4 q = lds128(xb_a + kXWord * w + nt * 8 * xstride + 16 * h);
-                        xf[nt][4 * h] = q.x; xf[nt][4 * h + 1] = q.y; xf[nt][4 * h + 2] = q.z; xf[nt][4 * h + 3] = q.w;
-                    }
+                for (int nt = 0; nt < NT; ++nt) {
+                    const uint4 q = lds128(xb_a + kXWord * w + nt * 8 * xstride + 8 * i);
+                    const int at = XP ? 0 : 2 * i;
+                    xf[nt][at] = q.x; xf[nt][at + 1] = q.y; xf[nt][at + 2] = q.z; xf[nt][at + 3] = q.w;
+                }
             }
         }
         uint32_t d[CA][8];   // the word's fragment bytes, rows g: two registers per k-block
