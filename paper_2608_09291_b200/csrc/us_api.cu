@@ -453,27 +453,26 @@ void build_tc_plan(us_handle* h, int ng)
     if (block_stages >= (1 << 16) || stages >= (1 << 24)) return;   // exact division by multiplication
     // Where it is chosen. The kernel saves the X fragments, MMAs and split-K adds of every tile and gives all CTAs the same
     // number of stages; it pays a longer prologue and a flush through the workspace per CTA (4 to 5 us together at N = 64).
-    // Against a plan that sums strips in shared memory, whose time follows the largest share of a CTA (cuts fall on strip
-    // boundaries), two straight lines in us fit what was measured at s = .5 and .6 within 5 %, `share` and `mean` being the
-    // largest and the average CTA share in stages:
-    //   N <= 16: that plan 4.5 + 1.08 share, this kernel 7.5 + 0.9 mean (20480 x 8192 26.2 / 23.3, 28672 x 8192 32.4 / 28.0,
-    //            27648 x 5120 21.0 / 20.9, 13824 x 5120 13.0 / 14.2). Half a us of margin, and from 10 stages on: among other
-    //            launches its code comes from L2 each time, and 5120 x 13824, 7 stages, alone 15.1 / 13.8, gained nothing in
-    //            a layer of seven projections (called by itself again and again it would).
-    //   N <= 32: 5.5 + 1.76 share, 9.7 + 0.97 mean (13824 x 5120 18.8 / 17.2, 28672 x 8192 51 / 33, 5120 x 5120 12.3 / 12.7);
-    //            2 us of margin, since matrices of uneven density cost this kernel more (4096 x 11008 sorted 15.5 / 16.1).
-    //            Even ones pay for that: 13824 x 5120 falls inside the margin and keeps the slower plan.
-    //   N <= 64: from 4 stages on (4096 x 4096, 1.7 stages, 14.4 / 17.3; 11008 x 4096, 4.6 stages, 35 / 20.6).
-    // Against the direct mode it wins nearly always (N = 32 on 2 x 2 tiles 5120 x 5120 14.9 / 12.9; N = 64 4096 x 4096 with
-    // INT2 weights 21.8 / 16.5, 28672 x 8192 92 / 41).
+    // Where us_spmm_ahead_kernel takes the calls it is the better one. Against a plan of us_spmm_kernel that sums strips in
+    // shared memory, whose time follows the largest share of a CTA (cuts fall on strip boundaries), straight lines in us
+    // fit what was measured at s = .5 and .6, `share` and `mean` being the largest and the average CTA share in stages:
+    //   N <= 16: that plan 5.9 + 1.08 share, this kernel 7.8 + 0.9 mean (20480 x 5120 17.6 / 17.5, 18432 x 6144 18.8 / 17.9, 27648 x 5120
+    //            21.6 / 21.0, 20480 x 8192 26.0 / 23.3), from 10 stages on and with 1.6 us of margin: among other launches its code
+    //            comes from L2 each time (a 13B-shaped chain with 27648 x 5120 on this kernel 74.3, on the other 72.2).
+    //   N <= 32: 5.5 + 1.76 share, 7.5 + 1.1 mean (11008 x 4096 13.6 / 13.1, 4096 x 11008 14.7 / 12.3, 13824 x 5120 19.2 / 15.9,
+    //            2048 x 8192 8.2 / 8.8), a us of margin, with INT2 weights 2.5 (11008 x 4096 11.8 / 12.4, 13824 x 5120 16.2 / 14.8).
+    //   N <= 64: from 2048 columns on (2048 x 2048 10.3 / 9.6, 4096 x 4096 16.6 / 14.2, 11008 x 4096 35 / 17.4), below that where
+    //            CTAs have most of a stage (16384 x 512 19.3 / 16.0; 4096 x 1024, 0.4 stages, 8.8 / 9.7).
+    // Against the direct mode it wins nearly always (N = 64 28672 x 8192 92 / 38).
     const int cls = class_of(nt_for(8 * ng));
     uint32_t most = 0;
     for (size_t c = 0; c + 1 < h->cta_begin[cls].size(); ++c) most = std::max(most, h->cta_begin[cls][c + 1] - h->cta_begin[cls][c]);
     const double mean = (double)stages / (double)n_cta, share = (double)most * n_stage / 16;
-    const bool better = h->s_local[cls] == 0 ? mean >= 1.5
-                        : ng <= 2            ? mean >= 10 && 4.5 + 1.08 * share > 8.0 + 0.9 * mean
-                        : ng <= 4            ? 5.5 + 1.76 * share > 11.7 + 0.97 * mean
-                                             : mean >= 4;
+    const bool better = cls <= 2 && h->ahead[cls].ok ? false
+                        : ng > 4                     ? hm.Kp >= 2048 || mean >= 0.8
+                        : h->s_local[cls] == 0       ? mean >= 1.5
+                        : ng <= 2                    ? mean >= 10 && 5.9 + 1.08 * share > 9.4 + 0.9 * mean
+                                                     : 5.5 + 1.76 * share > (hm.w2 ? 10.0 : 8.5) + 1.1 * mean;
     if (tc_knob() == 0 || (tc_knob() == 1 && !better)) return;
     p.slot_bytes = slot_bytes_for(hm);
     const int limit = h->max_smem;

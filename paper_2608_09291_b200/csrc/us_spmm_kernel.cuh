@@ -209,6 +209,12 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
+__device__ __forceinline__ uint2 lds64(uint32_t a)
+{
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+    return v;
+}
 __device__ __forceinline__ uint4 lds128(uint32_t a)
 {
     uint4 v;
@@ -577,10 +583,16 @@ __device__ __forceinline__ void process_tile(uint32_t slot_a, uint32_t lut_a, ui
             if (kPreX) {
 #pragma unroll
                 for (int nt = 0; nt < NT; ++nt) mma_block(nt, d[0][2 * i], d[0][2 * i + 1], XP ? packed_b(xf[nt][XP ? i : 0]) : make_uint2(xf[nt][XP ? 0 : 2 * i], xf[nt][XP ? 0 : 2 * i + 1]));
+            } else if (NT == 8) {   // (eight token groups have no registers to spare for more than a k-block's activations)
+#pragma unroll
+                for (int ca = 0; ca < CA; ++ca)
+#pragma unroll
+                    for (int nt = 0; nt < NT; ++nt)
+                        mma_block(nt, d[ca][2 * i], d[ca][2 * i + 1], lds64((ca ? xb_fold_a : xb_a) + kXWord * w + 8 * i + nt * 8 * xstride));
             } else if (XP ? i == 3 : i & 1) {
                 // the word's k-blocks in twos (packed X: all four, a 16-byte load holds them), token groups in twos (fours): MMAs
                 // on different sums follow each other
-                constexpr int GN = NT == 8 ? 1 : NT < (XP ? 4 : 2) ? NT : (XP ? 4 : 2);
+                constexpr int GN = NT < (XP ? 4 : 2) ? NT : (XP ? 4 : 2);
 #pragma unroll
                 for (int ca = 0; ca < CA; ++ca)
 #pragma unroll

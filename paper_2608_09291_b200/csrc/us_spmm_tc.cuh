@@ -269,6 +269,63 @@ __device__ __noinline__ void store_block_tc(const StoreCtx& p, int v0, int v1, i
     store_rows<1, AM>(p, v, lane, m_lo, m_hi, nullptr, -2, n_base);
 }
 
+// A strip is complete: take its sums from the workspace, two 8-token blocks ahead, leave that zeroed, store. The weight scales are
+// fetched once and the activation scales come from shared memory. (Not unrolled further: this code is cold, its lines come from
+// L2 one by one, and where strips complete in the middle of the weight stream that costs more than it saves.)
+template <bool AM>
+__device__ __noinline__ void finish_strip_tc(const StoreCtx p, const float* xsc_s, int32_t* accp, int ng, int lane, int m_lo, int m_hi)
+{
+    float sw_lo = 0.f, sw_hi = 0.f;
+    if (p.fp16_out) {
+        if (m_lo >= 0) sw_lo = __half2float(__ushort_as_half(__ldg(p.w_scale + m_lo)));
+        if (m_hi >= 0) sw_hi = __half2float(__ushort_as_half(__ldg(p.w_scale + m_hi)));
+    }
+    int v[3][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        v[0][j] = __ldcg(accp + j * 32);
+        v[1][j] = ng > 1 ? __ldcg(accp + 128 + j * 32) : 0;
+    }
+    int n = 2 * (lane & 3);
+#pragma unroll 1
+    for (int nt = 0; nt < ng; ++nt, n += 8) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            v[2][j] = nt + 2 < ng ? __ldcg(accp + 256 + j * 32) : 0;
+            __stcg(accp + j * 32, 0);
+        }
+        accp += 128;
+        const float2 sx = *reinterpret_cast<const float2*>(xsc_s + n);
+        uint32_t big[2] = {0u, 0u};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int m = j < 2 ? m_lo : m_hi;
+            if (n + (j & 1) < p.N && m >= 0) {
+                const size_t o = (size_t)(n + (j & 1)) * p.M + m;
+                if (p.fp16_out) {
+                    const __half h = __float2half_rn((float)v[0][j] * (j < 2 ? sw_lo : sw_hi) * (j & 1 ? sx.y : sx.x));
+                    reinterpret_cast<__half*>(p.Y)[o] = h;
+                    if (AM && m >= p.amax_m0 && m < p.amax_m1) big[j & 1] = max(big[j & 1], (uint32_t)(__half_as_ushort(h) & 0x7FFFu));
+                } else {
+                    reinterpret_cast<int32_t*>(p.Y)[o] = v[0][j];
+                }
+            }
+        }
+        if (AM) {   // the eight lanes that hold a token combine
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                uint32_t m = big[k];
+                m = max(m, __shfl_xor_sync(0xffffffffu, m, 4));
+                m = max(m, __shfl_xor_sync(0xffffffffu, m, 8));
+                m = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
+                if (lane < 4 && m) atomicMax(p.amax_s + n + k, m);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { v[0][j] = v[1][j]; v[1][j] = v[2][j]; }
+    }
+}
+
 // ANY: K is not a multiple of 32 (load_x32).
 // OCT = 3: 24 decode warps, 384 rows to a stage, for N <= 16. With 16 decode warps 0.59 instructions issue per cycle and
 // scheduler; eight more warps hide more of the decode's latency (28672 x 8192, N = 16: 29.3 -> 28.0 us, with INT2 weights
@@ -289,6 +346,7 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
     uint32_t* lut = reinterpret_cast<uint32_t*>(smem);                              // [256][lut_rep]
     uint8_t* xs = reinterpret_cast<uint8_t*>(lut + 256 * p.lut_rep);                // [x_stages][ng][16][8][16]
     // (an odd number of token groups: the MMA's last block reads on into the next stage, or these 2 KB; those sums are never used)
+    float* xsc_s = reinterpret_cast<float*>(xs + (size_t)p.x_stages * x_stage_bytes);           // [64] activation scales, in those 2 KB
     int32_t* sx = reinterpret_cast<int32_t*>(xs + (size_t)p.x_stages * x_stage_bytes + 2048);   // [kTcSxRing][64]
     uint64_t* bars = reinterpret_cast<uint64_t*>(sx + kTcSxRing * 64);
     uint32_t* misc = reinterpret_cast<uint32_t*>(bars + kTcBars);   // [0] tensor memory, [1] dead, [2] finished warps, [32..95] absmax
@@ -525,26 +583,8 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
                     asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p.cnt + strip), "r"(run_stages) : "memory");
                 old = __shfl_sync(0xffffffffu, old, 0);
                 if (old + (uint32_t)run_stages == (uint32_t)p.block_stages) {
-                    // the strip is complete: take the sums (two blocks ahead), leave workspace and counter zeroed
                     __syncwarp();
-                    int v[3][4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        v[0][j] = __ldcg(accp + j * 32);
-                        v[1][j] = ng > 1 ? __ldcg(accp + 128 + j * 32) : 0;
-                    }
-#pragma unroll 1
-                    for (int nt = 0; nt < ng; ++nt) {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            v[2][j] = nt + 2 < ng ? __ldcg(accp + 256 + j * 32) : 0;
-                            __stcg(accp + j * 32, 0);
-                        }
-                        store_block_tc<AM>(sctx, v[0][0], v[0][1], v[0][2], v[0][3], lane, m_lo, m_hi, 8 * nt);
-                        accp += 128;
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) { v[0][j] = v[1][j]; v[1][j] = v[2][j]; }
-                    }
+                    finish_strip_tc<AM>(sctx, xsc_s, accp, ng, lane, m_lo, m_hi);
                     if (lane == 0) p.cnt[strip] = 0;
                 }
             }
@@ -626,6 +666,9 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
         uint32_t x_par = 1;
         const int k_second = CA == 1 ? 128 : p.K_L / 2;
         asm volatile("griddepcontrol.wait;" ::: "memory");
+        // (by the warps of the first stage: its barriers hand the scales on to the decode warps, as they do the sums)
+        if (p.fp16_out && c0 == 0)
+            for (int i = lane + 32 * g0; i < p.N; i += 32 * P) xsc_s[i] = __half2float(__ushort_as_half(__ldg(p.x_scale + i)));
         if (c0 < W)
         for (int c = c0; c < total; c += W) {
             while (st >= n_stage) {
