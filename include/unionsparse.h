@@ -246,7 +246,8 @@ us_status us_debug_withhold_copy(us_handle* h, int64_t position, int64_t wait_us
  * and from [12] five words per CTA (192 CTAs), in ns after the first warp's start: CTA start, first
  * warp's end, activations staged, CTA end, past the wait for the stream's earlier work.
  * Recording costs a few clock reads per tile; off by default. Calls that run on the tensor-memory
- * kernel (wide batches) and variants without a timer build record nothing.
+ * kernel (wide batches) and variants without a timer build record nothing; calls that otherwise
+ * run on the decode-ahead kernel take the other one's plan while the timers are on.
  */
 us_status us_stage_timers(us_handle* h, int32_t enable, uint64_t* out, int32_t n_out);
 

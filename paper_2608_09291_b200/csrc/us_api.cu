@@ -460,7 +460,8 @@ void build_tc_plan(us_handle* h, int ng)
     //            21.6 / 21.0, 20480 x 8192 26.0 / 23.3), from 10 stages on and with 1.6 us of margin: among other launches its code
     //            comes from L2 each time (a 13B-shaped chain with 27648 x 5120 on this kernel 74.3, on the other 72.2).
     //   N <= 32: 5.5 + 1.76 share, 7.5 + 1.1 mean (11008 x 4096 13.6 / 13.1, 4096 x 11008 14.7 / 12.3, 13824 x 5120 19.2 / 15.9,
-    //            2048 x 8192 8.2 / 8.8), a us of margin, with INT2 weights 2.5 (11008 x 4096 11.8 / 12.4, 13824 x 5120 16.2 / 14.8).
+    //            2048 x 8192 8.2 / 8.8), a us of margin, with INT2 weights 2.5 (11008 x 4096 11.8 / 12.4, 13824 x 5120 16.2 / 14.8). Tiles of
+    //            uneven size leave it fewer slots (4096 x 11008, rows sorted, largest tile 1.3 times the average, 15.3 / 15.6).
     //   N <= 64: from 2048 columns on (2048 x 2048 10.3 / 9.6, 4096 x 4096 16.6 / 14.2, 11008 x 4096 35 / 17.4), below that where
     //            CTAs have most of a stage (16384 x 512 19.3 / 16.0; 4096 x 1024, 0.4 stages, 8.8 / 9.7).
     // Against the direct mode it wins nearly always (N = 64 28672 x 8192 92 / 38).
@@ -468,11 +469,12 @@ void build_tc_plan(us_handle* h, int ng)
     uint32_t most = 0;
     for (size_t c = 0; c + 1 < h->cta_begin[cls].size(); ++c) most = std::max(most, h->cta_begin[cls][c + 1] - h->cta_begin[cls][c]);
     const double mean = (double)stages / (double)n_cta, share = (double)most * n_stage / 16;
+    const double uneven = (double)hm.max_item_bytes * (double)hm.n_items / (double)std::max<uint64_t>(1, hm.blob_bytes);   // largest tile / average
     const bool better = cls <= 2 && h->ahead[cls].ok ? false
                         : ng > 4                     ? hm.Kp >= 2048 || mean >= 0.8
                         : h->s_local[cls] == 0       ? mean >= 1.5
                         : ng <= 2                    ? mean >= 10 && 5.9 + 1.08 * share > 9.4 + 0.9 * mean
-                                                     : 5.5 + 1.76 * share > (hm.w2 ? 10.0 : 8.5) + 1.1 * mean;
+                                                     : 5.5 + 1.76 * share > (hm.w2 ? 10.0 : 8.5) + 1.1 * mean + 12 * std::max(0.0, uneven - 1.1);
     if (tc_knob() == 0 || (tc_knob() == 1 && !better)) return;
     p.slot_bytes = slot_bytes_for(hm);
     const int limit = h->max_smem;
@@ -545,13 +547,16 @@ void build_ahead_plan(us_handle* h, int cls)
     const int places = us::kAheadCols / p.tile_cols;   // of parked tiles in each quarter of the tensor memory
     // The fewest K ranges whose X leaves room for six tile slots (5120 x 13824, N = 8: one range with five 16.3 us, two with
     // eight 12.5; N = 16: two with four 16.2, three with six 15.1).
+    if (hm.n_items > (int64_t)us::kAheadMaxTiles * h->sm_count || hm.n_items * hm.fmt.K_L > 64 * 1024 * (int64_t)h->sm_count) return;
     int64_t most = 0;
     int warps = 8;
     for (int64_t r = 1; r <= 8 && p.n_ranges == 0; ++r) {
         const int64_t G = (hm.n_segs + r - 1) / r;
         if ((hm.n_segs + G - 1) / G != r) continue;
         const int64_t x = (int64_t)nt * 8 * us::ahead_x_row((int)std::min<int64_t>(G * hm.fmt.K_L, 1 << 20), hm.K % 32 != 0);
-        if (x > kHalfSmBytes) continue;
+        // (no schedule is laid for ranges that cannot do: where not all can be parked, X and six slots beside it)
+        const bool all_parked = hm.n_items <= 4 * places * (int64_t)h->sm_count;
+        if (us::ahead_fixed_smem(nt, 1) + x + (all_parked ? 0 : 6 * (int64_t)p.slot_bytes) > kHalfSmBytes) continue;
         const Schedule& sc = schedule(h, (int)G);
         const std::vector<uint32_t>& begin = sc.begin;
         const int strips = sc.strips;

@@ -10,10 +10,14 @@
 // it is, and the MMAs: per k-block two masks, the two halves of a word of X per 8 tokens and the MMA.
 //
 //   decode    W warps; tile j of the CTA belongs to warp j % W. The first tiles are parked ahead, later ones when their turn
-//             comes, in the place of the warp's first. Tile j is copied to slot j % n_slots, by the warp that has emptied the slot; every tile
-//             has a barrier of its own, used once.
-//   helpers   the last T - W warps: tensor memory, row numbers and scales of the CTA's strips, X (one bulk copy per token; ragged
-//             rows go through everyone's registers).
+//             comes, in the place of the warp's first. Tile j is copied to slot j % n_slots; every tile has a barrier of its
+//             own, used once, and one that says that it is decoded.
+//   helpers   the last T - W warps. All: row numbers and scales of the CTA's strips. The first: tensor memory, X (one bulk copy per
+//             token; ragged rows are shifted into place by everyone) and its scales. The others: copies into slots that
+//             come free (a copy takes the warp that issues it some 500 cycles: 20480 x 5120, N = 16 20.5 us with one of them, 18.5 with three).
+//
+// 4096 x 4096, N = 8: 4.75 us a call with us_spmm_kernel's half-SM plan, 3.8 so (7.4 MB: 1.95 TB/s); 13824 x 5120, N = 8: 11.2, 10.0; what is left
+// of the former is the end of one kernel up to the end of the next one's wait (2), X (0.7), MMAs and stores (1).
 //
 // A CTA sums its part of each strip in shared memory. With one K range the cuts fall on strip boundaries: it stores its strips,
 // and nothing goes through the split-K workspace. Where X does not leave room (N = 16 from K = 6000 or so), K is cut in ranges as
@@ -429,8 +433,8 @@ __global__ void __launch_bounds__(32 * T, 2) us_spmm_ahead_kernel(const __grid_c
                 for (int i = 0; i < 4; ++i) atomicAdd(al + nt * 128 + i * 32, y[nt][i]);
         }
         if (!ok) *dead = 1;
-        // All decode warps together store the CTA's strips, 32 results of a strip and token group at a time. (With a counter
-        // per strip, as where warps end at different times, the last warp of a strip stored all of it: 4096 x 4096, N = 8.)
+        // All decode warps together store the CTA's strips, 32 results of a strip and token group at a time. (With a counter per
+        // strip, as where warps end at different times, its last warp stored all of it: 1024 x 1024, N = 8 2.37 us, like this 2.29.)
         asm volatile("bar.sync 1, %0;" ::"n"(32 * W) : "memory");
         // (a result: fragment value i of token group nt of the CTA's strip ls)
         auto store = [&](int ls, int nt, int i, int v) {

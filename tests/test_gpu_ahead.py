@@ -1,0 +1,77 @@
+"""The decode-ahead kernel at its edges: one tile and many rounds per warp, tiles parked and not, activations over the tile
+slots and beside them, K cut in ranges (sums through the workspace), ragged rows, every format, chained calls among plain ones."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2608_09291_b200 import workloads
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+# (half an SM's shared memory, and the threads: 384 and 512 at N <= 8 and N <= 16, 320 with two column areas and at N <= 32)
+@pytest.mark.parametrize("M,K,fmt,w2,N,block", [
+    (16, 256, (16, 128, 2, 1), False, 8, 384),         # one CTA, two tiles
+    (2300, 1100, (16, 128, 2, 1), False, 7, 384),      # nine segments, ragged rows
+    (4096, 4096, None, False, 1, 384),
+    (11008, 2048, None, False, 3, 384),
+    (4096, 3000, (16, 384, 2, 1), False, 9, 512),      # three mask words, columns past K
+    (9000, 5120, None, False, 16, 512),                # later tiles decoded when their turn comes
+    (2048, 16384, None, False, 16, 512),               # K in ranges
+    (1600, 16001, (16, 1024, 2, 1), False, 11, 512),   # the same with ragged rows
+    (3000, 4096, None, False, 32, 320),                # activations over the slots
+    (3000, 4095, (16, 1024, 2, 2), False, 25, 320),
+    (5003, 3001, (16, 1024, 2, 2), False, 8, 320),
+    (4096, 4096, (16, 512, 2, 2), True, 8, 320),
+    (1500, 2100, (16, 2048, 2, 2), True, 16, 320),     # parked tiles of 128 columns
+])
+def test_decode_ahead(M, K, fmt, w2, N, block):
+    from paper_2608_09291_b200 import binding as b
+    W = (workloads.make_weight_w2 if w2 else workloads.make_weight)(M, K, 0.5, seed=M + K)
+    X = workloads.make_x(K, N, seed=K)
+    s_w, s_x = workloads.make_scales(M, N, seed=K)
+    sw = b.SparseWeight(W, s_w, fmt=fmt, max_N=N, flags=b.US_ENCODE_W2 if w2 else 0)
+    try:
+        info = b.us_launch_info(sw.handle, N)
+        assert info["block"] == block and info["smem_bytes"] <= 114 * 1024, info
+        ref = oracle.spmm_dense(W, X)
+        Xd, sd = torch.from_numpy(b.pack_int4(X)).cuda(), torch.from_numpy(s_x).cuda()
+        outs = [sw.spmm(Xd, N) if i % 2 else sw.spmm(Xd, N, sd) for i in range(6)]   # back to back: each beside the one before
+        torch.cuda.synchronize()
+        sw.check()
+        for i, y in enumerate(outs):
+            if i % 2:
+                assert (y.cpu().numpy() == ref).all(), i
+            else:   # (one rounding to fp16)
+                assert oracle.fp16_within_tolerance(y.cpu().numpy(), ref, s_w, s_x).all(), i
+    finally:
+        sw.close()
+
+
+@pytest.mark.parametrize("M,K,N", [(1024, 1024, 8), (2304, 2304, 16), (2048, 2048, 32)])
+def test_dependent_chain_of_decode_ahead_calls(M, K, N):
+    """Every call reads what the one before wrote, and the weights of several handles are decoded meanwhile."""
+    from paper_2608_09291_b200 import binding as b
+    s_w = workloads.make_chain_weight_scales(M, K, 3)
+    Ws = [workloads.make_weight(M, K, 0.5, seed=i) for i in range(3)]
+    sws = [b.SparseWeight(W, s_w, max_N=N) for W in Ws]
+    try:
+        x0 = workloads.make_x_f16(K, N, seed=1)
+        a, src, ys, amaxes = b.absmax_f16(torch.from_numpy(x0).cuda()), torch.from_numpy(x0).cuda(), [], []
+        for sw in sws:
+            left = b.new_amax()
+            y = sw.spmm_requant(src, N, a, y_amax=left, amax_range=(0, M))
+            ys.append(y); amaxes.append(left)
+            src, a = y, left
+        torch.cuda.synchronize()
+        prev = x0
+        for W, sw, y, left in zip(Ws, sws, ys, amaxes):
+            sw.check()
+            q, s = oracle.requant_int4(prev)
+            prev = y.cpu().numpy()
+            assert oracle.fp16_within_tolerance(prev, oracle.spmm_dense(W, q), s_w, s).all()
+            assert (b.amax_values(left, N) == oracle.absmax_f16(prev).view(np.uint16)).all()
+    finally:
+        for sw in sws:
+            sw.close()
