@@ -432,7 +432,10 @@ __global__ void __launch_bounds__(32 * T, 2) us_spmm_ahead_kernel(const __grid_c
 #pragma unroll
                 for (int i = 0; i < 4; ++i) atomicAdd(al + nt * 128 + i * 32, y[nt][i]);
         }
-        if (!ok) *dead = 1;
+        if (!ok) {
+            *dead = 1;
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");   // (the first step of a tile that is not multiplied)
+        }
         // All decode warps together store the CTA's strips, 32 results of a strip and token group at a time. (With a counter per
         // strip, as where warps end at different times, its last warp stored all of it: 1024 x 1024, N = 8 2.37 us, like this 2.29.)
         asm volatile("bar.sync 1, %0;" ::"n"(32 * W) : "memory");
@@ -531,10 +534,13 @@ __global__ void __launch_bounds__(32 * T, 2) us_spmm_ahead_kernel(const __grid_c
         p.y_amax[64 + 64 * blockIdx.x + threadIdx.x] = threadIdx.x < NT * 8 ? misc[32 + threadIdx.x] : 0u;
         if (blockIdx.x == 0 && threadIdx.x == 0) p.y_amax[0] = gridDim.x;
     }
-    // After a wait ran out: the copies that were issued must land before the CTA exits.
-    if (*dead && warp == 0 && lane == 0)
+    // After a wait ran out: the copies that were issued must land before the CTA exits, those of X among them (the first
+    // helper warp has issued them, whatever became of the others): the next CTA here has its own data in this memory.
+    if (*dead && warp == 0 && lane == 0) {
         for (uint32_t j = 0; j < n; ++j)
             if (issued[j]) mbar_wait_bounded(bar0 + 8u * j, 0u, p.wait_ns_hi);
+        mbar_wait_bounded(b_x, 0u, p.wait_ns_hi);
+    }
 }
 
 }  // namespace us

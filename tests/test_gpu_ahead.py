@@ -75,3 +75,43 @@ def test_dependent_chain_of_decode_ahead_calls(M, K, N):
     finally:
         for sw in sws:
             sw.close()
+
+
+@pytest.mark.parametrize("M,K,fmt,N", [
+    (1024, 4096, None, 8),                    # one K range, activations beside the slots, every tile parked
+    (2048, 16384, None, 16),                  # K in ranges: partial sums and arrivals are left in the workspace
+    (3000, 4096, None, 32),                   # activations over the slots: they are fetched as the wait runs out
+    (1600, 16001, (16, 1024, 2, 1), 11),      # K in ranges, ragged rows
+    (9000, 5120, None, 16),                   # later tiles, for which helpers wait on slots
+    (5003, 3001, (16, 1024, 2, 2), 8),        # two column areas, ragged rows
+])
+def test_withheld_tile_ends_the_call_and_leaves_its_neighbours_alone(M, K, fmt, N):
+    """A tile that is never copied: the call ends with its error, nothing of it (activations still on their way) reaches the
+    CTAs of the calls behind it on the stream, and the handle's next call is correct."""
+    from paper_2608_09291_b200 import binding as b
+    W, V = workloads.make_weight(M, K, 0.5, seed=M + K), workloads.make_weight(4096, 2048, 0.5, seed=5)
+    X, Z = workloads.make_x(K, N, seed=K), workloads.make_x(2048, 8, seed=6)
+    sw, other = b.SparseWeight(W, None, fmt=fmt, max_N=N), b.SparseWeight(V, None, max_N=8)
+    try:
+        ref, ref_other = oracle.spmm_dense(W, X), oracle.spmm_dense(V, Z)
+        Xd, Zd = torch.from_numpy(b.pack_int4(X)).cuda(), torch.from_numpy(b.pack_int4(Z)).cuda()
+        n_tiles = sw.stats["n_tiles"]
+        for position in (0, n_tiles // 2 + 3, n_tiles - 1):
+            b.us_debug_withhold_copy(sw.handle, position, wait_us=2000)
+            sw.spmm(Xd, N)
+            ys = [other.spmm(Zd, 8) for _ in range(4)]
+            torch.cuda.synchronize()
+            assert b.us_last_error(sw.handle) == 7, position      # US_ERR_DEVICE_TIMEOUT
+            assert b.us_last_error(sw.handle) == 0
+            other.check()
+            for y in ys:
+                assert (y.cpu().numpy() == ref_other).all(), position
+            b.us_debug_withhold_copy(sw.handle, -1)
+            for _ in range(2):
+                y = sw.spmm(Xd, N)
+            torch.cuda.synchronize()
+            sw.check()
+            assert (y.cpu().numpy() == ref).all(), position
+    finally:
+        sw.close()
+        other.close()
