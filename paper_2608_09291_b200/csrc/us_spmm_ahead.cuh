@@ -181,7 +181,8 @@ template <bool ANY>
 struct AheadX {
     const uint8_t* from;
     const uint16_t* scale;
-    int64_t end;
+    const uint8_t* tail;   // ANY: a byte past the last 16-byte unit of X, lane h's if it is one of these columns
+    uint8_t* tail_dst;
     uint32_t dst, bytes;
 
     // (of columns k0 .. k0 + cols, k0 a multiple of 128)
@@ -190,12 +191,13 @@ struct AheadX {
         bytes = 0;
         from = nullptr;
         scale = nullptr;
+        tail = nullptr;
+        tail_dst = xs;
         dst = 0;
-        end = 0;
+        const int64_t ldx = ((int64_t)p.K + 1) / 2, whole = (int64_t)p.N * ldx & ~(int64_t)15;   // 16-byte units of X
+        const int64_t row_bytes = min((int64_t)cols / 2, ldx - k0 / 2);
         if (h < p.N) {
-            const int64_t ldx = ((int64_t)p.K + 1) / 2, whole = (int64_t)p.N * ldx & ~(int64_t)15;   // 16-byte units of X
-            const int64_t begin = h * ldx + k0 / 2;
-            end = begin + min((int64_t)cols / 2, ldx - k0 / 2);
+            const int64_t begin = h * ldx + k0 / 2, end = begin + row_bytes;
             const int64_t b = ANY ? begin & ~(int64_t)15 : begin, e = ANY ? min((end + 15) & ~(int64_t)15, whole) : end;
             from = p.X + b;
             dst = smem_u32(xs + h * xstride);
@@ -205,6 +207,15 @@ struct AheadX {
             }
         }
         if (p.fp16_out && h < p.N) scale = p.x_scale + h;
+        if (ANY && whole + h < (int64_t)p.N * ldx) {   // (15 bytes at most)
+            const int64_t at = whole + h;
+            const int row = (int)((uint32_t)at / (uint32_t)ldx);   // (eight ranges at most, each of which fits shared memory: 32 bits hold it)
+            const int64_t begin = row * ldx + k0 / 2;
+            if (at >= begin && at < begin + row_bytes) {
+                tail = p.X + at;
+                tail_dst = xs + row * xstride + (at - (begin & ~(int64_t)15));
+            }
+        }
         // columns past K, which the copies do not write: they meet zero weights, and the sums count them
         if (!ANY && k0 + cols > p.K) {
             const int rest = (k0 + cols - p.K) / 32;   // 16-byte units
@@ -213,15 +224,14 @@ struct AheadX {
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    __device__ __forceinline__ void fetch(const AheadParams& p, uint8_t* xs, int xstride, float* xsc_s, uint32_t b_x, int h)
+    __device__ __forceinline__ void fetch(float* xsc_s, uint32_t b_x, int h)
     {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         if (bytes) bulk_g2s(dst, from, bytes, b_x);
-        if (scale) xsc_s[h] = __half2float(__ushort_as_half(__ldg(scale)));
-        if (ANY && from) {   // the last bytes of X
-            const int64_t whole = (int64_t)p.N * (((int64_t)p.K + 1) / 2) & ~(int64_t)15, b = from - p.X;
-            for (int64_t i = max(b, whole); i < end; ++i) xs[h * xstride + (i - b)] = __ldg(p.X + i);
-        }
+        const unsigned short s = ld16_if(scale, scale != nullptr);
+        const uint8_t last = ANY ? ld8_if(tail, tail != nullptr) : (uint8_t)0;
+        if (scale) xsc_s[h] = __half2float(__ushort_as_half(s));
+        if (ANY && tail) *tail_dst = last;
         __syncwarp();
         if (h == 0) mbar_arrive(b_x);
     }
@@ -498,7 +508,7 @@ __global__ void __launch_bounds__(32 * T, 2) us_spmm_ahead_kernel(const __grid_c
             if (p.x_over) asm volatile("bar.sync 2, %0;" ::"n"(32 * (W + 1)) : "memory");
             AheadX<ANY> x;
             x.prepare(p, kr * p.G * p.K_L, (int)g * p.K_L, xs, xstride, b_x, lane);
-            x.fetch(p, xs, xstride, xsc_s, b_x, lane);
+            x.fetch(xsc_s, b_x, lane);
             if (ANY) {
                 ok = tc_wait_warp(b_x, 0u, p.wait_ns_hi, dead);
                 if (ok) ahead_shift_rows(xs, xstride, p.K, p.N, (int)g * (p.K_L / 32), warp, W + 1, lane);

@@ -221,6 +221,31 @@ __device__ __forceinline__ uint4 lds128(uint32_t a)
     asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
     return v;
 }
+// X and its scales may be written by the stream's earlier work while this kernel is already resident: they are read with
+// ordinary loads, which the dependency wait orders behind that work, not with the read-only kind, which takes for granted that
+// nothing is written while the kernel runs. (Loads past L1 by their kind, ld.global.cg, made the N <= 16 kernels 0.8 us a call
+// slower: 8192 x 8192 12.9 -> 13.7.) Zero where !ok, and no branch: with one every load of a batch waits for the one before
+// (13B-shaped chain, N = 16 72.4 -> 77.7 us a layer).
+__device__ __forceinline__ uint4 ld128_if(const void* a, bool ok)
+{
+    uint4 v;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\tmov.u32 %0, 0;\n\tmov.u32 %1, 0;\n\tmov.u32 %2, 0;\n\tmov.u32 %3, 0;\n\t"
+                 "@p ld.global.v4.u32 {%0,%1,%2,%3}, [%4];\n\t}"
+                 : "=&r"(v.x), "=&r"(v.y), "=&r"(v.z), "=&r"(v.w) : "l"(a), "r"((uint32_t)ok));
+    return v;
+}
+__device__ __forceinline__ unsigned short ld16_if(const uint16_t* a, bool ok)
+{
+    unsigned short v;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\tmov.u16 %0, 0;\n\t@p ld.global.u16 %0, [%1];\n\t}" : "=&h"(v) : "l"(a), "r"((uint32_t)ok));
+    return v;
+}
+__device__ __forceinline__ uint8_t ld8_if(const uint8_t* a, bool ok)
+{
+    unsigned short v;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\tmov.u16 %0, 0;\n\t@p ld.global.u8 %0, [%1];\n\t}" : "=&h"(v) : "l"(a), "r"((uint32_t)ok));
+    return (uint8_t)v;
+}
 __device__ __forceinline__ void mma_s8(int (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
                                        uint32_t a3, uint32_t b0, uint32_t b1)
 {
@@ -303,7 +328,7 @@ __device__ __forceinline__ void stage_x_any(const uint8_t* X, int K, int N, int 
         } else {
             uint4 v = make_uint4(0, 0, 0, 0);
             if (n < N && left > 0) {
-                const uint4 lo = __ldg(reinterpret_cast<const uint4*>(X + a)), hi = __ldg(reinterpret_cast<const uint4*>(X + a + 16));
+                const uint4 lo = *reinterpret_cast<const uint4*>(X + a), hi = *reinterpret_cast<const uint4*>(X + a + 16);
                 uint32_t w[7] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z};
                 if (at & 8) { w[0] = w[2]; w[1] = w[3]; w[2] = w[4]; w[3] = w[5]; w[4] = w[6]; w[5] = hi.w; }
                 if (at & 4) { w[0] = w[1]; w[1] = w[2]; w[2] = w[3]; w[3] = w[4]; w[4] = w[5]; }
@@ -356,14 +381,10 @@ __device__ __forceinline__ void stage_x(const SpmmParams& p, int seg0, int n_seg
 #pragma unroll
         for (int b = 0; b < kBatch; ++b) {
             const int u = u0 + b * blockDim.x;
-            v[b] = make_uint4(0, 0, 0, 0);
-            if (u < total) {
-                const int pi = u / upr, q = u - pi * upr;
-                const int sgl = pi / rows, n = pi - sgl * rows;
-                const int64_t k = (int64_t)(seg0 + sgl) * p.K_L + 32 * q;
-                if (n < p.N && k < p.K)
-                    v[b] = __ldg(reinterpret_cast<const uint4*>(p.X + (int64_t)n * ldx + k / 2));
-            }
+            const int pi = u / upr, q = u - pi * upr;
+            const int sgl = pi / rows, n = pi - sgl * rows;
+            const int64_t k = (int64_t)(seg0 + sgl) * p.K_L + 32 * q;
+            v[b] = ld128_if(p.X + (int64_t)n * ldx + k / 2, u < total && n < p.N && k < p.K);
         }
 #pragma unroll
         for (int b = 0; b < kBatch; ++b) {
@@ -453,7 +474,7 @@ __device__ __forceinline__ void store_rows(const StoreCtx p, const int (&v)[NT][
             if (p.fp16_out) {
                 float sx;
                 if (ScalePre<NT>::kSx && pre && pre->have_sx) sx = __half2float(__ushort_as_half(pre->sx[ScalePre<NT>::kSx ? nt : 0][j & 1]));
-                else sx = __half2float(__ushort_as_half(__ldg(p.x_scale + n)));
+                else sx = __half2float(__ushort_as_half(ld16_if(p.x_scale + n, true)));
                 const float r = (float)v[nt][j] * ((j < 2) ? sw_lo : sw_hi) * sx;
                 const __half h = __float2half_rn(r);
                 reinterpret_cast<__half*>(p.Y)[o] = h;
@@ -897,12 +918,12 @@ __global__ void __launch_bounds__(kMaxThreads<ANY, NT, STAGES, LA, TIMED, CA, W2
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 const int n = nt * 8 + (lane & 3) * 2 + j;
-                spre.sx[nt][j] = n < p.N ? __ldg(p.x_scale + n) : (unsigned short)0;
+                spre.sx[nt][j] = ld16_if(p.x_scale + n, n < p.N);
             }
         spre.have_sx = true;
     }
     const int g_first = (kr_first == n_kr - 1) ? g_last : p.G;   // segments in that range
-    constexpr int kXPre = NT <= 4 && !ANY ? 8 : 0;   // 16-byte units of X a thread prefetches
+    constexpr int kXPre = NT <= 2 && !ANY ? 8 : 0;   // 16-byte units of X a thread prefetches (N <= 32: 4096 x 11008, rows sorted, 15.5 with, 15.3 without)
     const int x_sh = 31 - __clz(p.K_L / 32);   // log2(units per (segment, token)) when a power of two
     const bool x_early = kXPre > 0 && (1 << x_sh) == p.K_L / 32;
     uint4 xpre[kXPre > 0 ? kXPre : 1];
@@ -912,14 +933,10 @@ __global__ void __launch_bounds__(kMaxThreads<ANY, NT, STAGES, LA, TIMED, CA, W2
 #pragma unroll
         for (int b = 0; b < kXPre; ++b) {
             const int u = threadIdx.x + b * blockDim.x;
-            xpre[b] = make_uint4(0, 0, 0, 0);
-            if (u < x_total) {
-                const int pi = u >> x_sh, q = u & (x_upr - 1);
-                const int sgl = pi / (NT * 8), n = pi & (NT * 8 - 1);
-                const int64_t k = (int64_t)(kr_first * p.G + sgl) * p.K_L + 32 * q;
-                if (n < p.N && k < p.K)
-                    xpre[b] = __ldg(reinterpret_cast<const uint4*>(p.X + (int64_t)n * ldx + k / 2));
-            }
+            const int pi = u >> x_sh, q = u & (x_upr - 1);
+            const int sgl = pi / (NT * 8), n = pi & (NT * 8 - 1);
+            const int64_t k = (int64_t)(kr_first * p.G + sgl) * p.K_L + 32 * q;
+            xpre[b] = ld128_if(p.X + (int64_t)n * ldx + k / 2, u < x_total && n < p.N && k < p.K);
         }
     }
     uint32_t phase = 0;   // bit s = parity to wait for on stage s

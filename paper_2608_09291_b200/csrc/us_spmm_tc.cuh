@@ -222,10 +222,10 @@ inline __device__ __noinline__ uint4 load_x_tail(const uint8_t* src, int left)
     }
     return make_uint4(o[0], o[1], o[2], o[3]);
 }
-__device__ __forceinline__ uint4 ldg_now(const uint8_t* a)
+__device__ __forceinline__ uint4 ld_now(const uint8_t* a)
 {
     uint4 v;
-    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(a));
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(a));
     return v;
 }
 template <bool ANY>
@@ -236,10 +236,10 @@ __device__ __forceinline__ UnitX load_x32(const TcParams& p, int64_t ldx, int n,
     if (n >= p.N || k >= p.K) return u;
     const int64_t b = (int64_t)n * ldx + (k >> 1);
     if (!ANY) {
-        u.lo = ldg_now(p.X + b);
+        u.lo = ld_now(p.X + b);
     } else if (p.K - k >= 32 && (b & ~(int64_t)15) + 32 <= (int64_t)p.N * ldx) {
-        u.lo = ldg_now(p.X + (b & ~(int64_t)15));
-        u.hi = ldg_now(p.X + (b & ~(int64_t)15) + 16);
+        u.lo = ld_now(p.X + (b & ~(int64_t)15));
+        u.hi = ld_now(p.X + (b & ~(int64_t)15) + 16);
     } else {
         u.lo = load_x_tail(p.X + b, p.K - k);
     }
@@ -668,7 +668,7 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
         asm volatile("griddepcontrol.wait;" ::: "memory");
         // (by the warps of the first stage: its barriers hand the scales on to the decode warps, as they do the sums)
         if (p.fp16_out && c0 == 0)
-            for (int i = lane + 32 * g0; i < p.N; i += 32 * P) xsc_s[i] = __half2float(__ushort_as_half(__ldg(p.x_scale + i)));
+            for (int i = lane + 32 * g0; i < p.N; i += 32 * P) xsc_s[i] = __half2float(__ushort_as_half(p.x_scale[i]));
         if (c0 < W)
         for (int c = c0; c < total; c += W) {
             while (st >= n_stage) {

@@ -203,3 +203,33 @@ def test_half_sm_plan_counts_the_registers_of_every_kernel(b, M, K, fmt, warps):
             _check_requant_call(b, sw, W, s_w, workloads.make_x_f16(K, 8, seed=2), 8, 0, M)
     finally:
         sw.close()
+
+
+@pytest.mark.parametrize("M,K,fmt,N", [(1024, 1024, None, 8), (2048, 4096, None, 16), (2048, 2048, None, 32),   # resident beside two launches
+                                       (24000, 1024, None, 8),                                                  # half an SM, the other kernel
+                                       (1600, 4001, None, 5), (4001, 2500, (16, 512, 2, 2), 3),                 # ragged rows
+                                       (2048, 4096, None, 64), (1100, 4099, None, 40)])                         # the tensor-memory kernel
+def test_activations_are_written_while_the_call_is_resident(b, M, K, fmt, N):
+    """Chained calls on one handle, back to back: the quantiser writes the same buffer of codes and steps again for every one
+    of them, while the product that reads it is already resident and the one before has just read the old ones."""
+    W = workloads.make_weight(M, K, 0.5, seed=M + K)
+    s_w = workloads.make_chain_weight_scales(M, K, 5)
+    sw = b.SparseWeight(W, s_w, fmt=fmt, max_N=N)
+    try:
+        xs = [workloads.make_x_f16(K, N, seed=10 + i) * np.float16(2.0 ** (i % 5 - 2)) for i in range(6)]
+        Xd = [torch.from_numpy(x).cuda() for x in xs]
+        amax = [b.absmax_f16(x) for x in Xd]
+        ref = []
+        for x, a in zip(Xd, amax):
+            torch.cuda.synchronize()
+            ref.append(sw.spmm_requant(x, N, a))
+        torch.cuda.synchronize()
+        ys = [sw.spmm_requant(x, N, a) for _ in range(4) for x, a in zip(Xd, amax)]
+        torch.cuda.synchronize()
+        sw.check()
+        for i, y in enumerate(ys):
+            assert torch.equal(y, ref[i % 6]), i
+        q, st = oracle.requant_int4(xs[0])
+        assert oracle.fp16_within_tolerance(ref[0].cpu().numpy(), oracle.spmm_dense(W, q), s_w, st, rel=2e-3).all()
+    finally:
+        sw.close()
