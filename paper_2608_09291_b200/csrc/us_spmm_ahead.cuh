@@ -522,7 +522,8 @@ __global__ void __launch_bounds__(32 * T, 2) us_spmm_ahead_kernel(const __grid_c
                     const uint32_t t = tile_index(j);
                     o0 = __ldg(p.item_off + t); o1 = __ldg(p.item_off + t + 1);
                 }
-                ok = tc_wait_warp(b_e + 8u * (j - (uint32_t)p.n_slots), 0u, p.wait_ns_hi, dead);
+                // (the slot of a tile that is not parked comes free behind the MMAs)
+                ok = tc_wait_warp(b_e + 8u * (j - (uint32_t)p.n_slots), 0u, p.wait_ns_hi, dead, j >= (uint32_t)(p.n_slots + p.parked));
                 if (!ok) break;
                 if (lane == 0) {
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

@@ -82,10 +82,12 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 // Bounded wait for a whole warp, with one verdict for all its lanes (warp-wide tcgen05 instructions follow); gives up
-// too when another warp of the CTA did.
-__device__ __forceinline__ bool tc_wait_warp(uint32_t bar, uint32_t parity, uint32_t limit_hi, volatile uint32_t* dead)
+// too when another warp of the CTA did. after: the wait cannot end before the stream's earlier work has, whose time is not
+// counted, however long it runs with this kernel resident.
+__device__ __forceinline__ bool tc_wait_warp(uint32_t bar, uint32_t parity, uint32_t limit_hi, volatile uint32_t* dead, bool after = false)
 {
     if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if (after) asm volatile("griddepcontrol.wait;" ::: "memory");
     const uint64_t t0 = global_timer_ns();
     const uint32_t nap = limit_hi < 64u ? 1000u : 20000u;
 #pragma unroll 1
@@ -96,9 +98,10 @@ __device__ __forceinline__ bool tc_wait_warp(uint32_t bar, uint32_t parity, uint
     return false;
 }
 // Waits, bounded, until a counter in shared memory has reached n.
-__device__ __forceinline__ bool tc_wait_count(volatile uint32_t* count, uint32_t n, uint32_t limit_hi, volatile uint32_t* dead)
+__device__ __forceinline__ bool tc_wait_count(volatile uint32_t* count, uint32_t n, uint32_t limit_hi, volatile uint32_t* dead, bool after)
 {
     if (__all_sync(0xffffffffu, *count >= n)) return true;
+    if (after) asm volatile("griddepcontrol.wait;" ::: "memory");
     const uint64_t t0 = global_timer_ns();
 #pragma unroll 1
     for (uint32_t it = 0; it < (1u << 24); ++it) {
@@ -467,9 +470,10 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
         constexpr int WPS = CA == 1 ? 2 : 1;  // mask words per stage
 
         // The warp's i-th tile is in its slot: another warp may not even have had its own tile there yet, and the barrier's
-        // parity alone could not tell, so wait for the pass to begin, then for its copy.
+        // parity alone could not tell, so wait for the pass to begin, then for its copy. (From the second pass on that may take MMAs
+        // in another warp's way, and those X.)
         auto wait_tile = [&](uint32_t i) {
-            ok = tc_wait_count(issued + slot, pass + 1u, p.wait_ns_hi, dead) && tc_wait_warp(b_w + 8u * slot, pass & 1u, p.wait_ns_hi, dead);
+            ok = tc_wait_count(issued + slot, pass + 1u, p.wait_ns_hi, dead, pass > 0) && tc_wait_warp(b_w + 8u * slot, pass & 1u, p.wait_ns_hi, dead);
             if (ok && i == 0 && lane > 0 && tile_first != kNone) copy_tile(tile_first, of0, of1, t_first);
             return ok;
         };
@@ -514,7 +518,7 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
             for (int s = 0; s < SR; ++s) { cw0[s] = lds32(a0 + 128u * s); cw1[s] = lds32(a0 + 128u * (SR + s)); }
             const int n_here = min(n_stage - st, left);
             for (int j = 0; j < n_here; ++j) {
-                ok = tc_wait_warp(b_ae + 8u * (o * kTcAStages + as), a_par, p.wait_ns_hi, dead);
+                ok = tc_wait_warp(b_ae + 8u * (o * kTcAStages + as), a_par, p.wait_ns_hi, dead, true);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t dst = tm_a + 64u * as;
@@ -601,7 +605,7 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
             const int n_here = min(n_stage - st, left);
 #pragma unroll 1
             for (int j = 0; j < n_here && ok; ++j) {
-                ok = tc_wait_warp(b_ae + 8u * (o * kTcAStages + as), a_par, p.wait_ns_hi, dead);
+                ok = tc_wait_warp(b_ae + 8u * (o * kTcAStages + as), a_par, p.wait_ns_hi, dead, true);
                 if (!ok) break;
                 if (lane == 0) mbar_arrive(b_af + 8u * (o * kTcAStages + as));
                 if (++as == kTcAStages) { as = 0; a_par ^= 1u; }
@@ -626,7 +630,7 @@ __global__ void __launch_bounds__(TcShape<OCT>::kThreads, 1) us_spmm_tc_kernel(c
         for (int s = 0; s < total && ok; ++s) {
             const bool half = odd && st == n_stage - 1;   // the tile's last stage holds one mask word only
             const bool last = --left_block == 0 || s == total - 1;   // end of the run of this row block
-            ok = tc_wait_warp(b_xf + 8u * xst, x_par, p.wait_ns_hi, dead);
+            ok = tc_wait_warp(b_xf + 8u * xst, x_par, p.wait_ns_hi, dead, true);
             const uint64_t b = bd0 + (uint64_t)((xst * x_stage_bytes) >> 4);
 #pragma unroll
             for (int o = 0; o < OCT; ++o) {

@@ -115,3 +115,29 @@ def test_withheld_tile_ends_the_call_and_leaves_its_neighbours_alone(M, K, fmt, 
     finally:
         sw.close()
         other.close()
+
+
+def test_time_of_earlier_work_is_not_counted_against_a_wait():
+    """Two calls that take two seconds each by giving up (test hook), a third behind them, resident from the start: its helpers
+    wait for slots that come free behind its own MMAs, four seconds later, with a limit of two for what is its own."""
+    from paper_2608_09291_b200 import binding as b
+    M, K, N = 148 * 96, 5120, 16           # six strips, 30 tiles to each of 148 CTAs, of which 16 are parked; seven slots
+    W, X = workloads.make_weight(M, K, 0.5, seed=3), workloads.make_x(K, N, seed=3)
+    sws = [b.SparseWeight(W, None, max_N=N) for _ in range(3)]
+    try:
+        info = b.us_launch_info(sws[0].handle, N)
+        if info["grid"] != 148:
+            pytest.skip("laid out for 148 SMs")
+        Xd = torch.from_numpy(b.pack_int4(X)).cuda()
+        ys = [torch.empty((N, M), dtype=torch.int32, device="cuda") for _ in sws]
+        torch.cuda.synchronize()
+        b.us_debug_withhold_copy(sws[0].handle, 0, wait_us=2_000_000)      # a tile that is decoded ahead
+        b.us_debug_withhold_copy(sws[1].handle, 29, wait_us=2_000_000)     # one whose turn comes when the first call has ended
+        for sw, y in zip(sws, ys):
+            sw.spmm(Xd, N, out=y)
+        torch.cuda.synchronize()
+        assert [b.us_last_error(sw.handle) for sw in sws] == [7, 7, 0]     # US_ERR_DEVICE_TIMEOUT where a tile was withheld
+        assert (ys[2].cpu().numpy() == oracle.spmm_dense(W, X)).all()
+    finally:
+        for sw in sws:
+            sw.close()
