@@ -139,6 +139,12 @@ us_status us_get_row_order(const us_handle* h, int32_t* perm_out);
  * arrival counters belong to the handle and are left zeroed by each call.
  * The handle's device must be the current device. After a call that us_last_error reports as
  * failed, the workspace has been cleared again and the handle can be used as before.
+ * The kernel is launched with programmatic stream serialization: its CTAs may start, and take shared memory and up to 512
+ * columns of tensor memory, while the kernel before it on the stream still runs, and they hold them until that kernel has
+ * ended. A kernel that lets its dependents start (griddepcontrol.launch_dependents) and allocates tensor memory of its own
+ * must therefore allocate first, as this library's do: a later allocation could wait for columns that are held for the end
+ * of the very kernel that waits. Where a program runs other such kernels before us_spmm, the environment variable US_PDL=0
+ * (read once per process) launches this library's the ordinary way.
  * Errors: INVALID_ARG (also: another device is current), UNSUPPORTED (host-only handle, or a
  * format no kernel reads), CUDA.
  */
