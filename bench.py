@@ -496,9 +496,7 @@ def report(out, rows):
 def kernel_label(binding, handle, N):
     """The dominant (only) kernel of a call and its launch geometry."""
     g = binding.us_launch_info(handle, N)
-    # (two or three octets; no other block is as wide. Half an SM's shared memory: all but a few shapes of one segment.)
-    name = ("us_spmm_tc_kernel" if g["block"] in (800, 896) else
-            "us_spmm_ahead_kernel" if g["smem_bytes"] <= 114 * 1024 else "us_spmm_kernel")
+    name = binding.us_launch_kernel(handle, N)
     return (f"{name} (n-tiles {max(1, 1 << (max(N, 1) - 1).bit_length()) // 8 or 1}, {g['grid']} CTAs x "
             f"{g['block'] // 32} warps, {g['smem_bytes']} B shared memory)")
 

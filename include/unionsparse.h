@@ -268,6 +268,11 @@ int64_t us_spmm_bytes(const us_handle* h, int32_t N, int32_t fp16_out);
 us_status us_launch_info(const us_handle* h, int32_t N, int32_t* grid, int32_t* block,
                          int32_t* smem_bytes);
 
+/* The kernel of that launch: "us_spmm_kernel", "us_spmm_ahead_kernel" or "us_spmm_tc_kernel"; NULL where us_launch_info
+ * returns an error. (Chained calls, and calls while the stage timers are on, may run on us_spmm_kernel where this names
+ * us_spmm_ahead_kernel.) */
+const char* us_launch_kernel(const us_handle* h, int32_t N);
+
 const char* us_status_string(us_status s);
 
 #ifdef __cplusplus

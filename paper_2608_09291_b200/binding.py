@@ -28,7 +28,8 @@ US_ENCODE_W2 = 8
 
 EXPORTS = ["us_encode", "us_get_stats", "us_decode", "us_get_row_order", "us_spmm", "us_spmm_static_scratch",
            "us_spmm_requant", "us_absmax_f16", "us_quantize_f16",
-           "us_last_error", "us_debug_withhold_copy", "us_stage_timers", "us_destroy", "us_spmm_bytes", "us_launch_info", "us_status_string"]
+           "us_last_error", "us_debug_withhold_copy", "us_stage_timers", "us_destroy", "us_spmm_bytes", "us_launch_info", "us_launch_kernel",
+           "us_status_string"]
 
 
 class us_format(ctypes.Structure):
@@ -63,6 +64,8 @@ _lib.us_debug_withhold_copy.argtypes = [_vp, ctypes.c_int64, ctypes.c_int64]
 _lib.us_spmm_bytes.argtypes = [_vp, ctypes.c_int32, ctypes.c_int32]
 _lib.us_spmm_bytes.restype = ctypes.c_int64
 _lib.us_launch_info.argtypes = [_vp, ctypes.c_int32] + [ctypes.POINTER(ctypes.c_int32)] * 3
+_lib.us_launch_kernel.argtypes = [_vp, ctypes.c_int32]
+_lib.us_launch_kernel.restype = ctypes.c_char_p
 _lib.us_status_string.argtypes = [ctypes.c_int]
 _lib.us_status_string.restype = ctypes.c_char_p
 
@@ -220,6 +223,14 @@ def us_launch_info(h: int, N: int) -> dict:
     _check(_lib.us_launch_info(h, int(N), ctypes.byref(g), ctypes.byref(b), ctypes.byref(s)),
            "us_launch_info")
     return {"grid": g.value, "block": b.value, "smem_bytes": s.value}
+
+
+def us_launch_kernel(h: int, N: int) -> str:
+    """Name of the kernel that us_spmm launches for N tokens."""
+    name = _lib.us_launch_kernel(h, int(N))
+    if name is None:
+        us_launch_info(h, N)   # (raises with the reason)
+    return name.decode()
 
 
 def pack_int4(X: np.ndarray) -> np.ndarray:

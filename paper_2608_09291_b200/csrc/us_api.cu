@@ -957,6 +957,13 @@ us_status us_launch_info(const us_handle* h, int32_t N, int32_t* grid, int32_t* 
     return US_OK;
 }
 
+const char* us_launch_kernel(const us_handle* h, int32_t N)
+{
+    if (us_launch_info(h, N, nullptr, nullptr, nullptr) != US_OK) return nullptr;
+    const int cls = class_of(nt_for(N));
+    return h->tc[(N + 7) / 8].ok ? "us_spmm_tc_kernel" : cls <= 2 && h->ahead[cls].ok ? "us_spmm_ahead_kernel" : "us_spmm_kernel";
+}
+
 us_status us_spmm(us_handle* h, const void* X, int32_t N, const void* x_scale, void* Y, void* stream)
 {
     const us_status s = check_spmm_args(h, X, N, x_scale, Y);

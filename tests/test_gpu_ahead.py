@@ -1,5 +1,10 @@
 """The decode-ahead kernel at its edges: one tile and many rounds per warp, tiles parked and not, activations over the tile
 slots and beside them, K cut in ranges (sums through the workspace), ragged rows, every format, chained calls among plain ones."""
+import os
+import subprocess
+import sys
+from pathlib import Path
+
 import numpy as np
 import pytest
 
@@ -8,6 +13,7 @@ from paper_2608_09291_b200 import workloads
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
+ROOT = Path(__file__).resolve().parent.parent
 
 
 # (half an SM's shared memory, and the threads: 384 and 512 at N <= 8 and N <= 16, 320 with two column areas and at N <= 32)
@@ -34,6 +40,7 @@ def test_decode_ahead(M, K, fmt, w2, N, block):
     sw = b.SparseWeight(W, s_w, fmt=fmt, max_N=N, flags=b.US_ENCODE_W2 if w2 else 0)
     try:
         info = b.us_launch_info(sw.handle, N)
+        assert b.us_launch_kernel(sw.handle, N) == "us_spmm_ahead_kernel"
         assert info["block"] == block and info["smem_bytes"] <= 114 * 1024, info
         ref = oracle.spmm_dense(W, X)
         Xd, sd = torch.from_numpy(b.pack_int4(X)).cuda(), torch.from_numpy(s_x).cuda()
@@ -77,22 +84,23 @@ def test_dependent_chain_of_decode_ahead_calls(M, K, N):
             sw.close()
 
 
-@pytest.mark.parametrize("M,K,fmt,N", [
+WITHHELD = [
     (1024, 4096, None, 8),                    # one K range, activations beside the slots, every tile parked
     (2048, 16384, None, 16),                  # K in ranges: partial sums and arrivals are left in the workspace
     (3000, 4096, None, 32),                   # activations over the slots: they are fetched as the wait runs out
     (1600, 16001, (16, 1024, 2, 1), 11),      # K in ranges, ragged rows
     (9000, 5120, None, 16),                   # later tiles, for which helpers wait on slots
     (5003, 3001, (16, 1024, 2, 2), 8),        # two column areas, ragged rows
-])
-def test_withheld_tile_ends_the_call_and_leaves_its_neighbours_alone(M, K, fmt, N):
-    """A tile that is never copied: the call ends with its error, nothing of it (activations still on their way) reaches the
-    CTAs of the calls behind it on the stream, and the handle's next call is correct."""
+]
+
+
+def run_withheld(M, K, fmt, N, kernel):
     from paper_2608_09291_b200 import binding as b
     W, V = workloads.make_weight(M, K, 0.5, seed=M + K), workloads.make_weight(4096, 2048, 0.5, seed=5)
     X, Z = workloads.make_x(K, N, seed=K), workloads.make_x(2048, 8, seed=6)
     sw, other = b.SparseWeight(W, None, fmt=fmt, max_N=N), b.SparseWeight(V, None, max_N=8)
     try:
+        assert b.us_launch_kernel(sw.handle, N) == kernel
         ref, ref_other = oracle.spmm_dense(W, X), oracle.spmm_dense(V, Z)
         Xd, Zd = torch.from_numpy(b.pack_int4(X)).cuda(), torch.from_numpy(b.pack_int4(Z)).cuda()
         n_tiles = sw.stats["n_tiles"]
@@ -115,6 +123,22 @@ def test_withheld_tile_ends_the_call_and_leaves_its_neighbours_alone(M, K, fmt, 
     finally:
         sw.close()
         other.close()
+
+
+@pytest.mark.parametrize("M,K,fmt,N", WITHHELD)
+def test_withheld_tile_ends_the_call_and_leaves_its_neighbours_alone(M, K, fmt, N):
+    """A tile that is never copied: the call ends with its error, nothing of it (activations still on their way) reaches the
+    CTAs of the calls behind it on the stream, and the handle's next call is correct."""
+    run_withheld(M, K, fmt, N, "us_spmm_ahead_kernel")
+
+
+def test_withheld_tile_of_the_other_kernel():
+    """The same shapes on us_spmm_kernel: sums in shared memory, K in ranges, half an SM and all of it. (A child process: which
+    kernels may run is read once.)"""
+    code = ("import sys; sys.path[:0] = ['.', 'tests']; import test_gpu_ahead as t\n"
+            "for case in t.WITHHELD + [(24000, 1024, None, 8)]: t.run_withheld(*case, 'us_spmm_kernel')")
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, US_AHEAD="0", US_TC="0"), capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stdout[-1500:] + r.stderr[-1500:]
 
 
 def test_time_of_earlier_work_is_not_counted_against_a_wait():
