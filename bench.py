@@ -501,10 +501,11 @@ def kernel_label(binding, handle, N):
             f"{g['block'] // 32} warps, {g['smem_bytes']} B shared memory)")
 
 
-# Measured DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch, from the ncu
-# captures of the same kernel build (one launch each; commands in the capture summaries).
-TRAFFIC_BYTES_PER_LAUNCH = 7_961_856          # 4096x4096, s = 0.5, N = 8, fp16: 7.9619 MB read, 0 written
-TRAFFIC_BYTES_PER_LAUNCH_LARGE = 101_812_736  # 28672x8192, s = 0.6, N = 8, int32: 98.01 MB read + 3.81 MB written
+# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch, where an ncu capture of the kernel that runs says it.
+# The headline's kernel, us_spmm_ahead_kernel, has none; us_spmm_kernel's of an earlier build on the large shape (28672x8192,
+# s = 0.6, N = 8, int32) was 98.01 MB read + 3.81 MB written, of the same stored bytes.
+TRAFFIC_BYTES_PER_LAUNCH = None
+TRAFFIC_BYTES_PER_LAUNCH_LARGE = 101_812_736
 
 
 def sweep(binding, torch, workloads, l2, peak_gbs):
