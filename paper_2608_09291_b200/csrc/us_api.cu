@@ -125,8 +125,8 @@ constexpr int kCoresidentTiles = 16;         // most tiles per CTA for the half-
 constexpr int kCoresidentK = 5120;           // ... and widest K: its few threads stage all of X (N = 8, half SM / whole: 2304 x 8192 6.8 / 5.9 us,
                                              // 2304 x 6144 6.4 / 5.6, 4096 x 4096 4.6 / 5.6)
 // The same where K is not a multiple of 32 and staging takes a thread one unit at a time (half SM / whole: N = 8
-// 1500 x 4500 6.7 / 5.8 (N = 1, which shares the plan, loses by it, 5.3 / 5.6), 2304 x 4500 7.3 / 6.5, 2304 x 3000 5.5 / 5.4; N = 1 there 4.4 / 5.2; N = 16 5003 x 3001 9.0 / 8.0).
-int64_t coresident_K(int64_t K, int nt) { return K % 32 == 0 ? kCoresidentK : nt == 1 ? 3072 : 2048; }
+// 1500 x 4500 6.7 / 5.8 (N = 1, which shares the plan, loses by it, 5.3 / 5.6), 2304 x 4500 7.3 / 6.5, 2304 x 3000 5.5 / 5.4; N = 1 there 4.4 / 5.2).
+int64_t coresident_K(int64_t K) { return K % 32 == 0 ? kCoresidentK : 3072; }
 constexpr int kHalfSmBytes = 228 * 1024 / 2 - 1024 - 512;   // shared memory of a half-SM CTA: 228 KB per SM, 1 KB reserved per CTA
 
 // Segments per K range for an N class. The int8 activations of one K range live in shared memory
@@ -272,16 +272,17 @@ bool plan_launch(const us_handle* h, int N, LaunchGeom* g)
     for (size_t c = 0; c + 1 < h->cta_begin[g->cls].size(); ++c)
         most = std::max<int64_t>(most, (int64_t)h->cta_begin[g->cls][c + 1] - h->cta_begin[g->cls][c]);
     int fixed = fixed_base + 32 * stages * 8;
-    // (us_spmm_ahead_kernel takes nearly all of these calls; what is left for this plan is said at build_ahead_plan.)
-    if (coresident_knob() && g->nt == 1 && most <= kCoresidentTiles && stages_knob() == 0 && h->host.Kp <= coresident_K(h->host.K, g->nt)) {
+    // (us_spmm_ahead_kernel takes nearly all of these calls; what is left for this plan is said at build_ahead_plan, and tiles of
+    // 2048 columns and more. At N = 9 .. 16 those leave too few slots, but at 90 % sparsity, and there half an SM is no better: 4096 x 4096
+    // 7.3 / 7.6, 2048 x 4096 8.7 / 7.2, 3072 x 4096 9.1 / 7.4.)
+    if (coresident_knob() && g->nt == 1 && most <= kCoresidentTiles && stages_knob() == 0 && h->host.Kp <= coresident_K(h->host.K)) {
         const int half = kHalfSmBytes;
         const int fixed8 = fixed_for(8) + 32 * 8;
         // (two column areas: 10 at most; 3001 x 2000, N = 8 4.10 us with 10, 4.18 with 12)
         int w = std::min({half_sm_warps(h, g->cls, s_local > 0, g->xp && s_local > 0), h->host.fmt.C_A == 2 ? 10 : 16, max_warps()});
         while (w >= 8 && fixed8 + w * (int)g->slot_bytes > half) --w;
-        // (only if every tile of the CTA finds a warp at once: 5120 x 5120 at 70 % sparsity, N = 16, has 11 tiles per CTA
-        // and room for 8 half-SM warps: 9.9 us against 8.9 with 16 warps on the whole SM; 1500 x 6000 has 12 and room for 10:
-        // N = 8 8.6 against 6.0)
+        // (only if every tile of the CTA finds a warp at once: 1500 x 6000 has 12 and room for 10: N = 8 8.6 us against 6.0 with
+        // 16 warps on the whole SM)
         if (w >= 8 && w >= most) { stages = 1; lut_rep = 8; warps = w; fixed = fixed8; }
     }
     g->stages = stages;
