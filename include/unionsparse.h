@@ -263,15 +263,18 @@ us_status us_destroy(us_handle* h);
 /* Algorithmic bytes one us_spmm call moves: encoded W as stored + X + Y + scales. */
 int64_t us_spmm_bytes(const us_handle* h, int32_t N, int32_t fp16_out);
 
-/* Launch geometry of the next us_spmm(N): CTAs, threads per CTA, dynamic shared memory. For a host-only handle, what a
- * handle on a B200 would have. */
+/* Launch geometry of us_spmm(N): CTAs, threads per CTA, dynamic shared memory. For a host-only handle, what a
+ * handle on a B200 would have. (Some handles have a second plan for calls right behind one whose CTAs take half an SM,
+ * see us_launch_kernel; this is the first.) */
 us_status us_launch_info(const us_handle* h, int32_t N, int32_t* grid, int32_t* block,
                          int32_t* smem_bytes);
 
-/* The kernel of that launch: "us_spmm_kernel", "us_spmm_ahead_kernel" or "us_spmm_tc_kernel"; NULL where us_launch_info
- * returns an error. (Chained calls, and calls while the stage timers are on, may run on us_spmm_kernel where this names
- * us_spmm_ahead_kernel.) */
-const char* us_launch_kernel(const us_handle* h, int32_t N);
+/* The kernel that the calling thread's next us_spmm(N) on the stream would launch: "us_spmm_kernel", "us_spmm_ahead_kernel"
+ * or "us_spmm_tc_kernel"; NULL where us_launch_info returns an error. It depends on the handle and, for some, on the
+ * thread's calls before it: one or two behind a call on the same stream whose CTAs take half an SM do so, too, and start
+ * beside those (the result is the same either way). While the stage timers are on, us_spmm_kernel runs where this names
+ * us_spmm_ahead_kernel; chained calls may, too. */
+const char* us_launch_kernel(const us_handle* h, int32_t N, void* stream);
 
 const char* us_status_string(us_status s);
 

@@ -64,7 +64,7 @@ _lib.us_debug_withhold_copy.argtypes = [_vp, ctypes.c_int64, ctypes.c_int64]
 _lib.us_spmm_bytes.argtypes = [_vp, ctypes.c_int32, ctypes.c_int32]
 _lib.us_spmm_bytes.restype = ctypes.c_int64
 _lib.us_launch_info.argtypes = [_vp, ctypes.c_int32] + [ctypes.POINTER(ctypes.c_int32)] * 3
-_lib.us_launch_kernel.argtypes = [_vp, ctypes.c_int32]
+_lib.us_launch_kernel.argtypes = [_vp, ctypes.c_int32, _vp]
 _lib.us_launch_kernel.restype = ctypes.c_char_p
 _lib.us_status_string.argtypes = [ctypes.c_int]
 _lib.us_status_string.restype = ctypes.c_char_p
@@ -225,9 +225,9 @@ def us_launch_info(h: int, N: int) -> dict:
     return {"grid": g.value, "block": b.value, "smem_bytes": s.value}
 
 
-def us_launch_kernel(h: int, N: int) -> str:
-    """Name of the kernel that us_spmm launches for N tokens."""
-    name = _lib.us_launch_kernel(h, int(N))
+def us_launch_kernel(h: int, N: int, stream: int | None = None) -> str:
+    """Name of the kernel that this thread's next us_spmm for N tokens on the stream would launch."""
+    name = _lib.us_launch_kernel(h, int(N), stream)
     if name is None:
         us_launch_info(h, N)   # (raises with the reason)
     return name.decode()

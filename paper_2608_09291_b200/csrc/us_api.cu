@@ -53,7 +53,9 @@ struct TcPlan {
 
 // The same for us_spmm_ahead_kernel, per N class.
 struct AheadPlan {
-    bool ok = false, chain_ok = false;   // chain_ok: chained calls, too
+    bool ok = false;
+    bool always = false;                 // whatever ran before; otherwise only behind a call of half an SM (ahead_plan)
+    bool chain_ok = false;               // chained calls, too
     int threads = 0, smem = 0;
     Kernel plain, chained;
     us::AheadParams p{};
@@ -471,7 +473,7 @@ void build_tc_plan(us_handle* h, int ng)
     for (size_t c = 0; c + 1 < h->cta_begin[cls].size(); ++c) most = std::max(most, h->cta_begin[cls][c + 1] - h->cta_begin[cls][c]);
     const double mean = (double)stages / (double)n_cta, share = (double)most * n_stage / 16;
     const double uneven = (double)hm.max_item_bytes * (double)hm.n_items / (double)std::max<uint64_t>(1, hm.blob_bytes);   // largest tile / average
-    const bool better = cls <= 2 && h->ahead[cls].ok ? false
+    const bool better = cls <= 2 && h->ahead[cls].always ? false
                         : ng > 4                     ? hm.Kp >= 2048 || mean >= 0.8
                         : h->s_local[cls] == 0       ? mean >= 1.5
                         : ng <= 2                    ? mean >= 10 && 5.9 + 1.08 * share > 9.4 + 0.9 * mean
@@ -532,6 +534,12 @@ void build_tc_plan(us_handle* h, int ng)
 //   N <= 32: where all tiles are parked (4096 x 4096 8.7 / 6.4, 5120 x 5120 11.6 / 9.3; 11008 x 4096, 20 tiles, 13.7 / 16.9).
 //   One segment to a strip and more than 8 tiles at N <= 8: not (24000 x 1024, 11 tiles, 4.9 / 5.6: the other half-SM plan has a warp
 //     for every tile).
+//   Otherwise, up to 64 tiles and with five slots at least: only behind calls of half an SM (ahead_plan), but at N = 9 .. 16 with two
+//     column areas. Alone these calls are slower so (27648 x 5120, N = 16 20.0 / 21.3 at .7, with five slots 21.1 / 25.8 at .5; 8192 x 8192
+//     12.9 / 13.5), among others the change of kind costs more: 13B-shaped layer, [Q;K;V] and [gate;up] stacked, N = 16, s = .3, .5, .6, .7,
+//     all as they are alone / these behind the others: 72.4, 69.4, 68.4, 65.5 / 64.3, 60.8, 56.5, 53.8; seven products at .7 77.3 / 61.4; N = 8
+//     stacked at .6, .7 57.4, 55.3 / 46.1, 44.6, 2 x 2 format at .5 54.0 / 45.7, INT2 50.6 / 42.0 (N = 16: 59.5 / 77.1, 50.5 / 68.4). With a
+//     foreign kernel between all of these, which the library cannot know, .5 77.9 / 83.9, .7 76.1 / 74.7.
 //   Chained calls: where all tiles are parked. The quantiser between two products takes the time in which later tiles would
 //     have been decoded (13B-shaped chain, all half 80, like this 72, all whole 74).
 void build_ahead_plan(us_handle* h, int cls)
@@ -551,13 +559,14 @@ void build_ahead_plan(us_handle* h, int cls)
     if (hm.n_items > (int64_t)us::kAheadMaxTiles * h->sm_count || hm.n_items * hm.fmt.K_L > 64 * 1024 * (int64_t)h->sm_count) return;
     int64_t most = 0;
     int warps = 8;
-    for (int64_t r = 1; r <= 8 && p.n_ranges == 0; ++r) {
+    int least = 6;   // tile slots
+    auto lay = [&](int64_t r) {
         const int64_t G = (hm.n_segs + r - 1) / r;
-        if ((hm.n_segs + G - 1) / G != r) continue;
+        if ((hm.n_segs + G - 1) / G != r) return;
         const int64_t x = (int64_t)nt * 8 * us::ahead_x_row((int)std::min<int64_t>(G * hm.fmt.K_L, 1 << 20), hm.K % 32 != 0);
         // (no schedule is laid for ranges that cannot do: where not all can be parked, X and six slots beside it)
         const bool all_parked = hm.n_items <= 4 * places * (int64_t)h->sm_count;
-        if (us::ahead_fixed_smem(nt, 1) + x + (all_parked ? 0 : 6 * (int64_t)p.slot_bytes) > kHalfSmBytes) continue;
+        if (us::ahead_fixed_smem(nt, 1) + x + (all_parked ? 0 : least * (int64_t)p.slot_bytes) > kHalfSmBytes) return;
         const Schedule& sc = schedule(h, (int)G);
         const std::vector<uint32_t>& begin = sc.begin;
         const int strips = sc.strips;
@@ -568,32 +577,46 @@ void build_ahead_plan(us_handle* h, int cls)
             most = std::max<int64_t>(most, (int64_t)begin[c + 1] - begin[c]);
             one_range = one_range && begin[c] / (hm.n_strips * G) == (begin[c + 1] - 1) / (hm.n_strips * G);
         }
-        if (!one_range || most > us::kAheadMaxTiles) continue;
+        if (!one_range || most > us::kAheadMaxTiles) return;
         // Twelve decode warps and three that copy where 64 registers a thread do and there is work for them (with eight: 11008 x 4096,
         // N = 8 7.05, with twelve 6.6; 13824 x 5120, N = 16 13.5 / 12.9; 2048 x 2048, N = 8 the other way, 2.5 / 2.6). One copying warp less
         // is slower (20480 x 5120, N = 16 20.5 with one, 18.5 with three): each copy takes the issuing warp some 500 cycles.
         const bool wide = plain && (nt == 1 ? hm.K > kCoresidentK || most > 16 : nt == 2);
         warps = wide ? 12 : 8;
         pl.threads = 32 * (wide ? 16 : nt == 1 && plain ? 12 : nt <= 2 && most > 16 ? 12 : 10);
-        if (4 * places < warps) continue;
+        if (4 * places < warps) return;
         const int64_t fixed = us::ahead_fixed_smem(nt, strips);
         auto slots_in = [&](int64_t bytes) { return (int32_t)std::min<int64_t>(most, std::max<int64_t>(0, bytes) / (int64_t)p.slot_bytes); };
         p.parked = (int32_t)std::min<int64_t>(most, 4 * places);
         p.n_slots = slots_in(kHalfSmBytes - fixed - x);
         p.x_over = p.parked == most && p.n_slots < std::min<int64_t>(most, warps) && fixed + x <= kHalfSmBytes ? 1 : 0;
         if (p.x_over) p.n_slots = slots_in(kHalfSmBytes - fixed);
-        if (p.n_slots < std::min<int64_t>(most, 6)) continue;
+        if (p.n_slots < std::min<int64_t>(most, least)) return;
         pl.smem = (int)(fixed + (p.x_over ? std::max<int64_t>(x, (int64_t)p.n_slots * p.slot_bytes) : x + (int64_t)p.n_slots * p.slot_bytes));
         std::copy(begin.begin(), begin.end(), p.cta_begin);
         p.n_ranges = (int32_t)r; p.G = (int32_t)G; p.s_local = strips;
-    }
-    if (p.n_ranges == 0) return;
+    };
+    auto fewest = [&](int slots, int ranges) {
+        least = slots;
+        for (int64_t r = 1; r <= ranges && p.n_ranges == 0; ++r) lay(r);
+        return p.n_ranges > 0;
+    };
+    const bool six = fewest(6, 8);
+    if (!six && !fewest(5, 8)) return;
     const int64_t share = most * hm.fmt.K_L / 1024;
     const bool more_ranges = p.n_ranges > 1 && h->s_local[cls] > 0 && h->G[cls] == hm.n_segs;   // than the other plan's one
-    const bool better = cls == 0   ? share <= (p.n_ranges > 1 || p.n_slots < 8 ? 40 : plain ? 64 : 46) && (hm.n_segs > 1 || most <= 8)
+    const bool better = !six       ? false
+                        : cls == 0 ? share <= (p.n_ranges > 1 || p.n_slots < 8 ? 40 : plain ? 64 : 46) && (hm.n_segs > 1 || most <= 8)
                         : cls == 1 ? share <= (more_ranges || (!plain && p.n_ranges > 1) ? 24 : plain ? 42 : 28)
                                    : p.parked == most;
-    if (ahead_knob() == 1 && !better) return;
+    const bool behind = (cls == 0 || (cls == 1 && plain)) && share <= 64 && h->plan[cls].g.smem > kHalfSmBytes && tc_knob() < 2;
+    if (ahead_knob() == 1 && !better && !behind) return;
+    if (!better && p.n_ranges > 1) {   // one range with five slots rather than more ranges
+        const int ranges = p.n_ranges, slots = least;
+        p.n_ranges = 0;
+        if (!fewest(5, 1)) { least = slots; lay(ranges); }
+    }
+    pl.always = better || ahead_knob() == 2;
     p.tm_cols = 32;
     while (p.tm_cols < (p.parked + 3) / 4 * p.tile_cols) p.tm_cols *= 2;
     p.blob = h->d_blob; p.item_off = h->d_item_off; p.row_order = h->d_row_order; p.w_scale = h->d_w_scale;
@@ -612,7 +635,7 @@ void build_ahead_plan(us_handle* h, int cls)
     pl.plain.symbol = symbol(false);
     pl.chained.symbol = symbol(true);
     pl.ok = true;
-    pl.chain_ok = p.parked == most;
+    pl.chain_ok = pl.always && p.parked == most;
 }
 
 // Loads a kernel, opted in to the device's full dynamic shared memory (once per device, with that device current), so that
@@ -697,13 +720,42 @@ us_status launch(us_handle* h, const Kernel& kernel, void* params, int threads, 
     return US_OK;
 }
 
+// The calling thread's last call: how many calls behind it on the stream take half an SM where they otherwise would not.
+// Two behind a call whose CTAs take half an SM anyhow, so that theirs can start beside them (a stacked [gate; up] and the down
+// projection behind it); such calls again and again go back to the whole SM. None where another kernel of the library, or a
+// clear, comes in between.
+struct LastCall {
+    int device = -1;
+    cudaStream_t stream = nullptr;
+    int beside = 0;
+};
+thread_local LastCall t_last;
+
+// The plan of us_spmm_ahead_kernel that a call on that stream takes, if any (see build_ahead_plan). timed: on the other
+// kernel's timer build.
+const AheadPlan* ahead_plan(const us_handle* h, int N, cudaStream_t st, bool chain, bool timed)
+{
+    const int cls = class_of(nt_for(N));
+    if (cls > 2 || !h->ahead[cls].ok) return nullptr;
+    const AheadPlan& a = h->ahead[cls];
+    if (chain) return a.chain_ok ? &a : nullptr;
+    if (timed && h->plan[cls].fn.timed.fn) return nullptr;
+    if (a.always) return h->tc[(N + 7) / 8].ok ? nullptr : &a;
+    return t_last.beside > 0 && t_last.stream == st && t_last.device == h->device ? &a : nullptr;
+}
+
 // The one launch path behind us_spmm, us_spmm_static_scratch and us_spmm_requant: fills the call's own
 // parameters into a copy of the class's plan and launches.
 us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_scale, void* Y, cudaStream_t st,
                        int32_t* acc, uint32_t* cnt, bool timers, const ChainArgs* chain = nullptr)
 {
+    const int cls = class_of(nt_for(N));
+    const ClassPlan& pl = h->plan[cls];
+    const AheadPlan* const ahead = ahead_plan(h, N, st, chain != nullptr, timers);
+    const bool half = ahead ? ahead->always : !h->tc[(N + 7) / 8].ok && pl.g.smem <= kHalfSmBytes;
+    t_last = {h->device, st, chain ? 0 : half ? 2 : ahead ? t_last.beside - 1 : 0};   // (behind a chained call a quantiser runs first)
     const TcPlan& tc = h->tc[(N + 7) / 8];
-    if (tc.ok) {
+    if (tc.ok && !ahead) {
         us::TcParams p = tc.p;
         p.X = static_cast<const uint8_t*>(X);
         p.x_scale = static_cast<const uint16_t*>(x_scale);
@@ -720,10 +772,8 @@ us_status enqueue_spmm(us_handle* h, const void* X, int32_t N, const void* x_sca
         if (!k.fn) return US_ERR_UNSUPPORTED;
         return launch(h, k, &p, tc.threads, tc.smem, st);
     }
-    const int cls = class_of(nt_for(N));
-    const ClassPlan& pl = h->plan[cls];
-    if (cls <= 2 && h->ahead[cls].ok && !(chain && !h->ahead[cls].chain_ok) && !(timers && !chain && pl.fn.timed.fn)) {   // (the stage timers are the other kernel's)
-        const AheadPlan& ah = h->ahead[cls];
+    if (ahead) {
+        const AheadPlan& ah = *ahead;
         us::AheadParams p = ah.p;
         p.X = static_cast<const uint8_t*>(X);
         p.x_scale = static_cast<const uint16_t*>(x_scale);
@@ -950,7 +1000,7 @@ us_status us_launch_info(const us_handle* h, int32_t N, int32_t* grid, int32_t* 
     const TcPlan& tc = h->tc[(N + 7) / 8];
     const int cls = class_of(nt_for(N));
     const ClassPlan& pl = h->plan[cls];
-    const AheadPlan* ah = cls <= 2 && h->ahead[cls].ok ? &h->ahead[cls] : nullptr;
+    const AheadPlan* ah = cls <= 2 && h->ahead[cls].always ? &h->ahead[cls] : nullptr;
     if (!tc.ok && !ah && !pl.ok) return US_ERR_UNSUPPORTED;
     if (grid) *grid = h->sm_count;
     if (block) *block = tc.ok ? tc.threads : ah ? ah->threads : pl.g.warps * 32;
@@ -958,11 +1008,12 @@ us_status us_launch_info(const us_handle* h, int32_t N, int32_t* grid, int32_t* 
     return US_OK;
 }
 
-const char* us_launch_kernel(const us_handle* h, int32_t N)
+const char* us_launch_kernel(const us_handle* h, int32_t N, void* stream)
 {
     if (us_launch_info(h, N, nullptr, nullptr, nullptr) != US_OK) return nullptr;
-    const int cls = class_of(nt_for(N));
-    return h->tc[(N + 7) / 8].ok ? "us_spmm_tc_kernel" : cls <= 2 && h->ahead[cls].ok ? "us_spmm_ahead_kernel" : "us_spmm_kernel";
+    return ahead_plan(h, N, static_cast<cudaStream_t>(stream), false, false) ? "us_spmm_ahead_kernel"
+           : h->tc[(N + 7) / 8].ok                                             ? "us_spmm_tc_kernel"
+                                                                               : "us_spmm_kernel";
 }
 
 us_status us_spmm(us_handle* h, const void* X, int32_t N, const void* x_scale, void* Y, void* stream)
@@ -1008,6 +1059,7 @@ us_status us_spmm_static_scratch(us_handle* h, const void* X, int32_t N, const v
     // The array keeps the previous call's contents: sums and counters must start at zero.
     const cudaError_t e = cudaMemsetAsync(scratch, 0, acc_bytes + cnt_bytes, st);
     if (e != cudaSuccess) { h->sticky = e; return US_ERR_CUDA; }
+    t_last.beside = 0;
     return enqueue_spmm(h, X, N, x_scale, Y, st, reinterpret_cast<int32_t*>(scratch),
                         reinterpret_cast<uint32_t*>(scratch + acc_bytes), false);
 }
@@ -1018,6 +1070,7 @@ cudaError_t launch_quantize(const uint16_t* X16, int64_t ldx, int32_t N, int64_t
                             uint16_t* x_scale, cudaStream_t st)
 {
     const int64_t units = (K + 7) / 8;
+    t_last.beside = 0;
     const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(64, (units + 255) / 256)), (unsigned)N);
     return launch_small(us::us_quantize_f16_kernel, grid, st, X16, ldx, K, amax, Xq, x_scale);
 }
@@ -1059,6 +1112,7 @@ us_status us_absmax_f16(const void* X16, int64_t ldx, int32_t N, int64_t K, void
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int64_t units = (K + 7) / 8;
     const unsigned gx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(16, (units + 255) / 256));
+    t_last.beside = 0;
     const cudaError_t e = launch_small(us::us_absmax_f16_kernel, dim3(gx, (unsigned)N), st, static_cast<const uint16_t*>(X16), ldx, K,
                                        (int)N, static_cast<uint32_t*>(amax));
     if (e != cudaSuccess) { cudaGetLastError(); return US_ERR_CUDA; }

@@ -165,3 +165,54 @@ def test_time_of_earlier_work_is_not_counted_against_a_wait():
     finally:
         for sw in sws:
             sw.close()
+
+
+@pytest.mark.parametrize("M,K,s", [(20480, 5120, 0.5), (27648, 5120, 0.5),     # 45 and 59 tiles to a CTA, six and five slots
+                                   (8192, 8192, 0.5), (8200, 8191, 0.5)])      # K in ranges where the other kernel has one; ragged rows
+def test_call_that_follows_its_neighbour_to_half_an_sm(M, K, s):
+    """Behind a call of half an SM on the same stream the call takes half an SM itself, twice running; on another stream, behind
+    another kernel of the library or a clear it does not. The sums are the same in both forms."""
+    from paper_2608_09291_b200 import binding as b
+    N = 16
+    W, (s_w, s_x) = workloads.make_weight(M, K, s, seed=M), workloads.make_scales(M, N, seed=K)
+    X = workloads.make_x(K, N, seed=K)
+    sw = b.SparseWeight(W, s_w, max_N=N)
+    small = b.SparseWeight(workloads.make_weight(2048, 2048, 0.5, seed=1), workloads.make_chain_weight_scales(2048, 2048, 1), max_N=N)
+    other = torch.cuda.Stream()
+    try:
+        Xd, xs = torch.from_numpy(b.pack_int4(X)).cuda(), torch.from_numpy(s_x.copy()).cuda()
+        Zd = torch.from_numpy(b.pack_int4(workloads.make_x(2048, N, seed=2))).cuda()
+        z16 = torch.from_numpy(workloads.make_x_f16(2048, N, seed=3)).cuda()
+        amax = b.absmax_f16(z16)
+        out = torch.empty((N, 2048), dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+
+        def kernel(stream=None):
+            return b.us_launch_kernel(sw.handle, N, stream)
+
+        ref = torch.from_numpy(oracle.spmm_dense(W, X)).cuda()
+        assert kernel() == "us_spmm_kernel"
+        first = sw.spmm(Xd, N, xs)
+        for _ in range(3):
+            assert torch.equal(sw.spmm(Xd, N), ref)
+            small.spmm(Zd, N, out=out)
+            assert kernel() == "us_spmm_ahead_kernel" and kernel(other.cuda_stream) == "us_spmm_kernel"
+            assert torch.equal(sw.spmm(Xd, N), ref)
+            assert kernel() == "us_spmm_ahead_kernel"
+            assert torch.equal(sw.spmm(Xd, N, xs), first)
+            assert kernel() == "us_spmm_kernel"
+            assert torch.equal(sw.spmm(Xd, N), ref)
+            for between in (lambda: small.spmm_requant(z16, N, amax), lambda: b.quantize_f16(z16, amax), lambda: b.absmax_f16(z16)):
+                small.spmm(Zd, N, out=out)
+                between()
+                assert kernel() == "us_spmm_kernel"
+            small.spmm(Zd, N, out=out)
+            y = torch.empty_like(ref)
+            b.us_spmm_static_scratch(sw.handle, Xd.data_ptr(), N, None, y.data_ptr())
+            assert kernel() == "us_spmm_kernel" and torch.equal(y, ref)
+        sw.check()
+        small.check()
+        assert oracle.fp16_within_tolerance(first.cpu().numpy(), ref.cpu().numpy(), s_w, s_x).all()
+    finally:
+        sw.close()
+        small.close()
