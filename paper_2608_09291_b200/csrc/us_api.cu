@@ -463,8 +463,10 @@ void build_tc_plan(us_handle* h, int ng)
     //            21.6 / 21.0, 20480 x 8192 26.0 / 23.3), from 10 stages on and with 1.6 us of margin: among other launches its code
     //            comes from L2 each time (a 13B-shaped chain with 27648 x 5120 on this kernel 74.3, on the other 72.2).
     //   N <= 32: 5.5 + 1.76 share, 7.5 + 1.1 mean (11008 x 4096 13.6 / 13.1, 4096 x 11008 14.7 / 12.3, 13824 x 5120 19.2 / 15.9,
-    //            2048 x 8192 8.2 / 8.8), a us of margin, with INT2 weights 2.5 (11008 x 4096 11.8 / 12.4, 13824 x 5120 16.2 / 14.8). Tiles of
-    //            uneven size leave it fewer slots (4096 x 11008, rows sorted, largest tile 1.3 times the average, 15.3 / 15.6).
+    //            2048 x 8192 8.2 / 8.8), a us of margin, with INT2 weights 2.5 (11008 x 4096 11.8 / 12.4, 13824 x 5120 16.2 / 14.8). Where the
+    //            order of the rows was changed its stores scatter, 7 us more here and 3 on a plan with one K range: 4 us of margin against those, 1.2 in ranges
+    //            (rows sorted, densities .3 to .7: 11008 x 4096 16.2 / 20.9, 12288 x 4096 18.0 / 21.2, 16384 x 4096 21.7 / 23.3; in ranges 4096 x
+    //            11008 19.5 / 19.5, with the weights in L2 15.3 / 15.7, at N = 20 17.0 / 15.5, 8192 x 8192 26.8 / 22.2; with .4 to .6 and .2 to .5 the same).
     //   N <= 64: from 2048 columns on (2048 x 2048 10.3 / 9.6, 4096 x 4096 16.6 / 14.2, 11008 x 4096 35 / 17.4), below that where
     //            CTAs have most of a stage (16384 x 512 19.3 / 16.0; 4096 x 1024, 0.4 stages, 8.8 / 9.7).
     // Against the direct mode it wins nearly always (N = 64 28672 x 8192 92 / 38).
@@ -472,12 +474,15 @@ void build_tc_plan(us_handle* h, int ng)
     uint32_t most = 0;
     for (size_t c = 0; c + 1 < h->cta_begin[cls].size(); ++c) most = std::max(most, h->cta_begin[cls][c + 1] - h->cta_begin[cls][c]);
     const double mean = (double)stages / (double)n_cta, share = (double)most * n_stage / 16;
-    const double uneven = (double)hm.max_item_bytes * (double)hm.n_items / (double)std::max<uint64_t>(1, hm.blob_bytes);   // largest tile / average
+    bool scattered = false;   // a strip's rows are not one run of output rows
+    for (int64_t i = 0; i + 16 <= hm.M && !scattered; i += 16)
+        for (int64_t j = i; j < i + 16; ++j) scattered = scattered || hm.row_order[j] < i || hm.row_order[j] >= i + 16;
+    const double margin = !scattered ? 0.0 : h->s_local[cls] > 0 && h->G[cls] == hm.n_segs ? 4.0 : 1.2;
     const bool better = cls <= 2 && h->ahead[cls].always ? false
                         : ng > 4                     ? hm.Kp >= 2048 || mean >= 0.8
                         : h->s_local[cls] == 0       ? mean >= 1.5
                         : ng <= 2                    ? mean >= 10 && 5.9 + 1.08 * share > 9.4 + 0.9 * mean
-                                                     : 5.5 + 1.76 * share > (hm.w2 ? 10.0 : 8.5) + 1.1 * mean + 12 * std::max(0.0, uneven - 1.1);
+                                                     : 5.5 + 1.76 * share > (hm.w2 ? 10.0 : 8.5) + 1.1 * mean + margin;
     if (tc_knob() == 0 || (tc_knob() == 1 && !better)) return;
     p.slot_bytes = slot_bytes_for(hm);
     const int limit = h->max_smem;

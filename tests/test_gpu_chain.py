@@ -2,6 +2,11 @@
 codes, steps and absmax words are integers decided in fp32 on both sides: they must agree bit for
 bit. The fp16 outputs are checked stage by stage from the device's own previous output, within
 max(2e-3 relative, 1 fp16 ulp) of the exactly rounded reference."""
+import os
+import subprocess
+import sys
+from pathlib import Path
+
 import numpy as np
 import pytest
 
@@ -11,6 +16,7 @@ from paper_2608_09291_b200 import workloads
 pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
+ROOT = Path(__file__).resolve().parent.parent
 
 
 @pytest.fixture(scope="module")
@@ -180,18 +186,14 @@ def test_layer_13b_chain(b, j, s):
             m["sw"].close()
 
 
-@pytest.mark.parametrize("M,K,fmt,warps", [(2048, 2048, None, 12),                    # local mode
-                                           (11500, 1000, (16, 512, 2, 1), 12),        # local mode, one range of two segments
-                                           (24000, 1024, None, 11),                   # direct mode, 11 tiles per CTA
-                                           (4001, 2500, (16, 512, 2, 2), 10)])        # two column areas, K no multiple of 32
-def test_half_sm_plan_counts_the_registers_of_every_kernel(b, M, K, fmt, warps):
-    """Plain, single-token and chained calls are different kernels under one plan: its warps are what two CTAs of each of
-    them share an SM with (2048 x 2048 had 11 while the direct mode's kernel was counted and the chained one was not)."""
+def run_half_sm_plan(M, K, fmt, warps):
+    from paper_2608_09291_b200 import binding as b
     W = workloads.make_weight(M, K, 0.5, seed=M + K)
     s_w = workloads.make_chain_weight_scales(M, K, 5)
     sw = b.SparseWeight(W, s_w, fmt=fmt, max_N=8)
     try:
         info = b.us_launch_info(sw.handle, 8)
+        assert b.us_launch_kernel(sw.handle, 8) == "us_spmm_kernel"
         assert info["smem_bytes"] <= 114 * 1024 and info["block"] == 32 * warps, info
         X = workloads.make_x(K, 8, seed=1)
         ref = oracle.spmm_dense(W, X)
@@ -203,6 +205,20 @@ def test_half_sm_plan_counts_the_registers_of_every_kernel(b, M, K, fmt, warps):
             _check_requant_call(b, sw, W, s_w, workloads.make_x_f16(K, 8, seed=2), 8, 0, M)
     finally:
         sw.close()
+
+
+@pytest.mark.parametrize("M,K,fmt,warps", [(2048, 2048, None, 10),                    # local mode
+                                           (10000, 1000, (16, 512, 2, 1), 10),        # local mode, one range of two segments, 10 tiles per CTA
+                                           (24000, 1024, None, 11),                   # direct mode, 11 tiles per CTA
+                                           (4001, 2500, (16, 512, 2, 2), 10)])        # two column areas, K no multiple of 32
+def test_half_sm_plan_counts_the_registers_of_every_kernel(M, K, fmt, warps):
+    """Plain, single-token and chained calls are different kernels under one plan: its warps are what two CTAs of each of
+    them share an SM with (10 in local mode, whose kernels take 81 to 96 registers since a mask word's activations are one load;
+    12 fit 80. 11500 x 1000, 12 tiles per CTA, has the whole SM so). The plan is us_spmm_kernel's: a child process keeps
+    the decode-ahead kernel off these shapes."""
+    code = f"import sys; sys.path[:0] = ['.', 'tests']; import test_gpu_chain; test_gpu_chain.run_half_sm_plan({M}, {K}, {fmt}, {warps})"
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, US_AHEAD="0"), capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout[-1500:] + r.stderr[-1500:]
 
 
 @pytest.mark.parametrize("M,K,fmt,N", [(1024, 1024, None, 8), (2048, 4096, None, 16), (2048, 2048, None, 32),   # resident beside two launches
